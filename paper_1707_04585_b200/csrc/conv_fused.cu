@@ -279,7 +279,7 @@ conv_fused_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_consta
     FusedShared *sh = (FusedShared *)(outb + p.aux_bytes);
     ItemRef *tab = (ItemRef *)(sh + 1);
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_index();
     const int etid = threadIdx.x & 127;                 // warps 0-3: accumulator row; all warps: index for the reductions
     const int cshift = p.KC == 64 ? 3 : (p.KC == 32 ? 2 : 1);     // 16-byte chunks per pixel = KC / 8
     const int pad = p.k >> 1;
@@ -416,21 +416,23 @@ conv_fused_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_consta
         }
         fence_proxy_async();
         __syncthreads();
-        if (threadIdx.x == 0) {
-            if (p.NB == 1 && nx1.t < NT) load_raw(nx1, 0);        // the raw buffer is free again
-            if (ti == 0 && !mbar_wait(&sh->w_full, 0)) ok = false;
-            tc_fence_after();
-            const uint32_t idesc = instr_desc(p.BN);
-            const int n_mma = taps * (p.KC >> 4);
-            const ulonglong2 *dsc = reinterpret_cast<const ulonglong2 *>(sh->desc);
-#pragma unroll 4
-            for (int i = 0; i < n_mma; i++) {
-                const ulonglong2 d = dsc[i];
-                mma_bf16(tmem_d, d.x, d.y, idesc, i ? 1u : 0u);
+        if (warp == 0) {
+            if (elect_one()) {
+                if (p.NB == 1 && nx1.t < NT) load_raw(nx1, 0);        // the raw buffer is free again
+                if (ti == 0 && !mbar_wait(&sh->w_full, 0)) ok = false;
+                tc_fence_after();
+                const uint32_t idesc = instr_desc(p.BN);
+                const int n_mma = taps * (p.KC >> 4);
+                const ulonglong2 *dsc = reinterpret_cast<const ulonglong2 *>(sh->desc);
+    #pragma unroll 4
+                for (int i = 0; i < n_mma; i++) {
+                    const ulonglong2 d = dsc[i];
+                    mma_bf16(tmem_d, d.x, d.y, idesc, i ? 1u : 0u);
+                }
+                mma_commit(&sh->mma_done);
+                tma_store_wait_read();                       // the previous tile's store has read the output buffer
+                ok = ok && mbar_wait(&sh->mma_done, ti & 1) && (!need_aux || mbar_wait(&sh->aux_full[b], u & 1));
             }
-            mma_commit(&sh->mma_done);
-            tma_store_wait_read();                       // the previous tile's store has read the output buffer
-            ok = ok && mbar_wait(&sh->mma_done, ti & 1) && (!need_aux || mbar_wait(&sh->aux_full[b], u & 1));
         }
         else if (threadIdx.x == 32 && p.NB == 2) {
             // meanwhile another thread issues the loads of the tiles ahead: this tile's raw buffer has been consumed,
@@ -460,7 +462,7 @@ conv_fused_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_consta
         fence_proxy_async();
         tc_fence_before();       // the next tile's MMAs overwrite the accumulator
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (warp == 0 && elect_one()) {
             for (int g = 0; g < p.BN / p.GW; g++) tma_store_4d(&map_out, outb + g * p.group_bytes, col0 + g * p.GW, 0, h0, n0);
             tma_store_commit();
         }
@@ -488,7 +490,7 @@ conv_fused_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_consta
         cur = nx1; nx1 = nx2;
         tile_next(p.g, step, G, nx2);
     }
-    if (threadIdx.x == 0) tma_store_wait_all();
+    if (warp == 0 && elect_one()) tma_store_wait_all();
     if (ok && e.part) {
         // per-CTA record: the threads that share a channel quad are added in order
         float *scratch = reinterpret_cast<float *>(abuf);

@@ -170,7 +170,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     float *gsums = (float *)(outr + 2 * p.group_bytes);
     TcShared *sh = p.epi_tma ? (TcShared *)(gsums + ng * 128 * 8) : (TcShared *)((uint8_t *)estage + kEpiStageBytes + kEpiSumFloats * 4);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int n_vt = p.n_cls * p.g.n_px_tiles;     // tiles of all classes
     uint32_t tmem_cols = 32;
     while ((int)tmem_cols < 2 * p.BN) tmem_cols <<= 1;
@@ -199,7 +199,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     // clocks.  So no divisions, no table look-ups and no descriptor construction inside them: the ring position is
     // stepped, tap data is read once per tap, descriptors are a base plus increments of the address field.
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             int s = 0; uint32_t round = 0;
             bool ok = true;
             const uint32_t tx = (uint32_t)(a_bytes + b_bytes);
@@ -223,7 +223,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = instr_desc(p.BN);
             const int row_bytes = p.KC * 2, nk = p.KC >> 4;
             const uint64_t da0 = smem_desc(smem_u32(tiles), row_bytes), db0 = smem_desc(smem_u32(tiles) + b_off, row_bytes);
@@ -440,7 +440,7 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     float *gsums = (float *)(outr + 2 * p.group_bytes);
     TcShared *sh = (TcShared *)(gsums + ng * 128 * 8);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const int pair = (int)blockIdx.x >> 1, n_pairs = (int)gridDim.x >> 1;
     const int n_pp = (p.g.n_px_tiles + 1) >> 1;                  // tile pairs per class
@@ -474,7 +474,7 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 
     // (single-thread loops kept lean, as in conv_tc_kernel)
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             int s = 0, as = 0; uint32_t round = 0, ar = 0;
             bool ok = true;
             const uint32_t full0 = mapa_shared(smem_u32(&sh->full[0]), 0), afull0 = mapa_shared(smem_u32(&sh->afull[0]), 0);   // the leader's barriers
@@ -517,7 +517,7 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             const uint32_t idesc = instr_desc_m256(p.BN);
             const int row_bytes = p.KC * 2, nk = p.KC >> 4;
             const uint64_t da0 = smem_desc(smem_u32(tiles), row_bytes), db0 = smem_desc(smem_u32(tiles) + b_off, row_bytes);
@@ -1114,7 +1114,7 @@ wgrad_tc_kernel(const __grid_constant__ WgBatch batch) {
     const int stage_bytes = a_region + ((256 * p.BN + 1023) & ~1023);
     TcShared *sh = (TcShared *)(tiles + p.stages * stage_bytes);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int bpg = 128 / p.blockC;                          // blocks per M group
     const int first_block = chunk * p.GM * bpg;
     int n_blocks = p.total_blocks - first_block; if (n_blocks > p.GM * bpg) n_blocks = p.GM * bpg;
@@ -1179,7 +1179,7 @@ wgrad_tc_kernel(const __grid_constant__ WgBatch batch) {
             if (++s == p.stages) { s = 0; round++; }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = instr_desc(p.BN, true);
             const int rba = p.blockC * 2, rbb = p.blockN * 2;
             // one thread issues everything: descriptors are a base plus increments of the address field (16-byte units),
@@ -1281,7 +1281,7 @@ wgrad_tc2_kernel(const __grid_constant__ WgBatch batch) {
     const int stage_bytes = a_region + ((256 * p.BN + 1023) & ~1023);
     TcShared *sh = (TcShared *)(tiles + p.stages * stage_bytes);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int bpg = 128 / p.blockC;                          // blocks per 128-row group
     const int first_block = chunk * 2 * p.GM * bpg;          // the pair's chunk: 2 * GM groups
     // blocks this CTA / the other CTA loads per pixel tile: group 2j + r holds the blocks first_block + (2j + r) * bpg ...
@@ -1348,7 +1348,7 @@ wgrad_tc2_kernel(const __grid_constant__ WgBatch batch) {
             if (++s == p.stages) { s = 0; round++; }
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             const uint32_t idesc = instr_desc_m256(2 * p.BN) | (3u << 15);     // both operands M / N-major
             const int rba = p.blockC * 2, rbb = p.blockN * 2;
             const uint64_t da0 = smem_desc_mn(smem_u32(tiles), rba, blk_bytes_a), db0 = smem_desc_mn(smem_u32(tiles) + a_region, rbb, blk_bytes_b);
