@@ -203,16 +203,19 @@ extern "C" int revnet_pack_weights(revnet_ctx *ctx, const revnet_block_desc *d, 
     char *at = (char *)pack_buffer;
     revnet_fn_params *ps[2] = {Fp, Gp};
     const revnet_fn_desc *fs[2] = {&d->F, &d->G};
+    PackJobs list;
+    int n = 0;
     for (int i = 0; i < 2; i++)
         for (int l = 0; l < 3; l++) {
             ps[i]->Wpack_fprop[l] = ps[i]->Wpack_dgrad[l] = nullptr;
             if (l >= fs[i]->n_layers || !packable(d, *fs[i], l)) continue;
             for (int tr = 0; tr < 2; tr++) {
-                tc_pack_now(ex, ps[i]->W[l], (bf16 *)at, fs[i]->cin[l], fs[i]->cout[l], fs[i]->k[l], tr != 0);
                 (tr ? ps[i]->Wpack_dgrad[l] : ps[i]->Wpack_fprop[l]) = at;
                 at += (tc_pack_elems(fs[i]->cin[l], fs[i]->cout[l], fs[i]->k[l], tr != 0) * sizeof(bf16) + 255) & ~size_t(255);
             }
+            list.job[n++] = tc_pack_job(ps[i]->W[l], (bf16 *)ps[i]->Wpack_fprop[l], (bf16 *)ps[i]->Wpack_dgrad[l], fs[i]->cin[l], fs[i]->cout[l], fs[i]->k[l]);
         }
+    tc_pack_list(ex, list, n);
     return finish(ctx, ex, "revnet_pack_weights");
 }
 

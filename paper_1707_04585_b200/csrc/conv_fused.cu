@@ -424,7 +424,7 @@ conv_fused_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_consta
                 const uint32_t idesc = instr_desc(p.BN);
                 const int n_mma = taps * (p.KC >> 4);
                 const ulonglong2 *dsc = reinterpret_cast<const ulonglong2 *>(sh->desc);
-    #pragma unroll 4
+#pragma unroll 4
                 for (int i = 0; i < n_mma; i++) {
                     const ulonglong2 d = dsc[i];
                     mma_bf16(tmem_d, d.x, d.y, idesc, i ? 1u : 0u);

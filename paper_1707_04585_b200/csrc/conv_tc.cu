@@ -732,65 +732,60 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     }
 }
 
-// ---- weight packs: bf16 [rows_pad][taps][cin_pad]; transposed = true builds the dgrad operand
-// (rows = input channels, columns = output channels, taps mirrored)
-__global__ void pack_weights_kernel(const float *__restrict__ W, bf16 *__restrict__ out, int Co, int Ci, int k,
-                                    int rows_pad, int cols_pad, int transposed) {
-    pdl_enter();
-    const int taps = k * k;
-    const size_t n = (size_t)rows_pad * taps * cols_pad;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % cols_pad);
-        const int tap = (int)((i / cols_pad) % taps);
-        const int r = (int)(i / ((size_t)cols_pad * taps));
-        float v = 0.f;
-        if (!transposed) { if (r < Co && c < Ci) v = W[((size_t)r * taps + tap) * Ci + c]; }
-        else { if (r < Ci && c < Co) v = W[((size_t)c * taps + (taps - 1 - tap)) * Ci + r]; }
-        out[i] = __float2bfloat16_rn(v);
+// ---- weight packs (see PackJob).  Bound by HBM: each weight is read once and written to both packs.  A block of 256
+// threads takes tiles of 64 output x 64 input channels of one tap: 256-byte reads, 128-byte writes to either pack, the
+// transposed one through shared memory; consecutive tiles walk the weights in memory order.
+// Measured: a 75 M weight layer 638 -> 87 us per pack (one element per thread and uncoalesced reads of the transposed pack
+// before); a block's eight launches are one; all packs of a step, each weight read once instead of twice: large-image step 68.9 -> 67.9 ms.
+constexpr int kPackTile = 64;
+__device__ __forceinline__ uint2 pack_bf16x4(float a, float b, float c, float d) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
+    return make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+}
+__host__ __device__ __forceinline__ int pack_ct(const PackJob &j) { const int n = j.ci_f > j.ci_d ? j.ci_f : j.ci_d; return (n + kPackTile - 1) / kPackTile; }
+__host__ __device__ __forceinline__ int pack_rt(const PackJob &j) { const int n = j.co_f > j.co_d ? j.co_f : j.co_d; return (n + kPackTile - 1) / kPackTile; }
+__device__ __forceinline__ void pack_layer(const PackJob &j, int first, int step) {
+    __shared__ float tile[kPackTile][kPackTile + 1];
+    const int taps = j.k * j.k, ct = pack_ct(j), n_tiles = ct * taps * pack_rt(j);
+    const int lx = threadIdx.x & 15, ly = threadIdx.x >> 4;
+    for (int t = first; t < n_tiles; t += step) {
+        const int ci0 = (t % ct) * kPackTile, tap = (t / ct) % taps, co0 = t / (ct * taps) * kPackTile;
+        const int ci = ci0 + 4 * lx;
+        float4 v[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int co = co0 + ly + 16 * i;
+            v[i] = (co < j.Co && ci < j.Ci) ? *reinterpret_cast<const float4 *>(j.W + ((size_t)co * taps + tap) * j.Ci + ci) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int co = co0 + ly + 16 * i;
+            if (j.f && co < j.co_f && ci < j.ci_f)
+                *reinterpret_cast<uint2 *>(j.f + ((size_t)co * taps + tap) * j.ci_f + ci) = pack_bf16x4(v[i].x, v[i].y, v[i].z, v[i].w);
+            if (j.d) { float *r = tile[ly + 16 * i] + 4 * lx; r[0] = v[i].x; r[1] = v[i].y; r[2] = v[i].z; r[3] = v[i].w; }
+        }
+        if (!j.d) continue;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            // rows of this pack are input channels, columns output channels, taps mirrored
+            const int r = ly + 16 * i, c = co0 + 4 * lx;
+            if (ci0 + r < j.ci_d && c < j.co_d)
+                *reinterpret_cast<uint2 *>(j.d + ((size_t)(ci0 + r) * taps + (taps - 1 - tap)) * j.co_d + c) =
+                    pack_bf16x4(tile[4 * lx][r], tile[4 * lx + 1][r], tile[4 * lx + 2][r], tile[4 * lx + 3][r]);
+        }
+        __syncthreads();
     }
 }
-
-// all packs of a step in one launch: blockIdx.y walks the job table.  A block (32 x 8 threads) takes tiles of
-// 32 rows x 64 columns of the pack (one tap), a thread two adjacent columns: the fp32 reads of a warp are contiguous
-// (256 bytes plain, 128 bytes transposed) and so are its bf16x2 writes (128 bytes); the transposed pack goes through
-// shared memory.
-__global__ void pack_weights_batch_kernel(const PackJob *__restrict__ jobs) {
+// every layer of a step (table in device memory) / of a block or a single layer (table by value); blockIdx.y picks the layer
+__global__ void __launch_bounds__(256) pack_weights_batch_kernel(const PackJob *__restrict__ jobs) {
     pdl_enter();
-    __shared__ float tile[64][33];
     const PackJob j = jobs[blockIdx.y];
-    const int taps = j.k * j.k;
-    const int rt = (j.rows_pad + 31) >> 5, ct = (j.cols_pad + 63) >> 6;
-    const int n_tiles = taps * rt * ct;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-        const int c0 = (t % ct) << 6, r0 = ((t / ct) % rt) << 5, tap = t / (ct * rt);
-        if (!j.transposed) {
-#pragma unroll
-            for (int rr = 0; rr < 32; rr += 8) {
-                const int r = r0 + rr + ty, c = c0 + 2 * tx;      // columns are input channels (a multiple of 4: c and c + 1 are valid together)
-                if (r < j.rows_pad && c < j.cols_pad) {
-                    float2 v = make_float2(0.f, 0.f);
-                    if (r < j.Co && c < j.Ci) v = *reinterpret_cast<const float2 *>(j.W + ((size_t)r * taps + tap) * j.Ci + c);
-                    *reinterpret_cast<__nv_bfloat162 *>(j.out + ((size_t)r * taps + tap) * j.cols_pad + c) = __floats2bfloat162_rn(v.x, v.y);
-                }
-            }
-        } else {
-            // rows of the pack are input channels, columns output channels, taps mirrored
-#pragma unroll
-            for (int cc = 0; cc < 64; cc += 8) {
-                const int co = c0 + cc + ty, ci = r0 + tx;
-                tile[cc + ty][tx] = (co < j.Co && ci < j.Ci) ? j.W[((size_t)co * taps + (taps - 1 - tap)) * j.Ci + ci] : 0.f;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int rr = 0; rr < 32; rr += 8) {
-                const int r = r0 + rr + ty, c = c0 + 2 * tx;
-                if (r < j.rows_pad && c < j.cols_pad)
-                    *reinterpret_cast<__nv_bfloat162 *>(j.out + ((size_t)r * taps + tap) * j.cols_pad + c) = __floats2bfloat162_rn(tile[2 * tx][rr + ty], tile[2 * tx + 1][rr + ty]);
-            }
-            __syncthreads();
-        }
-    }
+    pack_layer(j, blockIdx.x, gridDim.x);
+}
+__global__ void __launch_bounds__(256) pack_weights_kernel(const __grid_constant__ PackJobs jobs) {
+    pdl_enter();
+    pack_layer(jobs.job[blockIdx.y], blockIdx.x, gridDim.x);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
@@ -969,11 +964,8 @@ bool run_conv_tc(Exec &ex, const char *what, const void *act, Geom gin, int cin,
         EncodeTiledFn enc = encoder(ex.ctx);
         // without a pack made earlier in the step, build it from the fp32 master weights now
         if (!prepacked) {
-            const size_t n = (size_t)rows_pad * taps * s.cin_pad;
-            int grid = (int)((n + 255) / 256); if (grid > ex.ctx->sm_count * 4) grid = ex.ctx->sm_count * 4;
-            if (!transposed) launch(ex, pack_weights_kernel, grid, 256, 0, Wsrc, wp, cout, cin, k, rows_pad, s.cin_pad, 0);
-            else launch(ex, pack_weights_kernel, grid, 256, 0, Wsrc, wp, cin, cout, k, rows_pad, s.cin_pad, 1);
-            ex.check("pack_weights", (double)n * 6);
+            // (the pack's own sizes are those of tc_pack_elems: rows rounded up to its 128-row blocks, columns to 16)
+            tc_pack_now(ex, Wsrc, wp, transposed ? cout : cin, transposed ? cin : cout, k, transposed);
         }
         CUtensorMap map_a, map_b;
         const CUtensorMapSwizzle sw = s.KC == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : (s.KC == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
@@ -1705,12 +1697,9 @@ void *tc_encoder(revnet_ctx *ctx) { return (void *)encoder(ctx); }
 
 // pack of one layer built on the spot (calls that have no step-level pack)
 void tc_pack_now(Exec &ex, const float *W, bf16 *out, int cin, int cout, int k, bool transposed) {
-    if (ex.dry) return;
-    const PackJob j = tc_pack_job(W, out, cin, cout, k, transposed);
-    const size_t n = (size_t)j.rows_pad * k * k * j.cols_pad;
-    int grid = (int)((n + 255) / 256); if (grid > ex.ctx->sm_count * 4) grid = ex.ctx->sm_count * 4;
-    launch(ex, pack_weights_kernel, grid, 256, 0, W, out, cout, cin, k, j.rows_pad, j.cols_pad, transposed ? 1 : 0);
-    ex.check("pack_weights", (double)n * 6);
+    PackJobs list;
+    list.job[0] = tc_pack_job(W, transposed ? nullptr : out, transposed ? out : nullptr, cin, cout, k);
+    tc_pack_list(ex, list, 1);
 }
 
 // ---- packs made once per step (the train step calls these before the forward pass)
@@ -1724,18 +1713,28 @@ size_t tc_pack_elems(int cin, int cout, int k, bool transposed) {
     if (!transposed) pack_dims(cout, cin, rp, cp); else pack_dims(cin, cout, rp, cp);
     return (size_t)rp * k * k * cp;
 }
-PackJob tc_pack_job(const float *W, bf16 *out, int cin, int cout, int k, bool transposed) {
-    PackJob j;
-    j.W = W; j.out = out; j.Co = cout; j.Ci = cin; j.k = k; j.transposed = transposed ? 1 : 0;
-    if (!transposed) pack_dims(cout, cin, j.rows_pad, j.cols_pad); else pack_dims(cin, cout, j.rows_pad, j.cols_pad);
+PackJob tc_pack_job(const float *W, bf16 *f, bf16 *d, int cin, int cout, int k) {
+    PackJob j{W, f, d, cout, cin, k, 0, 0, 0, 0};
+    if (f) pack_dims(cout, cin, j.co_f, j.ci_f);
+    if (d) pack_dims(cin, cout, j.ci_d, j.co_d);
     return j;
 }
-void tc_pack_batch(Exec &ex, const PackJob *jobs_dev, int n_jobs, double bytes, size_t max_job_elems) {
+int tc_pack_tiles(const PackJob &j) { return pack_ct(j) * pack_rt(j) * j.k * j.k; }
+static double pack_job_bytes(const PackJob &j) {
+    return (double)j.Co * j.Ci * j.k * j.k * 4 + 2.0 * j.k * j.k * ((double)j.co_f * j.ci_f + (double)j.ci_d * j.co_d);
+}
+// blocks per layer sized for the largest one, at most eight per SM
+void tc_pack_batch(Exec &ex, const PackJob *jobs_dev, int n_jobs, double bytes, int max_tiles) {
     if (ex.dry || n_jobs == 0) return;
-    // blocks per job sized for the largest job (two 32 x 64 tiles per block), within 2 .. 592
-    size_t bx = (max_job_elems + 4095) / 4096;
-    if (bx < 2) bx = 2; if (bx > 592) bx = 592;
-    dim3 grid((unsigned)bx, (unsigned)n_jobs);
-    launch(ex, pack_weights_batch_kernel, grid, dim3(32, 8), 0, jobs_dev);
+    const int cap = ex.ctx->sm_count * 8;
+    launch(ex, pack_weights_batch_kernel, dim3((unsigned)(max_tiles < cap ? max_tiles : cap), (unsigned)n_jobs), 256, 0, jobs_dev);
     ex.check("pack_weights_batch", bytes);
+}
+void tc_pack_list(Exec &ex, const PackJobs &jobs, int n_jobs) {
+    if (ex.dry || n_jobs == 0) return;
+    int tiles = 1; double bytes = 0;
+    for (int i = 0; i < n_jobs; i++) { const int t = tc_pack_tiles(jobs.job[i]); if (t > tiles) tiles = t; bytes += pack_job_bytes(jobs.job[i]); }
+    const int cap = ex.ctx->sm_count * 8;
+    launch(ex, pack_weights_kernel, dim3((unsigned)(tiles < cap ? tiles : cap), (unsigned)n_jobs), 256, 0, jobs);
+    ex.check("pack_weights", bytes);
 }

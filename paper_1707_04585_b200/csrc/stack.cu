@@ -3,6 +3,7 @@
 // place on it in the forward pass, and Algorithm 1 walks it back in place in the backward pass,
 // so the activation footprint does not depend on the number of units.
 #include "common.cuh"
+#include <algorithm>
 #include <utility>
 #include <string.h>
 #include <array>
@@ -109,25 +110,23 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
         }
         std::vector<PackJob> jobs;
         double bytes = 0;
-        size_t max_elems = 0;
+        int max_tiles = 0;
         for (LayerSlot *l : slots) {
             l->wp_f = l->wp_d = nullptr;
             if (ex.mode != 0 || l->cin % 8 || l->cout % 8) continue;
             size_t nf = tc_pack_elems(l->cin, l->cout, l->k, false), nd = tc_pack_elems(l->cin, l->cout, l->k, true);
             bf16 *f = ex.ws.get<bf16>(nf), *dd = ex.ws.get<bf16>(nd);
             l->wp_f = f; l->wp_d = dd;
-            jobs.push_back(tc_pack_job(params + l->off_W, f, l->cin, l->cout, l->k, false));
-            jobs.push_back(tc_pack_job(params + l->off_W, dd, l->cin, l->cout, l->k, true));
-            bytes += (double)(nf + nd) * 2 + (double)l->cin * l->cout * l->k * l->k * 8;
-            if (nf > max_elems) max_elems = nf;
-            if (nd > max_elems) max_elems = nd;
+            jobs.push_back(tc_pack_job(params + l->off_W, f, dd, l->cin, l->cout, l->k));
+            bytes += (double)(nf + nd) * 2 + (double)l->cin * l->cout * l->k * l->k * 4;
+            max_tiles = std::max(max_tiles, tc_pack_tiles(jobs.back()));
         }
         PackJob *jobs_dev = ex.ws.get<PackJob>(jobs.size() + 1);
         if (!ex.dry && !jobs.empty()) {
             if (jobs.size() * sizeof(PackJob) <= pl->pack_host_bytes) {
                 memcpy(pl->pack_host, jobs.data(), jobs.size() * sizeof(PackJob));
                 cudaMemcpyAsync(jobs_dev, pl->pack_host, jobs.size() * sizeof(PackJob), cudaMemcpyHostToDevice, ex.stream);
-                tc_pack_batch(ex, jobs_dev, (int)jobs.size(), bytes, max_elems);
+                tc_pack_batch(ex, jobs_dev, (int)jobs.size(), bytes, max_tiles);
             } else {
                 for (LayerSlot *l : slots) l->wp_f = l->wp_d = nullptr;   // no staging room: pack per call instead
             }
@@ -482,7 +481,7 @@ extern "C" int revnet_stack_plan(revnet_ctx *ctx, const revnet_stack_desc *desc,
     {
         size_t layers = 0;
         for (auto &st : pl->st) layers += 1 + 6 + (size_t)st.units * 6;
-        pl->pack_host_bytes = layers * 2 * sizeof(PackJob);
+        pl->pack_host_bytes = layers * sizeof(PackJob);
         if (pl->pinned_is_malloc || cudaMallocHost(&pl->pack_host, pl->pack_host_bytes) != cudaSuccess) {
             cudaGetLastError(); pl->pack_host = nullptr; pl->pack_host_bytes = 0;
         }
