@@ -45,7 +45,7 @@ DEVICE_KERNEL = {
     "conv_fprop_tc": "conv_tc_kernel", "conv_dgrad_tc": "conv_tc_kernel", "conv_wgrad_tc": "wgrad_tc_kernel",
     "conv_fprop_tc2": "conv_tc2_kernel", "conv_dgrad_tc2": "conv_tc2_kernel", "conv_wgrad_tc2": "wgrad_tc2_kernel",
     "conv_fprop_simt": "gemm_simt_kernel", "conv_dgrad_simt": "gemm_simt_kernel", "conv_wgrad_simt": "gemm_simt_kernel",
-    "bn_stats_partial": "col_reduce_kernel", "bn_bwd_partial": "col_reduce_kernel",
+    "bn_stats": "col_reduce_kernel", "bn_bwd_sums": "col_reduce_kernel",
 }
 KERNEL_SOURCES = {
     "conv_fused_kernel": ("conv_fused.cu", "conv_epilogue.cuh", "tc_ptx.cuh"),

@@ -18,7 +18,7 @@ extern "C" int revnet_create(revnet_ctx **out, int device) {
         int sm = 0;
         if (cudaSetDevice(device) != cudaSuccess ||
             cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-            cudaMalloc(&c->dev_status, 1024) != cudaSuccess || cudaMemset(c->dev_status, 0, 1024) != cudaSuccess ||
+            cudaMalloc(&c->dev_status, revnet_ctx::kStatusBytes) != cudaSuccess || cudaMemset(c->dev_status, 0, revnet_ctx::kStatusBytes) != cudaSuccess ||
             cudaMalloc(&c->stamps, 2 * kStampSlots * sizeof(unsigned long long)) != cudaSuccess ||
             cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking) != cudaSuccess ||
             cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -361,7 +361,7 @@ extern "C" int revnet_check_device(revnet_ctx *ctx, void *stream) {
     if (st != 0) {
         // a kernel that gave up never counted itself out of its grid-wide reduction: zero the counter words as well,
         // or a later kernel handed the same word would elect its last CTA too early
-        cudaMemsetAsync(ctx->dev_status, 0, 1024, s);
+        cudaMemsetAsync(ctx->dev_status, 0, revnet_ctx::kStatusBytes, s);
         cudaStreamSynchronize(s);
         return fail(ctx, st, "a kernel gave up a bounded wait (device status " + std::to_string(st) + ")");
     }

@@ -21,8 +21,16 @@ struct revnet_ctx {
     int *dev_status = nullptr;   // device word for bounded-wait time-outs
     unsigned int *counters = nullptr;   // zeroed words the kernels' grid-wide reductions count on (each leaves its word zero)
     int next_counter = 0;
-    unsigned int *counter() { unsigned int *c = counters + next_counter; next_counter = (next_counter + 1) % kCounters; return c; }
-    static constexpr int kCounters = 192;
+    // n consecutive words, handed out in a ring: a word comes round again only after kCounters / n further reductions, far more
+    // than can be in flight on the context's streams
+    unsigned int *counter(int n = 1) {
+        if (next_counter + n > kCounters) next_counter = 0;
+        unsigned int *c = counters + next_counter;
+        next_counter += n;
+        return c;
+    }
+    static constexpr int kCounters = 8128;
+    static constexpr size_t kStatusBytes = (64 + kCounters) * sizeof(unsigned int);     // dev_status and, 64 words on, the counters
     void *encode_tiled = nullptr; // driver entry point for tensor-map encoding
     cudaStream_t capture_stream = nullptr;   // private stream on which a train step is captured into a graph
     cudaStream_t side_stream = nullptr;      // weight gradients run here, beside the data-gradient chain
@@ -304,8 +312,8 @@ struct Geom { int N, H, W; size_t P() const { return (size_t)N * H * W; } };
 Moments mom_alloc(Exec &ex, int C, bool with_part = false);
 // pending statistics -> mean / rstd (one small kernel); no-op otherwise
 void mom_finalize(Exec &ex, Moments &m, int C);
-// batch statistics of t ([P,C]) -> mean, rstd (two kernels; the convolution epilogues produce the
-// same quantities for the tensors they write)
+// batch statistics of t ([P,C]) -> mean, rstd (the convolution epilogues produce the same quantities for the
+// tensors they write)
 void bn_stats(Exec &ex, Pair t, size_t P, Moments m);
 // a = relu(scale*t + shift) written as one [P,C] tensor of float (strict) or bf16
 void bn_relu_apply(Exec &ex, Pair t, size_t P, BnRef bn, void *a, bool a_bf16);
