@@ -1,11 +1,17 @@
 // Convolution forward / data-gradient / weight-gradient as fp32 implicit GEMMs on the CUDA cores.
-// This is the strict-precision verification path, and the fallback for shapes the tensor-core
+// This is the strict-precision path, and the fallback for shapes the tensor-core
 // kernels do not take.  Products and sums are fp32 FMA; operands may be float or bf16.
 //
 //   fprop: out[p,co]   = sum_{kh,kw,ci} a[p (+) (kh,kw), ci] * W[co,kh,kw,ci]        (Eq. 2, Conv_kxk)
 //   dgrad: da[q,ci]    = sum_{kh,kw,co} g[p,co] * W[co,kh,kw,ci],  p*s + (kh,kw) - pad = q
 //   wgrad: dW[co,kh,kw,ci] = sum_p g[p,co] * a[p (+) (kh,kw), ci]
+//
+// Two kernels.  conv_gemm_kernel takes every layer whose channel counts are multiples of four (all BN-ReLU-conv layers):
+// quads of channels are loaded as vectors, a thread's pixel is decoded once, and the product is register-tiled.
+// gemm_simt_kernel loads element by element and is left for the stem convolution's odd channel counts (an image has
+// three), where the kernels of stem.cu do not take its size.
 #include "common.cuh"
+#include <algorithm>
 
 template <class T> __device__ __forceinline__ float ldf(const T *p);
 template <> __device__ __forceinline__ float ldf<float>(const float *p) { return *p; }
@@ -15,8 +21,290 @@ struct ConvGeom {
     int N, H, W, Ci, Ho, Wo, Co, k, s, pad;
 };
 
+// ------------------------------------------------------------------ channel counts that are multiples of four
+// C[M,N] = A[M,K] * B[K,N] in tiles of (64 WM) x (16 WN), 256 threads = 8 warps of which WK share the K range of a tile: a
+// warp holds 64 x 16 accumulators, 8 x 4 per thread, so that one K step costs three 16-byte shared-memory reads (one wavefront
+// each) per 32 FMAs.  K runs in chunks of 16 through two shared-memory buffers; the next chunk's quads are on their way
+// from global memory while this one is multiplied.
+// Bound by the FMA pipes (and by issue: 35 instructions per 32 FMAs).  Measured on the 3x3 layers of the CIFAR-sized
+// networks at batch 128: 16 channels at 32x32: 157 -> 33 us forward, 176 -> 27 us
+// data gradient, 371 -> 49 us weight gradient (the element-wise kernel spent its time on index divisions and scalar loads).
+struct FastDiv {                     // n / d for 0 <= n < 2^31 by multiplication (Granlund and Montgomery, 1994)
+    uint32_t d, mul, sh;
+    __device__ __forceinline__ uint32_t div(uint32_t n) const { return (__umulhi(mul, n) + n) >> sh; }
+    __device__ __forceinline__ void divmod(uint32_t n, uint32_t &q, uint32_t &r) const { q = div(n); r = n - q * d; }
+};
+static FastDiv fast_div(uint32_t d) {
+    FastDiv f; f.d = d; f.sh = 0;
+    while ((1ull << f.sh) < d) f.sh++;
+    f.mul = (uint32_t)(((1ull << 32) * ((1ull << f.sh) - d)) / d + 1);
+    return f;
+}
+template <class T> __device__ __forceinline__ float4 ldq(const T *p);
+template <> __device__ __forceinline__ float4 ldq<float>(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+template <> __device__ __forceinline__ float4 ldq<bf16>(const bf16 *p) {
+    const uint2 u = *reinterpret_cast<const uint2 *>(p);
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
+}
+__device__ __forceinline__ float round_w(float w, bool to_bf16) { return to_bf16 ? __bfloat162float(__float2bfloat16_rn(w)) : w; }
+__device__ __forceinline__ float4 round_w4(float4 w, bool b) { return make_float4(round_w(w.x, b), round_w(w.y, b), round_w(w.z, b), round_w(w.w, b)); }
+
+// Operands.  kAlongK: a quad is four consecutive K indices of one row (else four consecutive rows at one K index).
+// row(m): what a thread keeps of its row (quad of rows); quad(state, k): the four values, zeros outside.
+struct RowAt { int y, x; size_t base; bool ok; };
+template <class TA> struct FpropA {           // m = output pixel, k = (kh, kw, ci)
+    static constexpr bool kAlongK = true;
+    const TA *a; ConvGeom g; FastDiv wo, ho, ci, kk; int M, K;
+    __device__ __forceinline__ RowAt row(int m) const {
+        uint32_t t, x, n, y;
+        wo.divmod((uint32_t)m, t, x); ho.divmod(t, n, y);
+        return RowAt{(int)y * g.s - g.pad, (int)x * g.s - g.pad, (size_t)n * g.H * g.W * g.Ci, m < M};
+    }
+    __device__ __forceinline__ float4 quad(const RowAt &r, int k) const {
+        uint32_t tap, c, kh, kw;
+        ci.divmod((uint32_t)k, tap, c); kk.divmod(tap, kh, kw);
+        const int y = r.y + (int)kh, x = r.x + (int)kw;
+        if (!r.ok || k >= K || (unsigned)y >= (unsigned)g.H || (unsigned)x >= (unsigned)g.W) return make_float4(0.f, 0.f, 0.f, 0.f);
+        return ldq(a + r.base + ((size_t)y * g.W + x) * g.Ci + c);
+    }
+    __device__ __forceinline__ size_t out_row(int m) const { return (size_t)m; }
+    __device__ __forceinline__ bool skip(int, int, int) const { return false; }
+};
+// m = input pixel, k = (kh, kw, co).  With stride 2 the pixels are numbered parity class by parity class ((y & 1, x & 1), then
+// image, y / 2, x / 2), so that a tile lies in one class and the chunks of the taps that do not reach it are skipped.
+template <class TG> struct DgradA {
+    static constexpr bool kAlongK = true;
+    const TG *gq; ConvGeom g; FastDiv w, h, co, kk, cls; bool classes; int M, K;       // w, h: columns and rows of a class (stride 1: of the image)
+    __device__ __forceinline__ void place(int m, int &n, int &y, int &x) const {
+        uint32_t c = 0, r = (uint32_t)m, t, xx, nn, yy;
+        if (classes) cls.divmod(r, c, r);
+        w.divmod(r, t, xx); h.divmod(t, nn, yy);
+        n = (int)nn;
+        y = classes ? (int)(2 * yy + (c >> 1)) : (int)yy; x = classes ? (int)(2 * xx + (c & 1)) : (int)xx;
+    }
+    __device__ __forceinline__ RowAt row(int m) const {
+        int n, y, x;
+        place(m, n, y, x);
+        return RowAt{y + g.pad, x + g.pad, (size_t)n * g.Ho * g.Wo * g.Co, m < M};
+    }
+    __device__ __forceinline__ float4 quad(const RowAt &r, int k) const {
+        uint32_t tap, c, kh, kw;
+        co.divmod((uint32_t)k, tap, c); kk.divmod(tap, kh, kw);
+        int y = r.y - (int)kh, x = r.x - (int)kw;
+        bool ok = r.ok && k < K && y >= 0 && x >= 0;
+        if (g.s == 2) { ok = ok && !((y | x) & 1); y >>= 1; x >>= 1; }
+        if (!ok || y >= g.Ho || x >= g.Wo) return make_float4(0.f, 0.f, 0.f, 0.f);
+        return ldq(gq + r.base + ((size_t)y * g.Wo + x) * g.Co + c);
+    }
+    __device__ __forceinline__ size_t out_row(int m) const {
+        if (!classes) return (size_t)m;
+        int n, y, x;
+        place(m, n, y, x);
+        return ((size_t)n * g.H + y) * g.W + x;
+    }
+    // whether the chunk k .. k + 15 adds nothing to the rows m0 .. m1
+    __device__ __forceinline__ bool skip(int m0, int m1, int k) const {
+        if (!classes) return false;
+        const uint32_t c = cls.div((uint32_t)m0), tap = co.div((uint32_t)k);
+        if (c != cls.div((uint32_t)(m1 < M ? m1 : M - 1)) || tap != co.div((uint32_t)(k + 15))) return false;
+        uint32_t kh, kw;
+        kk.divmod(tap, kh, kw);
+        return (((c >> 1) + g.pad + kh) & 1) || (((c & 1) + g.pad + kw) & 1);
+    }
+};
+template <class TA> struct WgradA {           // m = (kh, kw, ci), k = output pixel
+    static constexpr bool kAlongK = false;
+    const TA *a; ConvGeom g; FastDiv wo, ho, ci, kk; int M, K;
+    __device__ __forceinline__ RowAt row(int m) const {
+        uint32_t tap, c, kh, kw;
+        ci.divmod((uint32_t)m, tap, c); kk.divmod(tap, kh, kw);
+        return RowAt{(int)kh - g.pad, (int)kw - g.pad, c, m < M};
+    }
+    __device__ __forceinline__ float4 quad(const RowAt &r, int k) const {
+        uint32_t t, xo, n, yo;
+        wo.divmod((uint32_t)k, t, xo); ho.divmod(t, n, yo);
+        const int y = (int)yo * g.s + r.y, x = (int)xo * g.s + r.x;
+        if (!r.ok || k >= K || (unsigned)y >= (unsigned)g.H || (unsigned)x >= (unsigned)g.W) return make_float4(0.f, 0.f, 0.f, 0.f);
+        return ldq(a + (((size_t)n * g.H + y) * g.W + x) * g.Ci + r.base);
+    }
+    __device__ __forceinline__ bool skip(int, int, int) const { return false; }
+};
+struct FpropB {                               // n = co, k = (kh, kw, ci): W[co][k];  wb: weights take part as bf16 values (mode 0)
+    static constexpr bool kAlongK = true;
+    const float *w; int N, K; bool wb;
+    __device__ __forceinline__ float4 quad(int n, int k) const {
+        return n < N && k < K ? round_w4(ldq(w + (size_t)n * K + k), wb) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+};
+struct DgradB {                               // n = ci (four of them), k = (kh, kw, co): W[co][tap][ci]
+    static constexpr bool kAlongK = false;
+    const float *w; FastDiv co; int taps, N, K; bool wb;
+    __device__ __forceinline__ float4 quad(int n, int k) const {
+        uint32_t tap, c;
+        co.divmod((uint32_t)k, tap, c);
+        return n < N && k < K ? round_w4(ldq(w + ((size_t)c * taps + tap) * N + n), wb) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+};
+template <class TG> struct WgradB {           // n = co (four of them), k = output pixel
+    static constexpr bool kAlongK = false;
+    const TG *gq; int N, K;
+    __device__ __forceinline__ float4 quad(int n, int k) const { return n < N && k < K ? ldq(gq + (size_t)k * N + n) : make_float4(0.f, 0.f, 0.f, 0.f); }
+};
+
+// Epilogues: four consecutive N of row m
+struct OutCouple {                            // out = partner + sign*acc (sign 0: plain store); out / partner may be split pairs
+    static constexpr bool kTransposed = false;
+    Pair out, partner; int sign;
+    __device__ __forceinline__ void store(size_t row, int n, float4 v) const { out.couple4(row, n, v, partner, sign); }
+};
+struct OutPlain {
+    static constexpr bool kTransposed = false;
+    float *out; int N;
+    __device__ __forceinline__ void store(size_t row, int n, float4 v) const { *reinterpret_cast<float4 *>(out + row * N + n) = v; }
+};
+struct OutSplit {                             // slice z of a split reduction: four consecutive M of column n, out[z][n][M]
+    static constexpr bool kTransposed = true;
+    float *out; int M; size_t slice;
+    __device__ __forceinline__ void store(int n, int m, float4 v, int z) const { *reinterpret_cast<float4 *>(out + z * slice + (size_t)n * M + m) = v; }
+};
+
+template <int WM, int WN, int WK> struct GemmTile {
+    static constexpr int BM = 64 * WM, BN = 16 * WN, BK = 16, PA = BM + 4, PB = BN + 4, kStage = BK * (PA + PB);
+    static constexpr int kReduce = (WK - 1) * WM * WN * 1024;
+    static constexpr int kSmem = (2 * kStage > kReduce ? 2 * kStage : kReduce) * 4;
+    static_assert(WM * WN * WK == 8, "eight warps");
+};
+
+template <int WM, int WN, int WK, class AL, class BL, class EP>
+__global__ void __launch_bounds__(256, 2) conv_gemm_kernel(AL al, BL bl, EP ep, int M, int N, int K, int k_per_split) {
+    pdl_enter();
+    using T = GemmTile<WM, WN, WK>;
+    constexpr int BM = T::BM, BN = T::BN, BK = T::BK, PA = T::PA, PB = T::PB;
+    constexpr int NA = BM / 64;               // A quads a thread loads per chunk
+    extern __shared__ float sm[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, lm = lane >> 2, ln = lane & 3;
+    const int wk = warp % WK, wn = (warp / WK) % WN, wm = warp / (WK * WN);
+    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
+    const int kbeg = blockIdx.z * k_per_split, kend = kbeg + k_per_split < K ? kbeg + k_per_split : K;
+    // this thread's A quads: along K, row tid % BM and K quads tid / BM + i * (256 / BM); along M, row quad tid % (BM / 4)
+    const int am = AL::kAlongK ? tid % BM : (tid % (BM / 4)) * 4;
+    const int ak = AL::kAlongK ? (tid / BM) * 4 : tid / (BM / 4);
+    constexpr int AKS = AL::kAlongK ? (BM < 256 ? 1024 / BM : 4) : 1024 / BM;      // K step between the quads of a thread
+    const bool b_on = tid < BN * 4;
+    const int bn = BL::kAlongK ? tid % BN : (tid % (BN / 4)) * 4;
+    const int bk = BL::kAlongK ? (tid / BN) * 4 : tid / (BN / 4);
+    const RowAt ra = al.row(m0 + am);
+    float4 va[NA], vb;
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int i = 0; i < NA; i++) va[i] = k0 + ak + i * AKS < kend ? al.quad(ra, k0 + ak + i * AKS) : make_float4(0.f, 0.f, 0.f, 0.f);
+        vb = b_on && k0 + bk < kend ? bl.quad(n0 + bn, k0 + bk) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    auto put = [&](float *As, float *Bs) {
+#pragma unroll
+        for (int i = 0; i < NA; i++) {
+            const int k = ak + i * AKS;
+            if (AL::kAlongK) { As[k * PA + am] = va[i].x; As[(k + 1) * PA + am] = va[i].y; As[(k + 2) * PA + am] = va[i].z; As[(k + 3) * PA + am] = va[i].w; }
+            else *reinterpret_cast<float4 *>(As + k * PA + am) = va[i];
+        }
+        if (b_on) {
+            if (BL::kAlongK) { Bs[bk * PB + bn] = vb.x; Bs[(bk + 1) * PB + bn] = vb.y; Bs[(bk + 2) * PB + bn] = vb.z; Bs[(bk + 3) * PB + bn] = vb.w; }
+            else *reinterpret_cast<float4 *>(Bs + bk * PB + bn) = vb;
+        }
+    };
+    float acc[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) acc[i][j] = 0.f;
+    auto next_chunk = [&](int k) { while (k < kend && al.skip(m0, m0 + BM - 1, k)) k += BK; return k; };
+    int k0 = next_chunk(kbeg), buf = 0;
+    if (k0 < kend) { fetch(k0); put(sm, sm + BK * PA); }
+    __syncthreads();
+    while (k0 < kend) {
+        const int kn = next_chunk(k0 + BK);
+        if (kn < kend) fetch(kn);
+        const float *As = sm + buf * T::kStage + wm * 64 + lm * 4, *Bs = sm + buf * T::kStage + BK * PA + wn * 16 + ln * 4;
+#pragma unroll
+        for (int kk = 0; kk < BK / WK; kk++) {
+            const int k = wk * (BK / WK) + kk;
+            const float4 a0 = *reinterpret_cast<const float4 *>(As + k * PA), a1 = *reinterpret_cast<const float4 *>(As + k * PA + 32);
+            const float4 b = *reinterpret_cast<const float4 *>(Bs + k * PB);
+            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                acc[i][0] = fmaf(a[i], b.x, acc[i][0]); acc[i][1] = fmaf(a[i], b.y, acc[i][1]);
+                acc[i][2] = fmaf(a[i], b.z, acc[i][2]); acc[i][3] = fmaf(a[i], b.w, acc[i][3]);
+            }
+        }
+        buf ^= 1;
+        if (kn < kend) put(sm + buf * T::kStage, sm + buf * T::kStage + BK * PA);
+        __syncthreads();
+        k0 = kn;
+    }
+    if (WK > 1) {
+        // the warps that share a tile are added in order
+        float *red = sm + (size_t)(wm * WN + wn) * 1024 + lane * 4;
+        if (wk > 0)
+#pragma unroll
+            for (int i = 0; i < 8; i++)
+                *reinterpret_cast<float4 *>(red + (size_t)(wk - 1) * WM * WN * 1024 + i * 128) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+        __syncthreads();
+        if (wk > 0) return;
+        for (int w = 0; w < WK - 1; w++)
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                const float4 v = *reinterpret_cast<const float4 *>(red + (size_t)w * WM * WN * 1024 + i * 128);
+                acc[i][0] += v.x; acc[i][1] += v.y; acc[i][2] += v.z; acc[i][3] += v.w;
+            }
+    }
+    const int n = n0 + wn * 16 + ln * 4;
+    if constexpr (EP::kTransposed) {
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int m = m0 + wm * 64 + h * 32 + lm * 4;
+            if (m < M)
+#pragma unroll
+                for (int j = 0; j < 4; j++)
+                    if (n + j < N) ep.store(n + j, m, make_float4(acc[4 * h][j], acc[4 * h + 1][j], acc[4 * h + 2][j], acc[4 * h + 3][j]), blockIdx.z);
+        }
+    } else if (n < N) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            const int m = m0 + wm * 64 + (i >> 2) * 32 + lm * 4 + (i & 3);
+            if (m < M) ep.store(al.out_row(m), n, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
+        }
+    }
+}
+
+template <int WM, int WN, int WK, class AL, class BL, class EP>
+static void launch_tile(Exec &ex, AL al, BL bl, EP ep, int M, int N, int K, int splits, int k_per_split) {
+    using T = GemmTile<WM, WN, WK>;
+    static OncePerDevice once;
+    if (T::kSmem > 48 * 1024 && once.first(ex.ctx->device))
+        cudaFuncSetAttribute(conv_gemm_kernel<WM, WN, WK, AL, BL, EP>, cudaFuncAttributeMaxDynamicSharedMemorySize, T::kSmem);
+    launch(ex, conv_gemm_kernel<WM, WN, WK, AL, BL, EP>, dim3((M + T::BM - 1) / T::BM, (N + T::BN - 1) / T::BN, splits), 256, T::kSmem, al, bl, ep, M, N, K, k_per_split);
+}
+// Tile of a forward / data-gradient GEMM (M = pixels): N tile as wide as the layer up to 64; the tallest M tile that still
+// gives every SM two CTAs (the warps it does not need for rows share the K range instead)
+template <class AL, class BL, class EP>
+static void launch_pixels(Exec &ex, AL al, BL bl, EP ep, int M, int N, int K) {
+    const long want = 2l * ex.ctx->sm_count;
+    const int nt = (N + 63) / 64;
+    if (N <= 16) {
+        if ((M + 255) / 256 >= want) launch_tile<4, 1, 2>(ex, al, bl, ep, M, N, K, 1, K);
+        else launch_tile<1, 1, 8>(ex, al, bl, ep, M, N, K, 1, K);
+    } else if (N <= 32) {
+        if ((M + 255) / 256 >= want) launch_tile<4, 2, 1>(ex, al, bl, ep, M, N, K, 1, K);
+        else launch_tile<1, 2, 4>(ex, al, bl, ep, M, N, K, 1, K);
+    } else if ((long)((M + 127) / 128) * nt >= want) launch_tile<2, 4, 1>(ex, al, bl, ep, M, N, K, 1, K);
+    else if ((long)((M + 63) / 64) * nt >= ex.ctx->sm_count) launch_tile<1, 4, 2>(ex, al, bl, ep, M, N, K, 1, K);
+    else launch_tile<1, 2, 4>(ex, al, bl, ep, M, N, K, 1, K);
+}
+
+// ------------------------------------------------------------------ any channel count, element by element
 // ---- operand loaders: element (m,k) of A and (k,n) of B of the implicit GEMM
-template <class TA> struct FpropA {           // m = output pixel, k = (kh,kw,ci)
+template <class TA> struct AnyFpropA {           // m = output pixel, k = (kh,kw,ci)
     const TA *a; ConvGeom g;
     static constexpr bool k_fast = true;
     __device__ float operator()(int m, int kk) const {
@@ -27,39 +315,17 @@ template <class TA> struct FpropA {           // m = output pixel, k = (kh,kw,ci
         return ldf(a + (((size_t)n * g.H + y) * g.W + x) * g.Ci + ci);
     }
 };
-__device__ __forceinline__ float round_w(float w, bool to_bf16) { return to_bf16 ? __bfloat162float(__float2bfloat16_rn(w)) : w; }
-struct FpropB {                               // k = (kh,kw,ci), n = co ; W[co][kh][kw][ci]
+struct AnyFpropB {                               // k = (kh,kw,ci), n = co ; W[co][kh][kw][ci]
     const float *w; int K; bool wb;           // wb: weights take part as bf16 values (mode 0)
     static constexpr bool k_fast = true;
     __device__ float operator()(int kk, int n) const { return round_w(w[(size_t)n * K + kk], wb); }
 };
-template <class TG> struct DgradA {           // m = input pixel, k = (kh,kw,co)
-    const TG *gq; ConvGeom g;
-    static constexpr bool k_fast = true;
-    __device__ float operator()(int m, int kk) const {
-        int x = m % g.W, t = m / g.W, y = t % g.H, n = t / g.H;
-        int co = kk % g.Co, tap = kk / g.Co, kw = tap % g.k, kh = tap / g.k;
-        int yy = y + g.pad - kh, xx = x + g.pad - kw;
-        if (yy < 0 || xx < 0 || yy % g.s || xx % g.s) return 0.f;
-        int ho = yy / g.s, wo = xx / g.s;
-        if (ho >= g.Ho || wo >= g.Wo) return 0.f;
-        return ldf(gq + (((size_t)n * g.Ho + ho) * g.Wo + wo) * g.Co + co);
-    }
-};
-struct DgradB {                               // k = (kh,kw,co), n = ci
-    const float *w; ConvGeom g; bool wb;
-    static constexpr bool k_fast = false;
-    __device__ float operator()(int kk, int n) const {
-        int co = kk % g.Co, tap = kk / g.Co;
-        return round_w(w[((size_t)co * g.k * g.k + tap) * g.Ci + n], wb);
-    }
-};
-template <class TG> struct WgradA {           // m = co, k = output pixel
+template <class TG> struct AnyWgradA {           // m = co, k = output pixel
     const TG *gq; ConvGeom g;
     static constexpr bool k_fast = false;
     __device__ float operator()(int m, int kk) const { return ldf(gq + (size_t)kk * g.Co + m); }
 };
-template <class TA> struct WgradB {           // k = output pixel, n = (kh,kw,ci)
+template <class TA> struct AnyWgradB {           // k = output pixel, n = (kh,kw,ci)
     const TA *a; ConvGeom g;
     static constexpr bool k_fast = false;
     __device__ float operator()(int kk, int n) const {
@@ -162,11 +428,20 @@ void conv_fprop_simt(Exec &ex, const void *a, bool a_bf16, Geom gi, const Layer 
     const int M = g.N * g.Ho * g.Wo, N = g.Co, K = g.k * g.k * g.Ci;
     ex.flops += 2ull * M * N * K;
     if (ex.dry) return;
-    EpiCouple ep{out, partner, sign};
-    FpropB bl{L.W, K, a_bf16};
     const double bytes = (double)g.N * g.H * g.W * g.Ci * (a_bf16 ? 2 : 4) + (double)M * N * (sign ? 8 : 4) + (double)N * K * 4;
-    if (a_bf16) launch_gemm(ex, "conv_fprop_simt", FpropA<bf16>{(const bf16 *)a, g}, bl, ep, M, N, K, 1, K, bytes);
-    else launch_gemm(ex, "conv_fprop_simt", FpropA<float>{(const float *)a, g}, bl, ep, M, N, K, 1, K, bytes);
+    if (g.Ci % 4) {
+        EpiCouple ep{out, partner, sign};
+        AnyFpropB bl{L.W, K, a_bf16};
+        if (a_bf16) launch_gemm(ex, "conv_fprop_simt", AnyFpropA<bf16>{(const bf16 *)a, g}, bl, ep, M, N, K, 1, K, bytes);
+        else launch_gemm(ex, "conv_fprop_simt", AnyFpropA<float>{(const float *)a, g}, bl, ep, M, N, K, 1, K, bytes);
+        return;
+    }
+    const FastDiv wo = fast_div(g.Wo), ho = fast_div(g.Ho), ci = fast_div(g.Ci), kk = fast_div(g.k);
+    const OutCouple ep{out, partner, sign};
+    const FpropB bl{L.W, N, K, a_bf16};
+    if (a_bf16) launch_pixels(ex, FpropA<bf16>{(const bf16 *)a, g, wo, ho, ci, kk, M, K}, bl, ep, M, N, K);
+    else launch_pixels(ex, FpropA<float>{(const float *)a, g, wo, ho, ci, kk, M, K}, bl, ep, M, N, K);
+    ex.check("conv_fprop_simt", bytes, 2.0 * M * N * (double)K);
 }
 
 void conv_dgrad_simt(Exec &ex, const void *gq, bool g_bf16, Geom gi, const Layer &L, float *da) {
@@ -174,48 +449,78 @@ void conv_dgrad_simt(Exec &ex, const void *gq, bool g_bf16, Geom gi, const Layer
     const int M = g.N * g.H * g.W, N = g.Ci, K = g.k * g.k * g.Co;
     ex.flops += 2ull * g.N * g.Ho * g.Wo * N * K;
     if (ex.dry) return;
-    EpiPlain ep{da, N, 0};
-    DgradB bl{L.W, g, g_bf16};
     const double bytes = (double)g.N * g.Ho * g.Wo * g.Co * (g_bf16 ? 2 : 4) + (double)M * N * 4 + (double)N * K * 4;
-    if (g_bf16) launch_gemm(ex, "conv_dgrad_simt", DgradA<bf16>{(const bf16 *)gq, g}, bl, ep, M, N, K, 1, K, bytes);
-    else launch_gemm(ex, "conv_dgrad_simt", DgradA<float>{(const float *)gq, g}, bl, ep, M, N, K, 1, K, bytes);
+    const OutPlain ep{da, N};
+    // stride 2: parity classes of (H + 1) / 2 x (W + 1) / 2 pixels would be ragged on odd sizes; those keep the plain numbering
+    const bool classes = g.s == 2 && g.H % 2 == 0 && g.W % 2 == 0;
+    const FastDiv w = fast_div(classes ? g.W / 2 : g.W), h = fast_div(classes ? g.H / 2 : g.H), co = fast_div(g.Co), kk = fast_div(g.k);
+    const FastDiv cls = fast_div(classes ? M / 4 : (uint32_t)M);
+    const DgradB bl{L.W, co, g.k * g.k, N, K, g_bf16};
+    if (g_bf16) launch_pixels(ex, DgradA<bf16>{(const bf16 *)gq, g, w, h, co, kk, cls, classes, M, K}, bl, ep, M, N, K);
+    else launch_pixels(ex, DgradA<float>{(const float *)gq, g, w, h, co, kk, cls, classes, M, K}, bl, ep, M, N, K);
+    ex.check("conv_dgrad_simt", bytes, 2.0 * g.N * g.Ho * g.Wo * N * (double)K);
 }
 
-// fixed-order sum of split-K slices
+// fixed-order sum of split-K slices: a block takes 32 elements, eight threads each (every eighth slice), added in order
 __global__ void splitk_reduce_kernel(const float *__restrict__ part, size_t n, int splits, float *__restrict__ out) {
     pdl_enter();
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        float s = 0.f;
-        for (int z = 0; z < splits; z++) s += part[(size_t)z * n + i];
+    __shared__ float sm[8][33];
+    const int e = threadIdx.x & 31, grp = threadIdx.x >> 5;
+    const size_t i = (size_t)blockIdx.x * 32 + e;
+    float s = 0.f;
+    if (i < n)
+#pragma unroll 4
+        for (int z = grp; z < splits; z += 8) s += part[(size_t)z * n + i];
+    sm[grp][e] = s;
+    __syncthreads();
+    if (grp == 0 && i < n) {
+        for (int g = 1; g < 8; g++) s += sm[g][e];
         out[i] = s;
     }
 }
 
+// dW as a GEMM of M = (tap, ci), N = co over the pixels; the pixels are split so that the grid fills the machine twice
+template <class TG, class TA>
+static void wgrad_launch(Exec &ex, const TG *gq, const TA *a, ConvGeom g, float *part, int splits, int kps) {
+    const int M = g.k * g.k * g.Ci, N = g.Co, K = g.N * g.Ho * g.Wo;
+    const WgradA<TA> al{a, g, fast_div(g.Wo), fast_div(g.Ho), fast_div(g.Ci), fast_div(g.k), M, K};
+    const WgradB<TG> bl{gq, N, K};
+    const OutSplit ep{part, M, (size_t)M * N};
+    if (N <= 16) launch_tile<1, 1, 8>(ex, al, bl, ep, M, N, K, splits, kps);
+    else if (N <= 32) launch_tile<1, 2, 4>(ex, al, bl, ep, M, N, K, splits, kps);
+    else launch_tile<1, 4, 2>(ex, al, bl, ep, M, N, K, splits, kps);
+}
 void conv_wgrad_simt(Exec &ex, const void *gq, bool g_bf16, const void *a, bool a_bf16, Geom gi, const Layer &L, float *dW) {
     ConvGeom g = geom_of(gi, L);
-    const int M = g.Co, N = g.k * g.k * g.Ci, K = g.N * g.Ho * g.Wo;
-    ex.flops += 2ull * M * N * (size_t)K;
-    // split the pixel sum so that the grid fills the machine; slices are summed in fixed order
-    int tiles = ((M + 63) / 64) * ((N + 63) / 64);
-    int splits = (ex.ctx->sm_count * 2 + tiles - 1) / tiles;
-    int max_splits = (K + 255) / 256; if (splits > max_splits) splits = max_splits; if (splits < 1) splits = 1;
-    int kps = (((K + splits - 1) / splits) + 15) / 16 * 16;
-    splits = (K + kps - 1) / kps;
+    const int Co = g.Co, KC = g.k * g.k * g.Ci, P = g.N * g.Ho * g.Wo;
+    ex.flops += 2ull * Co * KC * (size_t)P;
+    const bool quads = g.Ci % 4 == 0 && g.Co % 4 == 0;
+    const int bn = Co <= 16 ? 16 : (Co <= 32 ? 32 : 64);
+    const int tiles = quads ? ((KC + 63) / 64) * ((Co + bn - 1) / bn) : ((Co + 63) / 64) * ((KC + 63) / 64);
+    int splits = (ex.ctx->sm_count * (quads ? 4 : 2) + tiles - 1) / tiles;
+    int max_splits = (P + 255) / 256; if (splits > max_splits) splits = max_splits; if (splits < 1) splits = 1;
+    int kps = (((P + splits - 1) / splits) + 15) / 16 * 16;
+    splits = (P + kps - 1) / kps;
     size_t m = ex.ws.mark();
-    float *part = splits > 1 ? ex.ws.get<float>((size_t)splits * M * N) : dW;
+    float *part = splits > 1 ? ex.ws.get<float>((size_t)splits * Co * KC) : dW;
     if (!ex.dry) {
-        EpiPlain ep{part, N, (size_t)M * N};
-        const double bytes = (double)K * g.Co * (g_bf16 ? 2 : 4) + (double)g.N * g.H * g.W * g.Ci * (a_bf16 ? 2 : 4) + (double)M * N * 4;
-#define RV_WG(TG, TA) launch_gemm(ex, "conv_wgrad_simt", WgradA<TG>{(const TG *)gq, g}, WgradB<TA>{(const TA *)a, g}, ep, M, N, K, splits, kps, bytes)
-        if (g_bf16 && a_bf16) RV_WG(bf16, bf16);
-        else if (g_bf16) RV_WG(bf16, float);
-        else if (a_bf16) RV_WG(float, bf16);
-        else RV_WG(float, float);
+        const double bytes = (double)P * g.Co * (g_bf16 ? 2 : 4) + (double)g.N * g.H * g.W * g.Ci * (a_bf16 ? 2 : 4) + (double)Co * KC * 4;
+        if (quads && g_bf16 == a_bf16) {
+            if (g_bf16) wgrad_launch(ex, (const bf16 *)gq, (const bf16 *)a, g, part, splits, kps);
+            else wgrad_launch(ex, (const float *)gq, (const float *)a, g, part, splits, kps);
+            ex.check("conv_wgrad_simt", bytes, 2.0 * Co * KC * (double)P);
+        } else {
+            EpiPlain ep{part, KC, (size_t)Co * KC};
+#define RV_WG(TG, TA) launch_gemm(ex, "conv_wgrad_simt", AnyWgradA<TG>{(const TG *)gq, g}, AnyWgradB<TA>{(const TA *)a, g}, ep, Co, KC, P, splits, kps, bytes)
+            if (g_bf16 && a_bf16) RV_WG(bf16, bf16);
+            else if (g_bf16) RV_WG(bf16, float);
+            else if (a_bf16) RV_WG(float, bf16);
+            else RV_WG(float, float);
 #undef RV_WG
+        }
         if (splits > 1) {
-            size_t n = (size_t)M * N;
-            int grid = (int)((n + 255) / 256); if (grid > ex.ctx->sm_count * 8) grid = ex.ctx->sm_count * 8;
-            launch(ex, splitk_reduce_kernel, grid, 256, 0, part, n, splits, dW);
+            const size_t n = (size_t)Co * KC;
+            launch(ex, splitk_reduce_kernel, (unsigned)((n + 31) / 32), 256, 0, part, n, splits, dW);
             ex.check("splitk_reduce");
         }
     }
