@@ -306,6 +306,19 @@ __device__ __forceinline__ void bn_coef4(const BnRef &bn, int c, float4 &sc, flo
 }
 #endif
 
+struct FastDiv {                     // n / d for 0 <= n < 2^31 by multiplication (Granlund and Montgomery, 1994)
+    uint32_t d, mul, sh;
+#ifdef __CUDACC__
+    __device__ __forceinline__ uint32_t div(uint32_t n) const { return (__umulhi(mul, n) + n) >> sh; }
+    __device__ __forceinline__ void divmod(uint32_t n, uint32_t &q, uint32_t &r) const { q = div(n); r = n - q * d; }
+#endif
+};
+static inline FastDiv fast_div(uint32_t d) {
+    FastDiv f; f.d = d; f.sh = 0;
+    while ((1ull << f.sh) < d) f.sh++;
+    f.mul = (uint32_t)(((1ull << 32) * ((1ull << f.sh) - d)) / d + 1);
+    return f;
+}
 struct Geom { int N, H, W; size_t P() const { return (size_t)N * H * W; } };
 
 // ---------------------------------------------------------------- elementwise.cu

@@ -187,30 +187,38 @@ __device__ __forceinline__ void epilogue_tile(const EpiArgs &e, uint32_t tmem_ac
     }
 }
 
-// mean and 1 / sqrt(var + eps) from a channel's sum and second sum (double), rounded to float once
+// mean and 1 / sqrt(var + eps) from a channel's sum and second sum (double), rounded to float once.  The reciprocal root is
+// the single-precision one refined by two Newton steps in double (relative error below 1e-13): a double division and square
+// root would be a few hundred dependent instructions at the head of every convolution.
 __device__ __forceinline__ void moments_of(double sum, double sum2, double inv_count, float eps, float &mean, float &rstd) {
     const double m = sum * inv_count;
     double var = sum2 * inv_count - m * m;
     if (var < 0) var = 0;
-    mean = (float)m; rstd = (float)(1.0 / sqrt(var + (double)eps));
+    const double v = var + (double)eps;
+    double y = (double)rsqrtf((float)v);
+    y *= 1.5 - 0.5 * v * y * y;
+    y *= 1.5 - 0.5 * v * y * y;
+    mean = (float)m; rstd = (float)y;
 }
 
 // Adds the per-CTA records of a reduction.  A record is 2C floats = C/2 float4 slots (per channel
 // quad: sums, second sums); this call covers the slots slot0 .. slot0 + cw - 1 (cw <= 128, even).
-// Thread = (slot, sub), slot fastest so that a warp reads whole records: it adds the records sub,
-// sub + nsub, ... of its slot, ten loads in flight at a time; the subs are then added in order.
+// Thread = (sub, slot), slot fastest so that a warp reads whole records: it adds the records sub,
+// sub + nsub, ... of its slot, five loads in flight at a time; the subs of a warp are combined by
+// shuffles, the warps (or, of wide records, the subs) in order.
 // (Giving a slot to consecutive lanes and adding them by shuffles was measured slower: the loads
 // of a warp then touch 32 records.)  All in double precision, in an order that the number of
 // records, cw and NT fix.  Result: tot[slot - slot0][4].  Called by NT threads (tid = 0..NT-1)
 // that share named barrier 1; red: [NT][4] doubles, tot: [128][4] doubles of shared memory.
 template <int NT>
 __device__ __forceinline__ void reduce_records(const float *part, int parts, int C, int slot0, int cw, double *red, double *tot, int tid) {
-    const int nsub = NT / cw;
-    const int r = tid % cw, sub = tid / cw;
-    if (sub < nsub) {
-        double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
-        const float *src = part + (size_t)(slot0 + r) * 4;
-        constexpr int kInFlight = 10;
+    int rs = 4;
+    while (rs < cw) rs <<= 1;
+    const int slot = tid & (rs - 1), sub = tid / rs, nsub = NT / rs, lane = tid & 31;
+    double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
+    if (slot < cw) {
+        const float *src = part + (size_t)(slot0 + slot) * 4;
+        constexpr int kInFlight = 5;
         for (int i = sub; i < parts; i += kInFlight * nsub) {
             float4 v[kInFlight];
 #pragma unroll
@@ -221,23 +229,27 @@ __device__ __forceinline__ void reduce_records(const float *part, int parts, int
 #pragma unroll
             for (int k = 0; k < kInFlight; k++) { s0 += (double)v[k].x; s1 += (double)v[k].y; s2 += (double)v[k].z; s3 += (double)v[k].w; }
         }
-        red[tid * 4] = s0; red[tid * 4 + 1] = s1; red[tid * 4 + 2] = s2; red[tid * 4 + 3] = s3;
+    }
+    for (int o = rs; o < 32; o <<= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o); s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, o); s3 += __shfl_xor_sync(0xffffffffu, s3, o);
+    }
+    const int groups = rs <= 32 ? NT / 32 : nsub;
+    if (rs > 32 || lane < rs) {
+        double *d = red + ((rs <= 32 ? (tid >> 5) * rs + lane : sub * rs + slot)) * 4;
+        d[0] = s0; d[1] = s1; d[2] = s2; d[3] = s3;
     }
     named_barrier(1, NT);
-    if (tid < cw) {
-        double s0 = red[tid * 4], s1 = red[tid * 4 + 1], s2 = red[tid * 4 + 2], s3 = red[tid * 4 + 3];
-        for (int y = 1; y < nsub; y++) {
-            const double *o = red + (y * cw + tid) * 4;
-            s0 += o[0]; s1 += o[1]; s2 += o[2]; s3 += o[3];
-        }
-        double *d = tot + tid * 4;
-        d[0] = s0; d[1] = s1; d[2] = s2; d[3] = s3;
+    for (int i = tid; i < cw * 4; i += NT) {
+        double t = red[i];
+        for (int g = 1; g < groups; g++) t += red[g * rs * 4 + i];
+        tot[i] = t;
     }
     named_barrier(1, NT);
 }
 
-template <int NT>
-__device__ __forceinline__ void epilogue_publish(const EpiArgs &e, float *scratch, int etid);
+template <int NT, class E>
+__device__ __forceinline__ void epilogue_publish(const E &e, float *scratch, int etid);
 
 // After the last tile: per-CTA partials, grid-wide count, and the finalize by the CTA that comes last.
 __device__ __forceinline__ void epilogue_finish(const EpiArgs &e, int BN, int col0, float *stage, const float *sums, int etid) {
@@ -268,8 +280,8 @@ __device__ __forceinline__ void epilogue_finish(const EpiArgs &e, int BN, int co
 // Once every CTA has written its partial record into e.part: count, and let the CTA that comes
 // last reduce the records in a fixed order and write the results.  Called by NT threads (etid = 0..NT-1);
 // scratch: (NT + 128) * 32 bytes of shared memory.
-template <int NT>
-__device__ __forceinline__ void epilogue_publish(const EpiArgs &e, float *scratch, int etid) {
+template <int NT, class E>
+__device__ __forceinline__ void epilogue_publish(const E &e, float *scratch, int etid) {
     // publish, count, and let the last CTA of the grid reduce
     __threadfence();
     named_barrier(1, NT);

@@ -29,17 +29,6 @@ struct ConvGeom {
 // Bound by the FMA pipes (and by issue: 35 instructions per 32 FMAs).  Measured on the 3x3 layers of the CIFAR-sized
 // networks at batch 128: 16 channels at 32x32: 157 -> 33 us forward, 176 -> 27 us
 // data gradient, 371 -> 49 us weight gradient (the element-wise kernel spent its time on index divisions and scalar loads).
-struct FastDiv {                     // n / d for 0 <= n < 2^31 by multiplication (Granlund and Montgomery, 1994)
-    uint32_t d, mul, sh;
-    __device__ __forceinline__ uint32_t div(uint32_t n) const { return (__umulhi(mul, n) + n) >> sh; }
-    __device__ __forceinline__ void divmod(uint32_t n, uint32_t &q, uint32_t &r) const { q = div(n); r = n - q * d; }
-};
-static FastDiv fast_div(uint32_t d) {
-    FastDiv f; f.d = d; f.sh = 0;
-    while ((1ull << f.sh) < d) f.sh++;
-    f.mul = (uint32_t)(((1ull << 32) * ((1ull << f.sh) - d)) / d + 1);
-    return f;
-}
 template <class T> __device__ __forceinline__ float4 ldq(const T *p);
 template <> __device__ __forceinline__ float4 ldq<float>(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 template <> __device__ __forceinline__ float4 ldq<bf16>(const bf16 *p) {

@@ -142,13 +142,20 @@ __global__ void __launch_bounds__(256, 4) col_reduce_kernel(Pair t, const float 
     }
     float4 *sm4 = reinterpret_cast<float4 *>(red);       // [256][2]
     sm4[tid * 2] = s; sm4[tid * 2 + 1] = ss;
-    __syncthreads();
-    if (ty == 0 && valid) {
-        for (int y = 1; y < RPP; y++) {
-            const float4 a = sm4[(y * SW + tx) * 2], b = sm4[(y * SW + tx) * 2 + 1];
+    // the threads of a slab column, halved until one is left (narrow tensors: up to 128 of them)
+    for (int n = RPP; n > 1;) {
+        const int h = (n + 1) >> 1;
+        __syncthreads();
+        if (valid && ty + h < n) {
+            const float4 a = sm4[((ty + h) * SW + tx) * 2], b = sm4[((ty + h) * SW + tx) * 2 + 1];
             s.x += a.x; s.y += a.y; s.z += a.z; s.w += a.w;
             ss.x += b.x; ss.y += b.y; ss.z += b.z; ss.w += b.w;
+            sm4[tid * 2] = s; sm4[tid * 2 + 1] = ss;
         }
+        n = h;
+    }
+    __syncthreads();
+    if (ty == 0 && valid) {
         float *mine = part + ((size_t)blockIdx.x * C4 + q) * 8;
         st4(mine, s); st4(mine + 4, ss);
         __threadfence();
