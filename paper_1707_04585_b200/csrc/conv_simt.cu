@@ -26,6 +26,10 @@ struct ConvGeom {
 // warp holds 64 x 16 accumulators, 8 x 4 per thread, so that one K step costs three 16-byte shared-memory reads (one wavefront
 // each) per 32 FMAs.  K runs in chunks of 16 through two shared-memory buffers; the next chunk's quads are on their way
 // from global memory while this one is multiplied.
+// A sum of K products is taken in runs of 256 that are then added: the rounding error of one serial sum grows with the size
+// of the running value (K = 7488, a 3x3 layer of 832 channels: 2e-7 to 5e-7 of the result's deviation, enough to turn the sign
+// of a BN output close to zero), the runs keep it several times smaller, for 1.8 % of the time of a fp32 train
+// step of the 38-layer network.
 // Bound by the FMA pipes (and by issue: 35 instructions per 32 FMAs).  Measured on the 3x3 layers of the CIFAR-sized
 // networks at batch 128: 16 channels at 32x32: 157 -> 33 us forward, 176 -> 27 us
 // data gradient, 371 -> 49 us weight gradient (the element-wise kernel spent its time on index divisions and scalar loads).
@@ -164,6 +168,7 @@ template <int WM, int WN, int WK> struct GemmTile {
     static_assert(WM * WN * WK == 8, "eight warps");
 };
 
+constexpr int kRun = 16;            // chunks of 16
 template <int WM, int WN, int WK, class AL, class BL, class EP>
 __global__ void __launch_bounds__(256, 2) conv_gemm_kernel(AL al, BL bl, EP ep, int M, int N, int K, int k_per_split) {
     pdl_enter();
@@ -201,13 +206,13 @@ __global__ void __launch_bounds__(256, 2) conv_gemm_kernel(AL al, BL bl, EP ep, 
             else *reinterpret_cast<float4 *>(Bs + bk * PB + bn) = vb;
         }
     };
-    float acc[8][4];
+    float acc[8][4], sum[8][4];               // products of the current run of kRun chunks; sum of the runs before it
 #pragma unroll
     for (int i = 0; i < 8; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = 0.f;
+        for (int j = 0; j < 4; j++) acc[i][j] = sum[i][j] = 0.f;
     auto next_chunk = [&](int k) { while (k < kend && al.skip(m0, m0 + BM - 1, k)) k += BK; return k; };
-    int k0 = next_chunk(kbeg), buf = 0;
+    int k0 = next_chunk(kbeg), buf = 0, run = 0;
     if (k0 < kend) { fetch(k0); put(sm, sm + BK * PA); }
     __syncthreads();
     while (k0 < kend) {
@@ -226,11 +231,22 @@ __global__ void __launch_bounds__(256, 2) conv_gemm_kernel(AL al, BL bl, EP ep, 
                 acc[i][2] = fmaf(a[i], b.z, acc[i][2]); acc[i][3] = fmaf(a[i], b.w, acc[i][3]);
             }
         }
+        if (++run == kRun) {
+            run = 0;
+#pragma unroll
+            for (int i = 0; i < 8; i++)
+#pragma unroll
+                for (int j = 0; j < 4; j++) { sum[i][j] += acc[i][j]; acc[i][j] = 0.f; }
+        }
         buf ^= 1;
         if (kn < kend) put(sm + buf * T::kStage, sm + buf * T::kStage + BK * PA);
         __syncthreads();
         k0 = kn;
     }
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) acc[i][j] += sum[i][j];
     if (WK > 1) {
         // the warps that share a tile are added in order
         float *red = sm + (size_t)(wm * WN + wn) * 1024 + lane * 4;

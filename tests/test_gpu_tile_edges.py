@@ -1,0 +1,57 @@
+"""Blocks at the sizes where the tiles, splits and dispatch rules of the kernels end: one row or column
+more than a tile holds, widths that leave padded operand planes, reductions of one row and of many.
+Everything is compared with the float64 oracle under the stated tolerances (tests/parity.py: 1e-4 in the
+strict mode, 2e-2 outputs and 5e-2 gradients in the bf16 mode), which bound rounding at any size here:
+the longest sum has 1224 products."""
+import pytest
+
+from paper_1707_04585_b200 import binding as B
+from paper_1707_04585_b200 import synthetic as syn
+from tests import test_gpu_parity as tp
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = B.Context(0)
+    yield c
+    B.revnet_check_device(c)
+    c.close()
+
+
+@pytest.mark.parametrize("kind,N,H,W,c,w", [
+    ("basic", 2, 3, 3, 8, 0),             # one operand plane, less than one tile
+    ("basic", 2, 281, 283, 8, 0),         # rows longer than a tile; more tiles per CTA than one operand segment holds
+    ("basic", 3, 2, 200, 24, 0),          # three planes, two-row images
+    ("basic", 6, 9, 11, 40, 0),           # five planes
+    ("basic", 4, 13, 13, 56, 0),          # seven planes, 56 of 64 output columns
+    ("basic", 2, 16, 16, 64, 0),          # the widest layer with its BN and ReLU inside
+    ("bottleneck", 6, 9, 9, 32, 12),      # 1x1; rows of 48 bytes: 16-byte accesses
+    ("bottleneck", 8, 9, 9, 136, 72),     # weight packs with padded rows (136 -> 256, 72 -> 80) and columns (136 -> 144)
+])
+def test_bf16_blocks_at_tile_edges(ctx, kind, N, H, W, c, w):
+    tp.run_block_case(ctx, syn.BlockCfg(N, H, W, c, w, kind, seed=900 + c), 0, jitter=True, inplace=True)
+
+
+@pytest.mark.parametrize("kind,N,H,W,c,w", [
+    ("basic", 1, 5, 13, 4, 0),            # 65 pixels: one more than the shortest tile; columns 4 of 16
+    ("basic", 1, 275, 275, 16, 0),        # 256-row tiles, the last one of 105 rows
+    ("basic", 1, 150, 253, 20, 0),        # 32-column tiles, the tall ones
+    ("basic", 1, 139, 137, 36, 0),        # 64-column tiles
+    ("basic", 2, 11, 7, 68, 0),           # two column tiles, the second of 4 columns
+    ("bottleneck", 1, 3, 3, 132, 4),      # column sums of nine rows: two slabs of 17 and 16 quads, and one quad
+    ("bottleneck", 2, 37, 41, 260, 136),  # three slabs (22, 22, 21), several row ranges; sums of 1224 products
+])
+def test_strict_blocks_at_tile_edges(ctx, kind, N, H, W, c, w):
+    tp.run_block_case(ctx, syn.BlockCfg(N, H, W, c, w, kind, seed=900 + c), 1, jitter=True, inplace=True)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("N,H,cin,cout,stride", [
+    (3, 6, 8, 24, 2),                     # 27 pixels in each parity class of the data gradient
+    (2, 10, 40, 72, 2),
+    (2, 9, 24, 136, 1),
+])
+def test_transitions_at_tile_edges(ctx, mode, N, H, cin, cout, stride):
+    tp.run_transition_case(ctx, mode, N, H, cin, cout, 3, stride, False)
