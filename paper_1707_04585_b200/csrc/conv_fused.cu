@@ -110,26 +110,6 @@ __device__ __forceinline__ uint32_t relu_pack2(float lo, float hi) {
     asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
-// eight consecutive 32-bit words; wide: one 32-byte access (the address is a multiple of 32), else two of 16 bytes
-__device__ __forceinline__ void ld8(const void *p, uint32_t (&v)[8], bool wide) {
-    if (wide)
-        asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(p) : "memory");
-    else {
-        const uint4 a = reinterpret_cast<const uint4 *>(p)[0], b = reinterpret_cast<const uint4 *>(p)[1];
-        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-    }
-}
-__device__ __forceinline__ void st8(void *p, const uint32_t (&v)[8], bool wide) {
-    if (wide)
-        asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
-                     ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
-    else {
-        reinterpret_cast<uint4 *>(p)[0] = make_uint4(v[0], v[1], v[2], v[3]);
-        reinterpret_cast<uint4 *>(p)[1] = make_uint4(v[4], v[5], v[6], v[7]);
-    }
-}
-
 // a bounded wait of a whole warp: lane 0 polls
 __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, int lane) {
     bool ok = true;

@@ -1674,10 +1674,10 @@ bool conv_wgrad_tc_batch(Exec &ex, int n, const void *const *gq, const void *con
             if (max_slice >= 524288) {
                 size_t tiles = (max_slice + 1023) / 1024; if (tiles > (size_t)ex.ctx->sm_count * 8) tiles = (size_t)ex.ctx->sm_count * 8;
                 dim3 grid((unsigned)tiles, (unsigned)n_sums);
-                launch(ex, splitk_sum_tiled_kernel, grid, 256, 0, sums);
+                launch_stream(ex, sum_bytes, 20, splitk_sum_tiled_kernel, grid, 256, 0, sums);
             } else {
                 dim3 grid((unsigned)((max_slice + 31) / 32), (unsigned)n_sums);
-                launch(ex, splitk_sum_batch_kernel, grid, 256, 0, sums);
+                launch_stream(ex, sum_bytes, 6, splitk_sum_batch_kernel, grid, 256, 0, sums);
             }
             ex.check("splitk_sum", sum_bytes);
         }

@@ -28,6 +28,7 @@ def ctx():
     ("basic", 4, 13, 13, 56, 0),          # seven planes, 56 of 64 output columns
     ("basic", 2, 16, 16, 64, 0),          # the widest layer with its BN and ReLU inside
     ("bottleneck", 6, 9, 9, 32, 12),      # 1x1; rows of 48 bytes: 16-byte accesses
+    ("bottleneck", 1, 97, 99, 520, 8),    # streaming kernels with 32-byte accesses: 65 octets of channels, three rows per pass
     ("bottleneck", 8, 9, 9, 136, 72),     # weight packs with padded rows (136 -> 256, 72 -> 80) and columns (136 -> 144)
 ])
 def test_bf16_blocks_at_tile_edges(ctx, kind, N, H, W, c, w):
@@ -41,6 +42,7 @@ def test_bf16_blocks_at_tile_edges(ctx, kind, N, H, W, c, w):
     ("basic", 1, 139, 137, 36, 0),        # 64-column tiles
     ("basic", 2, 11, 7, 68, 0),           # two column tiles, the second of 4 columns
     ("bottleneck", 1, 3, 3, 132, 4),      # column sums of nine rows: two slabs of 17 and 16 quads, and one quad
+    ("bottleneck", 1, 97, 99, 520, 8),    # 32-byte accesses in the streaming kernels
     ("bottleneck", 2, 37, 41, 260, 136),  # three slabs (22, 22, 21), several row ranges; sums of 1224 products
 ])
 def test_strict_blocks_at_tile_edges(ctx, kind, N, H, W, c, w):
