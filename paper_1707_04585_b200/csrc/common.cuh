@@ -425,13 +425,14 @@ void tc_pack_now(Exec &ex, const float *W, bf16 *out, int cin, int cout, int k, 
 // bf16 weight packs of the tensor-core kernels, built once per train step
 // One layer's weights into its forward pack f [co_f][tap][ci_f] and / or its data-gradient pack d [ci_d][mirrored tap][co_d]
 // (either may be null); the pads of the packs are filled with zeros.
-struct PackJob { const float *W; bf16 *f, *d; int Co, Ci, k, co_f, ci_f, ci_d, co_d; };
+// tile0: tiles of the jobs before it in the table of a step.
+struct PackJob { const float *W; bf16 *f, *d; int Co, Ci, k, co_f, ci_f, ci_d, co_d, tile0; };
 constexpr int kPackJobs = 6;           // a block has at most two functions of three layers
 struct PackJobs { PackJob job[kPackJobs]; };
 size_t tc_pack_elems(int cin, int cout, int k, bool transposed);
 PackJob tc_pack_job(const float *W, bf16 *f, bf16 *d, int cin, int cout, int k);
 int tc_pack_tiles(const PackJob &j);                                          // tiles (blocks' worth of work) of a job
-void tc_pack_batch(Exec &ex, const PackJob *jobs_dev, int n_jobs, double bytes, int max_tiles);
+void tc_pack_batch(Exec &ex, const PackJob *jobs_dev, int n_jobs, double bytes, int tiles);      // tiles: of all jobs
 void tc_pack_list(Exec &ex, const PackJobs &jobs, int n_jobs);                // the same for a few layers, table passed by value
 
 // ---------------------------------------------------------------- block.cu

@@ -744,11 +744,11 @@ __device__ __forceinline__ uint2 pack_bf16x4(float a, float b, float c, float d)
 }
 __host__ __device__ __forceinline__ int pack_ct(const PackJob &j) { const int n = j.ci_f > j.ci_d ? j.ci_f : j.ci_d; return (n + kPackTile - 1) / kPackTile; }
 __host__ __device__ __forceinline__ int pack_rt(const PackJob &j) { const int n = j.co_f > j.co_d ? j.co_f : j.co_d; return (n + kPackTile - 1) / kPackTile; }
-__device__ __forceinline__ void pack_layer(const PackJob &j, int first, int step) {
+__device__ __forceinline__ void pack_layer(const PackJob &j, int first, int end, int step) {
     __shared__ float tile[kPackTile][kPackTile + 1];
-    const int taps = j.k * j.k, ct = pack_ct(j), n_tiles = ct * taps * pack_rt(j);
+    const int taps = j.k * j.k, ct = pack_ct(j);
     const int lx = threadIdx.x & 15, ly = threadIdx.x >> 4;
-    for (int t = first; t < n_tiles; t += step) {
+    for (int t = first; t < end; t += step) {
         const int ci0 = (t % ct) * kPackTile, tap = (t / ct) % taps, co0 = t / (ct * taps) * kPackTile;
         const int ci = ci0 + 4 * lx;
         float4 v[4];
@@ -777,15 +777,33 @@ __device__ __forceinline__ void pack_layer(const PackJob &j, int first, int step
         __syncthreads();
     }
 }
-// every layer of a step (table in device memory) / of a block or a single layer (table by value); blockIdx.y picks the layer
-__global__ void __launch_bounds__(256) pack_weights_batch_kernel(const PackJob *__restrict__ jobs) {
+// Every layer of a step (table in device memory): a CTA takes `run` consecutive tiles of all of them and finds its first layer
+// with a 32-way search.  (With one row of CTAs per layer, as many as the largest layer has tiles, the launch of nearly two
+// hundred thousand mostly empty CTAs took 202 us in the step of the 164-layer network; now 23 us.)
+__global__ void __launch_bounds__(256) pack_weights_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int tiles, int run) {
     pdl_enter();
-    const PackJob j = jobs[blockIdx.y];
-    pack_layer(j, blockIdx.x, gridDim.x);
+    int t = blockIdx.x * run;
+    const int end = t + run < tiles ? t + run : tiles, lane = threadIdx.x & 31;
+    int lo = 0, len = n_jobs;
+    while (true) {                               // the last job with tile0 <= t
+        const int step = (len + 31) >> 5;
+        const int n = __popc(__ballot_sync(0xffffffffu, lane * step < len && jobs[lo + lane * step].tile0 <= t)) - 1;
+        lo += n * step;
+        if (step <= 1) break;
+        len = len - n * step < step ? len - n * step : step;
+    }
+    while (t < end) {
+        const PackJob j = jobs[lo++];
+        const int job_end = j.tile0 + pack_ct(j) * pack_rt(j) * j.k * j.k, stop = job_end < end ? job_end : end;
+        pack_layer(j, t - j.tile0, stop - j.tile0, 1);
+        t = stop;
+    }
 }
+// the layers of a block, or a single one (table by value); blockIdx.y picks the layer
 __global__ void __launch_bounds__(256) pack_weights_kernel(const __grid_constant__ PackJobs jobs) {
     pdl_enter();
-    pack_layer(jobs.job[blockIdx.y], blockIdx.x, gridDim.x);
+    const PackJob &j = jobs.job[blockIdx.y];
+    pack_layer(j, blockIdx.x, pack_ct(j) * pack_rt(j) * j.k * j.k, gridDim.x);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
@@ -1714,7 +1732,7 @@ size_t tc_pack_elems(int cin, int cout, int k, bool transposed) {
     return (size_t)rp * k * k * cp;
 }
 PackJob tc_pack_job(const float *W, bf16 *f, bf16 *d, int cin, int cout, int k) {
-    PackJob j{W, f, d, cout, cin, k, 0, 0, 0, 0};
+    PackJob j{W, f, d, cout, cin, k, 0, 0, 0, 0, 0};
     if (f) pack_dims(cout, cin, j.co_f, j.ci_f);
     if (d) pack_dims(cin, cout, j.ci_d, j.co_d);
     return j;
@@ -1723,13 +1741,14 @@ int tc_pack_tiles(const PackJob &j) { return pack_ct(j) * pack_rt(j) * j.k * j.k
 static double pack_job_bytes(const PackJob &j) {
     return (double)j.Co * j.Ci * j.k * j.k * 4 + 2.0 * j.k * j.k * ((double)j.co_f * j.ci_f + (double)j.ci_d * j.co_d);
 }
-// blocks per layer sized for the largest one, at most eight per SM
-void tc_pack_batch(Exec &ex, const PackJob *jobs_dev, int n_jobs, double bytes, int max_tiles) {
+// one tile per CTA while that leaves at most 32 CTAs per SM, else four
+void tc_pack_batch(Exec &ex, const PackJob *jobs_dev, int n_jobs, double bytes, int tiles) {
     if (ex.dry || n_jobs == 0) return;
-    const int cap = ex.ctx->sm_count * 8;
-    launch(ex, pack_weights_batch_kernel, dim3((unsigned)(max_tiles < cap ? max_tiles : cap), (unsigned)n_jobs), 256, 0, jobs_dev);
+    const int run = tiles > ex.ctx->sm_count * 32 ? 4 : 1;
+    launch(ex, pack_weights_batch_kernel, (tiles + run - 1) / run, 256, 0, jobs_dev, n_jobs, tiles, run);
     ex.check("pack_weights_batch", bytes);
 }
+// blocks per layer sized for the largest one, at most eight per SM
 void tc_pack_list(Exec &ex, const PackJobs &jobs, int n_jobs) {
     if (ex.dry || n_jobs == 0) return;
     int tiles = 1; double bytes = 0;

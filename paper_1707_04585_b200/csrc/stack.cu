@@ -110,7 +110,7 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
         }
         std::vector<PackJob> jobs;
         double bytes = 0;
-        int max_tiles = 0;
+        int tiles = 0;
         for (LayerSlot *l : slots) {
             l->wp_f = l->wp_d = nullptr;
             if (ex.mode != 0 || l->cin % 8 || l->cout % 8) continue;
@@ -119,14 +119,15 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
             l->wp_f = f; l->wp_d = dd;
             jobs.push_back(tc_pack_job(params + l->off_W, f, dd, l->cin, l->cout, l->k));
             bytes += (double)(nf + nd) * 2 + (double)l->cin * l->cout * l->k * l->k * 4;
-            max_tiles = std::max(max_tiles, tc_pack_tiles(jobs.back()));
+            jobs.back().tile0 = tiles;
+            tiles += tc_pack_tiles(jobs.back());
         }
         PackJob *jobs_dev = ex.ws.get<PackJob>(jobs.size() + 1);
         if (!ex.dry && !jobs.empty()) {
             if (jobs.size() * sizeof(PackJob) <= pl->pack_host_bytes) {
                 memcpy(pl->pack_host, jobs.data(), jobs.size() * sizeof(PackJob));
                 cudaMemcpyAsync(jobs_dev, pl->pack_host, jobs.size() * sizeof(PackJob), cudaMemcpyHostToDevice, ex.stream);
-                tc_pack_batch(ex, jobs_dev, (int)jobs.size(), bytes, max_tiles);
+                tc_pack_batch(ex, jobs_dev, (int)jobs.size(), bytes, tiles);
             } else {
                 for (LayerSlot *l : slots) l->wp_f = l->wp_d = nullptr;   // no staging room: pack per call instead
             }
