@@ -103,6 +103,20 @@ struct Pair {
             *reinterpret_cast<int *>(o) = iv;
         }
     }
+    // the same for two channels, the partner's words already loaded
+    __device__ __forceinline__ void couple2_with(size_t row, int ch, float2 v, float2 p, int sign) const {
+        float *o = at(row, ch);
+        if (q == 0.f) {
+            if (sign > 0) v = make_float2(p.x + v.x, p.y + v.y);
+            else if (sign < 0) v = make_float2(p.x - v.x, p.y - v.y);
+            *reinterpret_cast<float2 *>(o) = v;
+        } else {
+            int2 iv = make_int2(__float2int_rn(v.x * (1.f / q)), __float2int_rn(v.y * (1.f / q)));
+            const int2 ip = make_int2(__float_as_int(p.x), __float_as_int(p.y));
+            if (sign) iv = sign > 0 ? make_int2(ip.x + iv.x, ip.y + iv.y) : make_int2(ip.x - iv.x, ip.y - iv.y);
+            *reinterpret_cast<int2 *>(o) = iv;
+        }
+    }
     // store v in the tensor's format; returns the values as stored (dequantised)
     __device__ __forceinline__ float4 store4(size_t row, int ch, float4 v) const {
         float *o = at(row, ch);

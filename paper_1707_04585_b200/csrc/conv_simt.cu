@@ -6,7 +6,7 @@
 //   dgrad: da[q,ci]    = sum_{kh,kw,co} g[p,co] * W[co,kh,kw,ci],  p*s + (kh,kw) - pad = q
 //   wgrad: dW[co,kh,kw,ci] = sum_p g[p,co] * a[p (+) (kh,kw), ci]
 //
-// Two kernels.  conv_gemm_kernel takes every layer whose channel counts are multiples of four (all BN-ReLU-conv layers):
+// Three kernels.  conv3x3_direct_kernel takes fp32 3x3 stride-1 layers (forward and data gradient), conv_gemm_kernel every other layer whose channel counts are multiples of four (all BN-ReLU-conv layers):
 // quads of channels are loaded as vectors, a thread's pixel is decoded once, and the product is register-tiled.
 // gemm_simt_kernel loads element by element and is left for the stem convolution's odd channel counts (an image has
 // three), where the kernels of stem.cu do not take its size.
@@ -33,6 +33,7 @@ struct ConvGeom {
 // Bound by the FMA pipes (and by issue: 35 instructions per 32 FMAs).  Measured on the 3x3 layers of the CIFAR-sized
 // networks at batch 128: 16 channels at 32x32: 157 -> 33 us forward, 176 -> 27 us
 // data gradient, 371 -> 49 us weight gradient (the element-wise kernel spent its time on index divisions and scalar loads).
+// The forward pass and the data gradient of most 3x3 stride-1 layers now take the direct kernel further down.
 template <class T> __device__ __forceinline__ float4 ldq(const T *p);
 template <> __device__ __forceinline__ float4 ldq<float>(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 template <> __device__ __forceinline__ float4 ldq<bf16>(const bf16 *p) {
@@ -149,11 +150,26 @@ struct OutCouple {                            // out = partner + sign*acc (sign 
     static constexpr bool kTransposed = false;
     Pair out, partner; int sign;
     __device__ __forceinline__ void store(size_t row, int n, float4 v) const { out.couple4(row, n, v, partner, sign); }
+    // eight rows `step` apart, columns n and n + 1; the partner's loads leave before the first store (it may be in place)
+    __device__ __forceinline__ void store8(size_t row, int step, int live, int n, const float (&v)[8][2]) const {
+        float2 p[8];
+        if (sign)
+#pragma unroll
+            for (int r = 0; r < 8; r++) p[r] = *reinterpret_cast<const float2 *>(partner.at(row + (size_t)(r < live ? r : 0) * step, n));
+#pragma unroll
+        for (int r = 0; r < 8; r++)
+            if (r < live) out.couple2_with(row + (size_t)r * step, n, make_float2(v[r][0], v[r][1]), p[r], sign);
+    }
 };
 struct OutPlain {
     static constexpr bool kTransposed = false;
     float *out; int N;
     __device__ __forceinline__ void store(size_t row, int n, float4 v) const { *reinterpret_cast<float4 *>(out + row * N + n) = v; }
+    __device__ __forceinline__ void store8(size_t row, int step, int live, int n, const float (&v)[8][2]) const {
+#pragma unroll
+        for (int r = 0; r < 8; r++)
+            if (r < live) *reinterpret_cast<float2 *>(out + (row + (size_t)r * step) * N + n) = make_float2(v[r][0], v[r][1]);
+    }
 };
 struct OutSplit {                             // slice z of a split reduction: four consecutive M of column n, out[z][n][M]
     static constexpr bool kTransposed = true;
@@ -307,6 +323,181 @@ static void launch_pixels(Exec &ex, AL al, BL bl, EP ep, int M, int N, int K) {
     else launch_tile<1, 2, 4>(ex, al, bl, ep, M, N, K, 1, K);
 }
 
+// ------------------------------------------------------------------ 3x3 stride 1, forward and data gradient: direct
+// out[p, n] = sum over taps and channels r of in[p + tap, r] * w[n][tap][r] with the input tile staged once, halo included,
+// instead of once per tap (the implicit GEMM above spends half its instructions on that).
+// A warp takes 8 rows x 4 columns of an image and 16 output channels: a lane one column, two output channels, eight rows.  Per
+// channel quad and column tap a lane reads ten input quads (eight rows and the halo, shared by the three row taps) and six weight
+// quads for 192 FMAs: 16 wavefronts of shared memory.  (Packed pairs, fma.rn.f32x2, reach 43.6 TFLOP/s here where single FMAs
+// reach 56, and need a second partial sum per output.)
+// A CTA is NW warps: CB groups of 16 output channels, NW / CB of those tiles (gx columns x gy rows x the rest images).  The input
+// channels are staged in chunks of up to 32 (pixel pitch: an odd number of quads, so that the four columns of a warp and their
+// 16-byte reads fall into different banks) by asynchronous copies into two buffers, the next chunk or tile while this one is
+// worked on; the sums of a chunk, at most 288 products each, are added to the running sums.
+// Bound by the FMA pipes, with about half of the time outside them: the start of a launch with one to four tiles per SM, the
+// copies' address arithmetic, and (8x8 images) too few warps.  Measured at batch 128, whole launches: 16 channels at 32x32
+// 33 -> 21 us, 32 at 16x16 41 -> 21 us, 56 at 8x8 41 -> 32 us against the implicit GEMM above.
+struct DirectGeom {
+    int N, H, W, Ci, Co;                          // Ci: channels summed over, Co: produced
+    int NW, gx, gy, gi, CB, kc, pitch;            // warps of a CTA, of a tile, channels per chunk, floats per staged pixel
+    int tx, ty, tiles;                            // tiles of an image, of all
+    FastDiv dtx, dty, dq, dcol, drow;             // by tx, ty, quads per chunk, staged columns, staged rows
+};
+// four channels r .. r + 3 of tap `tap` (of the sum above) for output n; forward: W[n][tap][r], data gradient: W[r][8 - tap][n]
+struct DirectFprop {
+    static constexpr bool kAlongK = true;
+    const float *w; int Ci;
+    __device__ __forceinline__ float4 along(int n, int tap, int r) const { return ldq(w + ((size_t)n * 9 + tap) * Ci + r); }
+};
+struct DirectDgrad {
+    static constexpr bool kAlongK = false;
+    const float *w; int Co;
+    __device__ __forceinline__ float4 along(int n, int tap, int r) const { return ldq(w + ((size_t)r * 9 + 8 - tap) * Co + n); }     // n .. n + 3
+};
+// weights of a chunk in shared memory: [tap][quad of r][output n of the CTA, in each 16 the even ones first][4]
+__device__ __forceinline__ int direct_slot(int n) { return (n & ~15) | ((n & 1) << 3) | ((n & 15) >> 1); }
+
+template <class WL, class EP>
+__global__ void __launch_bounds__(256, 2) conv3x3_direct_kernel(const float *__restrict__ in, WL wl, EP ep, const __grid_constant__ DirectGeom g) {
+    extern __shared__ float sm[];
+    const int tid = threadIdx.x, nth = blockDim.x, warp = tid >> 5, lane = tid & 31, lx = lane & 3, lg = lane >> 2;
+    const int wpx = g.NW / g.CB, wt = warp % wpx, wc = warp / wpx;                  // tile and channel group of this warp
+    const int wx = wt % g.gx, wy = (wt / g.gx) % g.gy, wi = wt / (g.gx * g.gy);
+    const int cols = g.gx * 4 + 2, rows = g.gy * 8 + 2, nb = g.CB * 16, n0 = blockIdx.y * nb;
+    const int quads = g.kc / 4, positions = rows * cols * g.gi, buf_floats = positions * g.pitch;
+    float *acts = sm + 9 * g.kc * nb;
+    const int at0 = ((wi * rows + wy * 8) * cols + wx * 4 + lx) * g.pitch;
+    const float *myw = sm + wc * 64 + lg * 4;
+    const int rowp = cols * g.pitch;
+    pdl_enter();
+    int x0, y0, i0;
+    auto place = [&](int t) {
+        uint32_t r0, bx, by, bi;
+        g.dtx.divmod((uint32_t)t, r0, bx); g.dty.divmod(r0, bi, by);
+        x0 = (int)bx * g.gx * 4; y0 = (int)by * g.gy * 8; i0 = (int)bi * g.gi;
+    };
+    // chunk c0 of tile t into buffer b; zeros outside the image and beyond the last channel
+    auto stage = [&](int t, int c0, int b) {
+        place(t);
+        float *dst = acts + b * buf_floats;
+        for (int e = tid; e < positions * quads; e += nth) {
+            uint32_t pos, q, row, col, img, ry;
+            g.dq.divmod((uint32_t)e, pos, q); g.dcol.divmod(pos, row, col); g.drow.divmod(row, img, ry);
+            const int x = x0 + (int)col - 1, y = y0 + (int)ry - 1, i = i0 + (int)img;
+            const bool ok = (unsigned)x < (unsigned)g.W && (unsigned)y < (unsigned)g.H && i < g.N && c0 + (int)q * 4 < g.Ci;
+            const float *src = in + (ok ? (((size_t)i * g.H + y) * g.W + x) * g.Ci + c0 + q * 4 : 0);
+            const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + (size_t)pos * g.pitch + q * 4);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
+        }
+    };
+    int t = blockIdx.x, c0 = 0, b = 0;
+    bool weights = true;
+    float sum[8][2];
+#pragma unroll
+    for (int r = 0; r < 8; r++) sum[r][0] = sum[r][1] = 0.f;
+    if (t < g.tiles) stage(t, 0, 0);
+    while (t < g.tiles) {
+        const int cq = (g.Ci - c0 < g.kc ? g.Ci - c0 : g.kc) / 4;                   // quads of this chunk
+        __syncthreads();                                                            // the chunk before has been read
+        if (weights) {
+            if (WL::kAlongK) {
+                for (int e = tid; e < 9 * nb * quads; e += nth) {
+                    uint32_t k, q; g.dq.divmod((uint32_t)e, k, q);
+                    const int tap = (int)k % 9, n = (int)k / 9;
+                    const float4 v = n0 + n < g.Co && (int)q < cq ? wl.along(n0 + n, tap, c0 + (int)q * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    *reinterpret_cast<float4 *>(sm + ((size_t)(tap * quads + (int)q) * nb + direct_slot(n)) * 4) = v;
+                }
+            } else {
+                const int nq = nb / 4;
+                for (int e = tid; e < 9 * g.kc * nq; e += nth) {
+                    const int n = e % nq * 4, k = e / nq, tap = k % 9, r = k / 9;
+                    const float4 v = n0 + n < g.Co && c0 + r < g.Ci ? wl.along(n0 + n, tap, c0 + r) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    float *d = sm + (size_t)(tap * quads + r / 4) * nb * 4 + (r & 3);
+                    d[direct_slot(n) * 4] = v.x; d[direct_slot(n + 1) * 4] = v.y; d[direct_slot(n + 2) * 4] = v.z; d[direct_slot(n + 3) * 4] = v.w;
+                }
+            }
+            weights = g.kc < g.Ci;
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        int tn = t, cn = c0 + g.kc;
+        if (cn >= g.Ci) { tn += gridDim.x; cn = 0; }
+        if (tn < g.tiles) stage(tn, cn, b ^ 1);
+        const float *myact = acts + b * buf_floats + at0;
+        float acc[8][2];
+#pragma unroll
+        for (int r = 0; r < 8; r++) acc[r][0] = acc[r][1] = 0.f;
+#pragma unroll 1
+        for (int q = 0; q < cq; q++) {
+#pragma unroll
+            for (int kw = 0; kw < 3; kw++) {
+                float4 a[10];
+#pragma unroll
+                for (int r = 0; r < 10; r++) a[r] = *reinterpret_cast<const float4 *>(myact + r * rowp + kw * g.pitch + q * 4);
+#pragma unroll
+                for (int kh = 0; kh < 3; kh++) {
+                    const float *w = myw + (size_t)((kh * 3 + kw) * quads + q) * nb * 4;
+                    const float4 w0 = *reinterpret_cast<const float4 *>(w), w1 = *reinterpret_cast<const float4 *>(w + 32);
+#pragma unroll
+                    for (int r = 0; r < 8; r++) { acc[r][0] = fmaf(a[r + kh].x, w0.x, acc[r][0]); acc[r][1] = fmaf(a[r + kh].x, w1.x, acc[r][1]); }
+#pragma unroll
+                    for (int r = 0; r < 8; r++) { acc[r][0] = fmaf(a[r + kh].y, w0.y, acc[r][0]); acc[r][1] = fmaf(a[r + kh].y, w1.y, acc[r][1]); }
+#pragma unroll
+                    for (int r = 0; r < 8; r++) { acc[r][0] = fmaf(a[r + kh].z, w0.z, acc[r][0]); acc[r][1] = fmaf(a[r + kh].z, w1.z, acc[r][1]); }
+#pragma unroll
+                    for (int r = 0; r < 8; r++) { acc[r][0] = fmaf(a[r + kh].w, w0.w, acc[r][0]); acc[r][1] = fmaf(a[r + kh].w, w1.w, acc[r][1]); }
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 8; r++) { sum[r][0] += acc[r][0]; sum[r][1] += acc[r][1]; }
+        if (tn != t) {
+            place(t);
+            const int n = n0 + wc * 16 + 2 * lg, x = x0 + wx * 4 + lx, y = y0 + wy * 8, i = i0 + wi;
+            if (n < g.Co && x < g.W && i < g.N) ep.store8(((size_t)i * g.H + y) * g.W + x, g.W, g.H - y, n, sum);
+#pragma unroll
+            for (int r = 0; r < 8; r++) sum[r][0] = sum[r][1] = 0.f;
+        }
+        t = tn; c0 = cn; b ^= 1;
+    }
+}
+
+// Tiles of a layer: false where less than half of their pixels would lie inside an image.  Four warps per CTA where eight would
+// leave SMs without one.
+static bool direct_shape(int N, int H, int W, int Ci, int Co, int sm, DirectGeom &g) {
+    g.N = N; g.H = H; g.W = W; g.Ci = Ci; g.Co = Co;
+    g.CB = Co > 16 ? 2 : 1;
+    g.kc = Ci < 32 ? Ci : 32;
+    g.pitch = (g.kc / 4) % 2 ? g.kc : g.kc + 4;
+    for (g.NW = 8; g.NW >= 4; g.NW -= 4) {
+        const int wpx = g.NW / g.CB, nbs = (Co + g.CB * 16 - 1) / (g.CB * 16);
+        g.gx = W <= 4 ? 1 : (W <= 8 ? 2 : 4);
+        if (g.gx > wpx) g.gx = wpx;
+        g.gy = wpx / g.gx;
+        while (g.gy > 1 && (g.gy >> 1) * 8 >= H) g.gy >>= 1;
+        g.gi = wpx / (g.gx * g.gy);
+        g.tx = (W + g.gx * 4 - 1) / (g.gx * 4); g.ty = (H + g.gy * 8 - 1) / (g.gy * 8);
+        const long long tiles = (long long)g.tx * g.ty * ((N + g.gi - 1) / g.gi);
+        if (tiles * wpx * 32 > 2ll * N * H * W || tiles > (1 << 28)) { if (g.NW == 8) continue; return false; }
+        g.tiles = (int)tiles;
+        if (tiles * nbs >= sm || g.NW == 4) break;
+    }
+    g.dtx = fast_div(g.tx); g.dty = fast_div(g.ty); g.dq = fast_div(g.kc / 4); g.dcol = fast_div(g.gx * 4 + 2); g.drow = fast_div(g.gy * 8 + 2);
+    return true;
+}
+template <class WL, class EP>
+static void launch_direct(Exec &ex, const float *in, WL wl, EP ep, const DirectGeom &g) {
+    const int smem = (9 * g.kc * g.CB * 16 + 2 * (g.gx * 4 + 2) * (g.gy * 8 + 2) * g.gi * g.pitch) * 4;      // at most 157 KB
+    static OncePerDevice once;
+    if (once.first(ex.ctx->device)) cudaFuncSetAttribute(conv3x3_direct_kernel<WL, EP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    const int nbs = (g.Co + g.CB * 16 - 1) / (g.CB * 16);
+    int per_sm = 16 / g.NW, fit = 227 * 1024 / (smem + 1024);
+    if (per_sm > fit) per_sm = fit;
+    int ctas = ex.ctx->sm_count * per_sm / nbs; if (ctas < 1) ctas = 1;
+    const int rounds = (g.tiles + ctas - 1) / ctas;
+    launch(ex, conv3x3_direct_kernel<WL, EP>, dim3((g.tiles + rounds - 1) / rounds, nbs), g.NW * 32, smem, in, wl, ep, g);
+}
+
 // ------------------------------------------------------------------ any channel count, element by element
 // ---- operand loaders: element (m,k) of A and (k,n) of B of the implicit GEMM
 template <class TA> struct AnyFpropA {           // m = output pixel, k = (kh,kw,ci)
@@ -443,6 +634,12 @@ void conv_fprop_simt(Exec &ex, const void *a, bool a_bf16, Geom gi, const Layer 
     }
     const FastDiv wo = fast_div(g.Wo), ho = fast_div(g.Ho), ci = fast_div(g.Ci), kk = fast_div(g.k);
     const OutCouple ep{out, partner, sign};
+    DirectGeom d;
+    if (g.k == 3 && g.s == 1 && !a_bf16 && direct_shape(g.N, g.H, g.W, g.Ci, g.Co, ex.ctx->sm_count, d)) {
+        launch_direct(ex, (const float *)a, DirectFprop{L.W, g.Ci}, ep, d);
+        ex.check("conv_fprop_simt", bytes, 2.0 * M * N * (double)K);
+        return;
+    }
     const FpropB bl{L.W, N, K, a_bf16};
     if (a_bf16) launch_pixels(ex, FpropA<bf16>{(const bf16 *)a, g, wo, ho, ci, kk, M, K}, bl, ep, M, N, K);
     else launch_pixels(ex, FpropA<float>{(const float *)a, g, wo, ho, ci, kk, M, K}, bl, ep, M, N, K);
@@ -456,6 +653,12 @@ void conv_dgrad_simt(Exec &ex, const void *gq, bool g_bf16, Geom gi, const Layer
     if (ex.dry) return;
     const double bytes = (double)g.N * g.Ho * g.Wo * g.Co * (g_bf16 ? 2 : 4) + (double)M * N * 4 + (double)N * K * 4;
     const OutPlain ep{da, N};
+    DirectGeom d;
+    if (g.k == 3 && g.s == 1 && !g_bf16 && g.Ci % 4 == 0 && direct_shape(g.N, g.H, g.W, g.Co, g.Ci, ex.ctx->sm_count, d)) {
+        launch_direct(ex, (const float *)gq, DirectDgrad{L.W, g.Ci}, ep, d);
+        ex.check("conv_dgrad_simt", bytes, 2.0 * g.N * g.Ho * g.Wo * N * (double)K);
+        return;
+    }
     // stride 2: parity classes of (H + 1) / 2 x (W + 1) / 2 pixels would be ragged on odd sizes; those keep the plain numbering
     const bool classes = g.s == 2 && g.H % 2 == 0 && g.W % 2 == 0;
     const FastDiv w = fast_div(classes ? g.W / 2 : g.W), h = fast_div(classes ? g.H / 2 : g.H), co = fast_div(g.Co), kk = fast_div(g.k);

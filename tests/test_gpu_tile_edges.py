@@ -41,6 +41,9 @@ def test_bf16_blocks_at_tile_edges(ctx, kind, N, H, W, c, w):
     ("basic", 1, 150, 253, 20, 0),        # 32-column tiles, the tall ones
     ("basic", 1, 139, 137, 36, 0),        # 64-column tiles
     ("basic", 2, 11, 7, 68, 0),           # two column tiles, the second of 4 columns
+    ("basic", 16, 5, 4, 8, 0),            # direct 3x3: eight images per tile, one column of warps
+    ("basic", 5, 7, 6, 20, 0),            # two images per tile, the last one of a tile missing
+    ("basic", 1, 33, 17, 100, 0),         # four chunks of input channels (the last of 4), four groups of outputs
     ("bottleneck", 1, 3, 3, 132, 4),      # column sums of nine rows: two slabs of 17 and 16 quads, and one quad
     ("bottleneck", 1, 97, 99, 520, 8),    # 32-byte accesses in the streaming kernels
     ("bottleneck", 2, 37, 41, 260, 136),  # three slabs (22, 22, 21), several row ranges; sums of 1224 products
