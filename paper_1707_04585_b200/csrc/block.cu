@@ -20,6 +20,7 @@ bool conv_wgrad_tc(Exec &ex, const void *g, const void *a, Geom gi, const Layer 
 bool conv_wgrad_tc_batch(Exec &ex, int n, const void *const *gq, const void *const *a, const Geom *gi, const Layer *const *L,
                          float *scratch, size_t *need);
 // one kernel for BN -> ReLU -> conv (at most 64 input channels, stride 1); likewise the data gradient of such a layer
+bool conv_fused_takes(Exec &ex, Geom gi, const Layer &L);
 bool conv_fprop_fused(Exec &ex, Pair t, BnRef bn, Geom gi, const Layer &L, Pair out, Pair partner, int sign, Moments *stats, bf16 *a_out);
 bool conv_dgrad_fused(Exec &ex, const void *g, Geom gi, const Layer &L, float *da, const BnBwdReq *bb);
 
@@ -89,7 +90,11 @@ void fn_forward(Exec &ex, Geom g, Pair u, const Moments *mom_in, const std::vect
         void *a = ex.ws.alloc(P * ly.cin * esz(ex));
         float *tn = last ? nullptr : ex.ws.get<float>(go.P() * ly.cout);
         Moments next;
-        if (!last) next = mom_alloc(ex, ly.cout, b16);      // with room for pending partials: the next layer consumes them
+        if (!last) {
+            next = mom_alloc(ex, ly.cout, b16);      // with room for pending partials: the next layer consumes them
+            const bool to_last = l + 1 == L - 1;
+            next.defer = b16 && !(to_last && (skip_last_conv || out.c1 || partner.c1)) && conv_fused_takes(ex, go, layers[l + 1]);
+        }
         const Pair o = last ? out : single(tn, ly.cout);
         bool fused = false;
         if (b16 && !(last && skip_last_conv))

@@ -310,6 +310,7 @@ struct Moments {
     int parts = 0;
     double inv_count = 0;          // 1 / pixels summed
     bool pending = false;
+    bool defer = false;            // the consumer adds pending records itself: any producer may leave them
 };
 // One BN as its consumers see it: scale = gamma*rstd, shift = beta - mean*scale are derived on the
 // fly, always with the same two roundings, so that the ReLU mask of the backward equals the forward's.

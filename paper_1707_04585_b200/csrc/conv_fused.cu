@@ -604,6 +604,12 @@ bool run_fused(Exec &ex, const char *what, int in_mode, const void *in, float in
 
 }  // namespace
 
+// whether conv_fprop_fused takes layer L on images gi (and so adds pending statistics of its input itself)
+bool conv_fused_takes(Exec &ex, Geom gi, const Layer &L) {
+    FusedShape s;
+    return L.stride == 1 && fused_shape(gi, L.cin, L.cout, L.k, ex.ctx->sm_count, s);
+}
+
 // out = partner + sign * conv(ReLU(BN(t)));  a_out (optional): the activated tensor, for the weight gradient
 bool conv_fprop_fused(Exec &ex, Pair t, BnRef bn, Geom gi, const Layer &L, Pair out, Pair partner, int sign, Moments *stats, bf16 *a_out) {
     if (L.stride != 1 || t.c1 != 0) return false;

@@ -12,8 +12,8 @@
 //
 // Roles inside a CTA: warp 0 issues TMA loads, warp 1 allocates tensor memory and issues the MMAs,
 // the remaining warps drain the accumulator (tcgen05.ld), apply the coupling epilogue (out = partner
-// +/- acc on the float or fixed-point state) and store: two groups of four warps (320 threads) where
-// the epilogue's tiles move through TMA, one group (192 threads) in the staged form.
+// +/- acc on the float or fixed-point state) and store: two or four groups of four warps where the
+// epilogue's tiles move through TMA, one group (192 threads) in the staged form.
 // Every mbarrier wait is bounded; on expiry the kernel records a status word and leaves.
 #include "common.cuh"
 #include "tc_ptx.cuh"
@@ -29,7 +29,8 @@ namespace {
 constexpr int kStages = 6;       // most operand stages of the convolution kernel
 constexpr int kWgStages = 4;     // ... of the weight-gradient kernel
 constexpr int kThreads = 192;      // TMA warp, MMA warp, four epilogue warps
-constexpr int kThreadsTma = 320;   // epilogue through TMA: two groups of four epilogue warps
+constexpr int kMaxGroups = 4;      // epilogue through TMA: two or four groups of four epilogue warps
+constexpr int kThreadsTma = 64 + kMaxGroups * 128;
 
 struct TcParams {
     int taps;        // k*k
@@ -47,9 +48,12 @@ struct TcParams {
     // partner, or BN input of a data gradient) arrives, as column groups of GW floats per pixel row
     int epi_tma;
     int GW;          // 32 or 16 floats: rows of 128 / 64 bytes, stored with the matching TMA swizzle
+    int epi_bytes;   // partner rings, output slots and sums of the TMA epilogue
     int group_bytes; // one column group of a tile (128 pixel rows), a multiple of 1024
     int need_aux;
-    int aux_slots;   // conv_tc2_kernel: slots of the partner ring (two interleaved rings, one per epilogue warp group)
+    int groups;      // epilogue warp groups
+    int aux_slots;   // slots of each group's partner ring
+    int inplace;     // coupling: the result is written over the partner group and stored from there (no output slots)
     int split_o, split_x;   // channels in the first tensor of a channel-split output / partner (0: one tensor)
     // the taps this launch sums: offset of the operand box in rows / columns of the operand tensor, and the tap's
     // place in the weight pack.  A plain convolution lists all k*k taps; one parity class of a stride-2 data
@@ -72,7 +76,8 @@ struct TcParams {
 struct __align__(8) TcShared {
     uint64_t full[kStages];
     uint64_t empty[kStages];
-    uint64_t acc_full[2];
+    uint64_t acc_full[4];            // by tile & 3: with four epilogue groups on alternate tiles each of them sees every phase of its own
+    
     uint64_t acc_empty[2];
     uint64_t aux_full[8];
     uint64_t afull[4], aempty[4];     // halo operand ring of conv_tc2_kernel
@@ -147,6 +152,197 @@ __device__ __forceinline__ void tma_pass_b(int GW, const uint8_t *ob, const uint
     }
 }
 
+// The epilogue of a CTA through TMA, by p.groups warp groups of four warps (wg; warps 2, 3, ... of the CTA).  A visit is one column
+// group of one tile: a chain of four barriers and two passes over shared memory whose time is latency, 3000 to 4700 clocks for 128 x
+// 32 floats, so its rate is set by how many groups work side by side.  With at least as many column groups as warp
+// groups, warp group wg takes the column groups wg, wg + groups, ... of every tile; with fewer, the warp groups also alternate
+// tiles (the host makes their number a multiple).  Partner groups arrive through a ring of aux_slots per warp group; a
+// coupling writes its result over the partner group and stores it from there, other modes have an output slot per warp group.
+// Four groups pay in the single-CTA kernel, whose tiles are short (large-image step: 16.1 -> 14.9 ms of its launches, 164-layer step
+// 4.86 -> 3.82 ms together with the records left to the consumer); the pair kernel has two: its tiles are bound by the MMAs,
+// and four would cost it operand stages (20.9 -> 22.3 ms).
+// PAIR: the tile of a CTA pair's tile pair (see conv_tc2_kernel).
+struct EpiMaps { const CUtensorMap *o0, *o1, *x0, *x1; };
+template <bool PAIR>
+__device__ __forceinline__ void tma_epilogue(const TcParams &p, TcShared *sh, const EpiMaps maps, uint8_t *auxr, uint32_t tmem_d, int col0, int warp, int lane,
+                                             int rank, int first, int step, int n_v, int per_cls) {
+    const int ng = p.BN / p.GW, NG = p.groups;
+    const int wg = (warp - 2) >> 2;
+    const int bar_a = 1 + 2 * wg, bar_b = 2 + 2 * wg, bar_all = 9;
+    const int etid = ((warp & 3) << 5) | lane;
+    const EpiArgs &e = p.epi;
+    const int GW = p.GW, QW = GW >> 2, rpp = 128 / QW;
+    const int jq = etid % QW, r0 = etid / QW;
+    const int box_px_o = p.g.BIMG * p.g.BH * p.g.W;
+    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+    const float out_q = e.out.q, out_s = out_q != 0.f ? 1.f / out_q : 0.f, t_q = e.t.q;
+    const uint32_t aux_tx = (uint32_t)(box_px_o * GW * 4);
+    const int SW = p.aux_slots;
+    uint8_t *auxg = auxr + wg * SW * p.group_bytes;                                  // this group's ring
+    uint8_t *outr = auxr + (p.need_aux ? NG * SW * p.group_bytes : 0);
+    uint8_t *out_slot = outr + wg * p.group_bytes;
+    float *gsums = (float *)(outr + (p.inplace ? 0 : NG * p.group_bytes));           // [ng][128][8], only if ng > groups
+    // this group's visits: column groups gi0, gi0 + gstep, ... < ng of the tiles first + step * (it0, it0 + itstep, ...)
+    const bool many = ng > NG;
+    const int gi0 = many || ng == NG ? wg : wg % ng, gstep = many ? NG : ng;
+    const int it0 = ng < NG ? wg / ng : 0, itstep = ng < NG ? NG / ng : 1;
+    // pixel of the tile's box (rows of W pixels) this thread's accumulator row holds; -1: padding
+    int srow = etid;
+    if (p.halo) { const int hh = etid / p.Wp, ww = etid - hh * p.Wp; srow = (hh < p.g.BH && ww < p.g.W) ? hh * p.g.W + ww : -1; }
+    const int prow = srow < 0 ? 0 : srow;
+    // class and pixel tile at place v of the tile list; false: the second tile of the last pair of an odd number
+    auto tile_of = [&](int v, int &cls, int &t) {
+        cls = v / per_cls;
+        t = PAIR ? 2 * (v - cls * per_cls) + rank : v - cls * per_cls;
+        return !PAIR || t < p.g.n_px_tiles;
+    };
+    // the partner groups in the order of the visits; visits beyond the valid channels and tiles have none
+    int l_v = first + it0 * step, l_gi = gi0, l_slot = 0;
+    auto load_next_aux = [&]() {                         // one thread; returns without loading once the visits are used up
+        while (l_v < n_v) {
+            int cls, t, n0, h0;
+            const int col = col0 + l_gi * GW;
+            const bool live = tile_of(l_v, cls, t) && col < e.n_cols;
+            l_gi += gstep;
+            const bool last_of_tile = l_gi >= ng;
+            if (live) {
+                tile_origin(p.g, t, n0, h0);
+                const bool second = p.split_x && col >= p.split_x;
+                uint64_t *bar = &sh->aux_full[wg * SW + l_slot];
+                mbar_expect_tx(bar, aux_tx);
+                tma_load_4d(auxg + l_slot * p.group_bytes, second ? maps.x1 : maps.x0, bar, second ? col - p.split_x : col, p.ox[cls], h0 * p.ostride + p.oy[cls], n0);
+                if (++l_slot == SW) l_slot = 0;
+            }
+            if (last_of_tile) { l_gi = gi0; l_v += itstep * step; }
+            if (live) return;
+        }
+    };
+    if (etid == 0 && p.need_aux)
+        for (int i = 0; i < SW; i++) load_next_aux();
+    if (many) {
+        for (int i = wg * 128 + etid; i < ng * 128 * 8; i += NG * 128) gsums[i] = 0.f;
+        named_barrier(bar_all, NG * 128);
+    }
+    float acc[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++) acc[j] = 0.f;
+    bool ok = true, refill = false;
+    int c_slot = 0; uint32_t c_par = 0;
+    int it = it0;
+#pragma unroll 1
+    for (int v = first + it0 * step; v < n_v; v += itstep * step, it += itstep) {
+        const int buf = it & 1;
+        int cls, t, n0, h0, valid_px = 0;
+        const bool in_range = tile_of(v, cls, t);
+        tile_origin(p.g, t, n0, h0);
+        if (in_range)
+            valid_px = p.g.BIMG > 1 ? (p.g.N - n0 < p.g.BIMG ? p.g.N - n0 : p.g.BIMG) * p.g.BH * p.g.W
+                                    : (p.g.H - h0 < p.g.BH ? p.g.H - h0 : p.g.BH) * p.g.W;
+        const uint32_t tm = tmem_d + lane_base + (uint32_t)(buf * p.BN);
+#pragma unroll 1
+        for (int gi = gi0; gi < ng; gi += gstep) {
+            const int col = col0 + gi * GW;
+            const bool live = in_range && col < e.n_cols;          // groups beyond the valid channels only drain their columns
+            const bool visit = p.need_aux && live;                 // the partner group sits in ring slot c_slot
+            const uint8_t *ax = auxg + c_slot * p.group_bytes;
+            uint8_t *ob = p.inplace ? auxg + c_slot * p.group_bytes : out_slot;
+            if (etid == 0) {
+                tma_store_wait_read();                             // this group's last store is done with its slot
+                if (refill) load_next_aux();                       // (in place: which can take the next partner group now)
+                ok = (PAIR ? mbar_wait_cluster(&sh->acc_full[it & 3], (it >> 2) & 1) : mbar_wait(&sh->acc_full[it & 3], (it >> 2) & 1)) && sh->failed == 0;
+                if (ok && visit) ok = mbar_wait(&sh->aux_full[wg * SW + c_slot], c_par);
+            }
+            refill = p.inplace && visit;
+            if (visit && ++c_slot == SW) { c_slot = 0; c_par ^= 1u; }
+            ok = named_barrier_and(bar_b, 128, ok);
+            if (!ok) break;
+            tc_fence_after();
+            const bool rowv = live && srow >= 0 && srow < valid_px;
+            const uint32_t tg = tm + (uint32_t)(gi * GW);
+            if (e.mode != EPI_COUPLE) {
+                if (out_q == 0.f) tma_pass_a<0>(tg, GW, prow, rowv, ax, ob, out_s); else tma_pass_a<1>(tg, GW, prow, rowv, ax, ob, out_s);
+            } else if (out_q == 0.f) {
+                if (e.sign > 0) tma_pass_a<2>(tg, GW, prow, rowv, ax, ob, out_s); else tma_pass_a<3>(tg, GW, prow, rowv, ax, ob, out_s);
+            } else {
+                if (e.sign > 0) tma_pass_a<4>(tg, GW, prow, rowv, ax, ob, out_s); else tma_pass_a<5>(tg, GW, prow, rowv, ax, ob, out_s);
+            }
+            tc_fence_before();
+            fence_proxy_async();
+            named_barrier(bar_a, 128);
+            if (etid == 0) {
+                // the columns of this group are drained: one arrival per column group
+                if (PAIR) mbar_arrive_cluster(mapa_shared(smem_u32(&sh->acc_empty[buf]), 0));
+                else mbar_arrive(&sh->acc_empty[buf]);
+                if (live) {
+                    const bool second = p.split_o && col >= p.split_o;
+                    tma_store_4d(second ? maps.o1 : maps.o0, ob, second ? col - p.split_o : col, p.ox[cls], h0 * p.ostride + p.oy[cls], n0);
+                    tma_store_commit();
+                }
+            }
+            if (e.part && live && col + jq * 4 < e.n_cols) {
+                float4 sc4 = make_float4(0, 0, 0, 0), sh4 = sc4, mu4 = sc4, rs4 = sc4;
+                if (e.mode == EPI_BNBWD) bn_coef4(e.bn, col + jq * 4, sc4, sh4, mu4, rs4);
+                float4 *slot = reinterpret_cast<float4 *>(gsums + (gi * 128 + etid) * 8);
+                if (many) {
+                    const float4 a0 = slot[0], a1 = slot[1];
+                    acc[0] = a0.x; acc[1] = a0.y; acc[2] = a0.z; acc[3] = a0.w; acc[4] = a1.x; acc[5] = a1.y; acc[6] = a1.z; acc[7] = a1.w;
+                }
+                if (e.mode == EPI_BNBWD) {
+                    if (t_q == 0.f) tma_pass_b<2>(GW, ob, ax, jq, r0, rpp, valid_px, 0.f, sc4, sh4, mu4, rs4, acc);
+                    else tma_pass_b<3>(GW, ob, ax, jq, r0, rpp, valid_px, t_q, sc4, sh4, mu4, rs4, acc);
+                } else if (out_q == 0.f) tma_pass_b<0>(GW, ob, ax, jq, r0, rpp, valid_px, 0.f, sc4, sh4, mu4, rs4, acc);
+                else tma_pass_b<1>(GW, ob, ax, jq, r0, rpp, valid_px, out_q, sc4, sh4, mu4, rs4, acc);
+                if (many) { slot[0] = make_float4(acc[0], acc[1], acc[2], acc[3]); slot[1] = make_float4(acc[4], acc[5], acc[6], acc[7]); }
+            }
+            named_barrier(bar_a, 128);                             // the partner group and the output slot have been read
+            if (etid == 0 && visit && !p.inplace) load_next_aux();
+        }
+        if (!ok) break;
+    }
+    if (etid == 0) tma_store_wait_read();
+    if (!ok && lane == 0) atomicExch(&sh->failed, 1u);
+    __threadfence_block();
+    named_barrier(bar_all, NG * 128);
+    if (!e.part) {
+        if (etid == 0) tma_store_wait_all();
+        return;
+    }
+    float *sums = many ? gsums : (float *)auxr;                    // (every load and store of the slots has completed)
+    if (!many) {
+        float4 *slot = reinterpret_cast<float4 *>(sums + (wg * 128 + etid) * 8);
+        slot[0] = make_float4(acc[0], acc[1], acc[2], acc[3]); slot[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+        named_barrier(bar_all, NG * 128);
+    }
+    ok = named_barrier_and(bar_all, NG * 128, *(volatile uint32_t *)&sh->failed == 0);
+    if (ok && wg == 0) {
+        // per-CTA record: the warp groups, then the threads, that share a channel quad are added in order
+        float *mine = e.part + (size_t)blockIdx.x * 2 * e.n_cols;
+        for (int gi = 0; gi < ng; gi++) {
+            const int col = col0 + gi * GW + jq * 4;
+            if (r0 == 0 && col < e.n_cols) {
+                float r[8];
+#pragma unroll
+                for (int j = 0; j < 8; j++) r[j] = 0.f;
+                for (int q = gi; q < (many ? gi + 1 : NG); q += many ? 1 : ng)
+                    for (int y = 0; y < rpp; y++)
+#pragma unroll
+                        for (int j = 0; j < 8; j++) r[j] += sums[(size_t)q * 128 * 8 + (y * QW + jq) * 8 + j];
+                *reinterpret_cast<float4 *>(mine + 2 * col) = make_float4(r[0], r[1], r[2], r[3]);
+                *reinterpret_cast<float4 *>(mine + 2 * col + 4) = make_float4(r[4], r[5], r[6], r[7]);
+            }
+        }
+    }
+    // the last CTA adds the records with all its epilogue threads (128 of them took four rounds of dependent reads for 148
+    // records); without a counter the records stay pending and their consumer adds them
+    if (ok && e.counter) {
+        float *scratch = reinterpret_cast<float *>(auxr + (many ? 0 : NG * 4096));
+        if (NG == 4) epilogue_publish<512>(e, scratch, wg * 128 + etid);
+        else if (NG == 2) epilogue_publish<256>(e, scratch, wg * 128 + etid);
+        else if (wg == 0) epilogue_publish<128>(e, scratch, etid);
+    }
+    if (etid == 0) tma_store_wait_all();
+}
+
 // Persistent CTA: walks the pixel tiles blockIdx.x, blockIdx.x + gridDim.x, ... of N tile blockIdx.y.
 // The operand ring runs on across tiles; the accumulator alternates between two tensor-memory
 // buffers so that the epilogue of one tile overlaps the MMAs of the next.
@@ -166,9 +362,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     float *estage = (float *)(tiles + p.stages * stage_bytes);
     const int ng = p.epi_tma ? p.BN / p.GW : 0;
     uint8_t *auxr = (uint8_t *)estage;
-    uint8_t *outr = auxr + (p.need_aux ? ng : 0) * p.group_bytes;
-    float *gsums = (float *)(outr + 2 * p.group_bytes);
-    TcShared *sh = p.epi_tma ? (TcShared *)(gsums + ng * 128 * 8) : (TcShared *)((uint8_t *)estage + kEpiStageBytes + kEpiSumFloats * 4);
+    TcShared *sh = p.epi_tma ? (TcShared *)(auxr + p.epi_bytes) : (TcShared *)((uint8_t *)estage + kEpiStageBytes + kEpiSumFloats * 4);
 
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int n_vt = p.n_cls * p.g.n_px_tiles;     // tiles of all classes
@@ -177,7 +371,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; s++) { mbar_init(&sh->full[s], 1); mbar_init(&sh->empty[s], 1); }
-        for (int b = 0; b < 2; b++) { mbar_init(&sh->acc_full[b], 1); mbar_init(&sh->acc_empty[b], p.epi_tma ? 256 : 128); }
+        for (int b = 0; b < 2; b++) mbar_init(&sh->acc_empty[b], p.epi_tma ? ng : 128);
+        for (int b = 0; b < 4; b++) mbar_init(&sh->acc_full[b], 1);
         for (int b = 0; b < 8; b++) mbar_init(&sh->aux_full[b], 1);
         sh->failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -249,7 +444,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     soff += stage16;
                     if (++s == p.stages) { s = 0; soff = 0; round++; }
                 }
-                if (ok) mma_commit(&sh->acc_full[buf]);
+                if (ok) mma_commit(&sh->acc_full[ti & 3]);
             }
         }
     } else if (!p.epi_tma) {
@@ -261,12 +456,12 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         bool ok = true;
         int ti = 0;
         for (int t = blockIdx.x; t < p.g.n_px_tiles; t += gridDim.x, ti++) {
-            const int buf = ti & 1; const uint32_t use = ti >> 1;
+            const int buf = ti & 1;
             int n0, h0;
             tile_origin(p.g, t, n0, h0);
             EpiPrefetch pre;
             epilogue_prefetch(p.epi, p.BN, col0, &sh->rows, p.g, n0, h0, etid, pre);     // before the accumulator is ready
-            if (etid == 0) ok = mbar_wait(&sh->acc_full[buf], use & 1) && sh->failed == 0;     // one thread polls, the rest block
+            if (etid == 0) ok = mbar_wait(&sh->acc_full[ti & 3], (ti >> 2) & 1) && sh->failed == 0;     // one thread polls, the rest block
             ok = named_barrier_and(2, 128, ok);
             if (!ok) break;
             tc_fence_after();
@@ -275,129 +470,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         if (ok) epilogue_finish(p.epi, p.BN, col0, estage, esums, etid);
         else if (lane == 0) atomicExch(&sh->failed, 1u);
     } else {
-        // epilogue through TMA: two groups of four warps; group wg takes the column groups wg, wg + 2, ... of every
-        // tile and owns output slot wg, so that one group's pass over shared memory overlaps the other's waits.
-        // Thread etid of a warp group owns accumulator row etid = pixel etid of the tile's box.
-        const int wg = (warp - 2) >> 2;
-        const int bar_a = 1 + 2 * wg, bar_b = 2 + 2 * wg;   // named barriers of this warp group; 5: both groups
-        const int etid = ((warp & 3) << 5) | lane;
-        const EpiArgs &e = p.epi;
-        const int GW = p.GW, QW = GW >> 2, rpp = 128 / QW;
-        const int jq = etid % QW, r0 = etid / QW;
-        const int box_px_o = p.g.BIMG * p.g.BH * p.g.W;
-        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const float out_q = e.out.q, out_s = out_q != 0.f ? 1.f / out_q : 0.f, t_q = e.t.q;
-        const uint32_t aux_tx = (uint32_t)(box_px_o * GW * 4);
-        for (int i = wg * 128 + etid; i < ng * 128 * 8; i += 256) gsums[i] = 0.f;
-        // column group gi of this N tile: which tensor of a channel-split pair, and the channel inside it
-        auto out_map = [&](int col) { return (p.split_o && col >= p.split_o) ? &map_o1 : &map_o0; };
-        auto aux_map = [&](int col) { return (p.split_x && col >= p.split_x) ? &map_x1 : &map_x0; };
-        auto col_out = [&](int col) { return (p.split_o && col >= p.split_o) ? col - p.split_o : col; };
-        auto col_aux = [&](int col) { return (p.split_x && col >= p.split_x) ? col - p.split_x : col; };
-        auto load_aux = [&](int gi, int cls, int n0, int h0) {     // one thread; (cls, n0, h0): class and origin of the tile
-            const int col = col0 + gi * GW;
-            if (col >= e.n_cols) return;
-            mbar_expect_tx(&sh->aux_full[gi], aux_tx);
-            tma_load_4d(auxr + gi * p.group_bytes, aux_map(col), &sh->aux_full[gi], col_aux(col), p.ox[cls], h0 * p.ostride + p.oy[cls], n0);
-        };
-        // class and origin of the tile at hand and of the one after it: worked out once per tile, so that the thread
-        // that issues the partner loads between two column groups has no divisions to do
-        int cls = 0, n0 = 0, h0 = 0, cls_n = 0, n0_n = 0, h0_n = 0;
-        if ((int)blockIdx.x < n_vt) {
-            cls_n = (int)blockIdx.x / p.g.n_px_tiles;
-            tile_origin(p.g, (int)blockIdx.x - cls_n * p.g.n_px_tiles, n0_n, h0_n);
-        }
-        if (etid == 0 && p.need_aux && (int)blockIdx.x < n_vt)
-            for (int gi = wg; gi < ng; gi += 2) load_aux(gi, cls_n, n0_n, h0_n);
-        named_barrier(5, 256);
-        bool ok = true;
-        int ti = 0;
-        uint8_t *ob = outr + wg * p.group_bytes;
-        for (int t = blockIdx.x; t < n_vt; t += gridDim.x, ti++) {
-            const int buf = ti & 1; const uint32_t use = ti >> 1;
-            cls = cls_n; n0 = n0_n; h0 = h0_n;
-            const int tn = t + (int)gridDim.x;
-            if (tn < n_vt) {
-                cls_n = tn / p.g.n_px_tiles;
-                tile_origin(p.g, tn - cls_n * p.g.n_px_tiles, n0_n, h0_n);
-            }
-            const int valid_px = p.g.BIMG > 1 ? (p.g.N - n0 < p.g.BIMG ? p.g.N - n0 : p.g.BIMG) * p.g.BH * p.g.W
-                                              : (p.g.H - h0 < p.g.BH ? p.g.H - h0 : p.g.BH) * p.g.W;
-            if (etid == 0) ok = mbar_wait(&sh->acc_full[buf], use & 1) && sh->failed == 0;     // one thread polls, the rest block
-            ok = named_barrier_and(bar_b, 128, ok);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t tm = tmem_d + lane_base + (uint32_t)(buf * p.BN);
-#pragma unroll 1
-            for (int gi = wg; gi < ng; gi += 2) {
-                const int col = col0 + gi * GW;
-                const bool live = col < e.n_cols;          // groups beyond the valid channels only drain their columns
-                const uint8_t *ax = auxr + gi * p.group_bytes;
-                if (etid == 0) {
-                    if (p.need_aux && live) ok = mbar_wait(&sh->aux_full[gi], ti & 1);
-                    tma_store_wait_read();                 // this group's last store is done with the output slot
-                }
-                ok = named_barrier_and(bar_b, 128, ok);
-                if (!ok) break;
-                const bool rowv = live && etid < valid_px;
-                const uint32_t tg = tm + (uint32_t)(gi * GW);
-                if (e.mode != EPI_COUPLE) {
-                    if (out_q == 0.f) tma_pass_a<0>(tg, GW, etid, rowv, ax, ob, out_s); else tma_pass_a<1>(tg, GW, etid, rowv, ax, ob, out_s);
-                } else if (out_q == 0.f) {
-                    if (e.sign > 0) tma_pass_a<2>(tg, GW, etid, rowv, ax, ob, out_s); else tma_pass_a<3>(tg, GW, etid, rowv, ax, ob, out_s);
-                } else {
-                    if (e.sign > 0) tma_pass_a<4>(tg, GW, etid, rowv, ax, ob, out_s); else tma_pass_a<5>(tg, GW, etid, rowv, ax, ob, out_s);
-                }
-                fence_proxy_async();
-                named_barrier(bar_a, 128);
-                if (etid == 0 && live) {
-                    tma_store_4d(out_map(col), ob, col_out(col), p.ox[cls], h0 * p.ostride + p.oy[cls], n0);
-                    tma_store_commit();
-                }
-                if (e.part && live && col + jq * 4 < e.n_cols) {
-                    float4 sc4 = make_float4(0, 0, 0, 0), sh4 = sc4, mu4 = sc4, rs4 = sc4;
-                    if (e.mode == EPI_BNBWD) bn_coef4(e.bn, col + jq * 4, sc4, sh4, mu4, rs4);
-                    float4 *slot = reinterpret_cast<float4 *>(gsums + (gi * 128 + etid) * 8);
-                    const float4 a0 = slot[0], a1 = slot[1];
-                    float acc[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                    if (e.mode == EPI_BNBWD) {
-                        if (t_q == 0.f) tma_pass_b<2>(GW, ob, ax, jq, r0, rpp, valid_px, 0.f, sc4, sh4, mu4, rs4, acc);
-                        else tma_pass_b<3>(GW, ob, ax, jq, r0, rpp, valid_px, t_q, sc4, sh4, mu4, rs4, acc);
-                    } else if (out_q == 0.f) tma_pass_b<0>(GW, ob, ax, jq, r0, rpp, valid_px, 0.f, sc4, sh4, mu4, rs4, acc);
-                    else tma_pass_b<1>(GW, ob, ax, jq, r0, rpp, valid_px, out_q, sc4, sh4, mu4, rs4, acc);
-                    slot[0] = make_float4(acc[0], acc[1], acc[2], acc[3]); slot[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
-                }
-                named_barrier(bar_a, 128);                 // the partner group and the output slot have been read
-                if (etid == 0 && p.need_aux && tn < n_vt) load_aux(gi, cls_n, n0_n, h0_n);
-            }
-            if (!ok) break;
-            // this warp group has drained its columns of the accumulator (the other group arrives for its own)
-            tc_fence_before();
-            mbar_arrive(&sh->acc_empty[buf]);
-        }
-        if (etid == 0) tma_store_wait_all();
-        if (!ok && lane == 0) atomicExch(&sh->failed, 1u);
-        __threadfence_block();
-        named_barrier(5, 256);
-        if (wg == 0 && e.part && sh->failed == 0) {
-            // per-CTA record: the threads that share a channel quad are added in order
-            float *mine = e.part + (size_t)blockIdx.x * 2 * e.n_cols;
-            for (int gi = 0; gi < ng; gi++) {
-                const int col = col0 + gi * GW + jq * 4;
-                if (r0 == 0 && col < e.n_cols) {
-                    const float *base = gsums + (size_t)gi * 128 * 8;
-                    float r[8];
-#pragma unroll
-                    for (int j = 0; j < 8; j++) r[j] = base[jq * 8 + j];
-                    for (int y = 1; y < rpp; y++)
-#pragma unroll
-                        for (int j = 0; j < 8; j++) r[j] += base[(y * QW + jq) * 8 + j];
-                    *reinterpret_cast<float4 *>(mine + 2 * col) = make_float4(r[0], r[1], r[2], r[3]);
-                    *reinterpret_cast<float4 *>(mine + 2 * col + 4) = make_float4(r[4], r[5], r[6], r[7]);
-                }
-            }
-            epilogue_publish<128>(e, reinterpret_cast<float *>(auxr), etid);
-        }
+        tma_epilogue<false>(p, sh, EpiMaps{&map_o0, &map_o1, &map_x0, &map_x1}, auxr, tmem_d, col0, warp, lane, 0, (int)blockIdx.x, (int)gridDim.x, n_vt, p.g.n_px_tiles);
     }
     tc_fence_before();
     __syncthreads();
@@ -436,9 +509,7 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const int wstage_bytes = (b_bytes + 1023) & ~1023;
     uint8_t *wring = tiles + (p.halo ? p.a_slots * p.a_slot_bytes : 0);
     uint8_t *auxr = p.halo ? wring + p.stages * wstage_bytes : tiles + p.stages * stage_bytes;
-    uint8_t *outr = auxr + (p.need_aux ? p.aux_slots : 0) * p.group_bytes;
-    float *gsums = (float *)(outr + 2 * p.group_bytes);
-    TcShared *sh = (TcShared *)(gsums + ng * 128 * 8);
+    TcShared *sh = (TcShared *)(auxr + p.epi_bytes);
 
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
@@ -450,8 +521,9 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; s++) { mbar_init(&sh->full[s], 1); mbar_init(&sh->empty[s], 1); }
-        // acc_empty (used in the leader): one arrival per epilogue warp group of either CTA
-        for (int b = 0; b < 2; b++) { mbar_init(&sh->acc_full[b], 1); mbar_init(&sh->acc_empty[b], 4); }
+        // acc_empty (used in the leader): one arrival per column group of either CTA
+        for (int b = 0; b < 2; b++) mbar_init(&sh->acc_empty[b], 2 * ng);
+        for (int b = 0; b < 4; b++) mbar_init(&sh->acc_full[b], 1);
         for (int b = 0; b < 8; b++) mbar_init(&sh->aux_full[b], 1);
         for (int b = 0; b < 4; b++) { mbar_init(&sh->afull[b], 1); mbar_init(&sh->aempty[b], 1); }
         sh->failed = 0;
@@ -560,7 +632,7 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                         aoff += aslot16;
                         if (++as == p.a_slots) { as = 0; aoff = 0; ar++; }
                     }
-                    if (ok) mma2_commit_both(&sh->acc_full[buf]);
+                    if (ok) mma2_commit_both(&sh->acc_full[ti & 3]);
                     continue;
                 }
                 const int iters = p.ntap[vp / n_pp] * p.chunks;
@@ -575,150 +647,12 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                     soff += stage16;
                     if (++s == p.stages) { s = 0; soff = 0; round++; }
                 }
-                if (ok) mma2_commit_both(&sh->acc_full[buf]);
+                if (ok) mma2_commit_both(&sh->acc_full[ti & 3]);
             }
         }
     } else {
-        // epilogue of this CTA's own tile: as in conv_tc_kernel (two groups of four warps, alternate column groups)
-        const int wg = (warp - 2) >> 2;
-        const int bar_a = 1 + 2 * wg, bar_b = 2 + 2 * wg;
-        const int etid = ((warp & 3) << 5) | lane;
-        const EpiArgs &e = p.epi;
-        const int GW = p.GW, QW = GW >> 2, rpp = 128 / QW;
-        const int jq = etid % QW, r0 = etid / QW;
-        const int box_px_o = p.g.BIMG * p.g.BH * p.g.W;
-        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const float out_q = e.out.q, out_s = out_q != 0.f ? 1.f / out_q : 0.f, t_q = e.t.q;
-        const uint32_t aux_tx = (uint32_t)(box_px_o * GW * 4);
-        const uint32_t acc_empty0[2] = {mapa_shared(smem_u32(&sh->acc_empty[0]), 0), mapa_shared(smem_u32(&sh->acc_empty[1]), 0)};
-        // pixel of the tile's box (rows of W pixels) this thread's accumulator row holds; -1: padding
-        int srow = etid;
-        if (p.halo) { const int hh = etid / p.Wp, ww = etid - hh * p.Wp; srow = (hh < p.g.BH && ww < p.g.W) ? hh * p.g.W + ww : -1; }
-        const int prow = srow < 0 ? 0 : srow;
-        for (int i = wg * 128 + etid; i < ng * 128 * 8; i += 256) gsums[i] = 0.f;
-        auto out_map = [&](int col) { return (p.split_o && col >= p.split_o) ? &map_o1 : &map_o0; };
-        auto aux_map = [&](int col) { return (p.split_x && col >= p.split_x) ? &map_x1 : &map_x0; };
-        auto col_out = [&](int col) { return (p.split_o && col >= p.split_o) ? col - p.split_o : col; };
-        auto col_aux = [&](int col) { return (p.split_x && col >= p.split_x) ? col - p.split_x : col; };
-        // The partner groups arrive through a ring of SW slots per warp group (slots wg, wg + 2, ...), filled in the
-        // order the group will visit them: its column groups of this tile, then of its next tile, ...; groups beyond
-        // the valid channels and tiles outside the tensor are not visited.  l_*: next visit to load (one thread),
-        // c_*: next visit to consume (all threads, uniform).
-        const int SW = p.aux_slots >> 1;
-        int l_vp = pair, l_gi = wg, l_slot = 0;
-        int c_slot = 0; uint32_t c_par = 0;
-        auto load_next_aux = [&]() {                         // one thread; returns without loading once the visits are used up
-            while (l_vp < n_vp) {
-                int cls, t, n0, h0;
-                my_tile(l_vp, cls, t);
-                const int col = col0 + l_gi * GW;
-                const bool live = col < e.n_cols && t < p.g.n_px_tiles;
-                l_gi += 2;
-                const bool last_of_tile = l_gi >= ng;
-                if (live) {
-                    tile_origin(p.g, t, n0, h0);
-                    const int slot = wg + 2 * l_slot;
-                    mbar_expect_tx(&sh->aux_full[slot], aux_tx);
-                    tma_load_4d(auxr + slot * p.group_bytes, aux_map(col), &sh->aux_full[slot], col_aux(col), p.ox[cls], h0 * p.ostride + p.oy[cls], n0);
-                    if (++l_slot == SW) l_slot = 0;
-                }
-                if (last_of_tile) { l_gi = wg; l_vp += n_pairs; }
-                if (live) return;
-            }
-        };
-        if (etid == 0 && p.need_aux && wg < ng)
-            for (int i = 0; i < SW; i++) load_next_aux();
-        named_barrier(5, 256);
-        bool ok = true;
-        int ti = 0;
-        uint8_t *ob = outr + wg * p.group_bytes;
-        for (int vp = pair; vp < n_vp; vp += n_pairs, ti++) {
-            const int buf = ti & 1; const uint32_t use = ti >> 1;
-            int cls, t, n0, h0;
-            my_tile(vp, cls, t);
-            const bool in_range = t < p.g.n_px_tiles;
-            tile_origin(p.g, t, n0, h0);
-            int valid_px = 0;
-            if (in_range)
-                valid_px = p.g.BIMG > 1 ? (p.g.N - n0 < p.g.BIMG ? p.g.N - n0 : p.g.BIMG) * p.g.BH * p.g.W
-                                        : (p.g.H - h0 < p.g.BH ? p.g.H - h0 : p.g.BH) * p.g.W;
-            if (etid == 0) ok = mbar_wait_cluster(&sh->acc_full[buf], use & 1) && sh->failed == 0;
-            ok = named_barrier_and(bar_b, 128, ok);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t tm = tmem_d + lane_base + (uint32_t)(buf * p.BN);
-#pragma unroll 1
-            for (int gi = wg; gi < ng; gi += 2) {
-                const int col = col0 + gi * GW;
-                const bool live = in_range && col < e.n_cols;
-                const bool visit = p.need_aux && live;       // this group's partner tile sits in ring slot c_slot
-                const uint8_t *ax = auxr + (wg + 2 * c_slot) * p.group_bytes;
-                if (etid == 0) {
-                    if (visit) ok = mbar_wait(&sh->aux_full[wg + 2 * c_slot], c_par);
-                    tma_store_wait_read();
-                }
-                if (visit && ++c_slot == SW) { c_slot = 0; c_par ^= 1u; }
-                ok = named_barrier_and(bar_b, 128, ok);
-                if (!ok) break;
-                const bool rowv = live && srow >= 0 && srow < valid_px;
-                const uint32_t tg = tm + (uint32_t)(gi * GW);
-                if (e.mode != EPI_COUPLE) {
-                    if (out_q == 0.f) tma_pass_a<0>(tg, GW, prow, rowv, ax, ob, out_s); else tma_pass_a<1>(tg, GW, prow, rowv, ax, ob, out_s);
-                } else if (out_q == 0.f) {
-                    if (e.sign > 0) tma_pass_a<2>(tg, GW, prow, rowv, ax, ob, out_s); else tma_pass_a<3>(tg, GW, prow, rowv, ax, ob, out_s);
-                } else {
-                    if (e.sign > 0) tma_pass_a<4>(tg, GW, prow, rowv, ax, ob, out_s); else tma_pass_a<5>(tg, GW, prow, rowv, ax, ob, out_s);
-                }
-                fence_proxy_async();
-                named_barrier(bar_a, 128);
-                if (etid == 0 && live) {
-                    tma_store_4d(out_map(col), ob, col_out(col), p.ox[cls], h0 * p.ostride + p.oy[cls], n0);
-                    tma_store_commit();
-                }
-                if (e.part && live && col + jq * 4 < e.n_cols) {
-                    float4 sc4 = make_float4(0, 0, 0, 0), sh4 = sc4, mu4 = sc4, rs4 = sc4;
-                    if (e.mode == EPI_BNBWD) bn_coef4(e.bn, col + jq * 4, sc4, sh4, mu4, rs4);
-                    float4 *slot = reinterpret_cast<float4 *>(gsums + (gi * 128 + etid) * 8);
-                    const float4 a0 = slot[0], a1 = slot[1];
-                    float acc[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                    if (e.mode == EPI_BNBWD) {
-                        if (t_q == 0.f) tma_pass_b<2>(GW, ob, ax, jq, r0, rpp, valid_px, 0.f, sc4, sh4, mu4, rs4, acc);
-                        else tma_pass_b<3>(GW, ob, ax, jq, r0, rpp, valid_px, t_q, sc4, sh4, mu4, rs4, acc);
-                    } else if (out_q == 0.f) tma_pass_b<0>(GW, ob, ax, jq, r0, rpp, valid_px, 0.f, sc4, sh4, mu4, rs4, acc);
-                    else tma_pass_b<1>(GW, ob, ax, jq, r0, rpp, valid_px, out_q, sc4, sh4, mu4, rs4, acc);
-                    slot[0] = make_float4(acc[0], acc[1], acc[2], acc[3]); slot[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
-                }
-                named_barrier(bar_a, 128);                 // the partner slot and the output slot have been read
-                if (etid == 0 && visit) load_next_aux();   // refill the slot just freed
-            }
-            if (!ok) break;
-            // this warp group has drained its columns of the accumulator: one arrival per group on the leader's barrier
-            tc_fence_before();
-            named_barrier(bar_a, 128);
-            if (etid == 0) mbar_arrive_cluster(acc_empty0[buf]);
-        }
-        if (etid == 0) tma_store_wait_all();
-        if (!ok && lane == 0) atomicExch(&sh->failed, 1u);
-        __threadfence_block();
-        named_barrier(5, 256);
-        if (wg == 0 && e.part && sh->failed == 0) {
-            float *mine = e.part + (size_t)blockIdx.x * 2 * e.n_cols;
-            for (int gi = 0; gi < ng; gi++) {
-                const int col = col0 + gi * GW + jq * 4;
-                if (r0 == 0 && col < e.n_cols) {
-                    const float *base = gsums + (size_t)gi * 128 * 8;
-                    float r[8];
-#pragma unroll
-                    for (int j = 0; j < 8; j++) r[j] = base[jq * 8 + j];
-                    for (int y = 1; y < rpp; y++)
-#pragma unroll
-                        for (int j = 0; j < 8; j++) r[j] += base[(y * QW + jq) * 8 + j];
-                    *reinterpret_cast<float4 *>(mine + 2 * col) = make_float4(r[0], r[1], r[2], r[3]);
-                    *reinterpret_cast<float4 *>(mine + 2 * col + 4) = make_float4(r[4], r[5], r[6], r[7]);
-                }
-            }
-            epilogue_publish<128>(e, reinterpret_cast<float *>(auxr), etid);
-        }
+        // epilogue of this CTA's own tile, as in conv_tc_kernel
+        tma_epilogue<true>(p, sh, EpiMaps{&map_o0, &map_o1, &map_x0, &map_x1}, auxr, tmem_d, col0, warp, lane, (int)rank, pair, n_pairs, n_vp, n_pp);
     }
     tc_fence_before();
     __syncthreads();
@@ -925,9 +859,6 @@ bool run_conv_tc(Exec &ex, const char *what, const void *act, Geom gin, int cin,
     // 16-row groups and there are at least two pixel tiles; REVNET_CONV_PAIR=0 keeps the single-CTA kernel (for comparison)
     // (1x1 layers are bound by the activations' way from HBM, which a pair does not shorten: measured 3-10 % slower there)
     bool pair = pair_enabled && epi_tma && (k == 3 || wide1) && s.BN % 32 == 0 && s.BN >= 64 && s.g.n_px_tiles >= 2 && ex.ctx->sm_count % 2 == 0;
-    // partner ring of the pair kernel: per epilogue warp group as many slots as it has column groups in a tile (at most 4)
-    int aux_slots = 0;
-    if (need_aux) { int sw = (ng + 1) / 2; if (sw > 4) sw = 4; aux_slots = 2 * sw; }
     // 3x3 stride-1 layers on a pair: the activations of a tile arrive once per channel chunk as one box with its halo
     // (see TcParams::halo); needs 64-channel chunks (128-byte operand rows) and tiles of whole image rows
     static const bool halo_enabled = [] { const char *v = getenv("REVNET_CONV_HALO"); return !(v && v[0] == '0'); }();
@@ -944,26 +875,41 @@ bool run_conv_tc(Exec &ex, const char *what, const void *act, Geom gin, int cin,
         a_box_bytes = box_rows * 128;
         a_slot_bytes = ((box_rows > read_rows ? box_rows : read_rows) * 128 + 1023) & ~1023;
     }
+    int groups = 2, aux_slots = 0, epi_bytes = 0;
+    bool inplace = false;
     if (epi_tma) {
-        stages = kStages;
         auto stage_bytes_of = [&](bool pr) {
             if (halo) return ((s.BN / 2) * s.KC * 2 + 1023) & ~1023;           // weight tiles only; the boxes are counted below
             return ((128 * s.KC * 2 + 1023) & ~1023) + (((pr ? s.BN / 2 : s.BN) * s.KC * 2 + 1023) & ~1023);
         };
-        auto smem_of = [&](int st, bool pr) { return 1024 + (halo ? a_slots * a_slot_bytes : 0) + st * stage_bytes_of(pr) + ((need_aux ? (pr ? aux_slots : ng) : 0) + 2) * group_bytes + ng * 128 * 32 + (int)sizeof(TcShared) + 64; };
-        // what does not fit gives way in this order: operand stages down to 3, partner slots down to 2 per warp group, stages down to 2
-        while (stages > 3 && smem_of(stages, pair) > 227 * 1024) stages--;
-        while (pair && aux_slots > 4 && smem_of(stages, pair) > 227 * 1024) aux_slots -= 2;
-        while (stages > 2 && smem_of(stages, pair) > 227 * 1024) stages--;
-        if (smem_of(stages, pair) > 227 * 1024) {
-            if (s.BN == 256) return false;      // (does not happen: three stages of a wide tile fit)
+        // Warp groups, partner slots per group and operand stages: the first of these that fits.  Single-CTA kernel: four groups (a
+        // divisor or a multiple of the column groups: three for three) as long as three operand stages remain (two if a tile has no more
+        // chunks); a coupling works in place in two slots per group.
+        const int iters = ntap_max * s.chunks, few = iters < 3 ? 2 : 3, want = pair ? 2 : (ng == 3 ? 3 : 4);
+        const struct { int groups, slots, stages; } tries[] = {{want, 2, few}, {want, 1, few}, {2, 2, few}, {2, 1, few}, {2, 2, 2}, {2, 1, 2}, {1, 1, 2}};
+        inplace = sign != 0;
+        bool fits = false;
+        for (const auto &y : tries) {
+            if (inplace && y.slots < 2) continue;
+            if (ng < y.groups && y.groups % ng) continue;
+            groups = y.groups; aux_slots = y.slots;
+            epi_bytes = ((need_aux ? groups * aux_slots : 0) + (inplace ? 0 : groups)) * group_bytes + (ng > groups ? ng * 4096 : 0);
+            const int least = groups * 4096 + (groups * 128 + 128) * 32;        // the sums at the end, and the last reduction
+            if (epi_bytes < least) epi_bytes = least;
+            auto smem_of = [&](int st) { return 1024 + (halo ? a_slots * a_slot_bytes : 0) + st * stage_bytes_of(pair) + epi_bytes + (int)sizeof(TcShared) + 64; };
+            stages = kStages;
+            while (stages > y.stages && smem_of(stages) > 227 * 1024) stages--;
+            if (smem_of(stages) <= 227 * 1024) { fits = true; s.smem = smem_of(stages); break; }
+        }
+        if (!fits) {
+            if (s.BN == 256) return false;      // (does not happen)
             epi_tma = false; pair = false; stages = 4;
             if (halo) { halo = false; tile_geom(g, s.g); }
-        } else s.smem = smem_of(stages, pair);
+        }
     }
     if ((s2 || s.BN == 256) && !epi_tma) return false;
     ex.flops += 2ull * g.P() * cout * cin * ntap_all;
-    int occ = (227 * 1024) / s.smem; if (occ > 2) occ = 2; if (occ < 1) occ = 1;
+    int occ = (227 * 1024) / s.smem; if (occ > 2) occ = 2; if (occ < 1 || groups > 2) occ = 1;      // (registers: 18 warps leave no room for a second CTA)
     int ctas = ex.ctx->sm_count * occ / s.n_tiles; if (ctas < 1) ctas = 1;
     if (ctas > s.g.n_px_tiles * n_cls) ctas = s.g.n_px_tiles * n_cls;
     if (pair) {
@@ -976,8 +922,13 @@ bool run_conv_tc(Exec &ex, const char *what, const void *act, Geom gin, int cin,
     size_t m = ex.ws.mark();
     bf16 *wp = prepacked ? const_cast<bf16 *>(prepacked) : ex.ws.get<bf16>((size_t)rows_pad * taps * s.cin_pad);
     const bool reduce = req.stats || req.bnbwd;
-    float *part = reduce ? ex.ws.get<float>((size_t)ctas * 2 * cout) : nullptr;
-    if (req.stats) req.stats->valid = true;
+    // statistics that the next layer's kernel adds up itself stay pending
+    const bool defer = req.stats && !req.bnbwd && epi_tma && req.stats->defer && req.stats->part && (size_t)ctas * 2 * cout <= req.stats->part_cap;
+    float *part = defer ? req.stats->part : (reduce ? ex.ws.get<float>((size_t)ctas * 2 * cout) : nullptr);
+    if (req.stats) {
+        req.stats->valid = true;
+        req.stats->pending = defer; req.stats->parts = ctas; req.stats->inv_count = 1.0 / ((double)g.P() * ostride * ostride);
+    }
     if (!ex.dry) {
         EncodeTiledFn enc = encoder(ex.ctx);
         // without a pack made earlier in the step, build it from the fp32 master weights now
@@ -1032,7 +983,7 @@ bool run_conv_tc(Exec &ex, const char *what, const void *act, Geom gin, int cin,
         }
         TcParams p;
         p.stages = stages; p.epi_tma = epi_tma ? 1 : 0; p.GW = GW; p.group_bytes = group_bytes; p.need_aux = need_aux ? 1 : 0;
-        p.aux_slots = aux_slots;
+        p.groups = groups; p.aux_slots = need_aux ? aux_slots : 0; p.inplace = inplace ? 1 : 0; p.epi_bytes = epi_bytes;
         p.split_o = out.c1 ? out.c0 : 0; p.split_x = (need_aux && auxp.c1) ? auxp.c0 : 0;
         memcpy(p.ntap, ntap, sizeof ntap); memcpy(p.tdy, tdy, sizeof tdy); memcpy(p.tdx, tdx, sizeof tdx); memcpy(p.tid, tid, sizeof tid);
         p.ostride = ostride; p.n_cls = n_cls;
@@ -1045,7 +996,7 @@ bool run_conv_tc(Exec &ex, const char *what, const void *act, Geom gin, int cin,
         memset(&e, 0, sizeof e);
         e.mode = req.bnbwd ? EPI_BNBWD : (sign ? EPI_COUPLE : EPI_PLAIN);
         e.out = out; e.partner = partner; e.sign = sign; e.n_cols = cout; e.pitch = kEpiPitch;
-        e.part = part; e.counter = reduce ? ex.ctx->counter() : nullptr;
+        e.part = part; e.counter = reduce && !defer ? ex.ctx->counter() : nullptr;
         e.inv_count = 1.0 / ((double)g.P() * ostride * ostride); e.eps = ex.eps;     // pixels of the output grid
         if (req.stats) { e.mean = req.stats->mean; e.rstd = req.stats->rstd; }
         if (req.bnbwd) { e.t = req.bnbwd->t; e.bn = req.bnbwd->bn; e.dgamma = req.bnbwd->dgamma; e.dbeta = req.bnbwd->dbeta; e.coef = req.bnbwd->coef; }
@@ -1055,8 +1006,8 @@ bool run_conv_tc(Exec &ex, const char *what, const void *act, Geom gin, int cin,
             cudaFuncSetAttribute(conv_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         }
         dim3 grid((unsigned)ctas, (unsigned)s.n_tiles);
-        if (pair) launch_cluster(ex, conv_tc2_kernel, grid, kThreadsTma, s.smem, 2, map_a, map_b, map_o[0], map_o[1], map_x[0], map_x[1], p);
-        else launch(ex, conv_tc_kernel, grid, epi_tma ? kThreadsTma : kThreads, s.smem, map_a, map_b, map_o[0], map_o[1], map_x[0], map_x[1], p);
+        if (pair) launch_cluster(ex, conv_tc2_kernel, grid, 64 + groups * 128, s.smem, 2, map_a, map_b, map_o[0], map_o[1], map_x[0], map_x[1], p);
+        else launch(ex, conv_tc_kernel, grid, epi_tma ? 64 + groups * 128 : kThreads, s.smem, map_a, map_b, map_o[0], map_o[1], map_x[0], map_x[1], p);
         const double bytes = (double)gin.P() * cin * 2 + (double)g.P() * cout * (sign || req.bnbwd ? 8 : 4) + (double)cout * taps * cin * 2;
         // (records of launches on a CTA pair carry the pair kernel's name)
         ex.check(!pair ? what : (transposed ? "conv_dgrad_tc2" : "conv_fprop_tc2"), bytes, 2.0 * g.P() * cout * cin * ntap_all);

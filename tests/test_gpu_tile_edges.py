@@ -28,6 +28,9 @@ def ctx():
     ("basic", 4, 13, 13, 56, 0),          # seven planes, 56 of 64 output columns
     ("basic", 2, 16, 16, 64, 0),          # the widest layer with its BN and ReLU inside
     ("bottleneck", 6, 9, 9, 32, 12),      # 1x1; rows of 48 bytes: 16-byte accesses
+    ("bottleneck", 10, 23, 9, 128, 32),   # one column group: four warp groups on alternate tiles, records left to the consumer
+    ("bottleneck", 10, 23, 9, 128, 64),   # two column groups
+    ("bottleneck", 10, 23, 9, 160, 96),   # three
     ("bottleneck", 1, 97, 99, 520, 8),    # streaming kernels with 32-byte accesses: 65 octets of channels, three rows per pass
     ("bottleneck", 8, 9, 9, 136, 72),     # weight packs with padded rows (136 -> 256, 72 -> 80) and columns (136 -> 144)
 ])
