@@ -1,9 +1,11 @@
 // The stem: a bare convolution of the 3-channel image (3x3 stride 1, or 7x7 stride 2), fp32 in both
 // precision modes, forward and weight gradient.  With so few input channels the contraction per
 // output pixel is short (K = k*k*3 = 27 or 147) and a tensor-core tile would be mostly padding, so
-// these are register-tiled CUDA-core kernels: the image patches of a tile of output pixels (128
-// forward, 64 for the weight gradient) are gathered into shared memory once and every thread keeps a
-// small block of the result in registers.
+// these are register-tiled CUDA-core kernels.  The stems that the networks have (three channels; 3x3
+// stride 1, 7x7 stride 2) take the row kernels: image rows in shared memory, a lane per one or two output
+// channels, a window of image values that slides along the row in registers.  Other shapes take the patch
+// kernels: the image patches of a tile of output pixels (128 forward, 64 for the weight gradient) are
+// gathered into shared memory once and every thread keeps a small block of the result in registers.
 //
 //   fprop: out[p, co]      = sum_{kh,kw,ci} img[p*s + (kh,kw) - pad, ci] * W[co, kh, kw, ci]
 //   wgrad: dW[co, kh,kw,ci] = sum_p g[p, co] * img[p*s + (kh,kw) - pad, ci]
@@ -183,6 +185,205 @@ __global__ void __launch_bounds__(256) stem_wgrad_kernel(const float *__restrict
         }
 }
 
+// ------------------------------------------------------------------ three channels, 3x3 stride 1 or 7x7 stride 2
+// Image rows y0 .. y0 + rows - 1 of image n into shared memory, element (row, column, channel) at
+// row * rp + (column + pad) * xp + channel * cp; rows outside the image become zeros, the columns beside it stay as they are
+// (zero since the start of the kernel).  Asynchronous: the caller waits.
+__device__ __forceinline__ void stage_rows(const float *__restrict__ img, const StemGeom &g, FastDiv rowdiv, int n, int y0, int rows, float *dst, int rp, int xp, int cp) {
+    const int row_e = g.W * 3;
+    for (int e = threadIdx.x; e < rows * row_e; e += blockDim.x) {
+        uint32_t r, q;
+        rowdiv.divmod((uint32_t)e, r, q);
+        const uint32_t x = q / 3, c = q - 3 * x;
+        const int y = y0 + (int)r;
+        const bool ok = (unsigned)y < (unsigned)g.H && n < g.N;
+        const float *src = img + (ok ? ((size_t)n * g.H + y) * row_e + q : 0);
+        const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + (int)r * rp + ((int)x + g.pad) * xp + (int)c * cp);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(ok ? 4 : 0) : "memory");
+    }
+}
+template <int K> struct StemRow {
+    static constexpr int S = K == 3 ? 1 : 2;
+    // weight gradient: KH rows of the filter per warp, RS output rows per CTA, U pixels per turn (a multiple of K: the window has
+    // turned), CBW channel groups of 32 at most per CTA
+    static constexpr int KH = K == 3 ? 3 : 1, HG = K / KH, RS = K == 3 ? 8 : 1, U = K == 3 ? 12 : 7, CBW = K == 3 ? 1 : 4;
+    // forward (7x7): output rows per CTA, warps
+    static constexpr int FR = 2, FW = 14;
+};
+
+// Weight gradient.  A warp has KH filter rows and 32 output channels, a lane each, and goes along output rows: per pixel S new image
+// columns and one gradient value come in, KH * K * 3 FMAs follow from registers.  Every 128 pixels or more the
+// sums are added to totals in shared memory, which are added over the warps of a filter row and written as one partial per CTA.
+// Bound by the FMA pipes.  Measured: 131072 pixels x 32 channels, 3x3: 59 -> 20 us; 802816 x 128, 7x7: 1405 -> 1045 us (29 TFLOP/s;
+// single FMAs reach 56).
+template <int K>
+__global__ void __launch_bounds__(K == 3 ? 256 : 896) stem_wgrad_row_kernel(const float *__restrict__ img, const float *__restrict__ gout, float *__restrict__ part,
+                                                                           StemGeom g, FastDiv rowdiv, int cols, int tiles_per_img, int n_tiles, int cbw) {
+    using T = StemRow<K>;
+    constexpr int S = T::S, KH = T::KH, A = KH * K * 3, U = T::U, ROWS = (T::RS - 1) * S + K;
+    extern __shared__ float sm[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
+    const int hg = warp % T::HG, cb = (warp / T::HG) % cbw, rs = warp / (T::HG * cbw);
+    const int co = ((int)blockIdx.y * cbw + cb) * 32 + lane;
+    const int rp = cols * 4, buf_floats = ROWS * rp;
+    float *tot = sm + 2 * buf_floats;                                  // [warp][A][32]
+    for (int i = tid; i < 2 * buf_floats + nw * A * 32; i += blockDim.x) sm[i] = 0.f;
+    __syncthreads();
+    pdl_enter();
+    float acc[A];
+#pragma unroll
+    for (int a = 0; a < A; a++) acc[a] = 0.f;
+    auto stage = [&](int t, int b) {
+        const int n = t / tiles_per_img, y0 = (t - n * tiles_per_img) * T::RS;
+        stage_rows(img, g, rowdiv, n, y0 * S - g.pad, ROWS, sm + b * buf_floats, rp, 4, 1);
+    };
+    float *mytot = tot + (size_t)warp * A * 32 + lane;
+    auto flush = [&]() {
+#pragma unroll
+        for (int a = 0; a < A; a++) { mytot[a * 32] += acc[a]; acc[a] = 0.f; }
+    };
+    int b = 0, held = 0;
+    if ((int)blockIdx.x < n_tiles) stage(blockIdx.x, 0);
+    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, b ^= 1) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        if (t + (int)gridDim.x < n_tiles) stage(t + gridDim.x, b ^ 1);
+        const int n = t / tiles_per_img, y = (t - n * tiles_per_img) * T::RS + rs;
+        if (y < g.Ho && co < g.Co) {
+            const float *gp = gout + (((size_t)n * g.Ho + y) * g.Wo) * g.Co + co;
+            const float *rowp = sm + b * buf_floats + (rs * S + hg * KH) * rp;
+            auto load_g = [&](int x, float (&v)[U]) {
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    const bool in = x + u < g.Wo;
+                    const float q = gp[(size_t)(in ? x + u : 0) * g.Co];
+                    v[u] = in ? q : 0.f;
+                }
+            };
+            float win[KH][K][3], gv[U], gn[U];
+            auto column = [&](int c, int slot) {
+#pragma unroll
+                for (int r = 0; r < KH; r++) {
+                    const float4 q = *reinterpret_cast<const float4 *>(rowp + r * rp + c * 4);
+                    win[r][slot][0] = q.x; win[r][slot][1] = q.y; win[r][slot][2] = q.z;
+                }
+            };
+#pragma unroll
+            for (int c = 0; c < K - S; c++) column(c, c);
+            load_g(0, gv);
+#pragma unroll 1
+            for (int x = 0; x < g.Wo; x += U) {
+                load_g(x + U, gn);
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+#pragma unroll
+                    for (int c = K - S; c < K; c++) column((x + u) * S + c, (u * S + c) % K);
+#pragma unroll
+                    for (int r = 0; r < KH; r++)
+#pragma unroll
+                        for (int kw = 0; kw < K; kw++)
+#pragma unroll
+                            for (int ci = 0; ci < 3; ci++)
+                                acc[(r * K + kw) * 3 + ci] = fmaf(gv[u], win[r][(u * S + kw) % K][ci], acc[(r * K + kw) * 3 + ci]);
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++) gv[u] = gn[u];
+            }
+            held += g.Wo;
+            if (held >= 128) { flush(); held = 0; }
+        }
+    }
+    flush();
+    __syncthreads();
+    // one partial per CTA: dW[co][kh][kw][ci], the row warps added in order
+    const int K27 = K * K * 3, n_co = cbw * 32, co0 = (int)blockIdx.y * n_co;
+    float *mine = part + (size_t)blockIdx.x * g.Co * K27;
+    const int n_rs = nw / (T::HG * cbw);
+    for (int e = tid; e < n_co * K27; e += blockDim.x) {
+        const int c = e / K27, kk = e - c * K27, h = kk / (KH * K * 3), a = kk - h * (KH * K * 3);
+        if (co0 + c >= g.Co) continue;
+        float v = 0.f;
+        for (int r = 0; r < n_rs; r++) v += tot[((size_t)((r * cbw + c / 32) * T::HG + h) * A + a) * 32 + c % 32];
+        mine[(size_t)(co0 + c) * K27 + kk] = v;
+    }
+}
+
+// Forward, 7x7.  A warp takes eight pixels of an output row and 32 COL output channels: per filter row and channel the image values of
+// its pixels (21 of them, planar rows in shared memory) and one weight row per column tap, 8 COL FMAs each.
+// Bound by the FMA pipes.  Measured: 802816 pixels x 128 channels: 1610 -> 890 us.
+template <int COL>
+__global__ void __launch_bounds__(StemRow<7>::FW * 32) stem_fprop_row_kernel(const float *__restrict__ img, const float *__restrict__ W, Pair out,
+                                                                           StemGeom g, FastDiv rowdiv, int cols, int tiles_per_img, int n_tiles, int cop) {
+    constexpr int K = 7;
+    using T = StemRow<K>;
+    constexpr int S = T::S, ROWS = (T::FR - 1) * S + K, NX = (7 * S + K + 3) / 4;
+    extern __shared__ float sm[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
+    float *Ws = sm;                                                    // [kh][ci][kw][cop]
+    float *rowsm = Ws + K * K * 3 * cop;                               // two buffers of [row][ci][cols]
+    const int buf_floats = ROWS * 3 * cols;
+    for (int i = tid; i < 2 * buf_floats; i += blockDim.x) rowsm[i] = 0.f;
+    for (int e = tid; e < K * K * 3 * cop; e += blockDim.x) {
+        const int co = e / (K * K * 3), kk = e - co * (K * K * 3), kh = kk / (K * 3), kw = kk / 3 % K, ci = kk % 3;
+        Ws[((kh * 3 + ci) * K + kw) * cop + co] = co < g.Co ? W[(size_t)co * (K * K * 3) + kk] : 0.f;
+    }
+    __syncthreads();
+    pdl_enter();
+    auto stage = [&](int t, int b) {
+        const int n = t / tiles_per_img, y0 = (t - n * tiles_per_img) * T::FR;
+        stage_rows(img, g, rowdiv, n, y0 * S - g.pad, ROWS, rowsm + b * buf_floats, 3 * cols, 1, cols);
+    };
+    const int segs = (g.Wo + 7) / 8, cbs = cop / (32 * COL), tasks = T::FR * segs * cbs;
+    int b = 0;
+    if ((int)blockIdx.x < n_tiles) stage(blockIdx.x, 0);
+    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, b ^= 1) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        if (t + (int)gridDim.x < n_tiles) stage(t + gridDim.x, b ^ 1);
+        const int n = t / tiles_per_img, y0 = (t - n * tiles_per_img) * T::FR;
+        for (int task = warp; task < tasks; task += nw) {
+            const int cb = task % cbs, q = task / cbs, seg = q % segs, r = q / segs;
+            const int co = cb * 32 * COL + lane * COL;
+            if (y0 + r >= g.Ho) break;
+            const float *xp = rowsm + b * buf_floats + r * S * 3 * cols + seg * 8 * S;
+            const float *wp = Ws + co;
+            float acc[8][COL];
+#pragma unroll
+            for (int i = 0; i < 8; i++)
+#pragma unroll
+                for (int j = 0; j < COL; j++) acc[i][j] = 0.f;
+#pragma unroll 3
+            for (int kc = 0; kc < K * 3; kc++) {                       // filter row and channel
+                float v[NX * 4];
+#pragma unroll
+                for (int i = 0; i < NX; i++) {
+                    const float4 u = *reinterpret_cast<const float4 *>(xp + kc * cols + 4 * i);
+                    v[4 * i] = u.x; v[4 * i + 1] = u.y; v[4 * i + 2] = u.z; v[4 * i + 3] = u.w;
+                }
+#pragma unroll
+                for (int kw = 0; kw < K; kw++) {
+                    float w[COL];
+                    if constexpr (COL == 2) { const float2 u = *reinterpret_cast<const float2 *>(wp + (kc * K + kw) * cop); w[0] = u.x; w[1] = u.y; }
+                    else w[0] = wp[(kc * K + kw) * cop];
+#pragma unroll
+                    for (int i = 0; i < 8; i++)
+#pragma unroll
+                        for (int j = 0; j < COL; j++) acc[i][j] = fmaf(v[i * S + kw], w[j], acc[i][j]);
+                }
+            }
+            if (co < g.Co)
+#pragma unroll
+                for (int i = 0; i < 8; i++) {
+                    const int x = seg * 8 + i;
+                    if (x >= g.Wo) continue;
+                    const size_t p = ((size_t)n * g.Ho + y0 + r) * g.Wo + x;
+                    if constexpr (COL == 2) out.couple2_with(p, co, make_float2(acc[i][0], acc[i][1]), make_float2(0.f, 0.f), 0);
+                    else out.couple(p, co, acc[i][0], out, 0);
+                }
+        }
+    }
+}
+
 // dW[i] = sum of the per-CTA partials, one warp per element: lane l adds the partials l, l + 32, ... and the
 // lanes are combined by a shuffle tree, so the order of additions is fixed by `parts` alone
 __global__ void stem_sum_kernel(const float *__restrict__ part, size_t n, int parts, float *__restrict__ out) {
@@ -208,10 +409,65 @@ int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
 }  // namespace
 
+// whether the row kernels take a stem, and their row pitch: columns -pad .. of the rows that the last turn of `turn` pixels reads
+static bool row_stem(const StemGeom &g, int turn, int &cols) {
+    if (g.Ci != 3 || !((g.k == 3 && g.s == 1) || (g.k == 7 && g.s == 2)) || (size_t)g.W * 3 * 32 > (1u << 30)) return false;
+    cols = round_up((round_up(g.Wo, turn) - 1) * g.s + g.k, 4) + 4;
+    if (cols < g.W + 2 * g.pad) cols = round_up(g.W + 2 * g.pad, 4);
+    return true;
+}
+template <class F> static int row_grid(Exec &ex, F kernel, int threads, size_t smem, int n_tiles, int blocks_y) {
+    int per_sm = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess || per_sm < 1) { cudaGetLastError(); per_sm = 1; }
+    int ctas = ex.ctx->sm_count * per_sm / blocks_y; if (ctas < 1) ctas = 1;
+    const int rounds = (n_tiles + ctas - 1) / ctas;
+    return (n_tiles + rounds - 1) / rounds;
+}
+// (3x3: the patch kernel is the quicker one, 18 against 24 us for 131072 x 32)
+template <int COL> static bool fprop_rows(Exec &ex, const float *img, const StemGeom &g, const float *W, Pair out) {
+    constexpr int K = 7;
+    using T = StemRow<K>;
+    int cols;
+    if (g.k != K || !row_stem(g, 8, cols)) return false;
+    const int cop = round_up(g.Co, 32 * COL), tiles_per_img = (g.Ho + T::FR - 1) / T::FR, n_tiles = g.N * tiles_per_img;
+    const size_t smem = ((size_t)g.K * cop + 2 * (size_t)((T::FR - 1) * T::S + K) * 3 * cols) * 4;
+    if (smem > 200 * 1024) return false;
+    if (ex.dry) return true;
+    static OncePerDevice once;
+    if (once.first(ex.ctx->device)) cudaFuncSetAttribute(stem_fprop_row_kernel<COL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    const int grid = row_grid(ex, stem_fprop_row_kernel<COL>, T::FW * 32, smem, n_tiles, 1);
+    launch(ex, stem_fprop_row_kernel<COL>, grid, T::FW * 32, smem, img, W, out, g, fast_div(g.W * 3), cols, tiles_per_img, n_tiles, cop);
+    return true;
+}
+// part: room for `cap` partials; the number written goes to `parts`
+template <int K> static bool wgrad_rows(Exec &ex, const float *img, const float *gout, const StemGeom &g, float *part, int cap, int &parts) {
+    using T = StemRow<K>;
+    int cols;
+    if (!row_stem(g, T::U, cols)) return false;
+    const int cbs = (g.Co + 31) / 32, cbw = cbs < T::CBW ? cbs : T::CBW, blocks_y = (cbs + cbw - 1) / cbw;
+    const int nw = T::HG * cbw * T::RS, tiles_per_img = (g.Ho + T::RS - 1) / T::RS, n_tiles = g.N * tiles_per_img;
+    const size_t smem = (2 * (size_t)((T::RS - 1) * T::S + K) * cols * 4 + (size_t)nw * T::KH * K * 3 * 32) * 4;
+    if (smem > 200 * 1024) return false;
+    if (ex.dry) return true;
+    static OncePerDevice once;
+    if (once.first(ex.ctx->device)) cudaFuncSetAttribute(stem_wgrad_row_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    parts = row_grid(ex, stem_wgrad_row_kernel<K>, nw * 32, smem, n_tiles, blocks_y);
+    if (parts > cap) parts = cap;
+    launch(ex, stem_wgrad_row_kernel<K>, dim3(parts, blocks_y), nw * 32, smem, img, gout, part, g, fast_div(g.W * 3), cols, tiles_per_img, n_tiles, cbw);
+    return true;
+}
+
 // image: fp32 [N,H,W,cin]; out: the stem's output (a plain tensor or the halves of stage 0's pair, float or fixed point)
 bool stem_fprop(Exec &ex, const float *img, Geom gi, const Layer &L, Pair out) {
     const StemGeom g = stem_geom(gi, L);
     if (L.cin > 255 || L.k > 255 || L.cout % 4 || (out.c1 && out.c0 % 4)) return false;
+    const bool wide = L.cout > 32;
+    if (wide ? fprop_rows<2>(ex, img, g, L.W, out) : fprop_rows<1>(ex, img, g, L.W, out)) {
+        const double P = (double)g.N * g.Ho * g.Wo;
+        ex.flops += 2ull * g.N * g.Ho * g.Wo * g.Co * g.K;
+        if (!ex.dry) ex.check("stem_fprop", (double)g.N * g.H * g.W * g.Ci * 4 + P * g.Co * 4 + (double)g.Co * g.K * 4, 2.0 * P * g.Co * g.K);
+        return true;
+    }
     const int CO_T = L.cout >= 64 ? 8 : 4;
     const int cop = round_up(L.cout, 8 * CO_T);
     const size_t smem = ((size_t)g.K * cop + (size_t)g.K * kFPx) * 4 + (size_t)g.K * 4;
@@ -240,23 +496,28 @@ bool stem_wgrad(Exec &ex, const float *img, const float *gout, Geom gi, const La
     const int CO_T = big ? 8 : 4, KK_T = big ? 12 : 4;
     const int cop = round_up(L.cout, CO_T), kp = round_up(g.K, KK_T);
     const int n_cg = cop / CO_T, n_kg = kp / KK_T, G = n_cg * n_kg;
-    if (G > 256) return false;
-    const int S = 256 / G;
-    const size_t smem = ((size_t)kPx * cop + (size_t)kPx * kp) * 4 + (size_t)g.K * 4;
-    if (smem > 200 * 1024) return false;
     const int P = g.N * g.Ho * g.Wo, n_chunks = (P + kPx - 1) / kPx;
-    int grid = ex.ctx->sm_count * 2; if (grid > n_chunks) grid = n_chunks;
+    const size_t smem = ((size_t)kPx * cop + (size_t)kPx * kp) * 4 + (size_t)g.K * 4;
+    int cols;
+    const bool rows = row_stem(g, 1, cols);
+    if (!rows && (G > 256 || smem > 200 * 1024)) return false;
+    int grid = ex.ctx->sm_count * (g.k == 3 ? 4 : 2); if (grid > n_chunks) grid = n_chunks;         // room for that many partials
     ex.flops += 2ull * P * g.Co * g.K;
     size_t m = ex.ws.mark();
     float *part = ex.ws.get<float>((size_t)grid * g.Co * g.K);
     if (!ex.dry) {
-        static OncePerDevice once;
-        if (once.first(ex.ctx->device)) {
-            cudaFuncSetAttribute(stem_wgrad_kernel<8, 12>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-            cudaFuncSetAttribute(stem_wgrad_kernel<4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        if (!(rows && (g.k == 3 ? wgrad_rows<3>(ex, img, gout, g, part, grid, grid) : wgrad_rows<7>(ex, img, gout, g, part, grid, grid)))) {
+            if (G > 256 || smem > 200 * 1024) { ex.ws.release(m); return false; }
+            if (grid > ex.ctx->sm_count * 2) grid = ex.ctx->sm_count * 2;
+            const int S = 256 / G;
+            static OncePerDevice once;
+            if (once.first(ex.ctx->device)) {
+                cudaFuncSetAttribute(stem_wgrad_kernel<8, 12>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+                cudaFuncSetAttribute(stem_wgrad_kernel<4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+            }
+            if (big) launch(ex, stem_wgrad_kernel<8, 12>, grid, 256, smem, img, gout, part, g, cop, kp, n_cg, G, S, n_chunks);
+            else launch(ex, stem_wgrad_kernel<4, 4>, grid, 256, smem, img, gout, part, g, cop, kp, n_cg, G, S, n_chunks);
         }
-        if (big) launch(ex, stem_wgrad_kernel<8, 12>, grid, 256, smem, img, gout, part, g, cop, kp, n_cg, G, S, n_chunks);
-        else launch(ex, stem_wgrad_kernel<4, 4>, grid, 256, smem, img, gout, part, g, cop, kp, n_cg, G, S, n_chunks);
         ex.check("stem_wgrad", (double)g.N * g.H * g.W * g.Ci * 4 + (double)P * g.Co * 4, 2.0 * P * g.Co * g.K);
         const size_t n = (size_t)g.Co * g.K;
         int sg = (int)((n + 7) / 8); if (sg > ex.ctx->sm_count * 8) sg = ex.ctx->sm_count * 8;      // eight warps per block

@@ -3,10 +3,13 @@ more than a tile holds, widths that leave padded operand planes, reductions of o
 Everything is compared with the float64 oracle under the stated tolerances (tests/parity.py: 1e-4 in the
 strict mode, 2e-2 outputs and 5e-2 gradients in the bf16 mode), which bound rounding at any size here:
 the longest sum has 1224 products."""
+from dataclasses import replace
+
 import pytest
 
 from paper_1707_04585_b200 import binding as B
 from paper_1707_04585_b200 import synthetic as syn
+from tests import helpers as hp
 from tests import test_gpu_parity as tp
 
 pytestmark = pytest.mark.gpu
@@ -53,6 +56,17 @@ def test_bf16_blocks_at_tile_edges(ctx, kind, N, H, W, c, w):
 ])
 def test_strict_blocks_at_tile_edges(ctx, kind, N, H, W, c, w):
     tp.run_block_case(ctx, syn.BlockCfg(N, H, W, c, w, kind, seed=900 + c), 1, jitter=True, inplace=True)
+
+
+@pytest.mark.parametrize("img,k,stem_c", [
+    (10, 3, 40),       # 3x3 row kernel: rows of ten pixels in turns of twelve, a second channel group of 8 lanes
+    (48, 7, 72),       # 7x7: rows of 24 pixels in turns of seven, three channel groups of the weight gradient
+    (56, 7, 8),        # one channel per lane, rows of 28 pixels in segments of eight
+])
+def test_stems_at_tile_edges(ctx, img, k, stem_c):
+    cfg = replace(hp.tiny_stack("bottleneck", k == 7, N=3), img=img, stem_cout=stem_c)
+    tp.run_stack_case(ctx, cfg, 1)
+    tp.ORACLE_RUNS.clear()
 
 
 @pytest.mark.parametrize("mode", [0, 1])
