@@ -800,6 +800,9 @@ bool run_conv_tc(Exec &ex, const char *what, const void *act, Geom gin, int cin,
                  const float *Wsrc, const bf16 *prepacked, bool transposed, Pair out, Pair partner, int sign, EpiReq req,
                  bool s2 = false) {
     TcShape s;
+    // a 1x1 layer has no neighbours: its pixels as one column, 128 of them per tile (by image rows a tile holds 112 of 56x56 or
+    // 28x28 images, 98 of 7x7)
+    if (k == 1 && stride == 1 && !s2 && gin.P() < (1u << 30)) gin = Geom{1, (int)gin.P(), 1};
     if (stride == 2 && (gin.H % 2 || gin.W % 2)) return false;
     if (s2 && (stride != 1 || k != 3 || !transposed || sign || req.stats || out.c1)) return false;
     const Geom g{gin.N, conv_out(gin.H, k, stride), conv_out(gin.W, k, stride)};   // geometry of the tiles
