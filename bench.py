@@ -43,7 +43,7 @@ ALU_KERNELS = ("gemm_simt_kernel",)   # fp32 CUDA-core GEMMs
 DEVICE_KERNEL = {
     "conv_fprop_fused": "conv_fused_kernel", "conv_dgrad_fused": "conv_fused_kernel",
     "conv_fprop_tc": "conv_tc_kernel", "conv_dgrad_tc": "conv_tc_kernel", "conv_wgrad_tc": "wgrad_tc_kernel",
-    "conv_fprop_tc2": "conv_tc2_kernel", "conv_dgrad_tc2": "conv_tc2_kernel", "conv_wgrad_tc2": "wgrad_tc2_kernel",
+    "conv_fprop_bn": "conv1x1_bn_kernel", "conv_fprop_tc2": "conv_tc2_kernel", "conv_dgrad_tc2": "conv_tc2_kernel", "conv_wgrad_tc2": "wgrad_tc2_kernel",
     "conv_fprop_simt": "gemm_simt_kernel", "conv_dgrad_simt": "gemm_simt_kernel", "conv_wgrad_simt": "gemm_simt_kernel",
     "bn_stats": "col_reduce_kernel", "bn_bwd_sums": "col_reduce_kernel",
 }
@@ -53,6 +53,7 @@ KERNEL_SOURCES = {
     "wgrad_tc_kernel": ("conv_tc.cu", "tc_ptx.cuh"),
     "conv_tc2_kernel": ("conv_tc.cu", "conv_epilogue.cuh", "tc_ptx.cuh"),
     "wgrad_tc2_kernel": ("conv_tc.cu", "tc_ptx.cuh"),
+    "conv1x1_bn_kernel": ("conv_tc.cu", "conv_epilogue.cuh", "tc_ptx.cuh"),
 }
 
 

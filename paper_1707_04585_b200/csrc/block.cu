@@ -21,6 +21,7 @@ bool conv_wgrad_tc_batch(Exec &ex, int n, const void *const *gq, const void *con
                          float *scratch, size_t *need);
 // one kernel for BN -> ReLU -> conv (at most 64 input channels, stride 1); likewise the data gradient of such a layer
 bool conv_fused_takes(Exec &ex, Geom gi, const Layer &L);
+bool conv_fprop_bn(Exec &ex, Pair t, BnRef bn, Geom gi, const Layer &L, Pair out, Moments *stats, bf16 *a_out);
 bool conv_fprop_fused(Exec &ex, Pair t, BnRef bn, Geom gi, const Layer &L, Pair out, Pair partner, int sign, Moments *stats, bf16 *a_out);
 bool conv_dgrad_fused(Exec &ex, const void *g, Geom gi, const Layer &L, float *da, const BnBwdReq *bb);
 
@@ -101,6 +102,7 @@ void fn_forward(Exec &ex, Geom g, Pair u, const Moments *mom_in, const std::vect
             fused = conv_fprop_fused(ex, t, bn, gi, ly, o, last ? partner : Pair{}, last ? sign : 0, last ? mom_out : &next,
                                      saved ? (bf16 *)a : nullptr);
         if (fused) cur.pending = false;     // the fused kernel has stored mean and rstd
+        else if (b16 && !last && !cur.pending && conv_fprop_bn(ex, t, bn, gi, ly, o, &next, saved ? (bf16 *)a : nullptr)) fused = true;
         else { mom_finalize(ex, cur, ly.cin); bn_relu_apply(ex, t, P, BnRef{ly.gamma, ly.beta, cur.mean, cur.rstd}, a, b16); }
         if (saved) { saved->a.push_back(a); saved->bn.push_back(cur); }
         if (last) {

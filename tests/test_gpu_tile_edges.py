@@ -34,6 +34,8 @@ def ctx():
     ("bottleneck", 10, 23, 9, 128, 32),   # one column group: four warp groups on alternate tiles, records left to the consumer
     ("bottleneck", 10, 23, 9, 128, 64),   # two column groups
     ("bottleneck", 10, 23, 9, 160, 96),   # three
+    ("bottleneck", 1, 9, 11, 128, 8),     # BN inside the wide 1x1: less than one tile, one 16-column group
+    ("bottleneck", 3, 61, 107, 448, 128), # 153 tiles: some CTAs take two; seven chunks through three raw slots, four column groups
     ("bottleneck", 1, 97, 99, 520, 8),    # streaming kernels with 32-byte accesses: 65 octets of channels, three rows per pass
     ("bottleneck", 8, 9, 9, 136, 72),     # weight packs with padded rows (136 -> 256, 72 -> 80) and columns (136 -> 144)
 ])
