@@ -80,7 +80,10 @@ void fn_forward(Exec &ex, Geom g, Pair u, const Moments *mom_in, const std::vect
         const Layer &ly = layers[l];
         const size_t P = gi.P();
         if (!cur.valid) {
-            cur = mom_alloc(ex, ly.cin);
+            // the fused kernel adds the records itself: they stay pending (small tensors have too few for that to pay: see bn_stats)
+            const bool defer = b16 && P * ly.cin > 65536 && t.c1 == 0 && !(l == L - 1 && (skip_last_conv || out.c1 || partner.c1)) && conv_fused_takes(ex, gi, ly);
+            cur = mom_alloc(ex, ly.cin, defer);
+            cur.defer = defer;
             bn_stats(ex, t, P, cur);
             cur.valid = true;
         }
@@ -91,16 +94,14 @@ void fn_forward(Exec &ex, Geom g, Pair u, const Moments *mom_in, const std::vect
         void *a = ex.ws.alloc(P * ly.cin * esz(ex));
         float *tn = last ? nullptr : ex.ws.get<float>(go.P() * ly.cout);
         Moments next;
-        if (!last) {
-            next = mom_alloc(ex, ly.cout, b16);      // with room for pending partials: the next layer consumes them
-            const bool to_last = l + 1 == L - 1;
-            next.defer = b16 && !(to_last && (skip_last_conv || out.c1 || partner.c1)) && conv_fused_takes(ex, go, layers[l + 1]);
-        }
+        if (!last) next = mom_alloc(ex, ly.cout, b16);      // with room for pending partials: the next layer consumes them
         const Pair o = last ? out : single(tn, ly.cout);
         bool fused = false;
         if (b16 && !(last && skip_last_conv))
             fused = conv_fprop_fused(ex, t, bn, gi, ly, o, last ? partner : Pair{}, last ? sign : 0, last ? mom_out : &next,
                                      saved ? (bf16 *)a : nullptr);
+        if (!fused && b16 && !last)         // whether the next layer adds the records of this one itself
+            next.defer = !(l + 1 == L - 1 && (skip_last_conv || out.c1 || partner.c1)) && conv_fused_takes(ex, go, layers[l + 1]);
         if (fused) cur.pending = false;     // the fused kernel has stored mean and rstd
         else if (b16 && !last && !cur.pending && conv_fprop_bn(ex, t, bn, gi, ly, o, &next, saved ? (bf16 *)a : nullptr)) fused = true;
         else { mom_finalize(ex, cur, ly.cin); bn_relu_apply(ex, t, P, BnRef{ly.gamma, ly.beta, cur.mean, cur.rstd}, a, b16); }

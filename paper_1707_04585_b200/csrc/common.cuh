@@ -383,7 +383,7 @@ Moments mom_alloc(Exec &ex, int C, bool with_part = false);
 void mom_finalize(Exec &ex, Moments &m, int C);
 // batch statistics of t ([P,C]) -> mean, rstd (the convolution epilogues produce the same quantities for the
 // tensors they write)
-void bn_stats(Exec &ex, Pair t, size_t P, Moments m);
+void bn_stats(Exec &ex, Pair t, size_t P, Moments &m);
 // a = relu(scale*t + shift) written as one [P,C] tensor of float (strict) or bf16
 void bn_relu_apply(Exec &ex, Pair t, size_t P, BnRef bn, void *a, bool a_bf16);
 // BN+ReLU backward: da [P,C] fp32; t the BN input.  Unless sums_done (a data-gradient epilogue

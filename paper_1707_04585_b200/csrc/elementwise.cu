@@ -79,13 +79,14 @@ __device__ __forceinline__ void st4(bf16 *p, float4 v) {
 // with the whole L1;
 // a row in flight per thread and a second kernel over uncoalesced partials before).
 struct RedShape { int SW, RPP, slabs, chunks, rows_per_cta; };
-static RedShape red_shape(size_t P, int C, int sm, int rows_in_flight) {
+static RedShape red_shape(size_t P, int C, int sm, int rows_in_flight, int max_chunks = 0) {
     RedShape r;
     const int C4 = C / 4;
     r.slabs = cdiv(C4, 32);
     r.SW = cdiv(C4, r.slabs);
     r.RPP = 256 / r.SW;
     size_t want = (size_t)sm * 4 / r.slabs; if (want < 1) want = 1;
+    if (max_chunks && want > (size_t)max_chunks) want = max_chunks;
     size_t rows = (P + want - 1) / want;
     const size_t pass = (size_t)r.RPP * rows_in_flight;       // rows of one pass over the loads in flight
     if (rows < pass) rows = pass;
@@ -161,6 +162,7 @@ __global__ void __launch_bounds__(256, 4) col_reduce_kernel(Pair t, const float 
         st4(mine, s); st4(mine + 4, ss);
         __threadfence();
     }
+    if (!counters) return;               // the records stay pending: their consumer adds them
     __syncthreads();
     if (tid == 0) last = atomicAdd(counters + blockIdx.y, 1u) == gridDim.x - 1 ? 1u : 0u;
     __syncthreads();
@@ -218,13 +220,20 @@ void mom_finalize(Exec &ex, Moments &m, int C) {
     m.pending = false;
 }
 
-void bn_stats(Exec &ex, Pair t, size_t P, Moments mo) {
+// A consumer that adds pending records takes 160 of them in one round of loads (see reduce_records: 32 threads per slot, five
+// each).  The last CTA's tail goes (basic block of 16 channels at 32x32: 260 -> 256 us for four such launches, of the odd-sized
+// one 177 -> 171); a handful of records stays with the last CTA.
+constexpr int kPendingRecords = 160, kFewRecords = 8;
+void bn_stats(Exec &ex, Pair t, size_t P, Moments &mo) {
     const int C = t.C();
     RedShape r = red_shape(P, C, ex.ctx->sm_count, kStatRows);
+    const bool defer = mo.defer && mo.part && (size_t)kPendingRecords * 2 * C <= mo.part_cap && r.chunks > kFewRecords;
+    if (defer) r = red_shape(P, C, ex.ctx->sm_count, kStatRows, kPendingRecords);
     size_t m = ex.ws.mark();
-    float *part = ex.ws.get<float>((size_t)r.chunks * 2 * C);
+    float *part = defer ? mo.part : ex.ws.get<float>((size_t)r.chunks * 2 * C);
+    mo.pending = defer; mo.parts = r.chunks; mo.inv_count = 1.0 / (double)P;
     if (!ex.dry) {
-        launch_stream(ex, (double)P * C * 4, 30, col_reduce_kernel<0>, dim3(r.chunks, r.slabs), 256, 0, t, nullptr, P, r.SW, r.rows_per_cta, BnRef{}, part, ex.ctx->counter(r.slabs),
+        launch_stream(ex, (double)P * C * 4, 30, col_reduce_kernel<0>, dim3(r.chunks, r.slabs), 256, 0, t, nullptr, P, r.SW, r.rows_per_cta, BnRef{}, part, defer ? nullptr : ex.ctx->counter(r.slabs),
                RedOut{mo.mean, mo.rstd, nullptr, nullptr, nullptr, 1.0 / (double)P, ex.eps});
         ex.check("bn_stats", (double)P * C * 4);
     }
