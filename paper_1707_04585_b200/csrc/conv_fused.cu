@@ -461,7 +461,14 @@ __global__ void __launch_bounds__(fused_threads(EW), 1) conv_fused_kernel(const 
                 float *mine = e.part + (size_t)blockIdx.x * 2 * e.n_cols + (c >> 2) * 8 + (c & 3);
                 mine[0] = a; mine[4] = b;
             }
-            if (ok && e.counter) { named_barrier(2, EW * 32); if (warp < 8) epilogue_publish<256>(e, reinterpret_cast<float *>(abuf), etid); }     // else the consumer adds the records
+            // (Without a counter the consumer adds the records.)  Layers of at most 64 columns have a record per SM or nearly so, and
+            // all sixteen warps add them (38-layer step 1899 -> 1875 us); of wider ones, split over fewer CTAs, eight warps are quicker
+            // (all sixteen everywhere: 164-layer step 0.6 % slower)
+            if (ok && e.counter) {
+                named_barrier(2, EW * 32);
+                if (EW == 16 && e.n_cols <= 64) epilogue_publish<512>(e, reinterpret_cast<float *>(abuf), etid);
+                else if (warp < 8) epilogue_publish<256>(e, reinterpret_cast<float *>(abuf), etid);
+            }
         }
     } else {
         const int bt = (int)threadIdx.x - kBuildWarp0 * 32;
@@ -522,7 +529,7 @@ bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count, FusedShape &s
         }
         g.seg_bytes = round_up(seg_of(g.S), 128);
         g.op_bytes = g.nseg * g.seg_bytes;
-        if (g.op_bytes < 12288) g.op_bytes = 12288;      // the last reduction borrows the region: (256 + 128) x 4 doubles
+        if (g.op_bytes < 20480) g.op_bytes = 20480;      // the last reduction borrows the region: (512 + 128) x 4 doubles
         s.smem = fixed + g.op_bytes;
         if (s.smem <= 227 * 1024 && g.plane16 < (1 << 14)) return true;
         if (g.BN < 32) return false;
