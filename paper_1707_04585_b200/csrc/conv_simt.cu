@@ -11,6 +11,7 @@
 // gemm_simt_kernel loads element by element and is left for the stem convolution's odd channel counts (an image has
 // three), where the kernels of stem.cu do not take its size.
 #include "common.cuh"
+#include "conv_direct.cuh"
 #include <algorithm>
 
 template <class T> __device__ __forceinline__ float ldf(const T *p);
@@ -150,7 +151,8 @@ struct OutCouple {                            // out = partner + sign*acc (sign 
     static constexpr bool kTransposed = false;
     Pair out, partner; int sign;
     __device__ __forceinline__ void store(size_t row, int n, float4 v) const { out.couple4(row, n, v, partner, sign); }
-    // eight rows `step` apart, columns n and n + 1; the partner's loads leave before the first store (it may be in place)
+    // the first `live` (one to eight) of eight rows `step` apart, columns n and n + 1; the partner's loads leave before the first
+    // store (it may be in place), those of the other rows repeat row 0
     __device__ __forceinline__ void store8(size_t row, int step, int live, int n, const float (&v)[8][2]) const {
         float2 p[8];
         if (sign)
@@ -337,12 +339,6 @@ static void launch_pixels(Exec &ex, AL al, BL bl, EP ep, int M, int N, int K) {
 // Bound by the FMA pipes, with about half of the time outside them: the start of a launch with one to four tiles per SM, the
 // copies' address arithmetic, and (8x8 images) too few warps.  Measured at batch 128, whole launches: 16 channels at 32x32
 // 33 -> 21 us, 32 at 16x16 41 -> 21 us, 56 at 8x8 41 -> 32 us against the implicit GEMM above.
-struct DirectGeom {
-    int N, H, W, Ci, Co;                          // Ci: channels summed over, Co: produced
-    int NW, gx, gy, gi, CB, kc, pitch;            // warps of a CTA, of a tile, channels per chunk, floats per staged pixel
-    int tx, ty, tiles;                            // tiles of an image, of all
-    FastDiv dtx, dty, dq, dcol, drow;             // by tx, ty, quads per chunk, staged columns, staged rows
-};
 // four channels r .. r + 3 of tap `tap` (of the sum above) for output n; forward: W[n][tap][r], data gradient: W[r][8 - tap][n]
 struct DirectFprop {
     static constexpr bool kAlongK = true;
@@ -454,7 +450,8 @@ __global__ void __launch_bounds__(256, 2) conv3x3_direct_kernel(const float *__r
         if (tn != t) {
             place(t);
             const int n = n0 + wc * 16 + 2 * lg, x = x0 + wx * 4 + lx, y = y0 + wy * 8, i = i0 + wi;
-            if (n < g.Co && x < g.W && i < g.N) ep.store8(((size_t)i * g.H + y) * g.W + x, g.W, g.H - y, n, sum);
+            const int live = direct_live_rows(g, n, x, y, i);
+            if (live > 0) ep.store8(((size_t)i * g.H + y) * g.W + x, g.W, live, n, sum);
 #pragma unroll
             for (int r = 0; r < 8; r++) sum[r][0] = sum[r][1] = 0.f;
         }
@@ -462,29 +459,6 @@ __global__ void __launch_bounds__(256, 2) conv3x3_direct_kernel(const float *__r
     }
 }
 
-// Tiles of a layer: false where less than half of their pixels would lie inside an image.  Four warps per CTA where eight would
-// leave SMs without one.
-static bool direct_shape(int N, int H, int W, int Ci, int Co, int sm, DirectGeom &g) {
-    g.N = N; g.H = H; g.W = W; g.Ci = Ci; g.Co = Co;
-    g.CB = Co > 16 ? 2 : 1;
-    g.kc = Ci < 32 ? Ci : 32;
-    g.pitch = (g.kc / 4) % 2 ? g.kc : g.kc + 4;
-    for (g.NW = 8; g.NW >= 4; g.NW -= 4) {
-        const int wpx = g.NW / g.CB, nbs = (Co + g.CB * 16 - 1) / (g.CB * 16);
-        g.gx = W <= 4 ? 1 : (W <= 8 ? 2 : 4);
-        if (g.gx > wpx) g.gx = wpx;
-        g.gy = wpx / g.gx;
-        while (g.gy > 1 && (g.gy >> 1) * 8 >= H) g.gy >>= 1;
-        g.gi = wpx / (g.gx * g.gy);
-        g.tx = (W + g.gx * 4 - 1) / (g.gx * 4); g.ty = (H + g.gy * 8 - 1) / (g.gy * 8);
-        const long long tiles = (long long)g.tx * g.ty * ((N + g.gi - 1) / g.gi);
-        if (tiles * wpx * 32 > 2ll * N * H * W || tiles > (1 << 28)) { if (g.NW == 8) continue; return false; }
-        g.tiles = (int)tiles;
-        if (tiles * nbs >= sm || g.NW == 4) break;
-    }
-    g.dtx = fast_div(g.tx); g.dty = fast_div(g.ty); g.dq = fast_div(g.kc / 4); g.dcol = fast_div(g.gx * 4 + 2); g.drow = fast_div(g.gy * 8 + 2);
-    return true;
-}
 template <class WL, class EP>
 static void launch_direct(Exec &ex, const float *in, WL wl, EP ep, const DirectGeom &g) {
     const int smem = (9 * g.kc * g.CB * 16 + 2 * (g.gx * 4 + 2) * (g.gy * 8 + 2) * g.gi * g.pitch) * 4;      // at most 157 KB

@@ -45,12 +45,14 @@ def test_bf16_blocks_at_tile_edges(ctx, kind, N, H, W, c, w):
 
 @pytest.mark.parametrize("kind,N,H,W,c,w", [
     ("basic", 1, 5, 13, 4, 0),            # 65 pixels: one more than the shortest tile; columns 4 of 16
-    ("basic", 1, 275, 275, 16, 0),        # 256-row tiles, the last one of 105 rows
+    ("basic", 1, 275, 275, 16, 0),        # 16-row tiles, the last one of 3 rows
     ("basic", 1, 150, 253, 20, 0),        # 32-column tiles, the tall ones
     ("basic", 1, 139, 137, 36, 0),        # 64-column tiles
     ("basic", 2, 11, 7, 68, 0),           # two column tiles, the second of 4 columns
     ("basic", 16, 5, 4, 8, 0),            # direct 3x3: eight images per tile, one column of warps
     ("basic", 5, 7, 6, 20, 0),            # two images per tile, the last one of a tile missing
+    ("basic", 75, 24, 16, 16, 0),         # direct 3x3, eight warps in two row groups: the second one of the last tile lies below the image
+    ("basic", 9, 20, 7, 8, 0),            # the same with narrow images and four warps
     ("basic", 1, 33, 17, 100, 0),         # four chunks of input channels (the last of 4), four groups of outputs
     ("bottleneck", 1, 3, 3, 132, 4),      # column sums of nine rows: two slabs of 17 and 16 quads, and one quad
     ("bottleneck", 1, 97, 99, 520, 8),    # 32-byte accesses in the streaming kernels
