@@ -31,6 +31,7 @@ constexpr int kWgStages = 4;     // ... of the weight-gradient kernel
 constexpr int kThreads = 192;      // TMA warp, MMA warp, four epilogue warps
 constexpr int kMaxGroups = 4;      // epilogue through TMA: two or four groups of four epilogue warps
 constexpr int kThreadsTma = 64 + kMaxGroups * 128;
+constexpr int kThreadsPair = 64 + 2 * 128;      // conv_tc2_kernel: two groups
 
 struct TcParams {
     int taps;        // k*k
@@ -44,9 +45,8 @@ struct TcParams {
     EpiArgs epi;
     int *status;
     int stages;      // operand ring depth (<= kStages)
-    // epilogue through TMA (epi_tma): the output tile leaves, and the tile read besides the accumulator (coupling
+    // epilogue through TMA: the output tile leaves, and the tile read besides the accumulator (coupling
     // partner, or BN input of a data gradient) arrives, as column groups of GW floats per pixel row
-    int epi_tma;
     int GW;          // 32 or 16 floats: rows of 128 / 64 bytes, stored with the matching TMA swizzle
     int epi_bytes;   // partner rings, output slots and sums of the TMA epilogue
     int group_bytes; // one column group of a tile (128 pixel rows), a multiple of 1024
@@ -63,7 +63,7 @@ struct TcParams {
     int n_cls;
     int ntap[4];
     signed char tdy[4][9], tdx[4][9], tid[4][9];
-    int ostride, oy[4], ox[4];    // epi_tma: output pixel = tile pixel * ostride + (oy, ox)
+    int ostride, oy[4], ox[4];    // epilogue through TMA: output pixel = tile pixel * ostride + (oy, ox)
     // conv_tc2_kernel, 3x3 stride 1 ("halo" operand): one box per channel chunk holds the tile's pixels WITH their
     // halo, (BH + 2) rows of Wp = W + 2 pixels; tap (kh, kw) reads the 128 rows that start kh * Wp + kw rows further
     // on, so the activations cross L2 -> shared memory once per chunk instead of once per tap.  Accumulator row m is
@@ -346,7 +346,12 @@ __device__ __forceinline__ void tma_epilogue(const TcParams &p, TcShared *sh, co
 // Persistent CTA: walks the pixel tiles blockIdx.x, blockIdx.x + gridDim.x, ... of N tile blockIdx.y.
 // The operand ring runs on across tiles; the accumulator alternates between two tensor-memory
 // buffers so that the epilogue of one tile overlaps the MMAs of the next.
-__global__ void __launch_bounds__(kThreadsTma, 1)
+// EPI_TMA: the epilogue through TMA; else the staged one, for channel-split tensors whose halves are no multiple of 16.  Two kernels,
+// so that each has the registers of its own block size: under the 576 threads of the other the staged one had 96 and
+// spilled, and its launches took 6 to 10 % longer than with the 133 that it has for its 192 (48 -> 1744 channels,
+// stride 2, 81 images of 28x28: 117 and 107 us forward).
+template <bool EPI_TMA>
+__global__ void __launch_bounds__(EPI_TMA ? kThreadsTma : kThreads, 1)
 conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_o0, const __grid_constant__ CUtensorMap map_o1,
                const __grid_constant__ CUtensorMap map_x0, const __grid_constant__ CUtensorMap map_x1, const TcParams p) {
@@ -357,12 +362,12 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const int a_bytes = box_px * p.KC * 2, b_bytes = p.BN * p.KC * 2;
     const int b_off = (128 * p.KC * 2 + 1023) & ~1023;
     const int stage_bytes = b_off + ((b_bytes + 1023) & ~1023);
-    // behind the operand ring: the staged epilogue's row stage and running sums, or (epi_tma) the partner ring,
+    // behind the operand ring: the staged epilogue's row stage and running sums, or (EPI_TMA) the partner ring,
     // two output groups and the running sums per column group
     float *estage = (float *)(tiles + p.stages * stage_bytes);
-    const int ng = p.epi_tma ? p.BN / p.GW : 0;
+    const int ng = EPI_TMA ? p.BN / p.GW : 0;
     uint8_t *auxr = (uint8_t *)estage;
-    TcShared *sh = p.epi_tma ? (TcShared *)(auxr + p.epi_bytes) : (TcShared *)((uint8_t *)estage + kEpiStageBytes + kEpiSumFloats * 4);
+    TcShared *sh = EPI_TMA ? (TcShared *)(auxr + p.epi_bytes) : (TcShared *)((uint8_t *)estage + kEpiStageBytes + kEpiSumFloats * 4);
 
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int n_vt = p.n_cls * p.g.n_px_tiles;     // tiles of all classes
@@ -371,13 +376,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; s++) { mbar_init(&sh->full[s], 1); mbar_init(&sh->empty[s], 1); }
-        for (int b = 0; b < 2; b++) mbar_init(&sh->acc_empty[b], p.epi_tma ? ng : 128);
+        for (int b = 0; b < 2; b++) mbar_init(&sh->acc_empty[b], EPI_TMA ? ng : 128);
         for (int b = 0; b < 4; b++) mbar_init(&sh->acc_full[b], 1);
         for (int b = 0; b < 8; b++) mbar_init(&sh->aux_full[b], 1);
         sh->failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         tma_prefetch_desc(&map_a); tma_prefetch_desc(&map_b);
-        if (p.epi_tma) { tma_prefetch_desc(&map_o0); tma_prefetch_desc(&map_o1); tma_prefetch_desc(&map_x0); tma_prefetch_desc(&map_x1); }
+        if (EPI_TMA) { tma_prefetch_desc(&map_o0); tma_prefetch_desc(&map_o1); tma_prefetch_desc(&map_x0); tma_prefetch_desc(&map_x1); }
     }
     if (warp == 1) tmem_alloc(&sh->tmem_base, tmem_cols);
     if (warp >= 2) build_row_map(p.g, &sh->rows, ((warp & 3) << 5) | lane);
@@ -447,7 +452,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 if (ok) mma_commit(&sh->acc_full[ti & 3]);
             }
         }
-    } else if (!p.epi_tma) {
+    } else if constexpr (!EPI_TMA) {
         // epilogue: this warp may touch accumulator lanes 32*(warp%4) .. +31
         const int etid = ((warp & 3) << 5) | lane;
         float *esums = estage + 128 * kEpiPitch;
@@ -677,7 +682,7 @@ conv1x1_bn_kernel(const __grid_constant__ CUtensorMap map_raw, const __grid_cons
 // own tile exactly as the single-CTA kernel does (epilogue through TMA only).
 // Tile pairs: class c, pair j holds the pixel tiles 2j and 2j + 1 of the class; with an odd tile count the last pair's
 // second tile lies outside the tensor (TMA delivers zeros, nothing is stored).
-__global__ void __launch_bounds__(kThreadsTma, 1)
+__global__ void __launch_bounds__(kThreadsPair, 1)
 conv_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                 const __grid_constant__ CUtensorMap map_o0, const __grid_constant__ CUtensorMap map_o1,
                 const __grid_constant__ CUtensorMap map_x0, const __grid_constant__ CUtensorMap map_x1, const TcParams p) {
@@ -1170,7 +1175,7 @@ bool run_conv_tc(Exec &ex, const char *what, const void *act, Geom gin, int cin,
             if (!ok) { ex.failed = true; ex.ctx->err = std::string(what) + ": tensor map (epilogue) rejected"; ex.ws.release(m); return true; }
         }
         TcParams p;
-        p.stages = stages; p.epi_tma = epi_tma ? 1 : 0; p.GW = GW; p.group_bytes = group_bytes; p.need_aux = need_aux ? 1 : 0;
+        p.stages = stages; p.GW = GW; p.group_bytes = group_bytes; p.need_aux = need_aux ? 1 : 0;
         p.groups = groups; p.aux_slots = need_aux ? aux_slots : 0; p.inplace = inplace ? 1 : 0; p.epi_bytes = epi_bytes;
         p.split_o = out.c1 ? out.c0 : 0; p.split_x = (need_aux && auxp.c1) ? auxp.c0 : 0;
         memcpy(p.ntap, ntap, sizeof ntap); memcpy(p.tdy, tdy, sizeof tdy); memcpy(p.tdx, tdx, sizeof tdx); memcpy(p.tid, tid, sizeof tid);
@@ -1190,12 +1195,13 @@ bool run_conv_tc(Exec &ex, const char *what, const void *act, Geom gin, int cin,
         if (req.bnbwd) { e.t = req.bnbwd->t; e.bn = req.bnbwd->bn; e.dgamma = req.bnbwd->dgamma; e.dbeta = req.bnbwd->dbeta; e.coef = req.bnbwd->coef; }
         static OncePerDevice once;
         if (once.first(ex.ctx->device)) {
-            cudaFuncSetAttribute(conv_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+            cudaFuncSetAttribute(conv_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+            cudaFuncSetAttribute(conv_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
             cudaFuncSetAttribute(conv_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         }
         dim3 grid((unsigned)ctas, (unsigned)s.n_tiles);
         if (pair) launch_cluster(ex, conv_tc2_kernel, grid, 64 + groups * 128, s.smem, 2, map_a, map_b, map_o[0], map_o[1], map_x[0], map_x[1], p);
-        else launch(ex, conv_tc_kernel, grid, epi_tma ? 64 + groups * 128 : kThreads, s.smem, map_a, map_b, map_o[0], map_o[1], map_x[0], map_x[1], p);
+        else launch(ex, epi_tma ? conv_tc_kernel<true> : conv_tc_kernel<false>, grid, epi_tma ? 64 + groups * 128 : kThreads, s.smem, map_a, map_b, map_o[0], map_o[1], map_x[0], map_x[1], p);
         const double bytes = (double)gin.P() * cin * 2 + (double)g.P() * cout * (sign || req.bnbwd ? 8 : 4) + (double)cout * taps * cin * 2;
         // (records of launches on a CTA pair carry the pair kernel's name)
         ex.check(!pair ? what : (transposed ? "conv_dgrad_tc2" : "conv_fprop_tc2"), bytes, 2.0 * g.P() * cout * cin * ntap_all);
@@ -1254,7 +1260,7 @@ bool run_bn_conv(Exec &ex, Pair t, BnRef bn, Geom gi, const Layer &L, Pair out, 
         }
         if (!ok) { ex.failed = true; ex.ctx->err = "conv1x1_bn: tensor map rejected"; ex.ws.release(m); return true; }
         p.taps = 1; p.k = 1; p.chunks = cin / 64; p.KC = 64; p.cin_pad = cin; p.BN = BN; p.stride = 1; p.g = tg;
-        p.status = ex.ctx->dev_status; p.stamp = ex.stamp_slot(); p.stages = stages; p.epi_tma = 1; p.groups = groups; p.epi_bytes = epi_bytes;
+        p.status = ex.ctx->dev_status; p.stamp = ex.stamp_slot(); p.stages = stages; p.groups = groups; p.epi_bytes = epi_bytes;
         p.GW = GW; p.group_bytes = group_bytes; p.n_cls = 1; p.ntap[0] = 1; p.ostride = 1;
         EpiArgs &e = p.epi;
         e.mode = EPI_PLAIN; e.out = out; e.n_cols = cout; e.part = part; e.counter = stats && !defer ? ex.ctx->counter() : nullptr;

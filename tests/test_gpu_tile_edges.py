@@ -74,10 +74,13 @@ def test_stems_at_tile_edges(ctx, img, k, stem_c):
 
 
 @pytest.mark.parametrize("mode", [0, 1])
-@pytest.mark.parametrize("N,H,cin,cout,stride", [
-    (3, 6, 8, 24, 2),                     # 27 pixels in each parity class of the data gradient
-    (2, 10, 40, 72, 2),
-    (2, 9, 24, 136, 1),
+@pytest.mark.parametrize("N,H,cin,cout,stride,split", [
+    (3, 6, 8, 24, 2, False),              # 27 pixels in each parity class of the data gradient
+    (2, 10, 40, 72, 2, False),
+    (2, 9, 24, 136, 1, False),
+    (5, 14, 48, 80, 2, True),             # halves of 24 and 40: the staged epilogue in both directions
+    (3, 10, 24, 400, 1, True),            # halves of 12 and 200, four column tiles
+    (4, 20, 96, 224, 2, True),            # halves of 48 and 112: 16-column groups on a pair, with and without a partner tile
 ])
-def test_transitions_at_tile_edges(ctx, mode, N, H, cin, cout, stride):
-    tp.run_transition_case(ctx, mode, N, H, cin, cout, 3, stride, False)
+def test_transitions_at_tile_edges(ctx, mode, N, H, cin, cout, stride, split):
+    tp.run_transition_case(ctx, mode, N, H, cin, cout, 3, stride, split)
