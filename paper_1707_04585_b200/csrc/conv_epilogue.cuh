@@ -204,7 +204,8 @@ __device__ __forceinline__ void moments_of(double sum, double sum2, double inv_c
 // Adds the per-CTA records of a reduction.  A record is 2C floats = C/2 float4 slots (per channel
 // quad: sums, second sums); this call covers the slots slot0 .. slot0 + cw - 1 (cw <= 128, even).
 // Thread = (sub, slot), slot fastest so that a warp reads whole records: it adds the records sub,
-// sub + nsub, ... of its slot, five loads in flight at a time; the subs of a warp are combined by
+// sub + nsub, ... of its slot, five loads in flight at a time (ten where only 128 threads share the work: 78.9 against 80.7 us
+// for a small strided 1x1 transition of 88 -> 168 channels); the subs of a warp are combined by
 // shuffles, the warps (or, of wide records, the subs) in order.
 // (Giving a slot to consecutive lanes and adding them by shuffles was measured slower: the loads
 // of a warp then touch 32 records.)  All in double precision, in an order that the number of
@@ -218,7 +219,7 @@ __device__ __forceinline__ void reduce_records(const float *part, int parts, int
     double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
     if (slot < cw) {
         const float *src = part + (size_t)(slot0 + slot) * 4;
-        constexpr int kInFlight = 5;
+        constexpr int kInFlight = NT == 128 ? 10 : 5;
         for (int i = sub; i < parts; i += kInFlight * nsub) {
             float4 v[kInFlight];
 #pragma unroll
