@@ -162,6 +162,8 @@ __device__ __forceinline__ void tma_pass_b(int GW, const uint8_t *ob, const uint
 // 4.86 -> 3.82 ms together with the records left to the consumer); the pair kernel has two: its tiles are bound by the MMAs,
 // and four would cost it operand stages (20.9 -> 22.3 ms).
 // PAIR: the tile of a CTA pair's tile pair (see conv_tc2_kernel).
+// warp groups that visit a tile, so the arrivals that free its accumulator
+__device__ __forceinline__ int epilogue_arrivals(const TcParams &p) { const int ng = p.BN / p.GW; return ng < p.groups ? ng : p.groups; }
 struct EpiMaps { const CUtensorMap *o0, *o1, *x0, *x1; };
 template <bool PAIR>
 __device__ __forceinline__ void tma_epilogue(const TcParams &p, TcShared *sh, const EpiMaps maps, uint8_t *auxr, uint32_t tmem_d, int col0, int warp, int lane,
@@ -244,19 +246,21 @@ __device__ __forceinline__ void tma_epilogue(const TcParams &p, TcShared *sh, co
             const int col = col0 + gi * GW;
             const bool live = in_range && col < e.n_cols;          // groups beyond the valid channels only drain their columns
             const bool visit = p.need_aux && live;                 // the partner group sits in ring slot c_slot
+            const bool last_of_tile = gi + gstep >= ng;            // this warp group's last visit to the tile
             const uint8_t *ax = auxg + c_slot * p.group_bytes;
             uint8_t *ob = p.inplace ? auxg + c_slot * p.group_bytes : out_slot;
             if (etid == 0) {
                 tma_store_wait_read();                             // this group's last store is done with its slot
                 if (refill) load_next_aux();                       // (in place: which can take the next partner group now)
-                ok = (PAIR ? mbar_wait_cluster(&sh->acc_full[it & 3], (it >> 2) & 1) : mbar_wait(&sh->acc_full[it & 3], (it >> 2) & 1)) && sh->failed == 0;
+                if (gi == gi0)                                     // (the accumulator is complete for the tile's later visits as well)
+                    ok = (PAIR ? mbar_wait_cluster(&sh->acc_full[it & 3], (it >> 2) & 1) : mbar_wait(&sh->acc_full[it & 3], (it >> 2) & 1)) && sh->failed == 0;
                 if (ok && visit) ok = mbar_wait(&sh->aux_full[wg * SW + c_slot], c_par);
             }
             refill = p.inplace && visit;
             if (visit && ++c_slot == SW) { c_slot = 0; c_par ^= 1u; }
             ok = named_barrier_and(bar_b, 128, ok);
             if (!ok) break;
-            tc_fence_after();
+            if (gi == gi0) tc_fence_after();
             const bool rowv = live && srow >= 0 && srow < valid_px;
             const uint32_t tg = tm + (uint32_t)(gi * GW);
             if (e.mode != EPI_COUPLE) {
@@ -266,17 +270,21 @@ __device__ __forceinline__ void tma_epilogue(const TcParams &p, TcShared *sh, co
             } else {
                 if (e.sign > 0) tma_pass_a<4>(tg, GW, prow, rowv, ax, ob, out_s); else tma_pass_a<5>(tg, GW, prow, rowv, ax, ob, out_s);
             }
-            tc_fence_before();
+            if (last_of_tile) tc_fence_before();
             fence_proxy_async();
             named_barrier(bar_a, 128);
             if (etid == 0) {
-                // the columns of this group are drained: one arrival per column group
-                if (PAIR) mbar_arrive_cluster(mapa_shared(smem_u32(&sh->acc_empty[buf]), 0));
-                else mbar_arrive(&sh->acc_empty[buf]);
                 if (live) {
                     const bool second = p.split_o && col >= p.split_o;
                     tma_store_4d(second ? maps.o1 : maps.o0, ob, second ? col - p.split_o : col, p.ox[cls], h0 * p.ostride + p.oy[cls], n0);
                     tma_store_commit();
+                }
+                // this warp group has drained its columns of the tile.  Once per tile and behind the store: on a pair the arrival
+                // is a release at cluster scope, and one per column group in front of the store cost 300 to 600 clocks each
+                // (32 -> 1248 channels, 12800 pixels, 16-column groups: 53 us, now 42)
+                if (last_of_tile) {
+                    if (PAIR) mbar_arrive_cluster(mapa_shared(smem_u32(&sh->acc_empty[buf]), 0));
+                    else mbar_arrive(&sh->acc_empty[buf]);
                 }
             }
             if (e.part && live && col + jq * 4 < e.n_cols) {
@@ -376,7 +384,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; s++) { mbar_init(&sh->full[s], 1); mbar_init(&sh->empty[s], 1); }
-        for (int b = 0; b < 2; b++) mbar_init(&sh->acc_empty[b], EPI_TMA ? ng : 128);
+        for (int b = 0; b < 2; b++) mbar_init(&sh->acc_empty[b], EPI_TMA ? epilogue_arrivals(p) : 128);
         for (int b = 0; b < 4; b++) mbar_init(&sh->acc_full[b], 1);
         for (int b = 0; b < 8; b++) mbar_init(&sh->aux_full[b], 1);
         sh->failed = 0;
@@ -521,7 +529,7 @@ conv1x1_bn_kernel(const __grid_constant__ CUtensorMap map_raw, const __grid_cons
         for (int s = 0; s < kStages; s++) { mbar_init(&sh->full[s], 1 + kBnBuildWarps / 2); mbar_init(&sh->empty[s], 1); }
         for (int b = 0; b < 8; b++) mbar_init(&sh->afull[b], 1);
         for (int b = 0; b < 4; b++) { mbar_init(&sh->aempty[b], kBnBuildWarps / 2); mbar_init(&sh->acc_full[b], 1); }
-        for (int b = 0; b < 2; b++) mbar_init(&sh->acc_empty[b], ng);
+        for (int b = 0; b < 2; b++) mbar_init(&sh->acc_empty[b], epilogue_arrivals(p));
         for (int b = 0; b < 8; b++) mbar_init(&sh->aux_full[b], 1);
         sh->failed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -693,7 +701,6 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const int a_bytes = box_px * p.KC * 2, b_bytes = BNH * p.KC * 2;
     const int b_off = (128 * p.KC * 2 + 1023) & ~1023;
     const int stage_bytes = b_off + ((b_bytes + 1023) & ~1023);
-    const int ng = p.BN / p.GW;
     // halo mode: the ring holds weight tiles only, the activation boxes have a ring of their own in front of it
     uint8_t *abuf = tiles;
     const int wstage_bytes = (b_bytes + 1023) & ~1023;
@@ -711,8 +718,7 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; s++) { mbar_init(&sh->full[s], 1); mbar_init(&sh->empty[s], 1); }
-        // acc_empty (used in the leader): one arrival per column group of either CTA
-        for (int b = 0; b < 2; b++) mbar_init(&sh->acc_empty[b], 2 * ng);
+        for (int b = 0; b < 2; b++) mbar_init(&sh->acc_empty[b], 2 * epilogue_arrivals(p));     // (used in the leader) those of either CTA
         for (int b = 0; b < 4; b++) mbar_init(&sh->acc_full[b], 1);
         for (int b = 0; b < 8; b++) mbar_init(&sh->aux_full[b], 1);
         for (int b = 0; b < 4; b++) { mbar_init(&sh->afull[b], 1); mbar_init(&sh->aempty[b], 1); }
