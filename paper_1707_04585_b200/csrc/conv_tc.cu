@@ -322,22 +322,19 @@ __device__ __forceinline__ void tma_epilogue(const TcParams &p, TcShared *sh, co
         named_barrier(bar_all, NG * 128);
     }
     ok = named_barrier_and(bar_all, NG * 128, *(volatile uint32_t *)&sh->failed == 0);
-    if (ok && wg == 0) {
-        // per-CTA record: the warp groups, then the threads, that share a channel quad are added in order
+    if (ok) {
+        // per-CTA record: the warp groups, then the threads, that share a channel quad are added in order; a thread per value (the
+        // eight sums of a quad lie side by side, in the slots as in the record)
         float *mine = e.part + (size_t)blockIdx.x * 2 * e.n_cols;
-        for (int gi = 0; gi < ng; gi++) {
-            const int col = col0 + gi * GW + jq * 4;
-            if (r0 == 0 && col < e.n_cols) {
-                float r[8];
-#pragma unroll
-                for (int j = 0; j < 8; j++) r[j] = 0.f;
-                for (int q = gi; q < (many ? gi + 1 : NG); q += many ? 1 : ng)
-                    for (int y = 0; y < rpp; y++)
-#pragma unroll
-                        for (int j = 0; j < 8; j++) r[j] += sums[(size_t)q * 128 * 8 + (y * QW + jq) * 8 + j];
-                *reinterpret_cast<float4 *>(mine + 2 * col) = make_float4(r[0], r[1], r[2], r[3]);
-                *reinterpret_cast<float4 *>(mine + 2 * col + 4) = make_float4(r[4], r[5], r[6], r[7]);
-            }
+        const int per = QW * 8;
+        for (int o = wg * 128 + etid; o < ng * per; o += NG * 128) {
+            const int gi = o / per, w = o - gi * per, col = col0 + gi * GW + (w >> 3) * 4;
+            if (col >= e.n_cols) continue;
+            float r = 0.f;
+            for (int q = gi; q < (many ? gi + 1 : NG); q += many ? 1 : ng)
+#pragma unroll 8
+                for (int y = 0; y < rpp; y++) r += sums[q * 128 * 8 + y * per + w];
+            mine[2 * col + (w & 7)] = r;
         }
     }
     // the last CTA adds the records with all its epilogue threads (128 of them took four rounds of dependent reads for 148
