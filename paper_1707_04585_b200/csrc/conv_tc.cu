@@ -1097,6 +1097,14 @@ bool run_conv_tc(Exec &ex, const char *what, const void *act, Geom gin, int cin,
             while (stages > y.stages && smem_of(stages) > 227 * 1024) stages--;
             if (smem_of(stages) <= 227 * 1024) { fits = true; s.smem = smem_of(stages); break; }
         }
+        // On a pair (two groups, eight partner barriers) room that the operand ring leaves goes to more partner slots, up to the four
+        // column groups that a warp group has in a tile: with two, narrow column groups or a result stored from its slot leave
+        // the next partner group too little time to arrive
+        for (int more = aux_slots + 1; fits && pair && need_aux && more <= 4 && more <= (ng + groups - 1) / groups + (inplace ? 1 : 0); more++) {
+            const int bytes = ((groups * more) + (inplace ? 0 : groups)) * group_bytes + (ng > groups ? ng * 4096 : 0), extra = bytes > epi_bytes ? bytes - epi_bytes : 0;
+            if (s.smem + extra > 227 * 1024) break;
+            aux_slots = more; epi_bytes += extra; s.smem += extra;
+        }
         if (!fits) {
             if (s.BN == 256) return false;      // (does not happen)
             epi_tma = false; pair = false; stages = 4;
