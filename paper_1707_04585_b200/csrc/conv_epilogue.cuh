@@ -11,6 +11,7 @@
 #pragma once
 #include "common.cuh"
 #include "tc_ptx.cuh"
+#include <math.h>
 
 namespace tc {
 
@@ -189,16 +190,21 @@ __device__ __forceinline__ void epilogue_tile(const EpiArgs &e, uint32_t tmem_ac
 
 // mean and 1 / sqrt(var + eps) from a channel's sum and second sum (double), rounded to float once.  The reciprocal root is
 // the single-precision one refined by two Newton steps in double (relative error below 1e-13): a double division and square
-// root would be a few hundred dependent instructions at the head of every convolution.
+// root would be a few hundred dependent instructions at the head of every convolution.  An argument outside the range of float
+// is scaled into it; zero and infinity (sums that overflowed) keep the exact results, infinity and zero, which a step would turn into NaN.
 __device__ __forceinline__ void moments_of(double sum, double sum2, double inv_count, float eps, float &mean, float &rstd) {
     const double m = sum * inv_count;
     double var = sum2 * inv_count - m * m;
     if (var < 0) var = 0;
     const double v = var + (double)eps;
-    double y = (double)rsqrtf((float)v);
-    y *= 1.5 - 0.5 * v * y * y;
-    y *= 1.5 - 0.5 * v * y * y;
-    mean = (float)m; rstd = (float)y;
+    const bool low = v < 1e-36, high = v > 1e36;
+    const double w = low ? v * 0x1p+120 : (high ? v * 0x1p-120 : v);
+    const float r = rsqrtf((float)w);
+    double y = (double)r;
+    y *= 1.5 - 0.5 * w * y * y;
+    y *= 1.5 - 0.5 * w * y * y;
+    if (!(r > 0.f && r < INFINITY)) y = (double)r;
+    mean = (float)m; rstd = (float)(low ? y * 0x1p+60 : (high ? y * 0x1p-60 : y));
 }
 
 // Adds the per-CTA records of a reduction.  A record is 2C floats = C/2 float4 slots (per channel

@@ -142,3 +142,29 @@ def test_timeline_mode_describes_the_last_step_and_changes_no_result(use_graph):
         assert loss == got[0][0] and np.array_equal(params, got[0][1])
     B.revnet_check_device(ctx)
     ctx.close()
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("kind,N,H,c,w", [
+    ("single", 2, 8, 16, 0),           # statistics finished by the reduction itself
+    ("basic", 8, 32, 16, 0),           # ... left as records for the fused convolution
+    ("bottleneck", 4, 16, 128, 32),    # ... read by the wide 1x1 kernel
+])
+def test_statistics_whose_sum_of_squares_overflows_switch_the_channel_off(mode, kind, N, H, c, w):
+    """A float state of 3e19 in one channel: the squares overflow, the variance is infinite, 1 / sqrt of it zero, and the channel's
+    activation is ReLU(beta), finite; the same bits as with that channel's gamma at zero."""
+    ctx = B.Context(0)
+    b = syn.BlockCfg(N, H, H, c, w, kind, seed=5)
+    inp = syn.make_block_inputs(b, affine_jitter=True)
+    inp["x2"][:, 2] = 3e19
+    ys = []
+    for zero in (False, True):
+        r = R.BlockRunner(ctx, b, mode, 0)
+        r.load(inp["params"])
+        r.F[0]["beta"][2] = 0.25
+        if zero:
+            r.F[0]["gamma"][2] = 0.0
+        ys.append(r.forward(inp["x1"], inp["x2"])[0])
+    assert np.isfinite(ys[0]).all() and np.array_equal(ys[0], ys[1])
+    B.revnet_check_device(ctx)
+    ctx.close()
