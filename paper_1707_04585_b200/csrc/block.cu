@@ -79,11 +79,19 @@ void fn_forward(Exec &ex, Geom g, Pair u, const Moments *mom_in, const std::vect
     for (int l = 0; l < L; l++) {
         const Layer &ly = layers[l];
         const size_t P = gi.P();
+        const size_t a_bytes = P * ly.cin * esz(ex);
+        void *a = nullptr;
         if (!cur.valid) {
-            // the fused kernel adds the records itself: they stay pending (small tensors have too few for that to pay: see bn_stats)
+            // the fused kernel adds the records itself: they stay pending (small tensors have too few for that to pay: see bn_stats).
+            // Without `saved` that kernel writes no activated tensor, so the records sit where it would be (more than 128 KB, the
+            // 160 records of 64 channels take 80): a forward pass needs no more scratch than one whose statistics are finished at once
             const bool defer = b16 && P * ly.cin > 65536 && t.c1 == 0 && !(l == L - 1 && (skip_last_conv || out.c1 || partner.c1)) && conv_fused_takes(ex, gi, ly);
-            cur = mom_alloc(ex, ly.cin, defer);
+            cur = mom_alloc(ex, ly.cin, defer && saved);
             cur.defer = defer;
+            if (defer && !saved) {
+                a = ex.ws.alloc(a_bytes);
+                cur.part = (float *)a; cur.part_cap = a_bytes / sizeof(float);
+            }
             bn_stats(ex, t, P, cur);
             cur.valid = true;
         }
@@ -91,7 +99,7 @@ void fn_forward(Exec &ex, Geom g, Pair u, const Moments *mom_in, const std::vect
         const bool last = l == L - 1;
         Geom go{gi.N, conv_out(gi.H, ly.k, ly.stride), conv_out(gi.W, ly.k, ly.stride)};
         // the activated tensor is materialised only where something reads it: the unfused convolution, or the weight gradient
-        void *a = ex.ws.alloc(P * ly.cin * esz(ex));
+        if (!a) a = ex.ws.alloc(a_bytes);
         float *tn = last ? nullptr : ex.ws.get<float>(go.P() * ly.cout);
         Moments next;
         if (!last) next = mom_alloc(ex, ly.cout, b16);      // with room for pending partials: the next layer consumes them

@@ -125,3 +125,10 @@ def test_pack_bytes_and_declared_buffer_sizes(ctx):
     plan = B.revnet_stack_plan(ctx, B.stack_desc(cfg, 0))
     plan.set_buffer_sizes(plan.activation_bytes, plan.workspace_bytes)
     plan.close()
+
+
+def test_forward_scratch_of_a_fused_block_holds_no_statistics_records(ctx):
+    """127 images of 32x32 x 64 channels: the bf16 activated tensor and the means fit the 16 MiB of revnet_block_fwd_noalloc with
+    130 KB to spare, which the records of pending statistics would take."""
+    fwd, _ = B.revnet_block_workspace_bytes(ctx, B.block_desc(syn.BlockCfg(127, 32, 32, 64, 0, "single", seed=0), 0, 16))
+    assert 127 * 32 * 32 * 64 * 2 <= fwd <= 16 << 20

@@ -15,10 +15,13 @@ from paper_1707_04585_b200 import synthetic as syn
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("mode", [0, 1])
-def test_noalloc_block_forward_matches_workspace_version_twice(mode):
+@pytest.mark.parametrize("mode,b", [
+    (0, syn.BlockCfg(8, 32, 32, 16, 0, "basic", seed=77)),
+    (1, syn.BlockCfg(8, 32, 32, 16, 0, "basic", seed=77)),
+    (0, syn.BlockCfg(127, 32, 32, 64, 0, "single", seed=77)),       # 130 KB below the limit
+])
+def test_noalloc_block_forward_matches_workspace_version_twice(mode, b):
     ctx = B.Context(0)
-    b = syn.BlockCfg(8, 32, 32, 16, 0, "basic", seed=77)
     for call in range(2):                                   # two calls in a row share the static array
         inp = syn.make_block_inputs(syn.BlockCfg(b.N, b.H, b.W, b.c, b.w, b.kind, seed=77 + call), affine_jitter=True)
         r = R.BlockRunner(ctx, b, mode)
