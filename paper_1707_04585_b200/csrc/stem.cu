@@ -439,22 +439,25 @@ template <int COL> static bool fprop_rows(Exec &ex, const float *img, const Stem
     launch(ex, stem_fprop_row_kernel<COL>, grid, T::FW * 32, smem, img, W, out, g, fast_div(g.W * 3), cols, tiles_per_img, n_tiles, cop);
     return true;
 }
-// part: room for `cap` partials; the number written goes to `parts`
-template <int K> static bool wgrad_rows(Exec &ex, const float *img, const float *gout, const StemGeom &g, float *part, int cap, int &parts) {
+// Launch of the row weight gradient; false: shape not taken (decided here alone, for the sizing run and the real one)
+struct RowWgrad { int cols, cbw, blocks_y, nw, tiles_per_img, n_tiles; size_t smem; };
+template <int K> static bool wgrad_rows_shape(const StemGeom &g, RowWgrad &w) {
     using T = StemRow<K>;
-    int cols;
-    if (!row_stem(g, T::U, cols)) return false;
-    const int cbs = (g.Co + 31) / 32, cbw = cbs < T::CBW ? cbs : T::CBW, blocks_y = (cbs + cbw - 1) / cbw;
-    const int nw = T::HG * cbw * T::RS, tiles_per_img = (g.Ho + T::RS - 1) / T::RS, n_tiles = g.N * tiles_per_img;
-    const size_t smem = (2 * (size_t)((T::RS - 1) * T::S + K) * cols * 4 + (size_t)nw * T::KH * K * 3 * 32) * 4;
-    if (smem > 200 * 1024) return false;
-    if (ex.dry) return true;
+    if (g.k != K || !row_stem(g, T::U, w.cols)) return false;
+    const int cbs = (g.Co + 31) / 32;
+    w.cbw = cbs < T::CBW ? cbs : T::CBW; w.blocks_y = (cbs + w.cbw - 1) / w.cbw;
+    w.nw = T::HG * w.cbw * T::RS; w.tiles_per_img = (g.Ho + T::RS - 1) / T::RS; w.n_tiles = g.N * w.tiles_per_img;
+    w.smem = (2 * (size_t)((T::RS - 1) * T::S + K) * w.cols * 4 + (size_t)w.nw * T::KH * K * 3 * 32) * 4;
+    return w.smem <= 200 * 1024;
+}
+// part: room for `cap` partials; returns the number written
+template <int K> static int wgrad_rows(Exec &ex, const float *img, const float *gout, const StemGeom &g, const RowWgrad &w, float *part, int cap) {
     static OncePerDevice once;
     if (once.first(ex.ctx->device)) cudaFuncSetAttribute(stem_wgrad_row_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    parts = row_grid(ex, stem_wgrad_row_kernel<K>, nw * 32, smem, n_tiles, blocks_y);
+    int parts = row_grid(ex, stem_wgrad_row_kernel<K>, w.nw * 32, w.smem, w.n_tiles, w.blocks_y);
     if (parts > cap) parts = cap;
-    launch(ex, stem_wgrad_row_kernel<K>, dim3(parts, blocks_y), nw * 32, smem, img, gout, part, g, fast_div(g.W * 3), cols, tiles_per_img, n_tiles, cbw);
-    return true;
+    launch(ex, stem_wgrad_row_kernel<K>, dim3(parts, w.blocks_y), w.nw * 32, w.smem, img, gout, part, g, fast_div(g.W * 3), w.cols, w.tiles_per_img, w.n_tiles, w.cbw);
+    return parts;
 }
 
 // image: fp32 [N,H,W,cin]; out: the stem's output (a plain tensor or the halves of stage 0's pair, float or fixed point)
@@ -498,16 +501,16 @@ bool stem_wgrad(Exec &ex, const float *img, const float *gout, Geom gi, const La
     const int n_cg = cop / CO_T, n_kg = kp / KK_T, G = n_cg * n_kg;
     const int P = g.N * g.Ho * g.Wo, n_chunks = (P + kPx - 1) / kPx;
     const size_t smem = ((size_t)kPx * cop + (size_t)kPx * kp) * 4 + (size_t)g.K * 4;
-    int cols;
-    const bool rows = row_stem(g, 1, cols);
+    RowWgrad w;
+    const bool rows = wgrad_rows_shape<3>(g, w) || wgrad_rows_shape<7>(g, w);
     if (!rows && (G > 256 || smem > 200 * 1024)) return false;
     int grid = ex.ctx->sm_count * (g.k == 3 ? 4 : 2); if (grid > n_chunks) grid = n_chunks;         // room for that many partials
     ex.flops += 2ull * P * g.Co * g.K;
     size_t m = ex.ws.mark();
     float *part = ex.ws.get<float>((size_t)grid * g.Co * g.K);
     if (!ex.dry) {
-        if (!(rows && (g.k == 3 ? wgrad_rows<3>(ex, img, gout, g, part, grid, grid) : wgrad_rows<7>(ex, img, gout, g, part, grid, grid)))) {
-            if (G > 256 || smem > 200 * 1024) { ex.ws.release(m); return false; }
+        if (rows) grid = g.k == 3 ? wgrad_rows<3>(ex, img, gout, g, w, part, grid) : wgrad_rows<7>(ex, img, gout, g, w, part, grid);
+        else {
             if (grid > ex.ctx->sm_count * 2) grid = ex.ctx->sm_count * 2;
             const int S = 256 / G;
             static OncePerDevice once;

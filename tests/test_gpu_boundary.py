@@ -1,6 +1,8 @@
 """Boundary behaviour on the device: pre-packed weights give the same bits as packing per call, a
 bounded wait that runs out is reported and leaves the context usable, a label out of range is
 reported instead of followed, undersized declared buffers are refused."""
+from dataclasses import replace
+
 import numpy as np
 import pytest
 import torch
@@ -168,3 +170,23 @@ def test_statistics_whose_sum_of_squares_overflows_switch_the_channel_off(mode, 
     assert np.isfinite(ys[0]).all() and np.array_equal(ys[0], ys[1])
     B.revnet_check_device(ctx)
     ctx.close()
+
+
+def test_flops_of_a_step_scale_with_the_image_where_the_stem_changes_kernels():
+    """Images of 896 pixels are too wide for the row kernel of the 7x7 stem's weight gradient and 32 channels too many for the patch
+    kernel: the general one takes over, and the step counts (and sizes scratch for) that one alone."""
+    per_pixel = []
+    for img in (64, 896):
+        cfg = replace(hp.tiny_stack("bottleneck", True, N=1), img=img, stem_cout=32)
+        ctx = B.Context(0)
+        r = R.StackRunner(ctx, cfg, 1)
+        inp = syn.make_stack_inputs(cfg)
+        r.load(inp["images"], inp["labels"], inp["params"])
+        st = r.step()
+        head = 4 * cfg.N * 2 * cfg.stages[-1].c * cfg.n_classes
+        per_pixel.append((st.flops_bwd - head) / img ** 2)
+        g = r.results()["grads"]["stem.W"]
+        assert np.isfinite(g).all() and np.abs(g).max() > 0
+        B.revnet_check_device(ctx)
+        ctx.close()
+    assert per_pixel[0] == per_pixel[1]
