@@ -6,8 +6,8 @@
 //   dgrad: da[q,ci]    = sum_{kh,kw,co} g[p,co] * W[co,kh,kw,ci],  p*s + (kh,kw) - pad = q
 //   wgrad: dW[co,kh,kw,ci] = sum_p g[p,co] * a[p (+) (kh,kw), ci]
 //
-// Three kernels.  conv3x3_direct_kernel takes fp32 3x3 stride-1 layers (forward and data gradient), conv_gemm_kernel every other layer whose channel counts are multiples of four (all BN-ReLU-conv layers):
-// quads of channels are loaded as vectors, a thread's pixel is decoded once, and the product is register-tiled.
+// Three kernels.  conv3x3_direct_kernel takes fp32 3x3 stride-1 layers (forward and data gradient), conv_gemm_kernel every
+// other layer whose channel counts are multiples of four (all BN-ReLU-conv layers): quads of channels are loaded as vectors, a thread's pixel is decoded once, and the product is register-tiled.
 // gemm_simt_kernel loads element by element and is left for the stem convolution's odd channel counts (an image has
 // three), where the kernels of stem.cu do not take its size.
 #include "common.cuh"
@@ -187,6 +187,7 @@ template <int WM, int WN, int WK> struct GemmTile {
 };
 
 constexpr int kRun = 16;            // chunks of 16
+// (127 registers, two CTAs per SM; the weight gradient of at most 16 output channels spills 52 bytes)
 template <int WM, int WN, int WK, class AL, class BL, class EP>
 __global__ void __launch_bounds__(256, 2) conv_gemm_kernel(AL al, BL bl, EP ep, int M, int N, int K, int k_per_split) {
     pdl_enter();
@@ -611,13 +612,13 @@ void conv_fprop_simt(Exec &ex, const void *a, bool a_bf16, Geom gi, const Layer 
     DirectGeom d;
     if (g.k == 3 && g.s == 1 && !a_bf16 && direct_shape(g.N, g.H, g.W, g.Ci, g.Co, ex.ctx->sm_count, d)) {
         launch_direct(ex, (const float *)a, DirectFprop{L.W, g.Ci}, ep, d);
-        ex.check("conv_fprop_simt", bytes, 2.0 * M * N * (double)K);
+        ex.check("conv_fprop_direct", bytes, 2.0 * M * N * (double)K);
         return;
     }
     const FpropB bl{L.W, N, K, a_bf16};
     if (a_bf16) launch_pixels(ex, FpropA<bf16>{(const bf16 *)a, g, wo, ho, ci, kk, M, K}, bl, ep, M, N, K);
     else launch_pixels(ex, FpropA<float>{(const float *)a, g, wo, ho, ci, kk, M, K}, bl, ep, M, N, K);
-    ex.check("conv_fprop_simt", bytes, 2.0 * M * N * (double)K);
+    ex.check("conv_fprop_gemm", bytes, 2.0 * M * N * (double)K);
 }
 
 void conv_dgrad_simt(Exec &ex, const void *gq, bool g_bf16, Geom gi, const Layer &L, float *da) {
@@ -630,7 +631,7 @@ void conv_dgrad_simt(Exec &ex, const void *gq, bool g_bf16, Geom gi, const Layer
     DirectGeom d;
     if (g.k == 3 && g.s == 1 && !g_bf16 && g.Ci % 4 == 0 && direct_shape(g.N, g.H, g.W, g.Co, g.Ci, ex.ctx->sm_count, d)) {
         launch_direct(ex, (const float *)gq, DirectDgrad{L.W, g.Ci}, ep, d);
-        ex.check("conv_dgrad_simt", bytes, 2.0 * g.N * g.Ho * g.Wo * N * (double)K);
+        ex.check("conv_dgrad_direct", bytes, 2.0 * g.N * g.Ho * g.Wo * N * (double)K);
         return;
     }
     // stride 2: parity classes of (H + 1) / 2 x (W + 1) / 2 pixels would be ragged on odd sizes; those keep the plain numbering
@@ -640,7 +641,7 @@ void conv_dgrad_simt(Exec &ex, const void *gq, bool g_bf16, Geom gi, const Layer
     const DgradB bl{L.W, co, g.k * g.k, N, K, g_bf16};
     if (g_bf16) launch_pixels(ex, DgradA<bf16>{(const bf16 *)gq, g, w, h, co, kk, cls, classes, M, K}, bl, ep, M, N, K);
     else launch_pixels(ex, DgradA<float>{(const float *)gq, g, w, h, co, kk, cls, classes, M, K}, bl, ep, M, N, K);
-    ex.check("conv_dgrad_simt", bytes, 2.0 * g.N * g.Ho * g.Wo * N * (double)K);
+    ex.check("conv_dgrad_gemm", bytes, 2.0 * g.N * g.Ho * g.Wo * N * (double)K);
 }
 
 // fixed-order sum of split-K slices: a block takes 32 elements, eight threads each (every eighth slice), added in order
@@ -690,7 +691,7 @@ void conv_wgrad_simt(Exec &ex, const void *gq, bool g_bf16, const void *a, bool 
         if (quads && g_bf16 == a_bf16) {
             if (g_bf16) wgrad_launch(ex, (const bf16 *)gq, (const bf16 *)a, g, part, splits, kps);
             else wgrad_launch(ex, (const float *)gq, (const float *)a, g, part, splits, kps);
-            ex.check("conv_wgrad_simt", bytes, 2.0 * Co * KC * (double)P);
+            ex.check("conv_wgrad_gemm", bytes, 2.0 * Co * KC * (double)P);
         } else {
             EpiPlain ep{part, KC, (size_t)Co * KC};
 #define RV_WG(TG, TA) launch_gemm(ex, "conv_wgrad_simt", AnyWgradA<TG>{(const TG *)gq, g}, AnyWgradB<TA>{(const TA *)a, g}, ep, Co, KC, P, splits, kps, bytes)

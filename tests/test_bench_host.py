@@ -31,7 +31,8 @@ def test_convolution_launch_shapes_are_split_by_what_binds_them():
 def test_roofline_that_binds_a_kernel():
     assert bench.binding_roofline("conv_tc_kernel", rec(1, 1.0, 1e9, 1e9), PEAKS) == "hbm"
     assert bench.binding_roofline("conv_tc_kernel", rec(1, 1.0, 1e6, 1e12), PEAKS) == "tensor"
-    assert bench.binding_roofline("gemm_simt_kernel", rec(1, 1.0, 1e6, 1e12), PEAKS) == "alu"
+    for k in ("conv3x3_direct_kernel", "conv_gemm_kernel", "gemm_simt_kernel"):
+        assert bench.binding_roofline(k, rec(1, 1.0, 1e6, 1e12), PEAKS) == "alu"
 
 
 def test_stored_traffic_is_reported_only_for_unchanged_kernel_sources(tmp_path, monkeypatch):
@@ -53,3 +54,10 @@ def test_committed_traffic_file_names_kernels_the_bench_knows():
         for k, v in kernels.items():
             assert k in bench.KERNEL_SOURCES, (workload, k)
             assert v["dram_bytes_per_launch"] > 0 and len(v["source_digest"]) == 16
+
+
+def test_every_convolution_record_of_the_library_names_a_device_kernel():
+    import re
+    src = "".join(open(bench.os.path.join(bench.ROOT, "paper_1707_04585_b200", "csrc", f)).read() for f in ("conv_simt.cu", "conv_tc.cu", "conv_fused.cu"))
+    names = set(re.findall(r'"(conv_(?:fprop|dgrad|wgrad)_\w+)"', src))
+    assert len(names) >= 12 and names <= set(bench.DEVICE_KERNEL), names - set(bench.DEVICE_KERNEL)
