@@ -41,8 +41,6 @@ struct TileGeom {
     int BH, BIMG;
     int tiles_per_img;       // BIMG == 1
     int n_px_tiles;
-    int hw_order;            // accumulator rows run (h, img, x) with x < Wp instead of (img, h, w)
-    int Wp;                  // hw_order: row pitch in pixels (W rounded up to a multiple of 8); columns >= W are padding
 };
 __device__ __forceinline__ void tile_origin(const TileGeom &g, int t, int &n0, int &h0) {
     if (g.BIMG > 1) { n0 = t * g.BIMG; h0 = 0; }
@@ -62,15 +60,8 @@ __device__ __forceinline__ float4 ldcg4(const float *p) { return __ldcg(reinterp
 // within the tile, for the bounds checks of ragged tiles.
 struct RowMap { int rel[128]; int hi[128]; };
 __device__ __forceinline__ void build_row_map(const TileGeom &g, RowMap *rm, int m) {
-    int img, h, w;
-    bool ok = true;
-    if (g.hw_order) {
-        w = m % g.Wp; img = (m / g.Wp) % g.BIMG; h = m / (g.BIMG * g.Wp);
-        ok = w < g.W && h < g.BH;
-    } else {
-        ok = m < g.BIMG * g.BH * g.W;
-        w = m % g.W; img = m / (g.BH * g.W); h = (m / g.W) % g.BH;
-    }
+    const bool ok = m < g.BIMG * g.BH * g.W;
+    const int w = m % g.W, img = m / (g.BH * g.W), h = (m / g.W) % g.BH;
     rm->rel[m] = ok ? (img * g.H + h) * g.W + w : -1;
     rm->hi[m] = h | (img << 16);
 }

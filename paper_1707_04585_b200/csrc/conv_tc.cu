@@ -955,7 +955,7 @@ int round_up(int x, int m) { return (x + m - 1) / m * m; }
 // that fall outside are padding: TMA fills their operand rows with zeros and the epilogue skips them.
 bool tile_geom(Geom g, TileGeom &t) {
     if (g.W > 128 || g.W < 1) return false;
-    t.N = g.N; t.H = g.H; t.W = g.W; t.hw_order = 0; t.Wp = g.W;
+    t.N = g.N; t.H = g.H; t.W = g.W;
     t.BH = 128 / g.W; if (t.BH > g.H) t.BH = g.H;
     t.BIMG = 1;
     if (t.BH == g.H) { t.BIMG = 128 / (g.H * g.W); if (t.BIMG > g.N) t.BIMG = g.N; if (t.BIMG < 1) t.BIMG = 1; }
