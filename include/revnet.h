@@ -64,8 +64,8 @@ typedef enum {
 typedef struct revnet_ctx revnet_ctx;
 typedef struct revnet_plan revnet_plan;
 
-/* Create / destroy a context bound to one CUDA device.  Creation allocates a few hundred
- * bytes of device memory for status words; nothing else is ever allocated by the library. */
+/* Create / destroy a context bound to one CUDA device.  Creation allocates 160 KB of
+ * device memory (status and counter words, timeline stamps); nothing else is ever allocated by the library. */
 int revnet_create(revnet_ctx **out, int device);
 int revnet_destroy(revnet_ctx *ctx);
 /* Text of the last error recorded on ctx (never NULL; valid until the next failing call on the same

@@ -336,6 +336,8 @@ __device__ __forceinline__ void column_sums(float (&a)[NC], int lane) {
     a[0] += __shfl_xor_sync(0xffffffffu, a[0], 16);
 }
 
+// Registers: 123 with eight epilogue warps; with sixteen the block of 768 threads leaves 80, and the epilogue, which holds 32 running sums,
+// 16 partner words and 8 values, spills 304 bytes.
 template <int EW>
 __global__ void __launch_bounds__(fused_threads(EW), 1) conv_fused_kernel(const __grid_constant__ FusedArgs A) {
     extern __shared__ uint8_t smem_raw[];

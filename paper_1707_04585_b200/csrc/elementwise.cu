@@ -123,6 +123,7 @@ struct RedPlan {
 };
 
 // CTAs run slab by slab along x (a tensor may have more slabs than a grid has rows)
+// (64 registers for four CTAs per SM: 44 bytes of spills in mode 0, 92 in mode 1, around the reduction behind the loop)
 template <int MODE>   // 0: sum t, sum t^2 ; 1: sum db, sum db*xhat (BN+ReLU backward)
 __global__ void __launch_bounds__(256, 4) col_reduce_kernel(Pair t, const float *__restrict__ da, size_t P, BnRef bn, const RedPlan pl, RedOut out) {
     pdl_enter();
@@ -239,7 +240,8 @@ Moments mom_alloc(Exec &ex, int C, bool with_part) {
     float *p = ex.ws.get<float>((size_t)2 * C);
     m.mean = p; m.rstd = p + C;
     if (with_part) {
-        // a fused convolution runs at most two CTAs per SM, one record of 2C floats each
+        // records of 2C floats that a producer may leave: one per CTA of a convolution (conv_tc_kernel runs at most two CTAs per SM, the
+        // others one), kPendingRecords of a stand-alone reduction
         m.part_cap = (size_t)2 * ex.ctx->sm_count * 2 * C;
         m.part = ex.ws.get<float>(m.part_cap);
     }
@@ -368,6 +370,7 @@ template <int V> struct BnCoef {
 };
 constexpr int kApplyRows = 4;
 
+// (64 registers for four CTAs per SM: with eight channels per thread the coefficients spill 20 to 24 bytes)
 template <class TO, int V>
 __global__ void __launch_bounds__(256, 4) bn_relu_apply_kernel(Pair t, size_t P, int SW, int rows, BnRef bn, TO *__restrict__ a, unsigned long long *stamp) {
     pdl_enter();
