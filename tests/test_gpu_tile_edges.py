@@ -30,6 +30,7 @@ def ctx():
     ("basic", 6, 9, 11, 40, 0),           # five planes
     ("basic", 4, 13, 13, 56, 0),          # seven planes, 56 of 64 output columns
     ("basic", 2, 16, 16, 64, 0),          # the widest layer with its BN and ReLU inside
+    ("basic", 1, 103, 103, 88, 0),        # column reductions in two levels: 121 records, the last group one CTA
     ("bottleneck", 6, 9, 9, 32, 12),      # 1x1; rows of 48 bytes: 16-byte accesses
     ("bottleneck", 10, 23, 9, 128, 32),   # one column group: four warp groups on alternate tiles, records left to the consumer
     ("bottleneck", 10, 23, 9, 128, 64),   # two column groups
@@ -44,16 +45,20 @@ def test_bf16_blocks_at_tile_edges(ctx, kind, N, H, W, c, w):
 
 
 @pytest.mark.parametrize("kind,N,H,W,c,w", [
-    ("basic", 1, 5, 13, 4, 0),            # 65 pixels: one more than the shortest tile; columns 4 of 16
-    ("basic", 1, 275, 275, 16, 0),        # 16-row tiles, the last one of 3 rows
-    ("basic", 1, 150, 253, 20, 0),        # 32-column tiles, the tall ones
-    ("basic", 1, 139, 137, 36, 0),        # 64-column tiles
+    ("basic", 1, 5, 13, 4, 0),            # direct 3x3: one tile, half of it inside the image, outputs 4 of 16; 65 pixels in the weight gradient
+    ("basic", 1, 275, 275, 16, 0),        # direct 3x3: 16-row tiles, the last one of 3 rows
+    ("basic", 1, 150, 253, 20, 0),        # direct 3x3: 20 of 32 outputs; weight gradient in 32-column tiles
+    ("basic", 1, 139, 137, 36, 0),        # direct 3x3: two groups of outputs, the second of 4; weight gradient in 64-column tiles
     ("basic", 2, 11, 7, 68, 0),           # two column tiles, the second of 4 columns
     ("basic", 16, 5, 4, 8, 0),            # direct 3x3: eight images per tile, one column of warps
     ("basic", 5, 7, 6, 20, 0),            # two images per tile, the last one of a tile missing
     ("basic", 75, 24, 16, 16, 0),         # direct 3x3, eight warps in two row groups: the second one of the last tile lies below the image
     ("basic", 9, 20, 7, 8, 0),            # the same with narrow images and four warps
     ("basic", 1, 33, 17, 100, 0),         # four chunks of input channels (the last of 4), four groups of outputs
+    ("basic", 1, 119, 122, 132, 0),       # column reductions in two levels, two slabs: 121 records (statistics) and 242 (backward sums)
+    ("bottleneck", 1, 277, 275, 16, 4),   # 1x1 GEMMs onto 4 and 16 channels in 256-row tiles, the last one of 143
+    ("bottleneck", 1, 277, 275, 32, 20),  # ... onto 20 and 32
+    ("bottleneck", 1, 195, 196, 64, 36),  # ... onto 36 and 64 in 128-row tiles, the last one of 76
     ("bottleneck", 1, 3, 3, 132, 4),      # column sums of nine rows: two slabs of 17 and 16 quads, and one quad
     ("bottleneck", 1, 97, 99, 520, 8),    # 32-byte accesses in the streaming kernels
     ("bottleneck", 2, 37, 41, 260, 136),  # three slabs (22, 22, 21), several row ranges; sums of 1224 products
