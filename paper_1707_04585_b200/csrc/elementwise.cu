@@ -106,6 +106,10 @@ static RedShape red_shape(size_t P, int C, int sm, int rows_in_flight, int max_c
 }
 // floats of scratch: the records, then the groups' sums in double precision
 static size_t red_floats(const RedShape &r, int C) { return (size_t)r.chunks * 2 * C + (size_t)r.groups * 4 * C; }
+static dim3 red_grid(const RedShape &r) {
+    const int z = cdiv(r.slabs, 65535);
+    return dim3(r.chunks, cdiv(r.slabs, z), z);
+}
 // counter words: per slab one for the slab and one for each group; a slab of one CTA counts nothing
 static int red_words(const RedShape &r) { return r.chunks > 1 ? r.slabs * (1 + r.groups) : 0; }
 constexpr int kStatRows = 8, kBwdRows = 4;
@@ -122,16 +126,19 @@ struct RedPlan {
     unsigned int *counters;       // per slab 1 + groups zeroed words, left zero
 };
 
-// CTAs run slab by slab along x (a tensor may have more slabs than a grid has rows)
-// (64 registers for four CTAs per SM: 44 bytes of spills in mode 0, 92 in mode 1, around the reduction behind the loop)
-template <int MODE>   // 0: sum t, sum t^2 ; 1: sum db, sum db*xhat (BN+ReLU backward)
+// Grid: chunks along x, slabs along y and, beyond 65535 of them, z
+// (64 registers for four CTAs per SM: 52 to 60 bytes of spills in mode 0, 92 to 96 in mode 1, around the reduction behind the loop.  Two
+// kernels, because a small launch fetches every instruction of its tail anew: with both forms in one, each launch of the smallest block
+// calls took 0.5 to 0.7 us longer)
+template <int MODE, bool GROUPS>   // MODE 0: sum t, sum t^2 ; 1: sum db, sum db*xhat (BN+ReLU backward); GROUPS: records added in two levels
 __global__ void __launch_bounds__(256, 4) col_reduce_kernel(Pair t, const float *__restrict__ da, size_t P, BnRef bn, const RedPlan pl, RedOut out) {
     pdl_enter();
     constexpr int NR = MODE == 0 ? kStatRows : kBwdRows;
     __shared__ double red[256 * 4], tot[128 * 4];
     __shared__ unsigned int last;
     const int C = t.C(), C4 = C / 4, SW = pl.SW, RPP = 256 / SW, tid = threadIdx.x;
-    const int slab = (int)blockIdx.x / pl.chunks, chunk = (int)blockIdx.x - slab * pl.chunks;
+    const int chunk = blockIdx.x, slab = blockIdx.y + blockIdx.z * gridDim.y;
+    if (slab * SW >= C4) return;
     const int tx = tid % SW, ty = tid / SW, q = slab * SW + tx;
     const bool valid = q < C4 && ty < RPP;
     const size_t r0 = (size_t)chunk * pl.rows;
@@ -187,21 +194,26 @@ __global__ void __launch_bounds__(256, 4) col_reduce_kernel(Pair t, const float 
     }
     if (pl.pending) return;
     const int q0 = slab * SW, nq = C4 - q0 < SW ? C4 - q0 : SW;
-    unsigned int *cnt = pl.counters + (size_t)slab * (1 + pl.groups);
+    unsigned int *cnt = pl.counters + (size_t)slab * (GROUPS ? 1 + pl.groups : 1);
     // whether this CTA is the last of n to come here (the word is left zero)
     auto last_of = [&](unsigned int *word, int n) {
         __syncthreads();
         if (tid == 0) {
-            // (one thread's fences, on either side, order what all the CTA's threads wrote before the barrier and read after the next)
-            __threadfence();
-            last = n == 1 || atomicAdd(word, 1u) == (unsigned int)n - 1 ? 1u : 0u;
-            if (last && n > 1) *word = 0u;
-            __threadfence();
+            // (one thread's fences, on either side, order what all the CTA's threads wrote before the barrier and read after the next;
+            // the word is cleared behind them: a fence waits for the stores in front of it)
+            bool l = true;
+            if (n > 1) {
+                __threadfence();
+                l = atomicAdd(word, 1u) == (unsigned int)n - 1;
+                __threadfence();
+                if (l) *word = 0u;
+            }
+            last = l ? 1u : 0u;
         }
         __syncthreads();
         return last != 0u;
     };
-    if (pl.group) {
+    if constexpr (GROUPS) {
         const int g = chunk / pl.group, first = g * pl.group, n = pl.chunks - first < pl.group ? pl.chunks - first : pl.group;
         if (!last_of(cnt + 1 + g, n)) return;
         tc::reduce_records<256>(pl.part + (size_t)first * 2 * C, n, C, 2 * q0, 2 * nq, red, tot, tid);
@@ -286,7 +298,7 @@ void bn_stats(Exec &ex, Pair t, size_t P, Moments &mo) {
     float *part = defer ? mo.part : ex.ws.get<float>(red_floats(r, C));
     mo.pending = defer; mo.parts = r.chunks; mo.inv_count = 1.0 / (double)P;
     if (!ex.dry) {
-        launch_stream(ex, (double)P * C * 4, 30, col_reduce_kernel<0>, r.chunks * r.slabs, 256, 0, t, nullptr, P, BnRef{}, red_plan(ex, r, C, part, defer),
+        launch_stream(ex, (double)P * C * 4, 30, r.group && !defer ? col_reduce_kernel<0, true> : col_reduce_kernel<0, false>, red_grid(r), 256, 0, t, nullptr, P, BnRef{}, red_plan(ex, r, C, part, defer),
                RedOut{mo.mean, mo.rstd, nullptr, nullptr, nullptr, 1.0 / (double)P, ex.eps});
         ex.check("bn_stats", (double)P * C * 4);
     }
@@ -476,7 +488,7 @@ void bn_relu_bwd(Exec &ex, const float *da, Pair t, size_t P, BnRef bn, float *d
     float *part = sums_done ? nullptr : ex.ws.get<float>(red_floats(r, C));
     if (!ex.dry) {
         if (!sums_done) {
-            launch_stream(ex, (double)P * C * 8, 30, col_reduce_kernel<1>, r.chunks * r.slabs, 256, 0, t, da, P, bn, red_plan(ex, r, C, part, false),
+            launch_stream(ex, (double)P * C * 8, 30, r.group ? col_reduce_kernel<1, true> : col_reduce_kernel<1, false>, red_grid(r), 256, 0, t, da, P, bn, red_plan(ex, r, C, part, false),
                    RedOut{nullptr, nullptr, dgamma, dbeta, coef, 1.0 / (double)P, ex.eps});
             ex.check("bn_bwd_sums", (double)P * C * 8);
         }
