@@ -188,14 +188,17 @@ __device__ __forceinline__ void moments_of(double sum, double sum2, double inv_c
     double var = sum2 * inv_count - m * m;
     if (var < 0) var = 0;
     const double v = var + (double)eps;
-    const bool low = v < 1e-36, high = v > 1e36;
-    const double w = low ? v * 0x1p+120 : (high ? v * 0x1p-120 : v);
-    const float r = rsqrtf((float)w);
-    double y = (double)r;
-    y *= 1.5 - 0.5 * w * y * y;
-    y *= 1.5 - 0.5 * w * y * y;
-    if (!(r > 0.f && r < INFINITY)) y = (double)r;
-    mean = (float)m; rstd = (float)(low ? y * 0x1p+60 : (high ? y * 0x1p-60 : y));
+    double y = (double)rsqrtf((float)v);
+    y *= 1.5 - 0.5 * v * y * y;
+    y *= 1.5 - 0.5 * v * y * y;
+    if (__builtin_expect(!(v >= 1e-36 && v <= 1e36), 0)) {
+        const double s = v < 1 ? 0x1p+60 : 0x1p-60, w = v * s * s;
+        const float r = rsqrtf((float)w);
+        y = (double)r;
+        if (r > 0.f && r < INFINITY) { y *= 1.5 - 0.5 * w * y * y; y *= 1.5 - 0.5 * w * y * y; }
+        y *= s;
+    }
+    mean = (float)m; rstd = (float)y;
 }
 
 // Adds the per-CTA records of a reduction.  A record is 2C floats = C/2 float4 slots (per channel
