@@ -65,7 +65,7 @@ static size_t esz(const Exec &ex) { return ex.mode == 0 ? 2 : 4; }
 
 // out = partner + sign * Fn(u).  With `saved`, every layer's activated input, BN input and BN
 // statistics are left in the workspace (the caller releases them after the backward).
-void fn_forward(Exec &ex, Geom g, Pair u, const Moments *mom_in, const std::vector<Layer> &layers, Pair partner, Pair out,
+void fn_forward(Exec &ex, Geom g, Pair u, Moments *mom_in, const std::vector<Layer> &layers, Pair partner, Pair out,
                 int sign, Moments *mom_out, FnSaved *saved, bool skip_last_conv) {
     const int L = (int)layers.size();
     const bool b16 = ex.mode == 0;
@@ -113,6 +113,7 @@ void fn_forward(Exec &ex, Geom g, Pair u, const Moments *mom_in, const std::vect
         if (fused) cur.pending = false;     // the fused kernel has stored mean and rstd
         else if (b16 && !last && !cur.pending && conv_fprop_bn(ex, t, bn, gi, ly, o, &next, saved ? (bf16 *)a : nullptr)) fused = true;
         else { mom_finalize(ex, cur, ly.cin); bn_relu_apply(ex, t, P, BnRef{ly.gamma, ly.beta, cur.mean, cur.rstd}, a, b16); }
+        if (l == 0 && mom_in) mom_in->pending = false;      // mean and rstd are stored by now
         if (saved) { saved->a.push_back(a); saved->bn.push_back(cur); }
         if (last) {
             if (!skip_last_conv && !fused) conv_fprop(ex, a, gi, ly, out, partner, sign, mom_out);
@@ -201,7 +202,7 @@ void fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
 }
 
 void block_forward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const std::vector<Layer> &G,
-                   float *x1, float *x2, float *y1, float *y2, const Moments *mx2, Moments *my1, Moments *my2) {
+                   float *x1, float *x2, float *y1, float *y2, Moments *mx2, Moments *my1, Moments *my2) {
     const float q = ex.q;
     // without hand-off (stand-alone call) the statistics of x2 and y1 come from the stand-alone reduction,
     // as they will in the reversal, which is handed y1 from outside
@@ -212,7 +213,7 @@ void block_forward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const s
 void block_backward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const std::vector<Layer> &G,
                     const float *y1, const float *y2, const float *dy1, const float *dy2,
                     float *x1, float *x2, float *dx1, float *dx2,
-                    Moments *m1, Moments *m2, const Moments *m2_use, const bf16 *dy2_cast, bf16 *dx2_cast,
+                    Moments *m1, Moments *m2, Moments *m2_use, const bf16 *dy2_cast, bf16 *dx2_cast,
                     Moments *m1_out, bool overlap) {
     FnSaved svG, svF;
     const float q = ex.q;   // format of the coupling state; gradients are always float
@@ -225,13 +226,14 @@ void block_backward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const 
     size_t m = ex.ws.mark();
     // x2 = y2 - G(z1), z1 = y1
     fn_forward(ex, g, single((float *)y1, c, q), m1, G, single((float *)y2, c, q), single(x2, c, q), -1, m2, &svG, false);
-    const Moments *mf = (m2_use && m2_use->valid) ? m2_use : m2;
+    Moments *mf = (m2_use && m2_use->valid) ? m2_use : m2;
+    Moments *mx1 = m1_out && !m1_out->mean ? nullptr : m1_out;
     if (!overlap) {
         // dz1 = dy1 + (dG/dz1)^T dy2 ; dW_G
         fn_backward(ex, g, single((float *)y1, c, q), G, svG, single((float *)dy2, c), dy2_cast, single((float *)dy1, c), single(dx1, c), dz1_cast);
         ex.ws.release(m);
         // x1 = z1 - F(x2)
-        fn_forward(ex, g, single(x2, c, q), mf, F, single((float *)y1, c, q), single(x1, c, q), -1, m1_out, &svF, false);
+        fn_forward(ex, g, single(x2, c, q), mf, F, single((float *)y1, c, q), single(x1, c, q), -1, mx1, &svF, false);
     } else {
         // x1 = z1 - F(x2) on the reconstruction stream (it needs x2 only), dz1 and dW_G meanwhile on the main stream;
         // F's internals are placed before G's gradient steps take their temporaries, so the arena stays a stack
@@ -244,7 +246,7 @@ void block_backward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const 
         // launches take short-lived scratch from the arena and hand it back at once, which is safe within one stream
         // only: what F's recomputation touched stays out of reach of the main stream's launches until the join
         ex.ws.high = ex.ws.off;
-        fn_forward(ex, g, single(x2, c, q), mf, F, single((float *)y1, c, q), single(x1, c, q), -1, m1_out, &svF, false);
+        fn_forward(ex, g, single(x2, c, q), mf, F, single((float *)y1, c, q), single(x1, c, q), -1, mx1, &svF, false);
         if (ex.ws.high > ex.ws.off) ex.ws.off = ex.ws.high;
         if (!ex.dry) { cudaEventRecord(ex.ctx->ev_rjoin, ex.ctx->recon_stream); ex.stream = main; }
         fn_backward(ex, g, single((float *)y1, c, q), G, svG, single((float *)dy2, c), dy2_cast, single((float *)dy1, c), single(dx1, c), dz1_cast);

@@ -379,6 +379,7 @@ struct Geom { int N, H, W; size_t P() const { return (size_t)N * H * W; } };
 
 // ---------------------------------------------------------------- elementwise.cu
 Moments mom_alloc(Exec &ex, int C, bool with_part = false);
+void mom_room(Exec &ex, Moments &m, int C);      // gives m room for pending records, and asks its producers to leave them
 // pending statistics -> mean / rstd (one small kernel); no-op otherwise
 void mom_finalize(Exec &ex, Moments &m, int C);
 // batch statistics of t ([P,C]) -> mean, rstd (the convolution epilogues produce the same quantities for the
@@ -454,10 +455,11 @@ void tc_pack_list(Exec &ex, const PackJobs &jobs, int n_jobs);                //
 struct FnSaved;   // activations kept from a residual function's (re)computation
 // out = partner + sign * Fn(u); if saved != nullptr the per-layer tensors stay in the workspace
 // skip_last_conv: only rebuild the saved tensors (used to re-derive a stored layer's operands)
-// mom_in: statistics of u if a kernel enqueued earlier provides them (else they are computed here);
+// mom_in: statistics of u if a kernel enqueued earlier provides them (else they are computed here); pending records of
+// theirs are added by the first layer's kernel, and mom_in is no longer pending on return;
 // mom_out: where the last convolution's epilogue should leave the statistics of `out`
-// (mom_out->valid tells whether it did).
-void fn_forward(Exec &ex, Geom g, Pair u, const Moments *mom_in, const std::vector<Layer> &layers, Pair partner, Pair out,
+// (mom_out->valid tells whether it did; mom_out->pending that their next reader has the records to add).
+void fn_forward(Exec &ex, Geom g, Pair u, Moments *mom_in, const std::vector<Layer> &layers, Pair partner, Pair out,
                 int sign, Moments *mom_out, FnSaved *saved, bool skip_last_conv);
 // dgin_out = add + (dFn/du)^T gup, parameter gradients written through the layers' pointers;
 // gup_cast: bf16 [P,C] copy of gup if the caller already has one; dgin_cast: if non-null, a bf16
@@ -475,17 +477,18 @@ struct FnSaved {
 //   backward: m1 in = statistics of y1, out = statistics of x1; m2 out = statistics of x2;
 //             m2_use: statistics F must use for x2 when the forward pass took them from elsewhere
 //             (the first block of a stage), so that F is recomputed bit for bit;
-//             m1_out: where the statistics of x1 go instead of m1 (default: m1 is overwritten)
+//             m1_out: where the statistics of x1 go instead of m1 (default: m1 is overwritten); m1_out->mean == nullptr, and
+//             m2 == nullptr beside a valid m2_use: nobody reads those of x1 / x2, they are not summed
 //   overlap : the recomputation of F (x1 = y1 - F(x2)) runs on the context's reconstruction stream beside
 //             the gradient steps of G, which still read y1 and its statistics: the caller must then pass
 //             x1 != y1 and m1_out != m1
 void block_forward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const std::vector<Layer> &G,
                    float *x1, float *x2, float *y1, float *y2,
-                   const Moments *mx2 = nullptr, Moments *my1 = nullptr, Moments *my2 = nullptr);
+                   Moments *mx2 = nullptr, Moments *my1 = nullptr, Moments *my2 = nullptr);
 void block_backward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const std::vector<Layer> &G,
                     const float *y1, const float *y2, const float *dy1, const float *dy2,
                     float *x1, float *x2, float *dx1, float *dx2,
-                    Moments *m1 = nullptr, Moments *m2 = nullptr, const Moments *m2_use = nullptr,
+                    Moments *m1 = nullptr, Moments *m2 = nullptr, Moments *m2_use = nullptr,
                     const bf16 *dy2_cast = nullptr, bf16 *dx2_cast = nullptr, Moments *m1_out = nullptr, bool overlap = false);
 
 static inline int conv_out(int in, int k, int s) { return (in + 2 * (k / 2) - k) / s + 1; }

@@ -10,6 +10,8 @@
 #include <stdlib.h>
 #include <math.h>
 
+bool conv_fused_takes(Exec &ex, Geom gi, const Layer &L);     // conv_fused.cu
+
 struct LayerSlot {
     int cin, cout, k, stride; size_t off_gamma, off_beta, off_W;   // offsets in floats; stem: gamma/beta unused
     const bf16 *wp_f = nullptr, *wp_d = nullptr;                  // bf16 packs of the current step (mode 0)
@@ -144,10 +146,11 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
     // batch statistics handed from kernel to kernel: per stage those of the current (x1,x2) pair (one
     // [2c] array each for mean and rstd, so that the pair reads as one tensor to a transition) and
     // those of the stage's input x2, which the reversal of the first unit needs again
-    struct StageMom { Moments m1, m2, cat, in_cat, in2, dy1; };      // dy1: statistics of a down-sampling unit's y1, kept for its backward
+    struct StageMom { Moments m1, m2, cat, in_cat, in2, dy1; bool defer; };      // dy1: statistics of a down-sampling unit's y1, kept for its backward
     std::vector<StageMom> sm(S);
     bf16 *gcast = nullptr;          // bf16 copy of the gradient w.r.t. x2 / y2, handed from unit to unit
-    float *x1_alt = nullptr, *m1_alt_buf = nullptr;
+    float *x1_alt = nullptr;
+    Moments m1_alt;
     bf16 *gcast2 = nullptr;         // stored-activation step: bf16 copy of the gradient w.r.t. z1 inside a unit
     // Stored-activation step (ordinary backprop): what every unit keeps from the forward pass.  The tensors
     // live in the workspace arena, unit after unit, and are released in reverse order by the backward pass.
@@ -167,12 +170,18 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
             sm[si].m2.mean = b + s.c; sm[si].m2.rstd = b + 3 * s.c;
             sm[si].in_cat.mean = b + 4 * s.c; sm[si].in_cat.rstd = b + 6 * s.c;
             sm[si].in2.mean = b + 5 * s.c; sm[si].in2.rstd = b + 7 * s.c;
+            // Where a unit's functions start with a fused convolution, the statistics of the pair between units stay the records of the
+            // convolution that coupled it: the next one adds them while its first rows are on the way (1.0 to 2.1 us), where the
+            // reduction by the producer's last CTA kept every other SM waiting for 4 us (count, records, result).
+            sm[si].defer = ex.mode == 0 && s.units > 0 && conv_fused_takes(ex, Geom{N, s.H, s.H}, bind(s.F[0][0], params, grads)) &&
+                           conv_fused_takes(ex, Geom{N, s.H, s.H}, bind(s.G[0][0], params, grads));
+            if (sm[si].defer) { mom_room(ex, sm[si].m1, s.c); mom_room(ex, sm[si].m2, s.c); }
             size_t e = (size_t)N * s.H * s.H * s.c; if (e > cmax) cmax = e;
         }
         if (ex.mode == 0) gcast = ex.ws.get<bf16>(cmax);
         // the reversal writes x1 beside y1 instead of over it (the two buffers change roles from unit to unit), and the
         // statistics of x1 beside those of y1, so that F can be recomputed while G's gradient steps still read y1
-        if (!d.store_activations) { x1_alt = ex.ws.get<float>(cmax); size_t c2 = 0; for (auto &st : pl->st) if ((size_t)st.c > c2) c2 = st.c; m1_alt_buf = ex.ws.get<float>(2 * c2); }
+        if (!d.store_activations) { x1_alt = ex.ws.get<float>(cmax); size_t c2 = 0; for (auto &st : pl->st) if ((size_t)st.c > c2) c2 = st.c; m1_alt = mom_alloc(ex, (int)c2); int cd = 0; for (int si = 0; si < S; si++) if (sm[si].defer && pl->st[si].c > cd) cd = pl->st[si].c; if (cd) mom_room(ex, m1_alt, cd); }
         if (ex.mode == 0 && d.store_activations) gcast2 = ex.ws.get<bf16>(cmax);
     }
     float *recon = ex.ws.get<float>(REVNET_MAX_STAGES);
@@ -201,7 +210,7 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
         StageMom &mo = sm[si];
         if (s.has_trans) {
             std::vector<Layer> T{bind(s.trans, params, grads)};
-            const Moments *min = si > 0 ? &sm[si - 1].cat : nullptr;
+            Moments *min = si > 0 ? &sm[si - 1].cat : nullptr;
             fn_forward(ex, Geom{N, prevH, prevH}, prev, min, T, Pair{}, halves(x1, x2, s.c, q), 0, &mo.in_cat, nullptr, false);
         }
         mo.in2.valid = mo.in_cat.valid;
@@ -225,16 +234,21 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
             cudaMemcpyAsync(actf(s.off_v2), x2, b, cudaMemcpyDeviceToDevice, ex.stream);
         }
         if (!stored) {
-            for (int u = 0; u < s.units; u++)
+            for (int u = 0; u < s.units; u++) {
+                // (the last unit's pair is read by a transition or a down-sampling unit, which want mean and rstd)
+                Moments my2 = mo.m2;
+                if (u == s.units - 1) { my2.part = nullptr; my2.defer = false; }
                 block_forward(ex, g, s.c, bind(s.F[u], params, grads), bind(s.G[u], params, grads), x1, x2, x1, x2,
-                              u == 0 ? &mo.in2 : &mo.m2, &mo.m1, &mo.m2);
+                              u == 0 ? &mo.in2 : &mo.m2, &mo.m1, &my2);
+                mo.m2.valid = my2.valid; mo.m2.pending = my2.pending; mo.m2.parts = my2.parts; mo.m2.inv_count = my2.inv_count;
+            }
             mo.cat.valid = mo.m1.valid && mo.m2.valid;
             prev = halves(x1, x2, s.c, q);
         } else {
             // every unit writes its outputs to fresh tensors and leaves the internals of F and G where they are
             kept[si].resize(s.units);
             float *c1 = x1, *c2 = x2;
-            const Moments *m_in = &mo.in2;
+            Moments *m_in = &mo.in2;
             const size_t half = g.P() * s.c;
             for (int u = 0; u < s.units; u++) {
                 StoredUnit &k = kept[si][u];
@@ -243,8 +257,8 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
                 const bool last_unit = u == s.units - 1;
                 k.y1 = ex.ws.get<float>(half); k.y2 = ex.ws.get<float>(half);
                 // the statistics of the stage's final pair go where the next transition expects them
-                if (last_unit) { k.my1 = mo.m1; k.my2 = mo.m2; }
-                else { k.my1 = mom_alloc(ex, s.c); k.my2 = mom_alloc(ex, s.c); }
+                if (last_unit) { k.my1 = mo.m1; k.my2 = mo.m2; k.my2.part = nullptr; k.my2.defer = false; }
+                else { k.my1 = mom_alloc(ex, s.c, mo.defer); k.my2 = mom_alloc(ex, s.c, mo.defer); k.my1.defer = k.my2.defer = mo.defer; }
                 fn_forward(ex, g, single(c2, s.c, q), m_in, bind(s.F[u], params, grads), single(c1, s.c, q), single(k.y1, s.c, q), +1, &k.my1, &k.svF, false);
                 fn_forward(ex, g, single(k.y1, s.c, q), &k.my1, bind(s.G[u], params, grads), single(c2, s.c, q), single(k.y2, s.c, q), +1, &k.my2, &k.svG, false);
                 if (last_unit) { mo.m1 = k.my1; mo.m2 = k.my2; }
@@ -277,12 +291,17 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
         StageMom &mo = sm[si];
         if (!stored) {
             Moments mcur = mo.m1, malt = mo.m1;
-            malt.mean = m1_alt_buf; malt.rstd = m1_alt_buf + s.c; malt.valid = false;
+            malt.mean = m1_alt.mean; malt.rstd = m1_alt.mean + s.c; malt.valid = false;
+            if (mo.defer) { malt.part = m1_alt.part; malt.part_cap = m1_alt.part_cap; }
             float *cur1 = x1, *alt1 = x1_alt;
             for (int u = s.units - 1; u >= 0; u--) {
-                // x1 alternates between the two buffers from unit to unit
+                // x1 alternates between the two buffers from unit to unit.  Nothing reads the statistics of the stage's input as the
+                // reversal returns it: the first unit's F takes those of the forward pass.  (The sizing run has them summed there as well:
+                // the scratch of a stage does not depend on its depth)
+                Moments none;
+                const bool unread = u == 0 && !ex.dry;
                 block_backward(ex, g, s.c, bind(s.F[u], params, grads), bind(s.G[u], params, grads), cur1, x2, d1, d2, alt1, x2, d1, d2,
-                               &mcur, &mo.m2, u == 0 ? &mo.in2 : nullptr, u == s.units - 1 ? nullptr : gcast, gcast, &malt, true);
+                               &mcur, unread ? nullptr : &mo.m2, u == 0 ? &mo.in2 : nullptr, u == s.units - 1 ? nullptr : gcast, gcast, unread ? &none : &malt, true);
                 std::swap(cur1, alt1);
                 std::swap(mcur, malt);
             }
