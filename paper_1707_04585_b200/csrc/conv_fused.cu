@@ -514,8 +514,9 @@ bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count, FusedShape &s
         s.n_tiles = (cout_pad + g.BN - 1) / g.BN;
         g.groups = g.BN / NC;
         int ctas = sm_count / s.n_tiles; if (ctas < 1) ctas = 1;
-        // a contiguous range of positions per CTA, half a tile at least
-        g.chunk = round_up((g.total + ctas - 1) / ctas, 8); if (g.chunk < 64) g.chunk = 64;
+        // a contiguous range of positions per CTA, a tile at least.  (Half tiles would put a small layer on every SM, but take as long and
+        // leave none to the launches beside it: 110-layer step 4964 -> 4877 us, odd-sized basic block 167 -> 164 with whole ones.)
+        g.chunk = round_up((g.total + ctas - 1) / ctas, 8); if (g.chunk < 128) g.chunk = 128;
         s.ctas = (g.total + g.chunk - 1) / g.chunk;
         g.wtile_bytes = (g.BN * g.KC * 2 + 1023) & ~1023;
         const int T = (g.chunk + 127) / 128, fixed = 1024 + k * k * g.wtile_bytes + (int)sizeof(FusedShared) + 64;
