@@ -23,7 +23,10 @@ bool conv_wgrad_tc_batch(Exec &ex, int n, const void *const *gq, const void *con
 bool conv_fused_takes(Exec &ex, Geom gi, const Layer &L);
 bool conv_fprop_bn(Exec &ex, Pair t, BnRef bn, Geom gi, const Layer &L, Pair out, Moments *stats, bf16 *a_out);
 bool conv_fprop_fused(Exec &ex, Pair t, BnRef bn, Geom gi, const Layer &L, Pair out, Pair partner, int sign, Moments *stats, bf16 *a_out);
-bool conv_dgrad_fused(Exec &ex, const void *g, Geom gi, const Layer &L, float *da, const BnBwdReq *bb);
+bool conv_dgrad_fused(Exec &ex, const void *g, Geom gi, const Layer &L, float *da, const BnBwdReq *bb, BwdSums *sums);
+bool conv_dgrad_fused_takes(Exec &ex, Geom gi, const Layer &L, bool behind);
+bool conv_dgrad_fused_behind(Exec &ex, const float *g, const BnBwdReq &behind, const BwdSums &bsums, bf16 *g_out, Geom gi, const Layer &L, float *da, const BnBwdReq *bb,
+                             BwdSums *sums);
 
 // stats: in = where the statistics of `out` should go (or nullptr); stats->valid says whether the kernel provides them
 static void conv_fprop(Exec &ex, const void *a, Geom gi, const Layer &L, Pair out, Pair partner, int sign, Moments *stats) {
@@ -34,9 +37,10 @@ static void conv_fprop(Exec &ex, const void *a, Geom gi, const Layer &L, Pair ou
     conv_fprop_simt(ex, a, b16, gi, L, out, partner, sign);
 }
 // returns true when the epilogue also produced the BN-backward sums asked for in bb
-static bool conv_dgrad(Exec &ex, const void *g, Geom gi, const Layer &L, float *da, const BnBwdReq *bb) {
+// (sums: conv_dgrad_fused takes the layer, and the sums stay records)
+static bool conv_dgrad(Exec &ex, const void *g, Geom gi, const Layer &L, float *da, const BnBwdReq *bb, BwdSums *sums) {
     const bool b16 = ex.mode == 0;
-    if (b16 && L.stride == 1 && conv_dgrad_fused(ex, g, gi, L, da, bb)) return bb != nullptr;
+    if (b16 && L.stride == 1 && conv_dgrad_fused(ex, g, gi, L, da, bb, sums)) return bb != nullptr;
     if (b16 && L.stride == 1 && conv_dgrad_tc(ex, g, gi, L, da, bb)) return bb != nullptr;
     // stride 2 on the tensor cores: the CTAs of one launch split into the parity classes of the input pixels
     bool fused = false;
@@ -163,35 +167,60 @@ bool fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
     for (int l = 0; l < L; l++) { lptr[l] = &layers[l]; aq[l] = saved.a[l]; }
     if (side && !conv_wgrad_tc_batch(ex, L, gq.data(), aq.data(), gin.data(), lptr.data(), nullptr, &wg_need)) side = false;
     float *wg_scratch = side && wg_need ? ex.ws.get<float>(wg_need) : nullptr;
+    // Where the data gradients are fused kernels, the sums of a layer's BN backward stay the records of its data gradient's CTAs, and the data
+    // gradient of the layer in front (or the last step, `add`) takes its input through that BN backward itself
+    BwdSums sums;                        // pending sums of layer l + 1
+    const float *da_behind = nullptr;    // da of that layer
+    BnBwdReq behind{};
+    const bool plain = b16 && u.c1 == 0 && add.p0 && add.c1 == 0 && add.q == 0.f && dgin_out.p0 && dgin_out.c1 == 0 && dgin_out.q == 0.f;
     for (int l = L - 1; l >= 0; l--) {
         const Layer &ly = layers[l];
         const size_t P = gin[l].P();
-        gq[l] = gcur;
-        if (!side) {
-            conv_wgrad(ex, gcur, saved.a[l], gin[l], ly, ly.dW);
-        } else if (l == 0) {
-            cudaStream_t main = ex.stream;
-            if (!ex.dry) {
-                cudaEventRecord(ex.ctx->ev_fork, main);
-                cudaStreamWaitEvent(ex.ctx->side_stream, ex.ctx->ev_fork, 0);
-                ex.stream = ex.ctx->side_stream;
-            }
-            conv_wgrad_tc_batch(ex, L, gq.data(), aq.data(), gin.data(), lptr.data(), wg_scratch, nullptr);
-            ex.stream = main;
-        }
+        const bool folded = sums.part != nullptr;
+        bf16 *dt = folded ? ex.ws.get<bf16>(P * ly.cout) : nullptr;
+        gq[l] = folded ? dt : gcur;
         float *da = ex.ws.get<float>(P * ly.cin);
         float *coef = ex.ws.get<float>((size_t)3 * ly.cin);
         const Pair tl = l == 0 ? u : single(saved.t[l - 1], ly.cin);
         const BnRef bn{ly.gamma, ly.beta, saved.bn[l].mean, saved.bn[l].rstd};
         const BnBwdReq bb{tl, bn, ly.dgamma, ly.dbeta, coef};
-        const bool sums_done = conv_dgrad(ex, gcur, gin[l], ly, da, &bb);
+        const bool leave = b16 && (folded || conv_dgrad_fused_takes(ex, gin[l], ly, false)) &&
+                           (l == 0 ? plain && bn_relu_bwd_sums_takes(P, ly.cin) : (l > 1 || u.c1 == 0) && conv_dgrad_fused_takes(ex, gin[l - 1], layers[l - 1], true));
+        BwdSums mine;
+        if (leave) mine.part = ex.ws.get<float>(bwd_sums_floats(ex, ly.cin));
+        auto wgrads = [&]() {            // as soon as every gradient operand exists
+            if (!side) {
+                conv_wgrad(ex, gq[l], saved.a[l], gin[l], ly, ly.dW);
+            } else if (l == 0) {
+                cudaStream_t main = ex.stream;
+                if (!ex.dry) {
+                    cudaEventRecord(ex.ctx->ev_fork, main);
+                    cudaStreamWaitEvent(ex.ctx->side_stream, ex.ctx->ev_fork, 0);
+                    ex.stream = ex.ctx->side_stream;
+                }
+                conv_wgrad_tc_batch(ex, L, gq.data(), aq.data(), gin.data(), lptr.data(), wg_scratch, nullptr);
+                ex.stream = main;
+            }
+        };
+        if (!folded) wgrads();
+        bool sums_done = true;
+        if (folded) {
+            if (!conv_dgrad_fused_behind(ex, da_behind, behind, sums, dt, gin[l], ly, da, &bb, leave ? &mine : nullptr) && !ex.failed) {
+                ex.failed = true; ex.ctx->err = "fn_backward: a fused data gradient was refused";      // (does not happen: asked above)
+            }
+        }
+        else sums_done = conv_dgrad(ex, gcur, gin[l], ly, da, &bb, leave ? &mine : nullptr);
+        if (folded) wgrads();
+        sums = mine;
+        da_behind = da; behind = bb;
         if (l == 0) {
             // add.p0 == nullptr: the gradient is stored without a partner (stored transitions)
-            bn_relu_bwd(ex, da, tl, P, bn, ly.dgamma, ly.dbeta, coef, sums_done, nullptr, false, add, dgin_out, b16 ? dgin_cast : nullptr);
-        } else {
-            void *dt = ex.ws.alloc(P * ly.cin * esz(ex));
-            bn_relu_bwd(ex, da, tl, P, bn, ly.dgamma, ly.dbeta, coef, sums_done, dt, b16, Pair{}, Pair{}, nullptr);
-            gcur = dt;
+            if (leave) bn_relu_bwd_sums(ex, da, tl, P, bn, ly.dgamma, ly.dbeta, sums, add, dgin_out, dgin_cast);
+            else bn_relu_bwd(ex, da, tl, P, bn, ly.dgamma, ly.dbeta, coef, sums_done, nullptr, false, add, dgin_out, b16 ? dgin_cast : nullptr);
+        } else if (!leave) {
+            void *dtn = ex.ws.alloc(P * ly.cin * esz(ex));
+            bn_relu_bwd(ex, da, tl, P, bn, ly.dgamma, ly.dbeta, coef, sums_done, dtn, b16, Pair{}, Pair{}, nullptr);
+            gcur = dtn;
         }
     }
     if (keep) return side;
@@ -219,6 +248,8 @@ void block_backward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const 
                     Moments *m1_out, bool overlap, const LateWgrad *late) {
     FnSaved svG, svF;
     const float q = ex.q;   // format of the coupling state; gradients are always float
+    // a block called by itself: the weight gradients of G run on beside F (joined with F's)
+    const bool late_g = late || (ex.mode == 0 && g.P() * c <= kLateWgradElems);
     size_t m0 = ex.ws.mark();
     if (!m1_out) m1_out = m1;
     // F may be recomputed beside G's gradient steps only if it leaves y1 and its statistics alone
@@ -233,8 +264,8 @@ void block_backward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const 
     Moments *mx1 = m1_out && !m1_out->mean ? nullptr : m1_out;
     if (!overlap) {
         // dz1 = dy1 + (dG/dz1)^T dy2 ; dW_G
-        on_side = fn_backward(ex, g, single((float *)y1, c, q), G, svG, single((float *)dy2, c), dy2_cast, single((float *)dy1, c), single(dx1, c), dz1_cast, late != nullptr);
-        if (!late) ex.ws.release(m);
+        on_side = fn_backward(ex, g, single((float *)y1, c, q), G, svG, single((float *)dy2, c), dy2_cast, single((float *)dy1, c), single(dx1, c), dz1_cast, late_g);
+        if (!late_g) ex.ws.release(m);
         // x1 = z1 - F(x2)
         fn_forward(ex, g, single(x2, c, q), mf, F, single((float *)y1, c, q), single(x1, c, q), -1, mx1, &svF, false);
     } else {
@@ -252,7 +283,7 @@ void block_backward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const 
         fn_forward(ex, g, single(x2, c, q), mf, F, single((float *)y1, c, q), single(x1, c, q), -1, mx1, &svF, false);
         if (ex.ws.high > ex.ws.off) ex.ws.off = ex.ws.high;
         if (!ex.dry) { cudaEventRecord(ex.ctx->ev_rjoin, ex.ctx->recon_stream); ex.stream = main; }
-        on_side = fn_backward(ex, g, single((float *)y1, c, q), G, svG, single((float *)dy2, c), dy2_cast, single((float *)dy1, c), single(dx1, c), dz1_cast, late != nullptr);
+        on_side = fn_backward(ex, g, single((float *)y1, c, q), G, svG, single((float *)dy2, c), dy2_cast, single((float *)dy1, c), single(dx1, c), dz1_cast, late_g);
         if (!ex.dry) cudaStreamWaitEvent(main, ex.ctx->ev_rjoin, 0);
     }
     // dx2 = dy2 + (dF/dx2)^T dz1 ; dW_F ; dx1 = dz1 (already in place)

@@ -434,6 +434,13 @@ bool stem_wgrad(Exec &ex, const float *img, const float *gout, Geom gi, const La
 // What a data-gradient epilogue needs to fuse the two sums of the BN+ReLU backward of the layer's
 // own BN: its input t, its coefficients, and where dgamma, dbeta and coef[3][C] go.
 struct BnBwdReq { Pair t; BnRef bn; float *dgamma, *dbeta, *coef; };
+// Sums of a BN backward left as per-CTA records of 2C floats (layout as for Moments): their consumer adds them, and stores dgamma and dbeta.
+// part: room for bwd_sums_floats() floats
+struct BwdSums { float *part = nullptr; int parts = 0; double inv_count = 0; };
+inline size_t bwd_sums_floats(const Exec &ex, int C) { return (size_t)ex.ctx->sm_count * 2 * C; }
+// whether bn_relu_bwd_sums takes the shape; out = add + dt from pending sums, optionally with a bf16 copy (all plain tensors)
+bool bn_relu_bwd_sums_takes(size_t P, int C);
+void bn_relu_bwd_sums(Exec &ex, const float *da, Pair t, size_t P, BnRef bn, float *dgamma, float *dbeta, const BwdSums &sums, Pair add, Pair out, bf16 *out_cast);
 // Reductions a convolution epilogue is asked to fuse.
 struct EpiReq {
     Moments *stats = nullptr;          // statistics of the stored result
@@ -477,6 +484,9 @@ bool fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
 // them; nothing they read (the unit's scratch, the bf16 gradient it was handed) may be overwritten before the main stream has waited
 // for it.  The units of a stage take two scratch regions in turn, and a unit waits for its predecessor's event (`before`) in front of
 // F's gradient steps.
+// kLateWgradElems: the largest half of a unit's pair for which they run on.  Both halves of a unit's scratch stay allocated for it; above, a
+// launch fills the GPU for so long that nothing is won by running two side by side.
+constexpr size_t kLateWgradElems = (size_t)1 << 23;
 struct LateWgrad { cudaEvent_t before = nullptr, done = nullptr; };      // (null: nothing to wait for, nothing to record)
 struct FnSaved {
     std::vector<void *> a;        // activated input of each conv

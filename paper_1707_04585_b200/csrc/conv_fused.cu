@@ -13,21 +13,28 @@
 // per row for every 8 channels: row l of plane j at j * plane + 16 l.  A tap's operand is the same planes from a row further
 // on, so every pixel is loaded, normalised and written once per range (plus the halo of W + 2 rows on either side), not
 // once per tap or per tile.
+// Input and partner rows arrive through shared memory, not through registers: the pixels of consecutive positions lie side by side in memory,
+// so the input of a range is a handful of bulk copies (pieces of about 12 KB), all of them under way as soon as the kernel before has ended,
+// and the partner rows of an epilogue warp's part of a tile are one TMA box of 32 rows x 64 bytes, in a ring of its own.
 // Roles (one CTA per SM):
-//   EW warps    epilogue (8, or 16 for more than 16 output columns), one accumulator row and 16 columns per thread, straight
+//   EW warps    epilogue (8, or 16 for 64 output columns), one accumulator row and 16 columns per thread, straight
 //               from tensor memory to global memory with 32-byte accesses: coupling on the float or fixed-point state, or plain
 //               store; the per-channel sums (batch statistics of the stored result, or the two sums of the BN+ReLU backward)
 //               stay in registers until the last tile.  Four warps make a group (128 rows x 16 columns); the groups split a
 //               tile's columns between them, and what is left over takes alternate tiles.  Before the first tile eight of
 //               them add the statistics records of the kernel before (BnRef::part).
-//   1 warp      weights (TMA, resident), tensor memory, MMA issue; two accumulators
-//   7 warps     build: 32-byte loads (8 channels of a pixel), four in flight per thread, scale*x + shift, ReLU, bf16 rounding,
-//               one 16-byte store to shared memory (and one to the activated tensor the weight gradient will read)
-// The same kernel computes data gradients: its input is then the bf16 upstream gradient, taken as it is, and the weights
-// are the mirrored, transposed pack.
-// Measured against the kernel with two CTAs of 256 threads that took turns at every step and built three shifted copies:
-// 16 channels at 32x32, batch 128: 19 -> 14 us per launch (nine MMAs of a tile issue in 500 clocks instead of 2200, a tile
-// every 1200 clocks and SM); basic block forward + backward there 307 -> 263 us, 16/32/56-channel step 2.13 -> 1.94 ms.
+//   1 warp      weights (TMA, resident), tensor memory, MMA issue; two or four accumulators
+//   1 warp      the input's pieces and the first partner rows
+//   6 warps     build: a row's 8 channels from shared memory, scale*x + shift, ReLU, bf16 rounding, one 16-byte store to the operand
+//               (and one to the activated tensor the weight gradient will read)
+// The same kernel computes data gradients: its input is then the bf16 upstream gradient, taken as it is, or (kInBwd) the gradient and
+// the BN input of the layer behind, whose BN + ReLU backward the build applies; the weights are the mirrored, transposed pack.
+// Measured, from the end of the wait for the kernel before to the last CTA's end, against the form whose seven build warps and epilogue warps
+// loaded from global memory into registers (four loads in flight per thread): data gradient of 16 channels at 32x32, batch 128, 12.3 -> 10.7 us,
+// of 32 at 16x16 12.3 -> 10.3, forward 12.0 -> 11.5; 32 -> 128 channels of the CIFAR-sized bottleneck network at 32x32 (1x1) 57.7 us by
+// events, 45 now.  Where a launch's time goes (16 channels, 32x32): first pieces there after 1.0 us, records added after 1.7, coefficients
+// after 2.2, first tile built after 3.4, last after 7.2, last accumulator drained after 8.5, sums 1.1 more.  The build is a chain of
+// latencies: 0.2 us per row and thread, 0.1 per tile signalled, 0.3 per piece.
 // Every mbarrier wait is bounded; on expiry the kernel records a status word and leaves.
 #include "common.cuh"
 #include "tc_ptx.cuh"
@@ -40,9 +47,13 @@ using namespace tc;
 namespace {
 
 constexpr int kFullBars = 16;             // tiles the build may run ahead of the MMAs
+constexpr int kRawSlots = 16;             // most pieces of the input in shared memory
+constexpr int kAuxSlots = 8;              // most tiles of an epilogue warp's partner rows in shared memory
+constexpr int kAccBufs = 4;               // most accumulators
 constexpr int NC = 16;                    // columns per epilogue thread
-constexpr int NBT = 224;                  // build threads: with the MMA warp a multiple of four warps, which keeps the most registers
-__host__ __device__ constexpr int fused_threads(int EW) { return EW * 32 + 32 + NBT; }
+constexpr int kAuxBytes = 32 * NC * 4;    // partner rows of an epilogue warp's part of a tile: 32 rows x 64 bytes
+constexpr int NBT = 192;                  // build threads
+__host__ __device__ constexpr int fused_threads(int EW) { return EW * 32 + 64 + NBT; }
 
 // What all layers of a launch share
 struct FusedGeom {
@@ -52,15 +63,22 @@ struct FusedGeom {
     int ksteps;            // MMA steps of 16 channels per tap
     int wpitch;            // channels per tap in the weight pack (cin rounded up to 16)
     int BN, groups;        // output columns per CTA; groups = BN / NC: warp groups that share a tile (1, 2 or 4)
+    int nacc, acc_shift;   // accumulators (2 or 4) and the logarithm of that
     int wtile_bytes;       // one tap of the weights: BN rows of KC bf16, rounded up to 1024
-    int N, H, W, pitch;    // pitch: positions per image row (W + 1; 1x1: unused)
-    int step_r, step_c;    // 3x3: the build's row stride in positions as whole image rows and columns
+    int N, H, W, P, pitch; // P: pixels; pitch: positions per image row (W + 1; 1x1: unused)
+    int nit, RS;           // the build: threads per row, rows in work at a time
+    int step_r, step_c;    // 3x3: RS positions as whole image rows and columns
     int halo;              // operand rows before a tile's first position (3x3: W + 2, else 0)
     int total;             // positions in all
     int chunk;             // positions per CTA
     int S, nseg;           // tiles per operand segment, segment buffers (1 or 2)
     int plane16, seg_bytes, op_bytes;     // plane stride in 16-byte units; bytes of a segment buffer, of the whole operand region
-    FastDiv dpitch, drows; // by positions per image row, by rows per image (H + 1)
+    int tab_bytes;         // 3x3: the build's table of pixels, one entry per row of a segment
+    int pps, pieces;       // pieces per full segment, in all
+    int piece, rowb;       // positions per piece of the input (a multiple of RS), bytes of a pixel of one input tensor
+    int raw_bytes, raw_slots;             // bytes of a piece's slot, slots
+    int aux_slots;         // tiles of partner rows that an epilogue warp holds
+    FastDiv dpitch, drows, dnit, dpps;    // by positions per image row, by rows per image (H + 1), by nit, by pps
 };
 // The epilogue of one layer (field names as epilogue_publish expects them)
 struct FusedEpi {
@@ -75,19 +93,25 @@ struct FusedEpi {
     BnRef bn;              // EPI_BNBWD
     float *dgamma, *dbeta, *coef;
 };
+// Input of a launch
+//   kInFloat, kInFixed   float / fixed-point tensor through BN + ReLU
+//   kInBf16              bf16 tensor as it is (the gradient entering a data gradient)
+//   kInBwd               gradient and BN input of the layer behind, through that layer's BN + ReLU backward
+enum { kInFloat = 0, kInBf16 = 1, kInFixed = 2, kInBwd = 3 };
 struct FusedLayer {
-    int in_mode;           // 0: float tensor through BN + ReLU; 2: fixed-point tensor likewise; 1: bf16 tensor as it is
-    int wide_in, wide_out; // 32-byte aligned rows: 32-byte accesses
+    int in_mode;
+    int wide_out;          // 32-byte aligned rows: 32-byte accesses
     int w_early;           // the weights were packed before the predecessor kernel: they may be loaded while it runs
     const void *in;
-    float in_q;            // in_mode 2: fixed-point step of the input
-    BnRef bn;              // in_mode 0, 2
-    bf16 *a_out;           // in_mode 0, 2, optional: the activated tensor [P, cin] (operand of the weight gradient)
-    const float *aux;      // coupling partner, or the BN input of a data gradient
+    const float *in_t;     // kInBwd: the BN input (in: the gradient w.r.t. the activated tensor)
+    float in_q;            // kInFixed: fixed-point step of the input
+    BnRef bn;              // all but kInBf16.  kInBwd: part holds the records of the backward sums
+    float *in_dgamma, *in_dbeta;          // kInBwd: where those sums go
+    bf16 *a_out;           // all but kInBf16, optional: the operand tensor [P, cin] (for the weight gradient)
     FusedEpi epi;
 };
 struct FusedArgs {
-    CUtensorMap map_w;
+    CUtensorMap map_w, map_x;     // weights; coupling partner, or the BN input of a data gradient
     FusedGeom g;
     FusedLayer ly;
     int *status;
@@ -95,19 +119,29 @@ struct FusedArgs {
 };
 
 struct __align__(16) FusedShared {
-    uint64_t full[kFullBars], seg_empty[2], acc_full[2], acc_empty[2], w_full;
+    uint64_t full[kFullBars], seg_empty[2], acc_full[kAccBufs], acc_empty[kAccBufs], w_full;
+    uint64_t raw_full[kRawSlots], raw_empty[kRawSlots], aux_full[16 * kAuxSlots];
+    int raw_px[kRawSlots];           // first pixel of a piece
     uint32_t tmem_base, failed;
-    __align__(16) float sc[64];      // BN scale and shift per input channel
-    __align__(16) float sf[64];
-    __align__(16) float4 coef[64];   // BN+ReLU backward: (scale, shift, mean, rstd) of each output column
-    __align__(16) float sums[16][2 * NC];     // per epilogue warp: NC sums, then NC second sums
-    __align__(16) double red[256 * 4], tot[32 * 4];    // statistics records
+    __align__(16) float cf[7][64];   // per input channel: BN scale and shift; kInBwd: also mean, rstd and the three coefficients of the backward
+    union {
+        struct { __align__(16) double red[256 * 4], tot[32 * 4]; };    // statistics records; done with when the coefficients are there
+        struct {
+            __align__(16) float4 coef[64];            // BN+ReLU backward: (scale, shift, mean, rstd) of each output column
+            __align__(16) float sums[16][2 * NC];     // per epilogue warp: NC sums, then NC second sums
+        };
+    };
 };
 
-// two floats -> ReLU -> bf16x2 (round to nearest even), one instruction
+// two floats -> (ReLU ->) bf16x2 (round to nearest even), one instruction
 __device__ __forceinline__ uint32_t relu_pack2(float lo, float hi) {
     uint32_t r;
     asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
 // a bounded wait of a whole warp: lane 0 polls
@@ -115,6 +149,11 @@ __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, int la
     bool ok = true;
     if (lane == 0) ok = mbar_wait(bar, parity);
     return __shfl_sync(0xffffffffu, ok, 0);
+}
+// bytes (a multiple of 16, both addresses too) from global to shared memory
+__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
 // pixel at position q, -1 for padding and for positions outside the batch
@@ -125,6 +164,16 @@ __device__ __forceinline__ int pixel_at(const FusedGeom &g, int q) {
     g.dpitch.divmod((uint32_t)q, row, c);
     g.drows.divmod(row, n, r);
     return (int)c < g.W && (int)r < g.H ? (int)(n * g.H + r) * g.W + (int)c : -1;
+}
+// pixels before position q
+__device__ __forceinline__ int pixels_before(const FusedGeom &g, int q) {
+    if (q <= 0) return 0;
+    if (q >= g.total) return g.P;
+    if (g.k == 1) return q;
+    uint32_t row, c, n, r;
+    g.dpitch.divmod((uint32_t)q, row, c);
+    g.drows.divmod(row, n, r);
+    return (int)(n * g.H + r) * g.W + ((int)r < g.H ? ((int)c < g.W ? (int)c : g.W) : 0);
 }
 // image, row and column of position q (3x3 layers; q may lie before the first image: image -1)
 __device__ __forceinline__ void place_at(const FusedGeom &g, int q, int &n, int &r, int &c) {
@@ -158,131 +207,198 @@ __device__ __forceinline__ void issue_tile(const FusedGeom &g, uint32_t acc, uin
     }
 }
 
-// The build of a CTA's operand rows.  A thread keeps its channel chunk ck and takes rows r0, r0 + RS, ... of each segment;
-// D loads are in flight while older rows are normalised and written.  IN: see FusedLayer::in_mode.
+// The input of a CTA arrives in pieces, through a ring.  The pixels of consecutive positions lie side by side in memory: a piece is one bulk
+// copy (kInBwd: two).  First and last pixel of piece n:
+__device__ __forceinline__ void piece_at(const FusedGeom &g, int pos0, int pos1, int n, int &a, int &b) {
+    uint32_t seg, j;
+    g.dpps.divmod((uint32_t)n, seg, j);
+    const int sb = pos0 + (int)seg * g.S * 128, own = pos1 - sb < g.S * 128 ? pos1 - sb : g.S * 128, rows = own + 2 * g.halo;
+    const int r0 = (int)j * g.piece, r1 = r0 + g.piece < rows ? r0 + g.piece : rows;
+    a = pixels_before(g, sb - g.halo + r0); b = pixels_before(g, sb - g.halo + r1);
+}
+__device__ __forceinline__ void load_piece(const FusedGeom &g, const FusedLayer &p, FusedShared *sh, uint8_t *raw, int slot, int a, int b) {      // one thread
+    const bool two = p.in_mode == kInBwd;
+    const uint32_t bytes = (uint32_t)((b - a) * g.rowb);
+    uint8_t *dst = raw + slot * g.raw_bytes;
+    sh->raw_px[slot] = a;
+    mbar_expect_tx(&sh->raw_full[slot], two ? 2 * bytes : bytes);
+    if (bytes) {
+        bulk_load(dst, reinterpret_cast<const uint8_t *>(p.in) + (size_t)a * g.rowb, bytes, &sh->raw_full[slot]);
+        if (two) bulk_load(dst + (g.raw_bytes >> 1), reinterpret_cast<const uint8_t *>(p.in_t) + (size_t)a * g.rowb, bytes, &sh->raw_full[slot]);
+    }
+}
+
+// The build of a CTA's operand rows.  A thread keeps its channels (eight; kInBwd: four) and takes rows r0, r0 + RS, ... of each
+// segment.  The pixels of its rows (-1: padding) stand in a table that it fills itself, for the first segment while the kernel
+// before this one still runs: six build warps are one or two per scheduler, so every instruction between a row's load and its
+// store costs its full latency.  One row per iteration: a loop that outgrows the scheduler's instruction buffer is slower than a
+// short one with nothing in flight.
+struct BuildPlace { int item, r0, low0; };
+__device__ __forceinline__ BuildPlace build_place(const FusedGeom &g, int bt) {
+    BuildPlace b;
+    uint32_t q, r;
+    g.dnit.divmod((uint32_t)bt, q, r);
+    b.item = (int)r; b.r0 = (int)q; b.low0 = (int)g.dnit.div((uint32_t)(bt & ~31));
+    return b;
+}
+__device__ __forceinline__ void build_table(const FusedGeom &g, int *tab, int r0, int first, int rows) {      // first: position of row 0
+    if (g.k == 1 || r0 >= g.RS) return;
+    int n, r, c;
+    place_at(g, first + r0, n, r, c);
+    for (int l = r0; l < rows; l += g.RS) {
+        tab[l] = c < g.W && (unsigned)r < (unsigned)g.H && (unsigned)n < (unsigned)g.N ? (n * g.H + r) * g.W + c : -1;
+        c += g.step_c; r += g.step_r;
+        if (c >= g.pitch) { c -= g.pitch; r++; }
+        while (r > g.H) { r -= g.H + 1; n++; }
+    }
+}
 template <int IN, int EW>
-__device__ __forceinline__ bool build_rows(const FusedGeom &g, const FusedLayer &p, FusedShared *sh, uint8_t *abuf, int pos0, int pos1, int bt, int lane) {
-    constexpr int NW = IN == 1 ? 4 : 8;                  // 32-bit words of an item
-    constexpr int D = 4;
-    const int nch = g.nch, RS = NBT / nch, ck = bt % nch, r0 = bt / nch, low0 = (bt & ~31) / nch;
-    const bool active = r0 < RS;
+__device__ __forceinline__ bool build_rows(const FusedGeom &g, const FusedLayer &p, FusedShared *sh, const uint8_t *raw, uint8_t *abuf, int *tab, int pos0, int pos1,
+                                           const BuildPlace bp, int lane) {
+    constexpr int V = IN == kInBwd ? 4 : 8;               // channels of a thread
+    const int RS = g.RS, it = bp.item;
     const int n_tiles = (pos1 - pos0 + 127) >> 7;
-    const bool wide = p.wide_in != 0;
-    float sc[8], sf[8];
+    float sc[V], sf[V], mu[V], rs[V], k0[V], k1[V], k2[V];       // (the last five: kInBwd)
     bool first = true;
+    int slot = 0; uint32_t round = 0;
     for (int t0 = 0, seg = 0; t0 < n_tiles; t0 += g.S, seg++) {
         const int T = n_tiles - t0 < g.S ? n_tiles - t0 : g.S;
         const int sb = pos0 + t0 * 128, own = pos1 - sb < T * 128 ? pos1 - sb : T * 128, rows = own + 2 * g.halo;
-        uint8_t *dst = abuf + (g.nseg == 2 ? (seg & 1) : 0) * g.seg_bytes + ck * g.plane16 * 16;
-        uint32_t raw[D][NW];
-        int pix[D];
-        // the place of the next row to load, stepped by RS positions without divisions
-        int lc = 0, lr = 0, ln = 0;
-        if (g.k == 3) place_at(g, sb - g.halo + r0, ln, lr, lc);
-        auto load = [&](int l, uint32_t (&v)[NW], int &px) {
-            px = -1;
-            if (g.k == 1) { if (active && l < rows && sb + l < g.total) px = sb + l; }
-            else {
-                if (active && l < rows && lc < g.W && (unsigned)lr < (unsigned)g.H && (unsigned)ln < (unsigned)g.N) px = (ln * g.H + lr) * g.W + lc;
-                lc += g.step_c; lr += g.step_r;
-                if (lc >= g.pitch) { lc -= g.pitch; lr++; }
-                while (lr > g.H) { lr -= g.H + 1; ln++; }
-            }
-            if (px >= 0) {
-                const size_t off = ((size_t)px * nch + ck) * (IN == 1 ? 16 : 32);
-                if constexpr (IN == 1) {
-                    const uint4 u = *reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(p.in) + off);
-                    v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
-                } else ld8(reinterpret_cast<const uint8_t *>(p.in) + off, v, wide);
-            }
-        };
-        int ll = r0, l = r0, low = low0, j = 0;
-#pragma unroll
-        for (int u = 0; u < D; u++) { load(ll, raw[u], pix[u]); ll += RS; }
-        if (first) {
-            first = false;
-            if (IN != 1) {
-                named_barrier(3, EW * 32 + NBT);         // scale and shift are there
-#pragma unroll
-                for (int i = 0; i < 8; i++) { sc[i] = sh->sc[ck * 8 + i] * (IN == 2 ? p.in_q : 1.f); sf[i] = sh->sf[ck * 8 + i]; }
-            }
-        }
+        const int my_rows = bp.r0 < RS ? rows : 0;
+        uint8_t *dst = abuf + (g.nseg == 2 ? (seg & 1) : 0) * g.seg_bytes + (IN == kInBwd ? (it >> 1) * g.plane16 * 16 + (it & 1) * 8 : it * g.plane16 * 16);
+        if (seg > 0) build_table(g, tab, bp.r0, sb - g.halo, rows);
         if (seg >= g.nseg && !warp_wait(&sh->seg_empty[g.nseg == 2 ? (seg & 1) : 0], (uint32_t)((g.nseg == 2 ? seg >> 1 : seg) - 1) & 1u, lane)) return false;
-        auto signal = [&](int tile) {
+        int l = bp.r0, low = bp.low0, j = 0, ready = 128 + 2 * g.halo;          // ready: rows that the tile to be signalled next needs
+        auto signal = [&]() {
             fence_proxy_async();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&sh->full[(t0 + tile) & (kFullBars - 1)]);
+            if (lane == 0) mbar_arrive(&sh->full[(t0 + j) & (kFullBars - 1)]);
+            j++; ready += 128;
         };
-        while (low < rows) {
+        for (int pr = 0; pr < rows; pr += g.piece) {
+            const bool here = mbar_wait(&sh->raw_full[slot], round & 1u);
+            if (first) {                                     // (also when the wait ran out: the epilogue warps stand at this barrier)
+                first = false;
+                if (IN != kInBf16) {
+                    named_barrier(3, EW * 32 + NBT + 32);         // the coefficients are there
 #pragma unroll
-            for (int u = 0; u < D; u++) {
-                if (low >= rows) break;
-                while (j < T && low >= (j + 1) * 128 + 2 * g.halo) signal(j++);
-                if (active && l < rows) {
-                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                    if (pix[u] >= 0) {
-                        if constexpr (IN == 1) v = make_uint4(raw[u][0], raw[u][1], raw[u][2], raw[u][3]);
-                        else {
-                            float x[8];
-#pragma unroll
-                            for (int i = 0; i < 8; i++) x[i] = fmaf(sc[i], IN == 2 ? __int2float_rn((int)raw[u][i]) : __uint_as_float(raw[u][i]), sf[i]);
-                            v = make_uint4(relu_pack2(x[0], x[1]), relu_pack2(x[2], x[3]), relu_pack2(x[4], x[5]), relu_pack2(x[6], x[7]));
-                            if (p.a_out && l >= g.halo && l < g.halo + own)
-                                *reinterpret_cast<uint4 *>(p.a_out + ((size_t)pix[u] * nch + ck) * 8) = v;
-                        }
+                    for (int i = 0; i < V; i++) {
+                        const int c = it * V + i;
+                        sc[i] = sh->cf[0][c] * (IN == kInFixed ? p.in_q : 1.f); sf[i] = sh->cf[1][c];
+                        if (IN == kInBwd) { mu[i] = sh->cf[2][c]; rs[i] = sh->cf[3][c]; k0[i] = sh->cf[4][c]; k1[i] = sh->cf[5][c]; k2[i] = sh->cf[6][c]; }
                     }
-                    *reinterpret_cast<uint4 *>(dst + l * 16) = v;
+                }
+            }
+            if (!__all_sync(0xffffffffu, here)) return false;
+            const int pxs = sh->raw_px[slot];
+            const uint8_t *src = raw + slot * g.raw_bytes + it * (IN == kInFloat || IN == kInFixed ? 32 : 16);
+#pragma unroll 1
+            for (int i = 0; i < g.piece && low < rows; i += RS) {
+                if (l < my_rows) {
+                    int px;
+                    if (g.k == 1) px = sb + l < g.total ? sb + l : -1;
+                    else px = tab[l];
+                    const uint8_t *s = src + (px - pxs) * g.rowb;
+                    const bool keep = p.a_out && (unsigned)(l - g.halo) < (unsigned)own;
+                    if constexpr (IN == kInBwd) {
+                        uint2 v = make_uint2(0u, 0u);
+                        if (px >= 0) {
+                            const float4 d4 = *reinterpret_cast<const float4 *>(s), t4 = *reinterpret_cast<const float4 *>(s + (g.raw_bytes >> 1));
+                            const float d[4] = {d4.x, d4.y, d4.z, d4.w}, t[4] = {t4.x, t4.y, t4.z, t4.w};
+                            float o[4];
+                            // (as bn_relu_bwd_apply_kernel has it)
+#pragma unroll
+                            for (int c = 0; c < 4; c++) o[c] = k0[c] * (fmaf(sc[c], t[c], sf[c]) > 0.f ? d[c] : 0.f) - k1[c] - k2[c] * ((t[c] - mu[c]) * rs[c]);
+                            v = make_uint2(pack2(o[0], o[1]), pack2(o[2], o[3]));
+                            if (keep) *reinterpret_cast<uint2 *>(p.a_out + (size_t)px * g.cin + it * 4) = v;
+                        }
+                        *reinterpret_cast<uint2 *>(dst + l * 16) = v;
+                    } else {
+                        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                        if (px >= 0) {
+                            v = *reinterpret_cast<const uint4 *>(s);
+                            if constexpr (IN != kInBf16) {
+                                const uint4 w = *reinterpret_cast<const uint4 *>(s + 16);
+                                const uint32_t r[8] = {v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w};
+                                float x[8];
+#pragma unroll
+                                for (int c = 0; c < 8; c++) x[c] = fmaf(sc[c], IN == kInFixed ? __int2float_rn((int)r[c]) : __uint_as_float(r[c]), sf[c]);
+                                v = make_uint4(relu_pack2(x[0], x[1]), relu_pack2(x[2], x[3]), relu_pack2(x[4], x[5]), relu_pack2(x[6], x[7]));
+                                if (keep) *reinterpret_cast<uint4 *>(p.a_out + (size_t)px * g.cin + it * 8) = v;
+                            }
+                        }
+                        *reinterpret_cast<uint4 *>(dst + l * 16) = v;
+                    }
                 }
                 l += RS; low += RS;
-                load(ll, raw[u], pix[u]);
-                ll += RS;
+                while (j < T && low >= ready) signal();
             }
+            if (g.pieces > g.raw_slots) {                    // (else nothing waits for the slot)
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sh->raw_empty[slot]);
+            }
+            if (++slot == g.raw_slots) { slot = 0; round++; }
         }
-        while (j < T) signal(j++);
+        while (j < T) signal();
     }
     return true;
+}
+
+// An epilogue warp's own ring of partner rows (its 32 rows and 16 columns of a tile): the copy of its k-th tile
+struct AuxRing { uint8_t *buf; uint64_t *bar; int col, on; };
+__device__ __forceinline__ AuxRing aux_ring(const FusedArgs &A, FusedShared *sh, uint8_t *auxb, int warp) {
+    const FusedGeom &g = A.g;
+    AuxRing x;
+    x.buf = auxb + warp * g.aux_slots * kAuxBytes; x.bar = sh->aux_full + warp * kAuxSlots;
+    x.col = (int)blockIdx.y * g.BN + ((warp >> 2) & (g.groups - 1)) * NC;
+    x.on = A.ly.epi.mode != EPI_PLAIN && x.col < A.ly.epi.n_cols;
+    return x;
+}
+__device__ __forceinline__ void aux_load(const FusedArgs &A, const AuxRing &x, int slot, int q) {       // one thread; q: the warp's first position
+    mbar_expect_tx(&x.bar[slot], kAuxBytes);
+    tma_load_2d(x.buf + slot * kAuxBytes, &A.map_x, &x.bar[slot], x.col, pixels_before(A.g, q));
 }
 
 // Epilogue of one warp's rows.  EK: 0 plain, 1 float coupling, 2 fixed-point coupling, 3 / 4 BN+ReLU backward with a float /
 // fixed-point BN input.
 template <int EW, int EK>
-__device__ __forceinline__ bool epilogue_loop(const FusedGeom &g, const FusedLayer &p, FusedShared *sh, int pos0, int pos1, int warp, int lane, uint32_t tmem_d,
+__device__ __forceinline__ bool epilogue_loop(const FusedArgs &A, FusedShared *sh, const AuxRing &ax, int pos0, int pos1, int warp, int lane, uint32_t tmem_d,
                                               float (&s)[NC], float (&ss)[NC]) {
+    const FusedGeom &g = A.g;
+    const FusedLayer &p = A.ly;
     const FusedEpi &e = p.epi;
-    const int grp = warp >> 2, row = (warp & 3) * 32 + lane;
+    const int grp = warp >> 2, wrow = (warp & 3) * 32;
     const int sets = EW / 4 / g.groups, set = grp / g.groups;                     // tiles set, set + sets, ...
     const bool wide = p.wide_out != 0;
-    const int lc = (grp % g.groups) * NC, col = (int)blockIdx.y * g.BN + lc;      // this thread's first column: in the CTA, in the tensor
+    const int lc = (grp & (g.groups - 1)) * NC, col = ax.col;                           // this thread's first column: in the CTA, in the tensor
     const float q = e.q, out_s = (EK <= 2 && q != 0.f) ? 1.f / q : 0.f, sgn = e.sign < 0 ? -1.f : 1.f;
     const int isgn = e.sign < 0 ? -1 : 1;
     const float4 *coef = sh->coef + lc;
     const int n_tiles = (pos1 - pos0 + 127) >> 7;
-    const uint32_t tm = tmem_d + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)lc;
+    const uint32_t tm = tmem_d + ((uint32_t)wrow << 16) + (uint32_t)lc;
+    int slot = 0; uint32_t round = 0;
     for (int ti = set; ti < n_tiles; ti += sets) {
-        const int q0 = pos0 + ti * 128 + row, px = q0 < pos1 ? pixel_at(g, q0) : -1;
+        const int qw = pos0 + ti * 128 + wrow, q0 = qw + lane, px = q0 < pos1 ? pixel_at(g, q0) : -1;
         const size_t off = (size_t)(px < 0 ? 0 : px) * e.n_cols + col;
-        // what the row needs besides the accumulator is on its way before the accumulator is complete
-        uint32_t x[NC];
-        if (EK > 0) {
-#pragma unroll
-            for (int c = 0; c < NC; c += 8) {
-                uint32_t v[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-                if (px >= 0) {
-                    if (col + c + 8 <= e.n_cols) ld8(p.aux + off + c, v, wide);
-                    else if (col + c < e.n_cols) { const uint4 a = *reinterpret_cast<const uint4 *>(p.aux + off + c); v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; }
-                }
-#pragma unroll
-                for (int i = 0; i < 8; i++) x[c + i] = v[i];
-            }
-        }
         const uint32_t keep = px >= 0 ? 0xffffffffu : 0u;      // rows that hold no pixel add nothing (a select, not a branch per column)
-        const int buf = ti & 1;
-        if (!warp_wait(&sh->acc_full[buf], (uint32_t)(ti >> 1) & 1u, lane)) return false;
+        const int xr = px < 0 ? 0 : px - pixels_before(g, qw);
+        const uint8_t *xrow = ax.buf + slot * kAuxBytes + xr * 64;
+        const int swz = (xr >> 1) & 3, buf = ti & (g.nacc - 1);
+        bool ok = true;
+        if (lane == 0) {
+            if (EK > 0 && ax.on) ok = mbar_wait(&ax.bar[slot], round & 1u);
+            ok = ok && mbar_wait(&sh->acc_full[buf], (uint32_t)(ti >> g.acc_shift) & 1u);
+        }
+        if (!__shfl_sync(0xffffffffu, ok, 0)) return false;
         tc_fence_after();
 #pragma unroll
         for (int c = 0; c < NC; c += 8) {
             float v[8];
-            uint32_t o[8];
+            uint32_t o[8], x[8];
+            if (EK > 0) {
+                const uint4 a = *reinterpret_cast<const uint4 *>(xrow + (((c >> 2) ^ swz) << 4)), b = *reinterpret_cast<const uint4 *>(xrow + ((((c >> 2) + 1) ^ swz) << 4));
+                x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+            }
             tmem_ld8(tm + (uint32_t)(buf * g.BN + c), v);
 #pragma unroll
             for (int i = 0; i < 8; i++) {
@@ -291,10 +407,10 @@ __device__ __forceinline__ bool epilogue_loop(const FusedGeom &g, const FusedLay
                     if (q != 0.f) { const int iv = __float2int_rn(v[i] * out_s); o[i] = (uint32_t)iv; st = __int2float_rn(iv) * q; }
                     else { o[i] = __float_as_uint(v[i]); st = v[i]; }
                 } else if (EK == 1) {
-                    st = fmaf(sgn, v[i], __uint_as_float(x[c + i]));
+                    st = fmaf(sgn, v[i], __uint_as_float(x[i]));
                     o[i] = __float_as_uint(st);
                 } else if (EK == 2) {
-                    const int iv = (int)x[c + i] + isgn * __float2int_rn(v[i] * out_s);
+                    const int iv = (int)x[i] + isgn * __float2int_rn(v[i] * out_s);
                     o[i] = (uint32_t)iv; st = __int2float_rn(iv) * q;
                 } else o[i] = __float_as_uint(v[i]);
                 if (EK <= 2) {
@@ -302,7 +418,8 @@ __device__ __forceinline__ bool epilogue_loop(const FusedGeom &g, const FusedLay
                     s[c + i] += st;
                     ss[c + i] = fmaf(st, st, ss[c + i]);
                 } else {
-                    const float t = EK == 4 ? __int2float_rn((int)x[c + i]) * q : __uint_as_float(x[c + i]);
+                    const uint32_t xi = x[i] & keep;
+                    const float t = EK == 4 ? __int2float_rn((int)xi) * q : __uint_as_float(xi);
                     const float4 k = coef[c + i];           // scale, shift, mean, rstd
                     const float d = fmaf(k.x, t, k.y) > 0.f ? __uint_as_float(__float_as_uint(v[i]) & keep) : 0.f;
                     s[c + i] += d;
@@ -317,7 +434,11 @@ __device__ __forceinline__ bool epilogue_loop(const FusedGeom &g, const FusedLay
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sh->acc_empty[buf]);
+        if (lane == 0) {
+            mbar_arrive(&sh->acc_empty[buf]);
+            if (EK > 0 && ax.on && ti + g.aux_slots * sets < n_tiles) aux_load(A, ax, slot, qw + g.aux_slots * sets * 128);
+        }
+        if (++slot == g.aux_slots) { slot = 0; round++; }
     }
     return true;
 }
@@ -336,24 +457,27 @@ __device__ __forceinline__ void column_sums(float (&a)[NC], int lane) {
     a[0] += __shfl_xor_sync(0xffffffffu, a[0], 16);
 }
 
-// Registers: 123 with eight epilogue warps; with sixteen the block of 768 threads leaves 80, and the epilogue, which holds 32 running sums,
-// 16 partner words and 8 values, spills 304 bytes.
+// Registers: with eight epilogue warps 96 for 512 threads (the bound of 640 asks for that), which leaves an SM room for a CTA of
+// the weight gradients (72 for 192 threads) that run on another stream.
 template <int EW>
-__global__ void __launch_bounds__(fused_threads(EW), 1) conv_fused_kernel(const __grid_constant__ FusedArgs A) {
+__global__ void __launch_bounds__(EW == 8 ? 640 : fused_threads(EW), 1) conv_fused_kernel(const __grid_constant__ FusedArgs A) {
     extern __shared__ uint8_t smem_raw[];
     const FusedGeom &g = A.g;
     const FusedLayer &p = A.ly;
     const FusedEpi &e = p.epi;
     uint8_t *wres = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int taps = g.k * g.k;
-    uint8_t *abuf = wres + taps * g.wtile_bytes;
-    FusedShared *sh = (FusedShared *)(abuf + g.op_bytes);
+    uint8_t *auxb = wres + taps * g.wtile_bytes;                            // partner rings (512-byte aligned for their swizzle)
+    uint8_t *abuf = auxb + EW * g.aux_slots * kAuxBytes;
+    uint8_t *raw = abuf + g.op_bytes;
+    int *tab = (int *)(raw + g.raw_slots * g.raw_bytes);
+    FusedShared *sh = (FusedShared *)((uint8_t *)tab + g.tab_bytes);
 
-    constexpr int kMmaWarp = EW, kBuildWarp0 = EW + 1;
+    constexpr int kMmaWarp = EW, kLoadWarp = EW + 1, kBuildWarp0 = EW + 2;
     const int warp = warp_index(), lane = threadIdx.x & 31;
-    const bool direct = p.in_mode == 1;
+    const bool direct = p.in_mode == kInBf16;
     uint32_t tmem_cols = 32;
-    while ((int)tmem_cols < 2 * g.BN) tmem_cols <<= 1;
+    while ((int)tmem_cols < g.nacc * g.BN) tmem_cols <<= 1;
     const int col0 = blockIdx.y * g.BN;
     const int pos0 = (int)blockIdx.x * g.chunk, pos1 = pos0 + g.chunk < g.total ? pos0 + g.chunk : g.total;
     auto load_weights = [&]() {
@@ -361,23 +485,47 @@ __global__ void __launch_bounds__(fused_threads(EW), 1) conv_fused_kernel(const 
         for (int tap = 0; tap < taps; tap++) tma_load_2d(wres + tap * g.wtile_bytes, &A.map_w, &sh->w_full, tap * g.wpitch, col0);
     };
 
+    BuildPlace bp{};
+    AuxRing ax{};
+    int piece_a = 0, piece_b = 0;        // loader: lane n's piece of the first ringful
     if (warp == kMmaWarp) {
         if (elect_one()) {
             tma_prefetch_desc(&A.map_w);
             for (int b = 0; b < kFullBars; b++) mbar_init(&sh->full[b], NBT / 32);
-            for (int b = 0; b < 2; b++) { mbar_init(&sh->seg_empty[b], 1); mbar_init(&sh->acc_full[b], 1); mbar_init(&sh->acc_empty[b], 4 * g.groups); }
+            for (int b = 0; b < 2; b++) mbar_init(&sh->seg_empty[b], 1);
+            for (int b = 0; b < kAccBufs; b++) { mbar_init(&sh->acc_full[b], 1); mbar_init(&sh->acc_empty[b], 4 * g.groups); }
             mbar_init(&sh->w_full, 1);
             sh->failed = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             if (p.w_early) load_weights();
         }
         tmem_alloc(&sh->tmem_base, tmem_cols);
-    } else if (warp >= kBuildWarp0 && (g.nch & 1)) {
-        // an odd number of 8-channel planes: the one that fills up the last MMA step holds zeros for good
-        for (int b = 0; b < g.nseg; b++)
-            for (int l = (int)threadIdx.x - kBuildWarp0 * 32; l < g.plane16; l += NBT)
-                *reinterpret_cast<uint4 *>(abuf + b * g.seg_bytes + (g.nch * g.plane16 + l) * 16) = make_uint4(0u, 0u, 0u, 0u);
-        fence_proxy_async();
+    } else if (warp == kLoadWarp) {
+        if (lane < g.raw_slots) {
+            mbar_init(&sh->raw_full[lane], 1); mbar_init(&sh->raw_empty[lane], NBT / 32);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            piece_at(g, pos0, pos1, lane, piece_a, piece_b);
+        }
+    } else if (warp >= kBuildWarp0) {
+        bp = build_place(g, (int)threadIdx.x - kBuildWarp0 * 32);
+        {
+            const int own = pos1 - pos0 < g.S * 128 ? pos1 - pos0 : g.S * 128;
+            build_table(g, tab, bp.r0, pos0 - g.halo, own + 2 * g.halo);
+        }
+        if (g.nch & 1) {
+            // an odd number of 8-channel planes: the one that fills up the last MMA step holds zeros for good
+            for (int b = 0; b < g.nseg; b++)
+                for (int l = (int)threadIdx.x - kBuildWarp0 * 32; l < g.plane16; l += NBT)
+                    *reinterpret_cast<uint4 *>(abuf + b * g.seg_bytes + (g.nch * g.plane16 + l) * 16) = make_uint4(0u, 0u, 0u, 0u);
+            fence_proxy_async();
+        }
+    } else {
+        ax = aux_ring(A, sh, auxb, warp);
+        if (lane == 0 && ax.on) {
+            tma_prefetch_desc(&A.map_x);
+            for (int b = 0; b < g.aux_slots; b++) mbar_init(&ax.bar[b], 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -396,9 +544,9 @@ __global__ void __launch_bounds__(fused_threads(EW), 1) conv_fused_kernel(const 
             ok = mbar_wait(&sh->w_full, 0);
             int j = 0, sbuf = 0;                // tile within its segment, segment buffer
             for (int ti = 0; ti < n_tiles && ok; ti++) {
-                const int buf = ti & 1;
+                const int buf = ti & (g.nacc - 1);
                 if (!mbar_wait(&sh->full[ti & (kFullBars - 1)], (uint32_t)(ti / kFullBars) & 1u)) { ok = false; break; }
-                if (ti > 1 && !mbar_wait(&sh->acc_empty[buf], (uint32_t)((ti >> 1) - 1) & 1u)) { ok = false; break; }
+                if (ti >= g.nacc && !mbar_wait(&sh->acc_empty[buf], (uint32_t)((ti >> g.acc_shift) - 1) & 1u)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t acc = tmem_d + (uint32_t)(buf * g.BN);
                 const uint64_t a = a0 + (uint32_t)((sbuf * g.seg_bytes >> 4) + j * 128);
@@ -411,27 +559,66 @@ __global__ void __launch_bounds__(fused_threads(EW), 1) conv_fused_kernel(const 
             }
         }
         __syncwarp();
+    } else if (warp == kLoadWarp) {
+        // the first ringful, a lane per piece; the partner rows of every epilogue warp's first tiles; then piece after piece
+        const int n_tiles = (pos1 - pos0 + 127) >> 7, full = (pos1 - pos0) / (g.S * 128), rest = pos1 - pos0 - full * g.S * 128;
+        const int n = full * g.pps + (rest > 0 ? (rest + 2 * g.halo + g.piece - 1) / g.piece : 0);
+        if (lane < g.raw_slots && lane < n) load_piece(g, p, sh, raw, lane, piece_a, piece_b);
+        // (the partner rows wait until the records of the statistics are in: those, and the first rows, are needed first)
+        if (!direct) named_barrier(3, EW * 32 + NBT + 32);
+        if (e.mode != EPI_PLAIN) {
+            const int sets = EW / 4 / g.groups;
+            for (int i = lane; i < EW * g.aux_slots; i += 32) {
+                const int slot = i / EW, w = i & (EW - 1), ti = (w >> 2) / g.groups + slot * sets;
+                const AuxRing x = aux_ring(A, sh, auxb, w);
+                if (x.on && ti < n_tiles) aux_load(A, x, slot, pos0 + ti * 128 + (w & 3) * 32);
+            }
+        }
+        __syncwarp();
+        if (elect_one()) {
+            int slot = 0, round = 0;
+            for (int i = g.raw_slots; i < n && ok; i++) {
+                int a, b;
+                piece_at(g, pos0, pos1, i, a, b);
+                ok = mbar_wait(&sh->raw_empty[slot], (uint32_t)round & 1u);
+                if (ok) load_piece(g, p, sh, raw, slot, a, b);
+                if (++slot == g.raw_slots) { slot = 0; round++; }
+            }
+        }
+        __syncwarp();
     } else if (warp < EW) {
         const int etid = (int)threadIdx.x;
         if (!direct && warp < 8) {
+            // the statistics of the input (kInBwd: the sums of the BN backward) may still be per-CTA records of the kernel before: every
+            // CTA adds them, the same way, while its first rows are on the way, and the first CTA stores the result for later readers
+            const int c = etid;
+            const bool mine = c < g.cin;
+            float gam = 0.f, bet = 0.f, mean = 0.f, rstd = 0.f;
+            if (mine) {
+                gam = p.bn.gamma[c]; bet = p.bn.beta[c];
+                if (!p.bn.part || p.in_mode == kInBwd) { mean = p.bn.mean[c]; rstd = p.bn.rstd[c]; }
+            }
             if (p.bn.part) reduce_records<256>(p.bn.part, p.bn.parts, g.cin, 0, g.cin >> 1, sh->red, sh->tot, etid);
-            if (etid < 64) {
-                // the statistics of the input may still be per-CTA records of the kernel before: added above (every CTA the
-                // same way, while its first rows are on the way), and the first CTA stores mean and rstd for later readers
-                const int c = etid;
-                float sc = 0.f, sf = 0.f;
-                if (c < g.cin) {
-                    float mean, rstd;
-                    if (p.bn.part) {
-                        moments_of(sh->tot[(2 * (c >> 2)) * 4 + (c & 3)], sh->tot[(2 * (c >> 2) + 1) * 4 + (c & 3)], p.bn.inv_count, p.bn.eps, mean, rstd);
-                        if (blockIdx.x == 0 && blockIdx.y == 0) { const_cast<float *>(p.bn.mean)[c] = mean; const_cast<float *>(p.bn.rstd)[c] = rstd; }
-                    } else { mean = p.bn.mean[c]; rstd = p.bn.rstd[c]; }
-                    bn_sc_sh(p.bn.gamma[c], p.bn.beta[c], mean, rstd, sc, sf);
+            if (c < 64) {
+                float sc = 0.f, sf = 0.f, k0 = 0.f, k1 = 0.f, k2 = 0.f;
+                if (mine) {
+                    const double sum = p.bn.part ? sh->tot[(2 * (c >> 2)) * 4 + (c & 3)] : 0., sum2 = p.bn.part ? sh->tot[(2 * (c >> 2) + 1) * 4 + (c & 3)] : 0.;
+                    const bool store = blockIdx.x == 0 && blockIdx.y == 0;
+                    if (p.in_mode == kInBwd) {
+                        const double gr = (double)gam * (double)rstd;
+                        k0 = (float)gr; k1 = (float)(gr * sum * p.bn.inv_count); k2 = (float)(gr * sum2 * p.bn.inv_count);
+                        if (store) { p.in_dbeta[c] = (float)sum; p.in_dgamma[c] = (float)sum2; }
+                    } else if (p.bn.part) {
+                        moments_of(sum, sum2, p.bn.inv_count, p.bn.eps, mean, rstd);
+                        if (store) { const_cast<float *>(p.bn.mean)[c] = mean; const_cast<float *>(p.bn.rstd)[c] = rstd; }
+                    }
+                    bn_sc_sh(gam, bet, mean, rstd, sc, sf);
                 }
-                sh->sc[c] = sc; sh->sf[c] = sf;
+                sh->cf[0][c] = sc; sh->cf[1][c] = sf;
+                if (p.in_mode == kInBwd) { sh->cf[2][c] = mean; sh->cf[3][c] = rstd; sh->cf[4][c] = k0; sh->cf[5][c] = k1; sh->cf[6][c] = k2; }
             }
         }
-        if (!direct) named_barrier(3, EW * 32 + NBT);
+        if (!direct) named_barrier(3, EW * 32 + NBT + 32);
         float s[NC], ss[NC];
 #pragma unroll
         for (int i = 0; i < NC; i++) s[i] = ss[i] = 0.f;
@@ -443,12 +630,12 @@ __global__ void __launch_bounds__(fused_threads(EW), 1) conv_fused_kernel(const 
                 sh->coef[etid] = k;
             }
             named_barrier(2, EW * 32);
-            ok = e.q == 0.f ? epilogue_loop<EW, 3>(g, p, sh, pos0, pos1, warp, lane, tmem_d, s, ss)
-                            : epilogue_loop<EW, 4>(g, p, sh, pos0, pos1, warp, lane, tmem_d, s, ss);
+            ok = e.q == 0.f ? epilogue_loop<EW, 3>(A, sh, ax, pos0, pos1, warp, lane, tmem_d, s, ss)
+                            : epilogue_loop<EW, 4>(A, sh, ax, pos0, pos1, warp, lane, tmem_d, s, ss);
         } else if (e.mode == EPI_COUPLE) {
-            ok = e.q == 0.f ? epilogue_loop<EW, 1>(g, p, sh, pos0, pos1, warp, lane, tmem_d, s, ss)
-                            : epilogue_loop<EW, 2>(g, p, sh, pos0, pos1, warp, lane, tmem_d, s, ss);
-        } else ok = epilogue_loop<EW, 0>(g, p, sh, pos0, pos1, warp, lane, tmem_d, s, ss);
+            ok = e.q == 0.f ? epilogue_loop<EW, 1>(A, sh, ax, pos0, pos1, warp, lane, tmem_d, s, ss)
+                            : epilogue_loop<EW, 2>(A, sh, ax, pos0, pos1, warp, lane, tmem_d, s, ss);
+        } else ok = epilogue_loop<EW, 0>(A, sh, ax, pos0, pos1, warp, lane, tmem_d, s, ss);
         if (e.part) {
             // per-CTA record: rows of a warp by shuffles, then the warps that share a column in order
             column_sums(s, lane); column_sums(ss, lane);
@@ -457,8 +644,9 @@ __global__ void __launch_bounds__(fused_threads(EW), 1) conv_fused_kernel(const 
             if (ok && etid < g.BN && col0 + etid < e.n_cols) {
                 const int lc = etid % NC;
                 float a = 0.f, b = 0.f;
-                for (int gr = etid / NC; gr < EW / 4; gr += g.groups)
-                    for (int w = 4 * gr; w < 4 * gr + 4; w++) { a += sh->sums[w][lc]; b += sh->sums[w][NC + lc]; }
+#pragma unroll
+                for (int w = 0; w < EW; w++)
+                    if (((w >> 2) & (g.groups - 1)) == etid / NC) { a += sh->sums[w][lc]; b += sh->sums[w][NC + lc]; }
                 const int c = col0 + etid;
                 float *mine = e.part + (size_t)blockIdx.x * 2 * e.n_cols + (c >> 2) * 8 + (c & 3);
                 mine[0] = a; mine[4] = b;
@@ -473,10 +661,10 @@ __global__ void __launch_bounds__(fused_threads(EW), 1) conv_fused_kernel(const 
             }
         }
     } else {
-        const int bt = (int)threadIdx.x - kBuildWarp0 * 32;
-        if (direct) ok = build_rows<1, EW>(g, p, sh, abuf, pos0, pos1, bt, lane);
-        else if (p.in_mode == 2) ok = build_rows<2, EW>(g, p, sh, abuf, pos0, pos1, bt, lane);
-        else ok = build_rows<0, EW>(g, p, sh, abuf, pos0, pos1, bt, lane);
+        if (direct) ok = build_rows<kInBf16, EW>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane);
+        else if (p.in_mode == kInFixed) ok = build_rows<kInFixed, EW>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane);
+        else if (p.in_mode == kInFloat) ok = build_rows<kInFloat, EW>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane);
+        else ok = build_rows<kInBwd, EW>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane);
     }
     if (!ok) atomicExch(&sh->failed, 1u);
     tc_fence_before();
@@ -491,21 +679,29 @@ __global__ void __launch_bounds__(fused_threads(EW), 1) conv_fused_kernel(const 
 
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
-struct FusedShape { int n_tiles, ctas, smem; FusedGeom g; };
+struct FusedShape { int n_tiles, ctas, smem, EW; FusedGeom g; };
 
-bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count, FusedShape &s) {
+// aux: the epilogue reads a partner tensor.  The CTAs' ranges depend on geo, cin, cout, k and sm_count alone wherever the memory suffices.
+bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count, int in_mode, bool aux, FusedShape &s) {
     if ((k != 1 && k != 3) || cin % 8 || cout % 4 || cin < 8 || cin > 64) return false;
     FusedGeom &g = s.g;
     memset(&g, 0, sizeof g);
     g.k = k; g.cin = cin; g.nch = cin / 8; g.wpitch = round_up(cin, 16); g.ksteps = g.wpitch / 16;
     g.KC = cin <= 16 ? 16 : (cin <= 32 ? 32 : 64);
-    g.N = geo.N; g.H = geo.H; g.W = geo.W; g.pitch = geo.W + 1;
-    g.dpitch = fast_div(geo.W + 1); g.drows = fast_div(geo.H + 1);
-    g.step_r = (NBT / g.nch) / g.pitch; g.step_c = (NBT / g.nch) % g.pitch;
-    g.halo = k == 3 ? geo.W + 2 : 0;
     const size_t total = k == 3 ? (size_t)geo.N * (geo.H + 1) * (geo.W + 1) : geo.P();
     if (total >= (1u << 30)) return false;
+    g.N = geo.N; g.H = geo.H; g.W = geo.W; g.P = (int)geo.P(); g.pitch = geo.W + 1;
+    g.dpitch = fast_div(geo.W + 1); g.drows = fast_div(geo.H + 1);
+    g.nit = in_mode == kInBwd ? 2 * g.nch : g.nch; g.RS = NBT / g.nit; g.dnit = fast_div(g.nit);
+    g.step_r = g.RS / g.pitch; g.step_c = g.RS % g.pitch;
+    g.halo = k == 3 ? geo.W + 2 : 0;
     g.total = (int)total;
+    // pieces of about 12 KB
+    const int tensors = in_mode == kInBwd ? 2 : 1;
+    g.rowb = cin * (in_mode == kInBf16 ? 2 : 4);
+    g.piece = g.RS;
+    while (2 * g.piece * g.rowb * tensors <= 12800) g.piece *= 2;
+    g.raw_bytes = round_up(g.piece * g.rowb, 128) * tensors;
     const int cout_pad = round_up(cout, 16), tiles = (g.total + 127) / 128, nchp = (g.nch + 1) & ~1;
     g.BN = cout_pad <= 16 ? 16 : (cout_pad <= 32 ? 32 : 64);
     // few tiles (late stages): split the output channels so that more SMs take part
@@ -513,6 +709,8 @@ bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count, FusedShape &s
     for (;; g.BN /= 2) {
         s.n_tiles = (cout_pad + g.BN - 1) / g.BN;
         g.groups = g.BN / NC;
+        s.EW = g.BN == 64 ? 16 : 8;
+        g.nacc = g.BN == 64 ? 2 : 4; g.acc_shift = g.BN == 64 ? 1 : 2;
         int ctas = sm_count / s.n_tiles; if (ctas < 1) ctas = 1;
         // a contiguous range of positions per CTA, a tile at least.  (Half tiles would put a small layer on every SM, but take as long and
         // leave none to the launches beside it: 110-layer step 4964 -> 4877 us, odd-sized basic block 167 -> 164 with whole ones.)
@@ -520,21 +718,49 @@ bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count, FusedShape &s
         s.ctas = (g.total + g.chunk - 1) / g.chunk;
         g.wtile_bytes = (g.BN * g.KC * 2 + 1023) & ~1023;
         const int T = (g.chunk + 127) / 128, fixed = 1024 + k * k * g.wtile_bytes + (int)sizeof(FusedShared) + 64;
+        const int aux1 = aux ? s.EW * kAuxBytes : 0, sets = s.EW / 4 / g.groups, own_tiles = (T + sets - 1) / sets;
         // planes are skewed against each other so that the chunks of a pixel, written by adjacent threads, hit different banks
-        auto seg_of = [&](int S) { g.plane16 = round_up(S * 128 + 2 * g.halo, 8) + (g.nch <= 2 ? 4 : (g.nch <= 4 ? 2 : 1)); return nchp * g.plane16 * 16; };
-        const int room = 227 * 1024 - fixed;
-        // the whole range as one segment if it fits, else the longest segments of which two fit
-        if (T <= kFullBars && seg_of(T) <= room) { g.S = T; g.nseg = 1; }
+        auto plane_of = [&](int S) { return round_up(S * 128 + 2 * g.halo, 8) + (g.nch <= 2 ? 4 : (g.nch <= 4 ? 2 : 1)); };
+        auto seg_of = [&](int S) { return round_up(nchp * plane_of(S) * 16, 128); };
+        auto tab_of = [&](int S) { return k == 3 ? (((S * 128 < g.chunk ? S * 128 : g.chunk) + 2 * g.halo) * 4 + 127) & ~127 : 0; };
+        auto pieces_of = [&](int S) { return ((S * 128 < g.chunk ? S * 128 : g.chunk) + 2 * g.halo + g.piece - 1) / g.piece; };
+        const int room = 227 * 1024 - fixed, least = 20480;      // least: the last reduction borrows the operand region, (512 + 128) x 4 doubles
+        // the whole range as one segment if it fits, else the longest segments of which two fit; beside them two pieces of the
+        // input and, for each epilogue warp, one tile's partner rows at least
+        auto fits = [&](int S, int nseg) {
+            const int op = nseg * seg_of(S);
+            return (op < least ? least : op) + (T <= S && pieces_of(S) < 2 ? 1 : 2) * g.raw_bytes + aux1 + tab_of(S) <= room;
+        };
+        // (1x1: no halo to build twice, short segments leave the room to the rings)
+        if (T <= (k == 1 ? 2 : kFullBars) && fits(T, 1)) { g.S = T; g.nseg = 1; }
         else {
-            g.nseg = 2; g.S = kFullBars / 2;
-            while (g.S > 1 && 2 * seg_of(g.S) > room) g.S--;
-            if (2 * seg_of(g.S) > room) g.nseg = 1;
+            g.nseg = 2; g.S = k == 1 ? 2 : kFullBars / 2;
+            while (g.S > 1 && !fits(g.S, 2)) g.S--;
+            if (!fits(g.S, 2)) g.nseg = 1;
         }
-        g.seg_bytes = round_up(seg_of(g.S), 128);
+        g.plane16 = plane_of(g.S);
+        g.seg_bytes = seg_of(g.S);
         g.op_bytes = g.nseg * g.seg_bytes;
-        if (g.op_bytes < 20480) g.op_bytes = 20480;      // the last reduction borrows the region: (512 + 128) x 4 doubles
-        s.smem = fixed + g.op_bytes;
-        if (s.smem <= 227 * 1024 && g.plane16 < (1 << 14)) return true;
+        if (g.op_bytes < least) g.op_bytes = least;
+        g.tab_bytes = tab_of(g.S);
+        g.pps = pieces_of(g.S); g.dpps = fast_div(g.pps);
+        g.pieces = T <= g.S ? g.pps : 2 * kRawSlots;        // (more than the ring holds, or counted as if)
+        // what is left goes to more pieces and more partner rows in flight, whichever has less
+        const int most_raw = T <= g.S ? (pieces_of(g.S) < kRawSlots ? pieces_of(g.S) : kRawSlots) : kRawSlots;
+        const int most_aux = !aux ? 0 : (own_tiles < kAuxSlots ? own_tiles : kAuxSlots);
+        g.raw_slots = most_raw < 2 ? most_raw : 2; g.aux_slots = aux ? 1 : 0;
+        int left = room - g.op_bytes - g.tab_bytes - g.raw_slots * g.raw_bytes - g.aux_slots * aux1;
+        s.smem = 227 * 1024 - left;
+        if (left >= 0 && g.plane16 < (1 << 14)) {
+            while (true) {
+                const bool r = g.raw_slots < most_raw && left >= g.raw_bytes, x = g.aux_slots < most_aux && left >= aux1;
+                if (!r && !x) break;
+                if (r && (!x || g.raw_slots * g.raw_bytes <= g.aux_slots * aux1)) { g.raw_slots++; left -= g.raw_bytes; }
+                else { g.aux_slots++; left -= aux1; }
+            }
+            s.smem = 227 * 1024 - left;
+            return true;
+        }
         if (g.BN < 32) return false;
     }
 }
@@ -543,13 +769,16 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// in: [P, cin] float / fixed point (in_mode 0) or bf16 (in_mode 1); out, partner and the BN input of a
-// data gradient must be plain (unsplit) tensors of cout channels
+// in: [P, cin]; out, partner and the BN input of a data gradient must be plain (unsplit) tensors of cout channels
+// behind: kInBwd, the BN whose backward the input still has to go through (bn names it too).  sums: where the records of the fused backward
+// sums may stay for their consumer
 bool run_fused(Exec &ex, const char *what, int in_mode, const void *in, float in_q, BnRef bn, Geom geo, int cin, int cout, int k,
-               const float *Wsrc, const bf16 *prepacked, bool transposed, Pair out, Pair partner, int sign, EpiReq req, bf16 *a_out) {
+               const float *Wsrc, const bf16 *prepacked, bool transposed, Pair out, Pair partner, int sign, EpiReq req, bf16 *a_out,
+               const BnBwdReq *behind = nullptr, BwdSums *sums = nullptr) {
     FusedShape s;
     if (out.c1 != 0 || (sign && partner.c1 != 0) || (req.bnbwd && req.bnbwd->t.c1 != 0)) return false;
-    if (!fused_shape(geo, cin, cout, k, ex.ctx->sm_count, s)) return false;
+    const bool aux = sign != 0 || req.bnbwd;
+    if (!fused_shape(geo, cin, cout, k, ex.ctx->sm_count, in_mode, aux, s)) return false;
     EncodeTiledFn enc = nullptr;
     if (!ex.dry) { enc = (EncodeTiledFn)tc_encoder(ex.ctx); if (!enc) return false; }
     const int taps = k * k;
@@ -561,7 +790,8 @@ bool run_fused(Exec &ex, const char *what, int in_mode, const void *in, float in
     const bool reduce = req.stats || req.bnbwd;
     // statistics whose owner has room for the records stay pending: the kernel that consumes them adds the records
     const bool defer = req.stats && !req.bnbwd && req.stats->part && (size_t)ctas * 2 * cout <= req.stats->part_cap;
-    float *part = defer ? req.stats->part : (reduce ? ex.ws.get<float>((size_t)ctas * 2 * cout) : nullptr);
+    float *part = defer ? req.stats->part : (sums ? sums->part : (reduce ? ex.ws.get<float>((size_t)ctas * 2 * cout) : nullptr));
+    if (sums) { sums->parts = ctas; sums->inv_count = 1.0 / (double)geo.P(); }
     if (req.stats) {
         req.stats->valid = true;
         req.stats->pending = defer; req.stats->parts = ctas; req.stats->inv_count = 1.0 / (double)geo.P();
@@ -582,17 +812,24 @@ bool run_fused(Exec &ex, const char *what, int in_mode, const void *in, float in
                 sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
             ex.failed = true; ex.ctx->err = std::string(what) + ": tensor map rejected"; ex.ws.release(m); return true;
         }
+        if (aux) {
+            cuuint64_t xdims[2] = {(cuuint64_t)cout, (cuuint64_t)geo.P()}, xstrides[1] = {(cuuint64_t)cout * 4};
+            cuuint32_t xbox[2] = {NC, 32};
+            if (enc(&A.map_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void *)(req.bnbwd ? req.bnbwd->t.p0 : partner.p0), xdims, xstrides, xbox, es,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
+                ex.failed = true; ex.ctx->err = std::string(what) + ": tensor map (partner) rejected"; ex.ws.release(m); return true;
+            }
+        }
         FusedLayer &p = A.ly;
-        p.in_mode = in_mode == 0 && in_q != 0.f ? 2 : in_mode; p.in = in; p.in_q = in_q; p.bn = bn; p.a_out = a_out;
-        p.aux = req.bnbwd ? req.bnbwd->t.p0 : (sign ? partner.p0 : out.p0);
-        p.wide_in = ((uintptr_t)in & 31) == 0;
-        p.wide_out = ((uintptr_t)out.p0 & 31) == 0 && ((uintptr_t)p.aux & 31) == 0 && cout % 8 == 0;
+        p.in_mode = in_mode; p.in = in; p.in_q = in_q; p.bn = bn; p.a_out = a_out;
+        if (behind) { p.in_t = behind->t.p0; p.in_dgamma = behind->dgamma; p.in_dbeta = behind->dbeta; }
+        p.wide_out = ((uintptr_t)out.p0 & 31) == 0 && cout % 8 == 0;
         p.w_early = prepacked ? 1 : 0;
         A.status = ex.ctx->dev_status; A.stamp = ex.stamp_slot();
         FusedEpi &e = p.epi;
         e.mode = req.bnbwd ? EPI_BNBWD : (sign ? EPI_COUPLE : EPI_PLAIN);
         e.out = out.p0; e.q = req.bnbwd ? req.bnbwd->t.q : out.q; e.sign = sign; e.n_cols = cout;
-        e.part = part; e.counter = (reduce && !defer) ? ex.ctx->counter() : nullptr;
+        e.part = part; e.counter = (reduce && !defer && !sums) ? ex.ctx->counter() : nullptr;
         e.inv_count = 1.0 / (double)geo.P(); e.eps = ex.eps;
         if (req.stats) { e.mean = req.stats->mean; e.rstd = req.stats->rstd; }
         if (req.bnbwd) { e.bn = req.bnbwd->bn; e.dgamma = req.bnbwd->dgamma; e.dbeta = req.bnbwd->dbeta; e.coef = req.bnbwd->coef; }
@@ -602,9 +839,9 @@ bool run_fused(Exec &ex, const char *what, int in_mode, const void *in, float in
             cudaFuncSetAttribute(conv_fused_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         }
         dim3 grid((unsigned)ctas, (unsigned)s.n_tiles);
-        const int EW = s.g.BN == 16 ? 8 : 16;
+        const int EW = s.EW;
         launch(ex, EW == 16 ? conv_fused_kernel<16> : conv_fused_kernel<8>, grid, fused_threads(EW), s.smem, A);
-        const double bytes = (double)geo.P() * cin * (in_mode == 0 ? 4 : 2) + (double)geo.P() * cout * (sign || req.bnbwd ? 8 : 4) +
+        const double bytes = (double)geo.P() * cin * (in_mode == kInBf16 ? 2 : (in_mode == kInBwd ? 8 : 4)) + (double)geo.P() * cout * (sign || req.bnbwd ? 8 : 4) +
                              (double)cout * taps * cin * 2 + (a_out ? (double)geo.P() * cin * 2 : 0.0);
         ex.check(what, bytes, 2.0 * geo.P() * cout * cin * taps);
     }
@@ -617,19 +854,42 @@ bool run_fused(Exec &ex, const char *what, int in_mode, const void *in, float in
 // whether conv_fprop_fused takes layer L on images gi (and so adds pending statistics of its input itself)
 bool conv_fused_takes(Exec &ex, Geom gi, const Layer &L) {
     FusedShape s;
-    return L.stride == 1 && fused_shape(gi, L.cin, L.cout, L.k, ex.ctx->sm_count, s);
+    return L.stride == 1 && fused_shape(gi, L.cin, L.cout, L.k, ex.ctx->sm_count, kInFloat, true, s);
 }
 
 // out = partner + sign * conv(ReLU(BN(t)));  a_out (optional): the activated tensor, for the weight gradient
 bool conv_fprop_fused(Exec &ex, Pair t, BnRef bn, Geom gi, const Layer &L, Pair out, Pair partner, int sign, Moments *stats, bf16 *a_out) {
     if (L.stride != 1 || t.c1 != 0) return false;
     EpiReq req; req.stats = stats;
-    return run_fused(ex, "conv_fprop_fused", 0, t.p0, t.q, bn, gi, L.cin, L.cout, L.k, L.W, L.Wp_fprop, false, out, partner, sign, req, a_out);
+    return run_fused(ex, "conv_fprop_fused", t.q != 0.f ? kInFixed : kInFloat, t.p0, t.q, bn, gi, L.cin, L.cout, L.k, L.W, L.Wp_fprop, false, out, partner, sign, req, a_out);
 }
 
 // da = conv^T(g) for a stride-1 layer, g bf16 [P, cout]
-bool conv_dgrad_fused(Exec &ex, const void *g, Geom gi, const Layer &L, float *da, const BnBwdReq *bb) {
+bool conv_dgrad_fused(Exec &ex, const void *g, Geom gi, const Layer &L, float *da, const BnBwdReq *bb, BwdSums *sums) {
     if (L.stride != 1) return false;
     EpiReq req; req.bnbwd = bb;
-    return run_fused(ex, "conv_dgrad_fused", 1, g, 0.f, BnRef{}, gi, L.cout, L.cin, L.k, L.W, L.Wp_dgrad, true, single(da, L.cin), Pair{}, 0, req, nullptr);
+    return run_fused(ex, "conv_dgrad_fused", kInBf16, g, 0.f, BnRef{}, gi, L.cout, L.cin, L.k, L.W, L.Wp_dgrad, true, single(da, L.cin), Pair{}, 0, req, nullptr,
+                     nullptr, sums);
+}
+
+// whether conv_dgrad_fused takes the data gradient of L, with a bf16 input or (behind) through the BN backward of the layer behind
+bool conv_dgrad_fused_takes(Exec &ex, Geom gi, const Layer &L, bool behind) {
+    FusedShape s;
+    if (L.stride != 1 || !fused_shape(gi, L.cout, L.cin, L.k, ex.ctx->sm_count, behind ? kInBwd : kInBf16, true, s) || !(ex.dry || tc_encoder(ex.ctx))) return false;
+    // Through the BN backward only where a build thread has few rows: its pass costs 0.3 us per row and thread, twice that of a bf16 input with
+    // twice the threads per row, against 5 us for the launch that it saves.  Odd-sized block (24 channels, a tile per CTA, five and a half rows)
+    // 151 -> 144.5 us; 56 channels at 8x8 (eleven rows) and 16 at 32x32 (twenty-one): 38-layer step 1665 -> 1686.
+    return !behind || (long long)(s.g.chunk + 2 * s.g.halo) * s.g.nit <= 6 * NBT;
+}
+
+// The same where the gradient still has to go through the BN + ReLU backward of the layer behind L: g is da of that layer (float), `behind` its
+// BN with a plain float input, `bsums` its pending sums.  dgamma and dbeta of that BN are stored, and the bf16 gradient (for the
+// weight gradient) in g_out.
+// The pass over the tensor between the two data gradients goes, and with it its launch and the last CTA's reduction in front of it.
+bool conv_dgrad_fused_behind(Exec &ex, const float *g, const BnBwdReq &behind, const BwdSums &bsums, bf16 *g_out, Geom gi, const Layer &L, float *da, const BnBwdReq *bb,
+                             BwdSums *sums) {
+    EpiReq req; req.bnbwd = bb;
+    BnRef bn = behind.bn;
+    bn.part = bsums.part; bn.parts = bsums.parts; bn.inv_count = bsums.inv_count; bn.eps = ex.eps;
+    return run_fused(ex, "conv_dgrad_fused", kInBwd, g, 0.f, bn, gi, L.cout, L.cin, L.k, L.W, L.Wp_dgrad, true, single(da, L.cin), Pair{}, 0, req, g_out, &behind, sums);
 }

@@ -516,6 +516,86 @@ void bn_relu_bwd(Exec &ex, const float *da, Pair t, size_t P, BnRef bn, float *d
     ex.ws.release(m);
 }
 
+// The last step of a function's backward on tensors of at most 64 channels: out = add + dt (bn_relu_bwd_apply_kernel<float, 2>) from sums that are
+// still the records of the data gradient's CTAs.  Every CTA adds them, with its first rows already on the way: the records and the
+// coefficients take it 2 us, where the reduction by the last CTA of the data gradient kept the GPU waiting for 4.  So a CTA takes all its rows
+// in one or two rounds of loads, and the grid stays at two CTAs per SM.
+constexpr int kSumsRows = 4;
+template <bool CAST>
+__global__ void __launch_bounds__(256, 2) bn_relu_bwd_sums_kernel(const float *__restrict__ da, Pair t, int P, int rows, BnRef bn, float *__restrict__ dgamma,
+                                                                  float *__restrict__ dbeta, const float *__restrict__ add, float *__restrict__ out,
+                                                                  bf16 *__restrict__ cast, unsigned long long *stamp) {
+    __shared__ double red[256 * 4], tot[32 * 4];
+    __shared__ __align__(16) float cf[7][64];
+    pdl_enter();
+    stamp_begin(stamp);
+    const int C = t.c0, C4 = C >> 2, rpp = 256 / C4, tid = threadIdx.x, q = tid % C4, r = tid / C4;
+    const int r0 = (int)blockIdx.x * rows, r1 = r0 + rows < P ? r0 + rows : P;
+    float4 v[kSumsRows], g[kSumsRows], a[kSumsRows];
+    auto load = [&](int rb) {
+#pragma unroll
+        for (int j = 0; j < kSumsRows; j++) {
+            int row = rb + j * rpp; if (row >= r1) row = r1 - 1;
+            const size_t off = (size_t)row * C + q * 4;
+            v[j] = ld4(t.p0 + off); g[j] = ld4(da + off); a[j] = ld4(add + off);
+        }
+    };
+    if (r < rpp && r0 + r < r1) load(r0 + r);
+    float gam = 0.f, bet = 0.f, mean = 0.f, rstd = 0.f;
+    if (tid < C) { gam = bn.gamma[tid]; bet = bn.beta[tid]; mean = bn.mean[tid]; rstd = bn.rstd[tid]; }
+    tc::reduce_records<256>(bn.part, bn.parts, C, 0, C >> 1, red, tot, tid);
+    if (tid < C) {
+        const double sum = tot[(2 * (tid >> 2)) * 4 + (tid & 3)], sum2 = tot[(2 * (tid >> 2) + 1) * 4 + (tid & 3)], gr = (double)gam * (double)rstd;
+        float sc, sh;
+        bn_sc_sh(gam, bet, mean, rstd, sc, sh);
+        cf[0][tid] = sc; cf[1][tid] = sh; cf[2][tid] = mean; cf[3][tid] = rstd;
+        cf[4][tid] = (float)gr; cf[5][tid] = (float)(gr * sum * bn.inv_count); cf[6][tid] = (float)(gr * sum2 * bn.inv_count);
+        if (blockIdx.x == 0) { dbeta[tid] = (float)sum; dgamma[tid] = (float)sum2; }
+    }
+    __syncthreads();
+    if (r < rpp) {
+        float4 k[7];
+#pragma unroll
+        for (int i = 0; i < 7; i++) k[i] = ld4(&cf[i][q * 4]);
+#pragma unroll 1
+        for (int rb = r0 + r; rb < r1; rb += kSumsRows * rpp) {
+            if (rb != r0 + r) load(rb);
+#pragma unroll
+            for (int j = 0; j < kSumsRows; j++) {
+                const int row = rb + j * rpp;
+                if (row >= r1) continue;
+                float x[4] = {v[j].x, v[j].y, v[j].z, v[j].w}, o[4];
+                values<4>(x, t.q);
+                const float d[4] = {g[j].x, g[j].y, g[j].z, g[j].w}, p[4] = {a[j].x, a[j].y, a[j].z, a[j].w};
+#define RV_K(n, i) (i == 0 ? k[n].x : i == 1 ? k[n].y : i == 2 ? k[n].z : k[n].w)
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    o[i] = RV_K(4, i) * (fmaf(RV_K(0, i), x[i], RV_K(1, i)) > 0.f ? d[i] : 0.f) - RV_K(5, i) - RV_K(6, i) * ((x[i] - RV_K(2, i)) * RV_K(3, i));
+                    o[i] += p[i];
+                }
+#undef RV_K
+                const float4 s = make_float4(o[0], o[1], o[2], o[3]);
+                st4(out + (size_t)row * C + q * 4, s);
+                if (CAST) st4(cast + (size_t)row * C + q * 4, s);
+            }
+        }
+    }
+    stamp_end(stamp);
+}
+// (larger tensors: the streaming kernel's wider accesses are worth more than the reduction in front of it)
+bool bn_relu_bwd_sums_takes(size_t P, int C) { return C <= 64 && C % 4 == 0 && P * C <= (size_t)1 << 22; }
+void bn_relu_bwd_sums(Exec &ex, const float *da, Pair t, size_t P, BnRef bn, float *dgamma, float *dbeta, const BwdSums &sums, Pair add, Pair out, bf16 *out_cast) {
+    if (ex.dry) return;
+    const int C = t.C(), rpp = 256 / (C / 4);
+    int ctas = cdiv(P, (size_t)rpp * kSumsRows);
+    if (ctas > 2 * ex.ctx->sm_count) ctas = 2 * ex.ctx->sm_count;
+    const int rows = cdiv(P, ctas);
+    bn.part = sums.part; bn.parts = sums.parts; bn.inv_count = sums.inv_count; bn.eps = ex.eps;
+    unsigned long long *stamp = ex.stamp_slot();
+    launch(ex, out_cast ? bn_relu_bwd_sums_kernel<true> : bn_relu_bwd_sums_kernel<false>, dim3(cdiv(P, rows)), 256, 0, da, t, (int)P, rows, bn, dgamma, dbeta, (const float *)add.p0, out.p0, out_cast, stamp);
+    ex.check("bn_relu_bwd_apply", (double)P * C * (16 + (out_cast ? 2 : 0)));
+}
+
 template <class TO, int V>
 __global__ void __launch_bounds__(256) concat_cast_kernel(Pair src, size_t P, int SW, int rows, TO *__restrict__ dst) {
     pdl_enter();

@@ -55,10 +55,6 @@ struct revnet_plan {
     revnet_step_stats graph_stats = {};
 };
 
-// largest half of a unit's pair for which its weight gradients may run on into the next unit (LateWgrad).  Both halves of a unit's
-// scratch stay allocated for it; above, a launch fills the GPU for so long that nothing is won by running two side by side.
-constexpr size_t kLateWgradElems = (size_t)1 << 23;
-
 static std::vector<std::array<int, 3>> fn_shape(int kind, int c, int w) {
     if (kind == 0) return {{c, c, 3}};
     if (kind == 1) return {{c, c, 3}, {c, c, 3}};

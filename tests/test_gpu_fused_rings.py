@@ -1,0 +1,33 @@
+"""Fused BN-ReLU-conv layers at the sizes where their rings of input pieces and partner rows, their operand segments and the
+pass of a gradient through the BN backward of the layer behind begin and end.  Compared with the float64 oracle under the
+stated tolerances of the bf16 mode (2e-2 outputs, 5e-2 gradients); the longest sum has 576 products."""
+import pytest
+
+from paper_1707_04585_b200 import binding as B
+from paper_1707_04585_b200 import synthetic as syn
+from tests import test_gpu_parity as tp
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = B.Context(0)
+    yield c
+    B.revnet_check_device(c)
+    c.close()
+
+
+@pytest.mark.parametrize("kind,N,H,W,c,w", [
+    ("basic", 1, 1, 1, 8, 0),             # one pixel; one piece
+    ("basic", 37, 15, 21, 24, 0),         # one tile per CTA: the inner data gradient goes through the BN backward itself
+    ("basic", 3, 5, 78, 16, 0),           # the largest halo for which it does (six rows per build thread), and
+    ("basic", 3, 5, 79, 16, 0),           # one size on, where it does not
+    ("basic", 150, 33, 31, 16, 0),        # nine tiles per CTA: the range as one segment, the partner ring goes round
+    ("basic", 64, 32, 32, 64, 0),         # two operand segments in turn, two pieces of the input in flight
+    ("basic", 3, 40, 150, 48, 0),         # long rows: a halo of 152 rows, six planes
+    ("single", 9, 30, 33, 40, 0),         # one layer per function: sums of the only layer left to the last step
+    ("bottleneck", 64, 32, 32, 128, 32),  # 1x1 onto 128 columns: many tiles per CTA in segments of two, both rings go round
+])
+def test_fused_layers_at_ring_edges(ctx, kind, N, H, W, c, w):
+    tp.run_block_case(ctx, syn.BlockCfg(N, H, W, c, w, kind, seed=700 + c), 0, jitter=True, inplace=True)
