@@ -37,7 +37,7 @@ def load_peaks():
 # fp32 FMA peak of the CUDA cores: 148 SMs x 128 lanes x 2 flop x 1.965 GHz (max SM clock)
 ALU_FP32_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
 
-ALU_KERNELS = ("conv3x3_direct_kernel", "conv_gemm_kernel", "gemm_simt_kernel")   # fp32 convolutions on the CUDA cores
+ALU_KERNELS = ("conv3x3_direct_kernel", "wgrad3x3_strip_kernel", "conv_gemm_kernel", "gemm_simt_kernel")   # fp32 convolutions on the CUDA cores
 
 # profile record name (one per call site class) -> the CUDA kernel that runs it, and the source files it is built from
 DEVICE_KERNEL = {
@@ -45,7 +45,7 @@ DEVICE_KERNEL = {
     "conv_fprop_tc": "conv_tc_kernel", "conv_dgrad_tc": "conv_tc_kernel", "conv_wgrad_tc": "wgrad_tc_kernel",
     "conv_fprop_bn": "conv1x1_bn_kernel", "conv_fprop_tc2": "conv_tc2_kernel", "conv_dgrad_tc2": "conv_tc2_kernel", "conv_wgrad_tc2": "wgrad_tc2_kernel",
     "conv_fprop_direct": "conv3x3_direct_kernel", "conv_dgrad_direct": "conv3x3_direct_kernel",
-    "conv_fprop_gemm": "conv_gemm_kernel", "conv_dgrad_gemm": "conv_gemm_kernel", "conv_wgrad_gemm": "conv_gemm_kernel",
+    "conv_fprop_gemm": "conv_gemm_kernel", "conv_dgrad_gemm": "conv_gemm_kernel", "conv_wgrad_gemm": "conv_gemm_kernel", "conv_wgrad_strip": "wgrad3x3_strip_kernel",
     "conv_fprop_simt": "gemm_simt_kernel", "conv_wgrad_simt": "gemm_simt_kernel",
     "bn_stats": "col_reduce_kernel", "bn_bwd_sums": "col_reduce_kernel",
 }

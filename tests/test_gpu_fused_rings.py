@@ -1,6 +1,6 @@
-"""Fused BN-ReLU-conv layers at the sizes where their rings of input pieces and partner rows, their operand segments and the
+"""Fused BN-ReLU-conv layers (and, in the strict mode, the weight gradient in strips of image rows) at the sizes where their rings of input pieces and partner rows, their operand segments and the
 pass of a gradient through the BN backward of the layer behind begin and end.  Compared with the float64 oracle under the
-stated tolerances of the bf16 mode (2e-2 outputs, 5e-2 gradients); the longest sum has 576 products."""
+stated tolerances (bf16 mode: 2e-2 outputs, 5e-2 gradients; strict mode: 1e-4), which bound rounding at these sizes."""
 import pytest
 
 from paper_1707_04585_b200 import binding as B
@@ -31,3 +31,14 @@ def ctx():
 ])
 def test_fused_layers_at_ring_edges(ctx, kind, N, H, W, c, w):
     tp.run_block_case(ctx, syn.BlockCfg(N, H, W, c, w, kind, seed=700 + c), 0, jitter=True, inplace=True)
+
+
+@pytest.mark.parametrize("kind,N,H,W,c", [
+    ("basic", 2, 9, 5, 12),               # nine pairs of quads: three row slices of a warp, five idle lanes; rows of 3 + 2 pixels
+    ("basic", 3, 1, 7, 4),                # one row: one slice
+    ("basic", 150, 17, 16, 16),           # several strips per CTA, the last strip of an image one row
+    ("basic", 5, 6, 9, 44),               # 121 pairs in four blocks, the last of 25
+    ("basic", 2, 3, 31, 64),              # 24 warps
+])
+def test_strict_weight_gradient_strips(ctx, kind, N, H, W, c):
+    tp.run_block_case(ctx, syn.BlockCfg(N, H, W, c, 0, kind, seed=800 + c), 1, jitter=True, inplace=True)
