@@ -211,7 +211,8 @@ __device__ __forceinline__ void moments_of(double sum, double sum2, double inv_c
 // of a warp then touch 32 records.)  All in double precision, in an order that the number of
 // records, cw and NT fix.  Result: tot[slot - slot0][4].  Called by NT threads (tid = 0..NT-1)
 // that share named barrier 1; red: [NT][4] doubles, tot: [128][4] doubles of shared memory.
-template <int NT>
+// IF: loads in flight per thread.
+template <int NT, int IF = NT == 128 ? 10 : 5>
 __device__ __forceinline__ void reduce_records(const float *part, int parts, int C, int slot0, int cw, double *red, double *tot, int tid) {
     int rs = 4;
     while (rs < cw) rs <<= 1;
@@ -219,7 +220,7 @@ __device__ __forceinline__ void reduce_records(const float *part, int parts, int
     double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
     if (slot < cw) {
         const float *src = part + (size_t)(slot0 + slot) * 4;
-        constexpr int kInFlight = NT == 128 ? 10 : 5;
+        constexpr int kInFlight = IF;
         for (int i = sub; i < parts; i += kInFlight * nsub) {
             float4 v[kInFlight];
 #pragma unroll

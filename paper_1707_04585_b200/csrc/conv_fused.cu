@@ -354,9 +354,9 @@ __device__ __forceinline__ AuxRing aux_ring(const FusedArgs &A, FusedShared *sh,
     x.on = A.ly.epi.mode != EPI_PLAIN && x.col < A.ly.epi.n_cols;
     return x;
 }
-__device__ __forceinline__ void aux_load(const FusedArgs &A, const AuxRing &x, int slot, int q) {       // one thread; q: the warp's first position
+__device__ __forceinline__ void aux_load(const FusedArgs &A, const AuxRing &x, int slot, int row) {       // one thread; row: the first pixel
     mbar_expect_tx(&x.bar[slot], kAuxBytes);
-    tma_load_2d(x.buf + slot * kAuxBytes, &A.map_x, &x.bar[slot], x.col, pixels_before(A.g, q));
+    tma_load_2d(x.buf + slot * kAuxBytes, &A.map_x, &x.bar[slot], x.col, row);
 }
 
 // Epilogue of one warp's rows.  EK: 0 plain, 1 float coupling, 2 fixed-point coupling, 3 / 4 BN+ReLU backward with a float /
@@ -436,7 +436,7 @@ __device__ __forceinline__ bool epilogue_loop(const FusedArgs &A, FusedShared *s
         __syncwarp();
         if (lane == 0) {
             mbar_arrive(&sh->acc_empty[buf]);
-            if (EK > 0 && ax.on && ti + g.aux_slots * sets < n_tiles) aux_load(A, ax, slot, qw + g.aux_slots * sets * 128);
+            if (EK > 0 && ax.on && ti + g.aux_slots * sets < n_tiles) aux_load(A, ax, slot, pixels_before(g, qw + g.aux_slots * sets * 128));
         }
         if (++slot == g.aux_slots) { slot = 0; round++; }
     }
@@ -565,15 +565,17 @@ __global__ void __launch_bounds__(EW == 8 ? 640 : fused_threads(EW), 1) conv_fus
         const int n = full * g.pps + (rest > 0 ? (rest + 2 * g.halo + g.piece - 1) / g.piece : 0);
         if (lane < g.raw_slots && lane < n) load_piece(g, p, sh, raw, lane, piece_a, piece_b);
         // (the partner rows wait until the records of the statistics are in: those, and the first rows, are needed first)
+        const int sets = EW / 4 / g.groups, w = lane & (EW - 1);          // lane: slots lane / EW, + 32 / EW, ... of warp w's ring
+        const AuxRing x = aux_ring(A, sh, auxb, w);
+        int slot = lane / EW, ti = (w >> 2) / g.groups + slot * sets;
+        int row = pixels_before(g, pos0 + ti * 128 + (w & 3) * 32);
         if (!direct) named_barrier(3, EW * 32 + NBT + 32);
-        if (e.mode != EPI_PLAIN) {
-            const int sets = EW / 4 / g.groups;
-            for (int i = lane; i < EW * g.aux_slots; i += 32) {
-                const int slot = i / EW, w = i & (EW - 1), ti = (w >> 2) / g.groups + slot * sets;
-                const AuxRing x = aux_ring(A, sh, auxb, w);
-                if (x.on && ti < n_tiles) aux_load(A, x, slot, pos0 + ti * 128 + (w & 3) * 32);
+        if (x.on)
+            while (slot < g.aux_slots && ti < n_tiles) {
+                aux_load(A, x, slot, row);
+                slot += 32 / EW; ti += 32 / EW * sets;
+                row = pixels_before(g, pos0 + ti * 128 + (w & 3) * 32);
             }
-        }
         __syncwarp();
         if (elect_one()) {
             int slot = 0, round = 0;
@@ -598,7 +600,7 @@ __global__ void __launch_bounds__(EW == 8 ? 640 : fused_threads(EW), 1) conv_fus
                 gam = p.bn.gamma[c]; bet = p.bn.beta[c];
                 if (!p.bn.part || p.in_mode == kInBwd) { mean = p.bn.mean[c]; rstd = p.bn.rstd[c]; }
             }
-            if (p.bn.part) reduce_records<256>(p.bn.part, p.bn.parts, g.cin, 0, g.cin >> 1, sh->red, sh->tot, etid);
+            if (p.bn.part) reduce_records<256, 10>(p.bn.part, p.bn.parts, g.cin, 0, g.cin >> 1, sh->red, sh->tot, etid);
             if (c < 64) {
                 float sc = 0.f, sf = 0.f, k0 = 0.f, k1 = 0.f, k2 = 0.f;
                 if (mine) {
@@ -699,14 +701,14 @@ bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count, int in_mode, 
     // pieces of about 12 KB
     const int tensors = in_mode == kInBwd ? 2 : 1;
     g.rowb = cin * (in_mode == kInBf16 ? 2 : 4);
-    g.piece = g.RS;
-    while (2 * g.piece * g.rowb * tensors <= 12800) g.piece *= 2;
-    g.raw_bytes = round_up(g.piece * g.rowb, 128) * tensors;
+    int piece = g.RS;
+    while (2 * piece * g.rowb * tensors <= 12800) piece *= 2;
     const int cout_pad = round_up(cout, 16), tiles = (g.total + 127) / 128, nchp = (g.nch + 1) & ~1;
     g.BN = cout_pad <= 16 ? 16 : (cout_pad <= 32 ? 32 : 64);
     // few tiles (late stages): split the output channels so that more SMs take part
     while (g.BN > 16 && tiles * ((cout_pad + g.BN - 1) / g.BN) * 2 <= sm_count) g.BN /= 2;
     for (;; g.BN /= 2) {
+        g.piece = piece; g.raw_bytes = round_up(piece * g.rowb, 128) * tensors;
         s.n_tiles = (cout_pad + g.BN - 1) / g.BN;
         g.groups = g.BN / NC;
         s.EW = g.BN == 64 ? 16 : 8;
@@ -746,6 +748,15 @@ bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count, int in_mode, 
         g.pps = pieces_of(g.S); g.dpps = fast_div(g.pps);
         g.pieces = T <= g.S ? g.pps : 2 * kRawSlots;        // (more than the ring holds, or counted as if)
         // what is left goes to more pieces and more partner rows in flight, whichever has less
+        // (a range that fits in two pieces beside two tiles of partner rows comes in two, the first with the first tile's rows at least:
+        // every piece costs a build warp 0.3 us)
+        if (T <= g.S) {
+            const int rows = g.chunk + 2 * g.halo, first = 128 + 2 * g.halo, half = (rows + 1) / 2;
+            const int R = round_up(half < first && first < rows ? first : half, g.RS), bytes = round_up(R * g.rowb, 128) * tensors;
+            if (R > g.piece && g.op_bytes + g.tab_bytes + (R >= rows ? 1 : 2) * bytes + 2 * aux1 <= room) {
+                g.piece = R; g.raw_bytes = bytes; g.pps = g.pieces = pieces_of(g.S); g.dpps = fast_div(g.pps);
+            }
+        }
         const int most_raw = T <= g.S ? (pieces_of(g.S) < kRawSlots ? pieces_of(g.S) : kRawSlots) : kRawSlots;
         const int most_aux = !aux ? 0 : (own_tiles < kAuxSlots ? own_tiles : kAuxSlots);
         g.raw_slots = most_raw < 2 ? most_raw : 2; g.aux_slots = aux ? 1 : 0;
