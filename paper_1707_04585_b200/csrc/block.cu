@@ -184,8 +184,9 @@ bool fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
         const Pair tl = l == 0 ? u : single(saved.t[l - 1], ly.cin);
         const BnRef bn{ly.gamma, ly.beta, saved.bn[l].mean, saved.bn[l].rstd};
         const BnBwdReq bb{tl, bn, ly.dgamma, ly.dbeta, coef};
-        const bool leave = b16 && (folded || conv_dgrad_fused_takes(ex, gin[l], ly, false)) &&
-                           (l == 0 ? plain && bn_relu_bwd_sums_takes(P, ly.cin) : (l > 1 || u.c1 == 0) && conv_dgrad_fused_takes(ex, gin[l - 1], layers[l - 1], true));
+        // fold: the data gradient in front goes through this BN's backward; else the kernel between them adds the records
+        const bool fold = l > 0 && (l > 1 || u.c1 == 0) && conv_dgrad_fused_takes(ex, gin[l - 1], layers[l - 1], true);
+        const bool leave = b16 && (folded || conv_dgrad_fused_takes(ex, gin[l], ly, false)) && (fold || (bn_relu_bwd_sums_takes(P, ly.cin) && (l > 0 || plain)));
         BwdSums mine;
         if (leave) mine.part = ex.ws.get<float>(bwd_sums_floats(ex, ly.cin));
         auto wgrads = [&]() {            // as soon as every gradient operand exists
@@ -211,15 +212,16 @@ bool fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
         }
         else sums_done = conv_dgrad(ex, gcur, gin[l], ly, da, &bb, leave ? &mine : nullptr);
         if (folded) wgrads();
-        sums = mine;
+        sums = fold ? mine : BwdSums{};
         da_behind = da; behind = bb;
         if (l == 0) {
             // add.p0 == nullptr: the gradient is stored without a partner (stored transitions)
-            if (leave) bn_relu_bwd_sums(ex, da, tl, P, bn, ly.dgamma, ly.dbeta, sums, add, dgin_out, dgin_cast);
+            if (leave) bn_relu_bwd_sums(ex, da, tl, P, bn, ly.dgamma, ly.dbeta, mine, add, dgin_out, dgin_cast);
             else bn_relu_bwd(ex, da, tl, P, bn, ly.dgamma, ly.dbeta, coef, sums_done, nullptr, false, add, dgin_out, b16 ? dgin_cast : nullptr);
-        } else if (!leave) {
+        } else if (!leave || !fold) {
             void *dtn = ex.ws.alloc(P * ly.cin * esz(ex));
-            bn_relu_bwd(ex, da, tl, P, bn, ly.dgamma, ly.dbeta, coef, sums_done, dtn, b16, Pair{}, Pair{}, nullptr);
+            if (leave) bn_relu_bwd_sums(ex, da, tl, P, bn, ly.dgamma, ly.dbeta, mine, Pair{}, Pair{}, (bf16 *)dtn);
+            else bn_relu_bwd(ex, da, tl, P, bn, ly.dgamma, ly.dbeta, coef, sums_done, dtn, b16, Pair{}, Pair{}, nullptr);
             gcur = dtn;
         }
     }

@@ -438,7 +438,8 @@ struct BnBwdReq { Pair t; BnRef bn; float *dgamma, *dbeta, *coef; };
 // part: room for bwd_sums_floats() floats
 struct BwdSums { float *part = nullptr; int parts = 0; double inv_count = 0; };
 inline size_t bwd_sums_floats(const Exec &ex, int C) { return (size_t)ex.ctx->sm_count * 2 * C; }
-// whether bn_relu_bwd_sums takes the shape; out = add + dt from pending sums, optionally with a bf16 copy (all plain tensors)
+// whether bn_relu_bwd_sums takes the shape; out = add + dt from pending sums, optionally with a bf16 copy, or (add.p0 == nullptr) the bf16
+// copy of dt alone (all plain tensors)
 bool bn_relu_bwd_sums_takes(size_t P, int C);
 void bn_relu_bwd_sums(Exec &ex, const float *da, Pair t, size_t P, BnRef bn, float *dgamma, float *dbeta, const BwdSums &sums, Pair add, Pair out, bf16 *out_cast);
 // Reductions a convolution epilogue is asked to fuse.

@@ -516,12 +516,12 @@ void bn_relu_bwd(Exec &ex, const float *da, Pair t, size_t P, BnRef bn, float *d
     ex.ws.release(m);
 }
 
-// The last step of a function's backward on tensors of at most 64 channels: out = add + dt (bn_relu_bwd_apply_kernel<float, 2>) from sums that are
-// still the records of the data gradient's CTAs.  Every CTA adds them, with its first rows already on the way: the records and the
+// bn_relu_bwd_apply_kernel on tensors of at most 64 channels from sums that are still the records of the data gradient's CTAs:
+// ADD: the last step of a function's backward, out = add + dt, CAST: with a bf16 copy; else between its layers, the bf16 copy of dt alone.  Every CTA adds them, with its first rows already on the way: the records and the
 // coefficients take it 2 us, where the reduction by the last CTA of the data gradient kept the GPU waiting for 4.  So a CTA takes all its rows
 // in one or two rounds of loads, and the grid stays at two CTAs per SM.
 constexpr int kSumsRows = 4;
-template <bool CAST>
+template <bool ADD, bool CAST>
 __global__ void __launch_bounds__(256, 2) bn_relu_bwd_sums_kernel(const float *__restrict__ da, Pair t, int P, int rows, BnRef bn, float *__restrict__ dgamma,
                                                                   float *__restrict__ dbeta, const float *__restrict__ add, float *__restrict__ out,
                                                                   bf16 *__restrict__ cast, unsigned long long *stamp) {
@@ -537,7 +537,8 @@ __global__ void __launch_bounds__(256, 2) bn_relu_bwd_sums_kernel(const float *_
         for (int j = 0; j < kSumsRows; j++) {
             int row = rb + j * rpp; if (row >= r1) row = r1 - 1;
             const size_t off = (size_t)row * C + q * 4;
-            v[j] = ld4(t.p0 + off); g[j] = ld4(da + off); a[j] = ld4(add + off);
+            v[j] = ld4(t.p0 + off); g[j] = ld4(da + off);
+            if (ADD) a[j] = ld4(add + off);
         }
     };
     if (r < rpp && r0 + r < r1) load(r0 + r);
@@ -566,16 +567,16 @@ __global__ void __launch_bounds__(256, 2) bn_relu_bwd_sums_kernel(const float *_
                 if (row >= r1) continue;
                 float x[4] = {v[j].x, v[j].y, v[j].z, v[j].w}, o[4];
                 values<4>(x, t.q);
-                const float d[4] = {g[j].x, g[j].y, g[j].z, g[j].w}, p[4] = {a[j].x, a[j].y, a[j].z, a[j].w};
+                const float d[4] = {g[j].x, g[j].y, g[j].z, g[j].w}, p[4] = {ADD ? a[j].x : 0.f, ADD ? a[j].y : 0.f, ADD ? a[j].z : 0.f, ADD ? a[j].w : 0.f};
 #define RV_K(n, i) (i == 0 ? k[n].x : i == 1 ? k[n].y : i == 2 ? k[n].z : k[n].w)
 #pragma unroll
                 for (int i = 0; i < 4; i++) {
                     o[i] = RV_K(4, i) * (fmaf(RV_K(0, i), x[i], RV_K(1, i)) > 0.f ? d[i] : 0.f) - RV_K(5, i) - RV_K(6, i) * ((x[i] - RV_K(2, i)) * RV_K(3, i));
-                    o[i] += p[i];
+                    if (ADD) o[i] += p[i];
                 }
 #undef RV_K
                 const float4 s = make_float4(o[0], o[1], o[2], o[3]);
-                st4(out + (size_t)row * C + q * 4, s);
+                if (ADD) st4(out + (size_t)row * C + q * 4, s);
                 if (CAST) st4(cast + (size_t)row * C + q * 4, s);
             }
         }
@@ -592,8 +593,8 @@ void bn_relu_bwd_sums(Exec &ex, const float *da, Pair t, size_t P, BnRef bn, flo
     const int rows = cdiv(P, ctas);
     bn.part = sums.part; bn.parts = sums.parts; bn.inv_count = sums.inv_count; bn.eps = ex.eps;
     unsigned long long *stamp = ex.stamp_slot();
-    launch(ex, out_cast ? bn_relu_bwd_sums_kernel<true> : bn_relu_bwd_sums_kernel<false>, dim3(cdiv(P, rows)), 256, 0, da, t, (int)P, rows, bn, dgamma, dbeta, (const float *)add.p0, out.p0, out_cast, stamp);
-    ex.check("bn_relu_bwd_apply", (double)P * C * (16 + (out_cast ? 2 : 0)));
+    launch(ex, !add.p0 ? bn_relu_bwd_sums_kernel<false, true> : (out_cast ? bn_relu_bwd_sums_kernel<true, true> : bn_relu_bwd_sums_kernel<true, false>), dim3(cdiv(P, rows)), 256, 0, da, t, (int)P, rows, bn, dgamma, dbeta, (const float *)add.p0, out.p0, out_cast, stamp);
+    ex.check("bn_relu_bwd_apply", (double)P * C * (add.p0 ? 16 + (out_cast ? 2 : 0) : 10));
 }
 
 template <class TO, int V>
