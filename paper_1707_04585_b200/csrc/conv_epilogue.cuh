@@ -25,7 +25,7 @@ struct EpiArgs {
     int pitch;               // floats per staged row: min(N tile, 64) + 4
     // reductions (optional: part == nullptr switches them off; EPI_BNBWD always reduces)
     float *part;             // [gridDim.x][n_cols/4][2][4]: per channel quad, 4 sums then 4 second sums
-    unsigned int *counter;   // zero on entry, left zero
+    unsigned int *counter;   // a word per N tile, zero on entry, left zero
     double inv_count;        // 1 / pixels
     float eps;
     float *mean, *rstd;      // EPI_PLAIN / EPI_COUPLE: statistics of the stored result
@@ -251,7 +251,7 @@ __device__ __forceinline__ void reduce_records(const float *part, int parts, int
 }
 
 template <int NT, class E>
-__device__ __forceinline__ void epilogue_publish(const E &e, float *scratch, int etid);
+__device__ __forceinline__ void epilogue_publish(const E &e, int col0, int BN, float *scratch, int etid);
 
 // After the last tile: per-CTA partials, grid-wide count, and the finalize by the CTA that comes last.
 __device__ __forceinline__ void epilogue_finish(const EpiArgs &e, int BN, int col0, float *stage, const float *sums, int etid) {
@@ -276,51 +276,46 @@ __device__ __forceinline__ void epilogue_finish(const EpiArgs &e, int BN, int co
             *reinterpret_cast<float4 *>(mine + 2 * col + 4) = make_float4(r[4], r[5], r[6], r[7]);
         }
     }
-    epilogue_publish<128>(e, scratch, etid);
+    epilogue_publish<128>(e, col0, BN, scratch, etid);
 }
 
-// Once every CTA has written its partial record into e.part: count, and let the CTA that comes
-// last reduce the records in a fixed order and write the results.  Called by NT threads (etid = 0..NT-1);
-// scratch: (NT + 128) * 32 bytes of shared memory.
+// Once every CTA has written its partial record into e.part: count, and let the CTA that comes last of those of its N tile (blockIdx.y; the
+// columns col0 .. col0 + BN - 1) reduce the records of these columns in a fixed order and write the results.  A counter per N tile: with one
+// for the grid, its last CTA added the records of all columns alone (37 records of 512 channels: 150 KB through one SM) while the others waited.
+// Called by NT threads (etid = 0..NT-1); scratch: (NT + 128) * 32 bytes of shared memory.
 template <int NT, class E>
-__device__ __forceinline__ void epilogue_publish(const E &e, float *scratch, int etid) {
-    // publish, count, and let the last CTA of the grid reduce
-    __threadfence();
+__device__ __forceinline__ void epilogue_publish(const E &e, int col0, int BN, float *scratch, int etid) {
+    unsigned int *flag = reinterpret_cast<unsigned int *>(scratch), *counter = e.counter + blockIdx.y;
     named_barrier(1, NT);
-    unsigned int *flag = reinterpret_cast<unsigned int *>(scratch);
     if (etid == 0) {
-        const unsigned int total = gridDim.x * gridDim.y;
-        const unsigned int old = atomicAdd(e.counter, 1u);
-        *flag = (old == total - 1) ? 1u : 0u;
+        // (one thread's fences, on either side, order what the others wrote before the barrier and read after the next)
+        __threadfence();
+        const bool last = atomicAdd(counter, 1u) == gridDim.x - 1;
+        __threadfence();
+        if (last) *counter = 0u;
+        *flag = last ? 1u : 0u;
     }
     named_barrier(1, NT);
     const bool last = *flag != 0;
     named_barrier(1, NT);
-    if (!last) return;
-    __threadfence();
-    const int C = e.n_cols, R = C >> 1;
+    const int C = e.n_cols, width = C - col0 < BN ? C - col0 : BN;      // (at most 256 columns: 128 slots)
+    if (!last || width <= 0) return;
     double *red = reinterpret_cast<double *>(scratch);            // [NT][4]
     double *tot = red + NT * 4;                                   // [128][4]
-    for (int slot0 = 0; slot0 < R; slot0 += 128) {
-        const int cw = R - slot0 < 128 ? R - slot0 : 128;         // even
-        reduce_records<NT>(e.part, (int)gridDim.x, C, slot0, cw, red, tot, etid);
-        for (int lc = etid; lc < cw * 2; lc += NT) {              // one thread per channel of this slot range
-            const int k = lc >> 2, j = lc & 3;                    // local quad, lane within it
-            const int ch = (slot0 >> 1) * 4 + lc;
-            const double sum = tot[(2 * k) * 4 + j], sum2 = tot[(2 * k + 1) * 4 + j];
-            if (e.mode == EPI_BNBWD) {
-                e.dbeta[ch] = (float)sum; e.dgamma[ch] = (float)sum2;
-                const double gr = (double)e.bn.gamma[ch] * (double)e.bn.rstd[ch];
-                e.coef[ch] = (float)gr; e.coef[C + ch] = (float)(gr * sum * e.inv_count); e.coef[2 * C + ch] = (float)(gr * sum2 * e.inv_count);
-            } else {
-                float m, r;
-                moments_of(sum, sum2, e.inv_count, e.eps, m, r);
-                e.mean[ch] = m; e.rstd[ch] = r;
-            }
+    reduce_records<NT>(e.part, (int)gridDim.x, C, col0 >> 1, width >> 1, red, tot, etid);
+    for (int lc = etid; lc < width; lc += NT) {                   // one thread per channel
+        const int k = lc >> 2, j = lc & 3, ch = col0 + lc;        // local quad, lane within it
+        const double sum = tot[(2 * k) * 4 + j], sum2 = tot[(2 * k + 1) * 4 + j];
+        if (e.mode == EPI_BNBWD) {
+            e.dbeta[ch] = (float)sum; e.dgamma[ch] = (float)sum2;
+            const double gr = (double)e.bn.gamma[ch] * (double)e.bn.rstd[ch];
+            e.coef[ch] = (float)gr; e.coef[C + ch] = (float)(gr * sum * e.inv_count); e.coef[2 * C + ch] = (float)(gr * sum2 * e.inv_count);
+        } else {
+            float m, r;
+            moments_of(sum, sum2, e.inv_count, e.eps, m, r);
+            e.mean[ch] = m; e.rstd[ch] = r;
         }
-        named_barrier(1, NT);
     }
-    if (etid == 0) *e.counter = 0u;
 }
 
 }  // namespace tc

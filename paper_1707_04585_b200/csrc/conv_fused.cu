@@ -86,7 +86,7 @@ struct FusedEpi {
     float *out;            // [P, n_cols]
     float q;               // format of out (and of the coupling partner), or of the BN input of a data gradient: 0 float, else fixed-point step
     float *part;           // per-CTA records of the column sums, or null
-    unsigned int *counter; // null: the records stay pending, their consumer adds them
+    unsigned int *counter; // a word per N tile; null: the records stay pending, their consumer adds them
     double inv_count;
     float eps;
     float *mean, *rstd;
@@ -252,7 +252,8 @@ __device__ __forceinline__ void build_table(const FusedGeom &g, int *tab, int r0
         while (r > g.H) { r -= g.H + 1; n++; }
     }
 }
-template <int IN, int EW>
+// K1: 1x1 layers, where position and pixel are the same and no row is padding.
+template <int IN, int EW, bool K1>
 __device__ __forceinline__ bool build_rows(const FusedGeom &g, const FusedLayer &p, FusedShared *sh, const uint8_t *raw, uint8_t *abuf, int *tab, int pos0, int pos1,
                                            const BuildPlace bp, int lane) {
     constexpr int V = IN == kInBwd ? 4 : 8;               // channels of a thread
@@ -266,7 +267,7 @@ __device__ __forceinline__ bool build_rows(const FusedGeom &g, const FusedLayer 
         const int sb = pos0 + t0 * 128, own = pos1 - sb < T * 128 ? pos1 - sb : T * 128, rows = own + 2 * g.halo;
         const int my_rows = bp.r0 < RS ? rows : 0;
         uint8_t *dst = abuf + (g.nseg == 2 ? (seg & 1) : 0) * g.seg_bytes + (IN == kInBwd ? (it >> 1) * g.plane16 * 16 + (it & 1) * 8 : it * g.plane16 * 16);
-        if (seg > 0) build_table(g, tab, bp.r0, sb - g.halo, rows);
+        if (!K1 && seg > 0) build_table(g, tab, bp.r0, sb - g.halo, rows);
         if (seg >= g.nseg && !warp_wait(&sh->seg_empty[g.nseg == 2 ? (seg & 1) : 0], (uint32_t)((g.nseg == 2 ? seg >> 1 : seg) - 1) & 1u, lane)) return false;
         int l = bp.r0, low = bp.low0, j = 0, ready = 128 + 2 * g.halo;          // ready: rows that the tile to be signalled next needs
         auto signal = [&]() {
@@ -295,14 +296,12 @@ __device__ __forceinline__ bool build_rows(const FusedGeom &g, const FusedLayer 
 #pragma unroll 1
             for (int i = 0; i < g.piece && low < rows; i += RS) {
                 if (l < my_rows) {
-                    int px;
-                    if (g.k == 1) px = sb + l < g.total ? sb + l : -1;
-                    else px = tab[l];
+                    const int px = K1 ? sb + l : tab[l];
                     const uint8_t *s = src + (px - pxs) * g.rowb;
-                    const bool keep = p.a_out && (unsigned)(l - g.halo) < (unsigned)own;
+                    const bool keep = p.a_out && (K1 || (unsigned)(l - g.halo) < (unsigned)own);
                     if constexpr (IN == kInBwd) {
                         uint2 v = make_uint2(0u, 0u);
-                        if (px >= 0) {
+                        if (K1 || px >= 0) {
                             const float4 d4 = *reinterpret_cast<const float4 *>(s), t4 = *reinterpret_cast<const float4 *>(s + (g.raw_bytes >> 1));
                             const float d[4] = {d4.x, d4.y, d4.z, d4.w}, t[4] = {t4.x, t4.y, t4.z, t4.w};
                             float o[4];
@@ -315,7 +314,7 @@ __device__ __forceinline__ bool build_rows(const FusedGeom &g, const FusedLayer 
                         *reinterpret_cast<uint2 *>(dst + l * 16) = v;
                     } else {
                         uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                        if (px >= 0) {
+                        if (K1 || px >= 0) {
                             v = *reinterpret_cast<const uint4 *>(s);
                             if constexpr (IN != kInBf16) {
                                 const uint4 w = *reinterpret_cast<const uint4 *>(s + 16);
@@ -658,15 +657,17 @@ __global__ void __launch_bounds__(EW == 8 ? 640 : fused_threads(EW), 1) conv_fus
             // (all sixteen everywhere: 164-layer step 0.6 % slower)
             if (ok && e.counter) {
                 named_barrier(2, EW * 32);
-                if (EW == 16 && e.n_cols <= 64) epilogue_publish<512>(e, reinterpret_cast<float *>(abuf), etid);
-                else if (warp < 8) epilogue_publish<256>(e, reinterpret_cast<float *>(abuf), etid);
+                if (EW == 16 && e.n_cols <= 64) epilogue_publish<512>(e, col0, g.BN, reinterpret_cast<float *>(abuf), etid);
+                else if (warp < 8) epilogue_publish<256>(e, col0, g.BN, reinterpret_cast<float *>(abuf), etid);
             }
         }
     } else {
-        if (direct) ok = build_rows<kInBf16, EW>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane);
-        else if (p.in_mode == kInFixed) ok = build_rows<kInFixed, EW>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane);
-        else if (p.in_mode == kInFloat) ok = build_rows<kInFloat, EW>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane);
-        else ok = build_rows<kInBwd, EW>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane);
+#define RV_BUILD(IN) ok = g.k == 1 ? build_rows<IN, EW, true>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane) : build_rows<IN, EW, false>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane)
+        if (direct) RV_BUILD(kInBf16);
+        else if (p.in_mode == kInFixed) RV_BUILD(kInFixed);
+        else if (p.in_mode == kInFloat) RV_BUILD(kInFloat);
+        else RV_BUILD(kInBwd);
+#undef RV_BUILD
     }
     if (!ok) atomicExch(&sh->failed, 1u);
     tc_fence_before();
@@ -714,9 +715,11 @@ bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count, int in_mode, 
         s.EW = g.BN == 64 ? 16 : 8;
         g.nacc = g.BN == 64 ? 2 : 4; g.acc_shift = g.BN == 64 ? 1 : 2;
         int ctas = sm_count / s.n_tiles; if (ctas < 1) ctas = 1;
-        // a contiguous range of positions per CTA, a tile at least.  (Half tiles would put a small layer on every SM, but take as long and
-        // leave none to the launches beside it: 110-layer step 4964 -> 4877 us, odd-sized basic block 167 -> 164 with whole ones.)
-        g.chunk = round_up((g.total + ctas - 1) / ctas, 8); if (g.chunk < 128) g.chunk = 128;
+        // A contiguous range of positions per CTA, a tile at least.  (Half tiles would put a small layer on every SM, but take as long and
+        // leave none to the launches beside it: 110-layer step 4964 -> 4877 us, odd-sized basic block 167 -> 164 with whole ones.)  A layer
+        // of so few tiles that half ones leave half of the SMs takes those: 64 channels, 10 images of 22x8, forward 20.6 -> 19.2 us.
+        const int least_chunk = tiles * 4 * s.n_tiles <= sm_count ? 64 : 128;
+        g.chunk = round_up((g.total + ctas - 1) / ctas, 8); if (g.chunk < least_chunk) g.chunk = least_chunk;
         s.ctas = (g.total + g.chunk - 1) / g.chunk;
         g.wtile_bytes = (g.BN * g.KC * 2 + 1023) & ~1023;
         const int T = (g.chunk + 127) / 128, fixed = 1024 + k * k * g.wtile_bytes + (int)sizeof(FusedShared) + 64;
@@ -840,7 +843,7 @@ bool run_fused(Exec &ex, const char *what, int in_mode, const void *in, float in
         FusedEpi &e = p.epi;
         e.mode = req.bnbwd ? EPI_BNBWD : (sign ? EPI_COUPLE : EPI_PLAIN);
         e.out = out.p0; e.q = req.bnbwd ? req.bnbwd->t.q : out.q; e.sign = sign; e.n_cols = cout;
-        e.part = part; e.counter = (reduce && !defer && !sums) ? ex.ctx->counter() : nullptr;
+        e.part = part; e.counter = (reduce && !defer && !sums) ? ex.ctx->counter(s.n_tiles) : nullptr;
         e.inv_count = 1.0 / (double)geo.P(); e.eps = ex.eps;
         if (req.stats) { e.mean = req.stats->mean; e.rstd = req.stats->rstd; }
         if (req.bnbwd) { e.bn = req.bnbwd->bn; e.dgamma = req.bnbwd->dgamma; e.dbeta = req.bnbwd->dbeta; e.coef = req.bnbwd->coef; }

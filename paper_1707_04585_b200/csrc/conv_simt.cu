@@ -672,7 +672,7 @@ __global__ void splitk_reduce_kernel(const float *__restrict__ part, size_t n, i
 // buffers; the slices' sums are added through shared memory at the end, in order, and the CTAs' by splitk_reduce_kernel.
 // A lane's sum runs over its slice of the CTA's pixels: 64 products for 16 channels at 32x32 as for 56 at 8x8.
 // Bound by the FMA pipes, and by launch, first copies and the two reductions for a third of the time.  Measured by events at batch 128: 16
-// channels at 32x32 57.9 -> 26.7 us, 32 at 16x16 33.7 -> 28.7, 56 at 8x8 24.6 -> 23 against the implicit GEMM; fp32 step of the
+// channels at 32x32 57.9 -> 26.7 us, 32 at 16x16 33.7 -> 28.7, 56 at 8x8 24.6 -> 24.5 against the implicit GEMM; fp32 step of the
 // 38-layer network 5.61 -> 5.21 ms.
 struct WgStrip {
     int N, H, W, Ci, Co;

@@ -341,9 +341,9 @@ __device__ __forceinline__ void tma_epilogue(const TcParams &p, TcShared *sh, co
     // records); without a counter the records stay pending and their consumer adds them
     if (ok && e.counter) {
         float *scratch = reinterpret_cast<float *>(auxr + (many ? 0 : NG * 4096));
-        if (NG == 4) epilogue_publish<512>(e, scratch, wg * 128 + etid);
-        else if (NG == 2) epilogue_publish<256>(e, scratch, wg * 128 + etid);
-        else if (wg == 0) epilogue_publish<128>(e, scratch, etid);
+        if (NG == 4) epilogue_publish<512>(e, col0, p.BN, scratch, wg * 128 + etid);
+        else if (NG == 2) epilogue_publish<256>(e, col0, p.BN, scratch, wg * 128 + etid);
+        else if (wg == 0) epilogue_publish<128>(e, col0, p.BN, scratch, etid);
     }
     if (etid == 0) tma_store_wait_all();
 }
@@ -1200,7 +1200,7 @@ bool run_conv_tc(Exec &ex, const char *what, const void *act, Geom gin, int cin,
         memset(&e, 0, sizeof e);
         e.mode = req.bnbwd ? EPI_BNBWD : (sign ? EPI_COUPLE : EPI_PLAIN);
         e.out = out; e.partner = partner; e.sign = sign; e.n_cols = cout; e.pitch = kEpiPitch;
-        e.part = part; e.counter = reduce && !defer ? ex.ctx->counter() : nullptr;
+        e.part = part; e.counter = reduce && !defer ? ex.ctx->counter(s.n_tiles) : nullptr;
         e.inv_count = 1.0 / ((double)g.P() * ostride * ostride); e.eps = ex.eps;     // pixels of the output grid
         if (req.stats) { e.mean = req.stats->mean; e.rstd = req.stats->rstd; }
         if (req.bnbwd) { e.t = req.bnbwd->t; e.bn = req.bnbwd->bn; e.dgamma = req.bnbwd->dgamma; e.dbeta = req.bnbwd->dbeta; e.coef = req.bnbwd->coef; }
