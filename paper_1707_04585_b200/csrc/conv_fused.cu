@@ -25,7 +25,7 @@
 //               them add the statistics records of the kernel before (BnRef::part).
 //   1 warp      weights (TMA, resident), tensor memory, MMA issue; two or four accumulators
 //   1 warp      the input's pieces and the first partner rows
-//   6 warps     build: a row's 8 channels from shared memory, scale*x + shift, ReLU, bf16 rounding, one 16-byte store to the operand
+//   6 warps     (or 10) build: a row's 8 channels from shared memory, scale*x + shift, ReLU, bf16 rounding, one 16-byte store to the operand
 //               (and one to the activated tensor the weight gradient will read)
 // The same kernel computes data gradients: its input is then the bf16 upstream gradient, taken as it is, or (kInBwd) the gradient and
 // the BN input of the layer behind, whose BN + ReLU backward the build applies; the weights are the mirrored, transposed pack.
@@ -52,8 +52,7 @@ constexpr int kAuxSlots = 8;              // most tiles of an epilogue warp's pa
 constexpr int kAccBufs = 4;               // most accumulators
 constexpr int NC = 16;                    // columns per epilogue thread
 constexpr int kAuxBytes = 32 * NC * 4;    // partner rows of an epilogue warp's part of a tile: 32 rows x 64 bytes
-constexpr int NBT = 192;                  // build threads
-__host__ __device__ constexpr int fused_threads(int EW) { return EW * 32 + 64 + NBT; }
+__host__ __device__ constexpr int fused_threads(int EW, int NBT) { return EW * 32 + 64 + NBT; }      // NBT: build threads
 
 // What all layers of a launch share
 struct FusedGeom {
@@ -253,7 +252,7 @@ __device__ __forceinline__ void build_table(const FusedGeom &g, int *tab, int r0
     }
 }
 // K1: 1x1 layers, where position and pixel are the same and no row is padding.
-template <int IN, int EW, bool K1>
+template <int IN, int EW, int NBT, bool K1>
 __device__ __forceinline__ bool build_rows(const FusedGeom &g, const FusedLayer &p, FusedShared *sh, const uint8_t *raw, uint8_t *abuf, int *tab, int pos0, int pos1,
                                            const BuildPlace bp, int lane) {
     constexpr int V = IN == kInBwd ? 4 : 8;               // channels of a thread
@@ -456,10 +455,10 @@ __device__ __forceinline__ void column_sums(float (&a)[NC], int lane) {
     a[0] += __shfl_xor_sync(0xffffffffu, a[0], 16);
 }
 
-// Registers: with eight epilogue warps 96 for 512 threads (the bound of 640 asks for that), which leaves an SM room for a CTA of
-// the weight gradients (72 for 192 threads) that run on another stream.
-template <int EW>
-__global__ void __launch_bounds__(EW == 8 ? 640 : fused_threads(EW), 1) conv_fused_kernel(const __grid_constant__ FusedArgs A) {
+// Registers: with eight epilogue warps 96 for 512 or 640 threads; of 512 (the bound asks for it) that leaves an SM room for a CTA of the
+// weight gradients (72 for 192 threads) that run on another stream.
+template <int EW, int NBT>
+__global__ void __launch_bounds__(EW == 8 ? 640 : fused_threads(EW, NBT), 1) conv_fused_kernel(const __grid_constant__ FusedArgs A) {
     extern __shared__ uint8_t smem_raw[];
     const FusedGeom &g = A.g;
     const FusedLayer &p = A.ly;
@@ -662,7 +661,7 @@ __global__ void __launch_bounds__(EW == 8 ? 640 : fused_threads(EW), 1) conv_fus
             }
         }
     } else {
-#define RV_BUILD(IN) ok = g.k == 1 ? build_rows<IN, EW, true>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane) : build_rows<IN, EW, false>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane)
+#define RV_BUILD(IN) ok = g.k == 1 ? build_rows<IN, EW, NBT, true>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane) : build_rows<IN, EW, NBT, false>(g, p, sh, raw, abuf, tab, pos0, pos1, bp, lane)
         if (direct) RV_BUILD(kInBf16);
         else if (p.in_mode == kInFixed) RV_BUILD(kInFixed);
         else if (p.in_mode == kInFloat) RV_BUILD(kInFloat);
@@ -682,7 +681,7 @@ __global__ void __launch_bounds__(EW == 8 ? 640 : fused_threads(EW), 1) conv_fus
 
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
-struct FusedShape { int n_tiles, ctas, smem, EW; FusedGeom g; };
+struct FusedShape { int n_tiles, ctas, smem, EW, NBT; FusedGeom g; };
 
 // aux: the epilogue reads a partner tensor.  The CTAs' ranges depend on geo, cin, cout, k and sm_count alone wherever the memory suffices.
 bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count, int in_mode, bool aux, FusedShape &s) {
@@ -695,21 +694,17 @@ bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count, int in_mode, 
     if (total >= (1u << 30)) return false;
     g.N = geo.N; g.H = geo.H; g.W = geo.W; g.P = (int)geo.P(); g.pitch = geo.W + 1;
     g.dpitch = fast_div(geo.W + 1); g.drows = fast_div(geo.H + 1);
-    g.nit = in_mode == kInBwd ? 2 * g.nch : g.nch; g.RS = NBT / g.nit; g.dnit = fast_div(g.nit);
-    g.step_r = g.RS / g.pitch; g.step_c = g.RS % g.pitch;
+    g.nit = in_mode == kInBwd ? 2 * g.nch : g.nch; g.dnit = fast_div(g.nit);
     g.halo = k == 3 ? geo.W + 2 : 0;
     g.total = (int)total;
     // pieces of about 12 KB
     const int tensors = in_mode == kInBwd ? 2 : 1;
     g.rowb = cin * (in_mode == kInBf16 ? 2 : 4);
-    int piece = g.RS;
-    while (2 * piece * g.rowb * tensors <= 12800) piece *= 2;
     const int cout_pad = round_up(cout, 16), tiles = (g.total + 127) / 128, nchp = (g.nch + 1) & ~1;
     g.BN = cout_pad <= 16 ? 16 : (cout_pad <= 32 ? 32 : 64);
     // few tiles (late stages): split the output channels so that more SMs take part
     while (g.BN > 16 && tiles * ((cout_pad + g.BN - 1) / g.BN) * 2 <= sm_count) g.BN /= 2;
     for (;; g.BN /= 2) {
-        g.piece = piece; g.raw_bytes = round_up(piece * g.rowb, 128) * tensors;
         s.n_tiles = (cout_pad + g.BN - 1) / g.BN;
         g.groups = g.BN / NC;
         s.EW = g.BN == 64 ? 16 : 8;
@@ -721,6 +716,14 @@ bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count, int in_mode, 
         const int least_chunk = tiles * 4 * s.n_tiles <= sm_count ? 64 : 128;
         g.chunk = round_up((g.total + ctas - 1) / ctas, 8); if (g.chunk < least_chunk) g.chunk = least_chunk;
         s.ctas = (g.total + g.chunk - 1) / g.chunk;
+        // Six build warps, or ten where a CTA has a tile at most and so waits for its build (24 channels, 8 images of 9x17, forward: 19.7 against 18.8 us);
+        // with more tiles they cost the epilogue beside them more than they give (16 channels, 14 images of 47x44: 21.6 against 22.6 us), and beside sixteen
+        // epilogue warps there are no registers for them.
+        s.NBT = s.EW == 8 && g.chunk <= 128 ? 320 : 192;
+        g.RS = s.NBT / g.nit; g.step_r = g.RS / g.pitch; g.step_c = g.RS % g.pitch;
+        g.piece = g.RS;
+        while (2 * g.piece * g.rowb * tensors <= 12800) g.piece *= 2;
+        g.raw_bytes = round_up(g.piece * g.rowb, 128) * tensors;
         g.wtile_bytes = (g.BN * g.KC * 2 + 1023) & ~1023;
         const int T = (g.chunk + 127) / 128, fixed = 1024 + k * k * g.wtile_bytes + (int)sizeof(FusedShared) + 64;
         const int aux1 = aux ? s.EW * kAuxBytes : 0, sets = s.EW / 4 / g.groups, own_tiles = (T + sets - 1) / sets;
@@ -849,12 +852,12 @@ bool run_fused(Exec &ex, const char *what, int in_mode, const void *in, float in
         if (req.bnbwd) { e.bn = req.bnbwd->bn; e.dgamma = req.bnbwd->dgamma; e.dbeta = req.bnbwd->dbeta; e.coef = req.bnbwd->coef; }
         static OncePerDevice once;
         if (once.first(ex.ctx->device)) {
-            cudaFuncSetAttribute(conv_fused_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-            cudaFuncSetAttribute(conv_fused_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+            cudaFuncSetAttribute(conv_fused_kernel<16, 192>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+            cudaFuncSetAttribute(conv_fused_kernel<8, 192>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+            cudaFuncSetAttribute(conv_fused_kernel<8, 320>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         }
         dim3 grid((unsigned)ctas, (unsigned)s.n_tiles);
-        const int EW = s.EW;
-        launch(ex, EW == 16 ? conv_fused_kernel<16> : conv_fused_kernel<8>, grid, fused_threads(EW), s.smem, A);
+        launch(ex, s.EW == 16 ? conv_fused_kernel<16, 192> : (s.NBT == 320 ? conv_fused_kernel<8, 320> : conv_fused_kernel<8, 192>), grid, fused_threads(s.EW, s.NBT), s.smem, A);
         const double bytes = (double)geo.P() * cin * (in_mode == kInBf16 ? 2 : (in_mode == kInBwd ? 8 : 4)) + (double)geo.P() * cout * (sign || req.bnbwd ? 8 : 4) +
                              (double)cout * taps * cin * 2 + (a_out ? (double)geo.P() * cin * 2 : 0.0);
         ex.check(what, bytes, 2.0 * geo.P() * cout * cin * taps);
@@ -893,7 +896,7 @@ bool conv_dgrad_fused_takes(Exec &ex, Geom gi, const Layer &L, bool behind) {
     // Through the BN backward only where a build thread has few rows: its pass costs 0.3 us per row and thread, twice that of a bf16 input with
     // twice the threads per row, against 5 us for the launch that it saves.  Odd-sized block (24 channels, a tile per CTA, five and a half rows)
     // 151 -> 144.5 us; 56 channels at 8x8 (eleven rows) and 16 at 32x32 (twenty-one): 38-layer step 1665 -> 1686.
-    return !behind || (long long)(s.g.chunk + 2 * s.g.halo) * s.g.nit <= 6 * NBT;
+    return !behind || (long long)(s.g.chunk + 2 * s.g.halo) * s.g.nit <= 6 * 192;
 }
 
 // The same where the gradient still has to go through the BN + ReLU backward of the layer behind L: g is da of that layer (float), `behind` its
