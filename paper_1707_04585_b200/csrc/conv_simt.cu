@@ -7,7 +7,7 @@
 //   wgrad: dW[co,kh,kw,ci] = sum_p g[p,co] * a[p (+) (kh,kw), ci]
 //
 // Four kernels.  conv3x3_direct_kernel takes fp32 3x3 stride-1 layers (forward and data gradient), wgrad3x3_strip_kernel the weight
-// gradients of those of at most 64 channels, conv_gemm_kernel every other layer whose channel counts are multiples of four (all BN-ReLU-conv layers): quads of channels are loaded as vectors, a thread's pixel is decoded once, and the product is register-tiled.
+// gradients of those of at most 48, conv_gemm_kernel every other layer whose channel counts are multiples of four (all BN-ReLU-conv layers): quads of channels are loaded as vectors, a thread's pixel is decoded once, and the product is register-tiled.
 // gemm_simt_kernel loads element by element and is left for the stem convolution's odd channel counts (an image has
 // three), where the kernels of stem.cu do not take its size.
 #include "common.cuh"
@@ -663,17 +663,17 @@ __global__ void splitk_reduce_kernel(const float *__restrict__ part, size_t n, i
 }
 
 // ------------------------------------------------------------------ weight gradient of fp32 3x3 stride-1 layers
-// dW[co, (kh, kw), ci] = sum over pixels of g[y, x, co] a[y + kh - 1, x + kw - 1, ci], of at most 64 channels either way.
+// dW[co, (kh, kw), ci] = sum over pixels of g[y, x, co] a[y + kh - 1, x + kw - 1, ci], of at most 48 x 48 channels.
 // A lane keeps four input channels x four output channels x the three column taps of one row tap: walking along a row of the image
 // it reads one new quad of either tensor per pixel (the window of three input quads slides in registers) for 48 FMAs, where the
 // implicit GEMM above reads three per 32 and works out the pixel of every quad that it stages.
 // Warps: 3 row taps x nb blocks of 32 (input quad, output quad) pairs x R groups of rows; with at most 16 pairs a warp holds sl rows of
 // them.  The rows of a strip (BH rows of an image, and the halo rows of the input) arrive by asynchronous copies in two
 // buffers; the slices' sums are added through shared memory at the end, in order, and the CTAs' by splitk_reduce_kernel.
-// A lane's sum runs over its slice of the CTA's pixels: 64 products for 16 channels at 32x32 as for 56 at 8x8.
+// A lane's sum runs over its slice of the CTA's pixels: 64 products for 16 channels at 32x32.
 // Bound by the FMA pipes, and by launch, first copies and the two reductions for a third of the time.  Measured by events at batch 128: 16
-// channels at 32x32 57.9 -> 26.7 us, 32 at 16x16 33.7 -> 28.7, 56 at 8x8 24.6 -> 24.5 against the implicit GEMM; fp32 step of the
-// 38-layer network 5.61 -> 5.21 ms.
+// channels at 32x32 57.9 -> 26.7 us, 32 at 16x16 33.7 -> 28.7 against the implicit GEMM; fp32 step of the
+// 38-layer network 5.61 -> 5.15 ms.
 struct WgStrip {
     int N, H, W, Ci, Co;
     int cq, oq, pairs, sl, nb, R;         // quads per pixel, pairs of quads; slices per warp, blocks of pairs, row groups
@@ -681,7 +681,10 @@ struct WgStrip {
     int a_floats, g_floats;               // of a buffer
     FastDiv dcq, dw2, dpairs, dimg, dnb;  // by cq, by W + 2, by pairs, by per_img, by nb
 };
-constexpr int kWgStripThreads = 768;      // most threads of a CTA
+constexpr int kWgStripThreads = 768;      // (at most 480 are launched; the bound keeps the kernel at 80 registers, two CTAs of 384 threads per SM)
+// Most pairs of quads.  Above (56 channels and more) no two warps share a row and the implicit GEMM is as quick or quicker: 56 channels at
+// 8x8, batch 128, 24.6 against 24.5 us; fp32 stored step of the 110-layer network at batch 23 7.42 against 7.74 ms.
+constexpr int kWgStripPairs = 144;
 constexpr int kWgStripRun = 512;          // most products of one lane's sum (the error of a serial sum grows with it; see the runs of the implicit GEMM)
 __device__ __forceinline__ void cp_async16(float *dst, const float *src, bool ok) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");
@@ -802,18 +805,25 @@ static bool wg_strip_shape(const ConvGeom &g, int sm, WgStrip &p, int &ctas, int
     if (g.k != 3 || g.s != 1 || g.Ci % 4 || g.Co % 4 || g.Ci > 64 || g.Co > 64 || g.W > kWgStripRun) return false;
     p.N = g.N; p.H = g.H; p.W = g.W; p.Ci = g.Ci; p.Co = g.Co;
     p.cq = g.Ci / 4; p.oq = g.Co / 4; p.pairs = p.cq * p.oq;
+    if (p.pairs > kWgStripPairs) return false;
     p.sl = p.pairs <= 16 ? 32 / p.pairs : 1;
     p.nb = p.sl > 1 ? 1 : (p.pairs + 31) / 32;
     if (p.sl > p.H) p.sl = p.H;
     p.R = 4 / p.nb < 1 ? 1 : 4 / p.nb;               // about twelve warps
-    while (p.R > 1 && p.R * p.sl > p.H) p.R--;
+    while (p.R > 1 && (p.R * p.sl > p.H || p.N * ((p.H + p.R * p.sl - 1) / (p.R * p.sl)) < sm)) p.R--;      // (few images: smaller CTAs)
     threads = 96 * p.nb * p.R;
     const int slices = p.R * p.sl;
     // strips: as many rows, a multiple of the slices, as two CTAs per SM have room for in two buffers; a strip of one round of the slices at least
     auto floats = [&](int bh) { return (size_t)(bh + 2) * (g.W + 2) * g.Ci + (size_t)bh * g.W * g.Co; };
-    p.BH = slices;
-    while (p.BH < p.H && 2 * floats(p.BH + slices) * 4 <= 100 * 1024 && (p.BH / slices + 1) * g.W <= kWgStripRun) p.BH += slices;
-    if (p.BH > p.H) p.BH = p.H;
+    // (of these the height that gives a CTA the fewest rows, its strips' halos counted as one each)
+    const int room = sm * (threads <= 384 ? 2 : 1);
+    long long best = -1;
+    for (int bh = slices;; bh += slices) {
+        const int h = bh < p.H ? bh : p.H, strips = p.N * ((p.H + h - 1) / h);
+        const long long cost = (long long)((strips + room - 1) / room) * (h + 1);
+        if (best < 0 || cost <= best) { best = cost; p.BH = h; }
+        if (h == p.H || 2 * floats(bh + slices) * 4 > 100 * 1024 || (bh / slices + 1) * g.W > kWgStripRun) break;
+    }
     p.a_floats = (p.BH + 2) * (g.W + 2) * g.Ci; p.g_floats = p.BH * g.W * g.Co;
     size_t bytes = 2 * floats(p.BH) * 4;
     const size_t red = slices > 1 ? (size_t)slices * 9 * g.Ci * g.Co * 4 : 0;
@@ -821,9 +831,9 @@ static bool wg_strip_shape(const ConvGeom &g, int sm, WgStrip &p, int &ctas, int
     if (bytes > 200 * 1024) return false;
     smem = (int)bytes;
     p.per_img = (p.H + p.BH - 1) / p.BH; p.strips = p.N * p.per_img;
-    // as many CTAs as two per SM (one, where they do not fit), with the same number of strips each
-    const int room = sm * (threads <= 384 && smem <= 112 * 1024 ? 2 : 1);
-    p.per_cta = (p.strips + room - 1) / room;
+    // as many CTAs as there is room for, with the same number of strips each
+    const int fit = smem <= 112 * 1024 ? room : sm;
+    p.per_cta = (p.strips + fit - 1) / fit;
     const int run = (p.BH + slices - 1) / slices * g.W;              // products of a lane's sum per strip
     if (p.per_cta * run > kWgStripRun) p.per_cta = kWgStripRun / run;
     ctas = (p.strips + p.per_cta - 1) / p.per_cta;

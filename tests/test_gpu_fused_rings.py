@@ -38,7 +38,8 @@ def test_fused_layers_at_ring_edges(ctx, kind, N, H, W, c, w):
     ("basic", 3, 1, 7, 4),                # one row: one slice
     ("basic", 150, 17, 16, 16),           # several strips per CTA, the last strip of an image one row
     ("basic", 5, 6, 9, 44),               # 121 pairs in four blocks, the last of 25
-    ("basic", 2, 3, 31, 64),              # 24 warps
+    ("basic", 2, 3, 31, 48),              # the most pairs that it takes: five blocks, 15 warps
+    ("basic", 2, 3, 31, 52),              # one quad more: the implicit GEMM
 ])
 def test_strict_weight_gradient_strips(ctx, kind, N, H, W, c):
     tp.run_block_case(ctx, syn.BlockCfg(N, H, W, c, 0, kind, seed=800 + c), 1, jitter=True, inplace=True)
