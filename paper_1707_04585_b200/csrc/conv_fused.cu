@@ -176,10 +176,13 @@ __device__ __forceinline__ void load_piece(const FusedGeom &g, const FusedLayer 
 }
 
 // The build of a CTA's operand rows.  A thread keeps its channels (eight; kInBwd: four) and takes rows r0, r0 + RS, ... of each
-// segment.  The pixels of its rows (-1: padding) stand in a table that it fills itself, for the first segment while the kernel
-// before this one still runs: six build warps are one or two per scheduler, so every instruction between a row's load and its
+// segment.  The pixels of its rows (-1: padding) stand in a table, for the first segment filled while the kernel before this one
+// still runs: six build warps are one or two per scheduler, so every instruction between a row's load and its
 // store costs its full latency.  One row per iteration: a loop that outgrows the scheduler's instruction buffer is slower than a
 // short one with nothing in flight.
+// The nit threads of a row write the same entry.  Where nit does not divide 32 they can sit in two warps, and one warp may be a segment
+// ahead of the other: segments in two buffers then have a table each, filled behind the wait for the segment's buffer.  That wait
+// ends when the MMAs have read the segment that had the buffer before, so every warp has built all its rows and left its table.
 struct BuildPlace { int item, r0, low0; };
 __device__ __forceinline__ BuildPlace build_place(const FusedGeom &g, int bt) {
     BuildPlace b;
@@ -214,8 +217,9 @@ __device__ __forceinline__ bool build_rows(const FusedGeom &g, const FusedLayer 
         const int sb = pos0 + t0 * 128, own = pos1 - sb < T * 128 ? pos1 - sb : T * 128, rows = own + 2 * g.halo;
         const int my_rows = bp.r0 < RS ? rows : 0;
         uint8_t *dst = abuf + (g.nseg == 2 ? (seg & 1) : 0) * g.seg_bytes + (IN == kInBwd ? (it >> 1) * g.plane16 * 16 + (it & 1) * 8 : it * g.plane16 * 16);
-        if (!K1 && seg > 0) build_table(g, tab, bp.r0, sb - g.halo, rows);
         if (seg >= g.nseg && !warp_wait(&sh->seg_empty[g.nseg == 2 ? (seg & 1) : 0], (uint32_t)((g.nseg == 2 ? seg >> 1 : seg) - 1) & 1u, lane)) return false;
+        int *const place = tab + (g.tabs == 2 && (seg & 1) ? g.tab_bytes >> 2 : 0);
+        if (!K1 && seg > 0) build_table(g, place, bp.r0, sb - g.halo, rows);
         int l = bp.r0, low = bp.low0, j = 0, ready = 128 + 2 * g.halo;          // ready: rows that the tile to be signalled next needs
         auto signal = [&]() {
             fence_proxy_async();
@@ -243,7 +247,7 @@ __device__ __forceinline__ bool build_rows(const FusedGeom &g, const FusedLayer 
 #pragma unroll 1
             for (int i = 0; i < g.piece && low < rows; i += RS) {
                 if (l < my_rows) {
-                    const int px = K1 ? sb + l : tab[l];
+                    const int px = K1 ? sb + l : place[l];
                     const uint8_t *s = src + (px - pxs) * g.rowb;
                     const bool keep = p.a_out && (K1 || (unsigned)(l - g.halo) < (unsigned)own);
                     if constexpr (IN == kInBwd) {
@@ -417,7 +421,7 @@ __global__ void __launch_bounds__(EW == 8 ? 640 : fused_threads(EW, NBT), 1) con
     uint8_t *abuf = auxb + EW * g.aux_slots * kAuxBytes;
     uint8_t *raw = abuf + g.op_bytes;
     int *tab = (int *)(raw + g.raw_slots * g.raw_bytes);
-    FusedShared *sh = (FusedShared *)((uint8_t *)tab + g.tab_bytes);
+    FusedShared *sh = (FusedShared *)((uint8_t *)tab + g.tabs * g.tab_bytes);
 
     constexpr int kMmaWarp = EW, kLoadWarp = EW + 1, kBuildWarp0 = EW + 2;
     const int warp = warp_index(), lane = threadIdx.x & 31;

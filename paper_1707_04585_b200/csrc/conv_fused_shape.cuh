@@ -30,7 +30,7 @@ struct FusedGeom {
     int chunk;             // positions per CTA
     int S, nseg;           // tiles per operand segment, segment buffers (1 or 2)
     int plane16, seg_bytes, op_bytes;     // plane stride in 16-byte units; bytes of a segment buffer, of the whole operand region
-    int tab_bytes;         // 3x3: the build's table of pixels, one entry per row of a segment
+    int tab_bytes, tabs;   // 3x3: the build's table of pixels, one entry per row of a segment; tables (see build_table)
     int pps, pieces;       // pieces per full segment, in all
     int piece, rowb;       // positions per piece of the input (a multiple of RS), bytes of a pixel of one input tensor
     int raw_bytes, raw_slots;             // bytes of a piece's slot, slots
@@ -113,9 +113,10 @@ static inline bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count,
         const int room = 227 * 1024 - fixed, least = 20480;      // least: the last reduction borrows the operand region, (512 + 128) x 4 doubles
         // the whole range as one segment if it fits, else the longest segments of which two fit; beside them two pieces of the
         // input and, for each epilogue warp, one tile's partner rows at least
+        auto tabs_of = [&](int nseg) { return nseg == 2 && 32 % g.nit != 0 ? 2 : 1; };
         auto fits = [&](int S, int nseg) {
             const int op = nseg * seg_of(S);
-            return (op < least ? least : op) + (T <= S && pieces_of(S) < 2 ? 1 : 2) * g.raw_bytes + aux1 + tab_of(S) <= room;
+            return (op < least ? least : op) + (T <= S && pieces_of(S) < 2 ? 1 : 2) * g.raw_bytes + aux1 + tabs_of(nseg) * tab_of(S) <= room;
         };
         // (1x1: no halo to build twice, short segments leave the room to the rings)
         if (T <= (k == 1 ? 2 : kFullBars) && fits(T, 1)) { g.S = T; g.nseg = 1; }
@@ -128,7 +129,8 @@ static inline bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count,
         g.seg_bytes = seg_of(g.S);
         g.op_bytes = g.nseg * g.seg_bytes;
         if (g.op_bytes < least) g.op_bytes = least;
-        g.tab_bytes = tab_of(g.S);
+        g.tab_bytes = tab_of(g.S); g.tabs = tabs_of(g.nseg);
+        const int tab = g.tabs * g.tab_bytes;
         g.pps = pieces_of(g.S); g.dpps = fast_div(g.pps);
         g.pieces = T <= g.S ? g.pps : 2 * kRawSlots;        // (more than the ring holds, or counted as if)
         // what is left goes to more pieces and more partner rows in flight, whichever has less
@@ -137,14 +139,14 @@ static inline bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count,
         if (T <= g.S) {
             const int rows = g.chunk + 2 * g.halo, first = 128 + 2 * g.halo, half = (rows + 1) / 2;
             const int R = round_up(half < first && first < rows ? first : half, g.RS), bytes = round_up(R * g.rowb, 128) * tensors;
-            if (R > g.piece && g.op_bytes + g.tab_bytes + (R >= rows ? 1 : 2) * bytes + 2 * aux1 <= room) {
+            if (R > g.piece && g.op_bytes + tab + (R >= rows ? 1 : 2) * bytes + 2 * aux1 <= room) {
                 g.piece = R; g.raw_bytes = bytes; g.pps = g.pieces = pieces_of(g.S); g.dpps = fast_div(g.pps);
             }
         }
         const int most_raw = T <= g.S ? (pieces_of(g.S) < kRawSlots ? pieces_of(g.S) : kRawSlots) : kRawSlots;
         const int most_aux = !aux ? 0 : (own_tiles < kAuxSlots ? own_tiles : kAuxSlots);
         g.raw_slots = most_raw < 2 ? most_raw : 2; g.aux_slots = aux ? 1 : 0;
-        int left = room - g.op_bytes - g.tab_bytes - g.raw_slots * g.raw_bytes - g.aux_slots * aux1;
+        int left = room - g.op_bytes - tab - g.raw_slots * g.raw_bytes - g.aux_slots * aux1;
         s.smem = 227 * 1024 - left;
         if (left >= 0 && g.plane16 < (1 << 14)) {
             while (true) {

@@ -1,9 +1,11 @@
 """Fused BN-ReLU-conv layers (and, in the strict mode, the weight gradient in strips of image rows) at the sizes where their rings of input pieces and partner rows, their operand segments and the
 pass of a gradient through the BN backward of the layer behind begin and end.  Compared with the float64 oracle under the
 stated tolerances (bf16 mode: 2e-2 outputs, 5e-2 gradients; strict mode: 1e-4), which bound rounding at these sizes."""
+import numpy as np
 import pytest
 
 from paper_1707_04585_b200 import binding as B
+from paper_1707_04585_b200 import runner as R
 from paper_1707_04585_b200 import synthetic as syn
 from tests import test_gpu_parity as tp
 
@@ -24,13 +26,42 @@ def ctx():
     ("basic", 3, 5, 78, 16, 0),           # the largest halo for which it does (six rows per build thread), and
     ("basic", 3, 5, 79, 16, 0),           # one size on, where it does not
     ("basic", 150, 33, 31, 16, 0),        # nine tiles per CTA: the range as one segment, the partner ring goes round
-    ("basic", 64, 32, 32, 64, 0),         # two operand segments in turn, two pieces of the input in flight
+    ("basic", 64, 32, 32, 64, 0),         # four tiles per CTA as one segment, two pieces of the input in flight
     ("basic", 3, 40, 150, 48, 0),         # long rows: a halo of 152 rows, six planes
     ("single", 9, 30, 33, 40, 0),         # one layer per function: sums of the only layer left to the last step
     ("bottleneck", 64, 32, 32, 128, 32),  # 1x1 onto 128 columns: many tiles per CTA in segments of two, both rings go round
 ])
 def test_fused_layers_at_ring_edges(ctx, kind, N, H, W, c, w):
     tp.run_block_case(ctx, syn.BlockCfg(N, H, W, c, w, kind, seed=700 + c), 0, jitter=True, inplace=True)
+
+
+# 3x3 layers whose CTAs take their range in several operand segments, two buffers in turn (tests/test_fused_shapes_host.py holds the last
+# number, their segments, against the launch geometry).  With 24, 40, 48 and 56 channels the threads of a row sit in two warps
+SEGMENTED = [
+    ("single", 3, 133, 485, 24, 11),
+    ("basic", 3, 226, 119, 40, 5),
+    ("single", 37, 46, 64, 48, 3),
+    ("basic", 7, 114, 77, 56, 4),
+    ("single", 100, 24, 30, 64, 3),
+]
+
+
+@pytest.mark.parametrize("kind,N,H,W,c,segments", SEGMENTED)
+def test_segments_in_turn(ctx, kind, N, H, W, c, segments):
+    tp.run_block_case(ctx, syn.BlockCfg(N, H, W, c, 0, kind, seed=750 + c), 0, jitter=True, inplace=True)
+
+
+def test_segments_in_turn_give_the_same_bits_every_time(ctx):
+    b = syn.BlockCfg(3, 226, 119, 40, 0, "single", seed=790)
+    r, inp = R.BlockRunner(ctx, b, 0), syn.make_block_inputs(b)
+    r.load(inp["params"])
+    first = None
+    for _ in range(8):
+        y1, y2 = r.forward(inp["x1"], inp["x2"])
+        x1, x2, dx1, dx2, grads = r.backward(y1, y2, inp["dy1"], inp["dy2"])
+        out = dict(grads, y1=y1, y2=y2, x1=x1, x2=x2, dx1=dx1, dx2=dx2)
+        first = first or out
+        assert all(np.array_equal(out[k], first[k]) for k in first)
 
 
 @pytest.mark.parametrize("kind,N,H,W,c", [
