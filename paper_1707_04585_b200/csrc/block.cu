@@ -250,8 +250,9 @@ void block_backward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const 
                     Moments *m1_out, bool overlap, const LateWgrad *late) {
     FnSaved svG, svF;
     const float q = ex.q;   // format of the coupling state; gradients are always float
-    // a block called by itself: the weight gradients of G run on beside F (joined with F's)
-    const bool late_g = late || (ex.mode == 0 && g.P() * c <= kLateWgradElems);
+    // (a block called by itself joins the weight gradients of each function at its end: whether F's run on the side stream as well is F's own
+    // affair, so nothing later would be sure to wait for G's)
+    const bool late_g = late != nullptr;
     size_t m0 = ex.ws.mark();
     if (!m1_out) m1_out = m1;
     // F may be recomputed beside G's gradient steps only if it leaves y1 and its statistics alone

@@ -41,6 +41,47 @@ def test_prepacked_weights_give_the_same_bits(kind, N, H, c, w):
     ctx.close()
 
 
+@pytest.mark.parametrize("wF,wG", [(12, 16), (16, 12)])
+def test_block_bwd_is_joined_where_f_and_g_take_different_kernels(wF, wG):
+    """Inner widths of 16 and 12: the weight gradients of one function run on the side stream, those of the other do not.  What the caller
+    enqueues behind the call may read every gradient and reuse the workspace."""
+    ctx = B.Context(0)
+    N, H, W, c = 64, 32, 32, 16
+    rng = np.random.default_rng(5)
+    fn = {}
+    for name, w in (("F", wF), ("G", wG)):
+        fn[name] = [dict(name=f"{name}.l{i}", W=(rng.standard_normal((co, ci, 3, 3)) * np.sqrt(2.0 / (9 * ci))).astype(np.float32),
+                         gamma=np.ones(ci, np.float32), beta=np.zeros(ci, np.float32)) for i, (ci, co) in enumerate(((c, w), (w, c)))]
+    desc = B.block_desc(syn.BlockCfg(N, H, W, c, 0, "basic", seed=0), 0, 16)
+    for d, w in ((desc.F, wF), (desc.G, wG)):
+        d.cout[0] = d.cin[1] = w
+    ws = torch.empty(max(B.revnet_block_workspace_bytes(ctx, desc)), dtype=torch.uint8, device="cuda")
+    x1, x2, dy1, dy2 = (rng.standard_normal((N, c, H, W)).astype(np.float32) for _ in range(4))
+    params = {n: [dict(W=R._dev(B.w_to_abi(l["W"])), gamma=R._dev(l["gamma"]), beta=R._dev(l["beta"])) for l in fn[n]] for n in fn}
+    grads = {n: [{k: torch.zeros_like(v) for k, v in l.items()} for l in params[n]] for n in fn}
+    s1, s2 = R.to_state(x1, 16), R.to_state(x2, 16)
+    g1, g2 = R._dev(B.to_nhwc(dy1)), R._dev(B.to_nhwc(dy2))
+    B.revnet_block_fwd(ctx, desc, s1, s2, params["F"], params["G"], s1, s2, ws)
+    B.revnet_block_bwd(ctx, desc, s1, s2, g1, g2, params["F"], params["G"], s1, s2, g1, g2, grads["F"], grads["G"], ws)
+    got = {n: [l["W"].clone() for l in grads[n]] for n in fn}          # on the caller's stream, at once
+    ws.fill_(255)
+    for n in fn:
+        for l in grads[n]:
+            l["W"].fill_(float("nan"))
+    torch.cuda.synchronize()
+    num = dict(bf16_operands=True, frac_bits=16)
+    f64 = [np.rint(x.astype(np.float64) * 65536) / 65536 for x in (x1, x2)]
+    y1, y2 = orc.block_fwd(*f64, fn["F"], fn["G"], 1e-5, num=num)
+    og = {}
+    orc.block_bwd_reconstruct(y1, y2, dy1.astype(np.float64), dy2.astype(np.float64), fn["F"], fn["G"], 1e-5, og, num=num)
+    for n in fn:
+        for i in range(2):
+            assert hp.rel_l2(B.w_from_abi(got[n][i].cpu().numpy()), og[f"{n}.l{i}.W"]) <= 5e-2, (n, i)
+            assert torch.isnan(grads[n][i]["W"]).all(), (n, i)          # nothing of the call was still to come
+    B.revnet_check_device(ctx)
+    ctx.close()
+
+
 def test_pack_buffer_checks():
     ctx = B.Context(0)
     b = syn.BlockCfg(2, 8, 8, 32, 0, "basic", seed=9)
