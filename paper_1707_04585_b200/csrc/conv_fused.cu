@@ -218,8 +218,10 @@ __device__ __forceinline__ bool build_rows(const FusedGeom &g, const FusedLayer 
         const int my_rows = bp.r0 < RS ? rows : 0;
         uint8_t *dst = abuf + (g.nseg == 2 ? (seg & 1) : 0) * g.seg_bytes + (IN == kInBwd ? (it >> 1) * g.plane16 * 16 + (it & 1) * 8 : it * g.plane16 * 16);
         if (seg >= g.nseg && !warp_wait(&sh->seg_empty[g.nseg == 2 ? (seg & 1) : 0], (uint32_t)((g.nseg == 2 ? seg >> 1 : seg) - 1) & 1u, lane)) return false;
-        int *const place = tab + (g.tabs == 2 && (seg & 1) ? g.tab_bytes >> 2 : 0);
-        if (!K1 && seg > 0) build_table(g, place, bp.r0, sb - g.halo, rows);
+        if (!K1 && seg > 0) {
+            if (g.tabs == 2) tab += seg & 1 ? g.tab_bytes >> 2 : -(g.tab_bytes >> 2);
+            build_table(g, tab, bp.r0, sb - g.halo, rows);
+        }
         int l = bp.r0, low = bp.low0, j = 0, ready = 128 + 2 * g.halo;          // ready: rows that the tile to be signalled next needs
         auto signal = [&]() {
             fence_proxy_async();
@@ -247,7 +249,7 @@ __device__ __forceinline__ bool build_rows(const FusedGeom &g, const FusedLayer 
 #pragma unroll 1
             for (int i = 0; i < g.piece && low < rows; i += RS) {
                 if (l < my_rows) {
-                    const int px = K1 ? sb + l : place[l];
+                    const int px = K1 ? sb + l : tab[l];
                     const uint8_t *s = src + (px - pxs) * g.rowb;
                     const bool keep = p.a_out && (K1 || (unsigned)(l - g.halo) < (unsigned)own);
                     if constexpr (IN == kInBwd) {
