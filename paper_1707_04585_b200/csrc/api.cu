@@ -25,8 +25,6 @@ extern "C" int revnet_create(revnet_ctx **out, int device) {
             cudaStreamCreateWithFlags(&c->recon_stream, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&c->ev_rfork, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&c->ev_rjoin, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&c->ev_late[0], cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&c->ev_late[1], cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess) {
             cudaGetLastError();
@@ -50,7 +48,6 @@ extern "C" int revnet_destroy(revnet_ctx *ctx) {
     if (ctx->recon_stream) cudaStreamDestroy(ctx->recon_stream);
     if (ctx->ev_rfork) cudaEventDestroy(ctx->ev_rfork);
     if (ctx->ev_rjoin) cudaEventDestroy(ctx->ev_rjoin);
-    for (cudaEvent_t e : ctx->ev_late) if (e) cudaEventDestroy(e);
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
     delete ctx;

@@ -133,8 +133,8 @@ void fn_forward(Exec &ex, Geom g, Pair u, Moments *mom_in, const std::vector<Lay
 }
 
 // dgin_out = add + (dFn/du)^T gup ; parameter gradients through the layers' pointers.
-bool fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnSaved &saved, Pair gup, const bf16 *gup_cast,
-                 Pair add, Pair dgin_out, bf16 *dgin_cast, bool keep) {
+void fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnSaved &saved, Pair gup, const bf16 *gup_cast,
+                 Pair add, Pair dgin_out, bf16 *dgin_cast) {
     const int L = (int)layers.size();
     const bool b16 = ex.mode == 0;
     size_t outer = ex.ws.mark();
@@ -225,13 +225,11 @@ bool fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
             gcur = dtn;
         }
     }
-    if (keep) return side;
     if (side && !ex.dry) {
         cudaEventRecord(ex.ctx->ev_join, ex.ctx->side_stream);
         cudaStreamWaitEvent(ex.stream, ex.ctx->ev_join, 0);
     }
     ex.ws.release(outer);
-    return side;
 }
 
 void block_forward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const std::vector<Layer> &G,
@@ -247,12 +245,9 @@ void block_backward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const 
                     const float *y1, const float *y2, const float *dy1, const float *dy2,
                     float *x1, float *x2, float *dx1, float *dx2,
                     Moments *m1, Moments *m2, Moments *m2_use, const bf16 *dy2_cast, bf16 *dx2_cast,
-                    Moments *m1_out, bool overlap, const LateWgrad *late) {
+                    Moments *m1_out, bool overlap) {
     FnSaved svG, svF;
     const float q = ex.q;   // format of the coupling state; gradients are always float
-    // (a block called by itself joins the weight gradients of each function at its end: whether F's run on the side stream as well is F's own
-    // affair, so nothing later would be sure to wait for G's)
-    const bool late_g = late != nullptr;
     size_t m0 = ex.ws.mark();
     if (!m1_out) m1_out = m1;
     // F may be recomputed beside G's gradient steps only if it leaves y1 and its statistics alone
@@ -263,12 +258,11 @@ void block_backward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const 
     // x2 = y2 - G(z1), z1 = y1
     fn_forward(ex, g, single((float *)y1, c, q), m1, G, single((float *)y2, c, q), single(x2, c, q), -1, m2, &svG, false);
     Moments *mf = (m2_use && m2_use->valid) ? m2_use : m2;
-    bool on_side = false;
     Moments *mx1 = m1_out && !m1_out->mean ? nullptr : m1_out;
     if (!overlap) {
         // dz1 = dy1 + (dG/dz1)^T dy2 ; dW_G
-        on_side = fn_backward(ex, g, single((float *)y1, c, q), G, svG, single((float *)dy2, c), dy2_cast, single((float *)dy1, c), single(dx1, c), dz1_cast, late_g);
-        if (!late_g) ex.ws.release(m);
+        fn_backward(ex, g, single((float *)y1, c, q), G, svG, single((float *)dy2, c), dy2_cast, single((float *)dy1, c), single(dx1, c), dz1_cast);
+        ex.ws.release(m);
         // x1 = z1 - F(x2)
         fn_forward(ex, g, single(x2, c, q), mf, F, single((float *)y1, c, q), single(x1, c, q), -1, mx1, &svF, false);
     } else {
@@ -286,12 +280,10 @@ void block_backward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const 
         fn_forward(ex, g, single(x2, c, q), mf, F, single((float *)y1, c, q), single(x1, c, q), -1, mx1, &svF, false);
         if (ex.ws.high > ex.ws.off) ex.ws.off = ex.ws.high;
         if (!ex.dry) { cudaEventRecord(ex.ctx->ev_rjoin, ex.ctx->recon_stream); ex.stream = main; }
-        on_side = fn_backward(ex, g, single((float *)y1, c, q), G, svG, single((float *)dy2, c), dy2_cast, single((float *)dy1, c), single(dx1, c), dz1_cast, late_g);
+        fn_backward(ex, g, single((float *)y1, c, q), G, svG, single((float *)dy2, c), dy2_cast, single((float *)dy1, c), single(dx1, c), dz1_cast);
         if (!ex.dry) cudaStreamWaitEvent(main, ex.ctx->ev_rjoin, 0);
     }
     // dx2 = dy2 + (dF/dx2)^T dz1 ; dW_F ; dx1 = dz1 (already in place)
-    if (late && late->before && !ex.dry) cudaStreamWaitEvent(ex.stream, late->before, 0);
-    on_side = fn_backward(ex, g, single(x2, c, q), F, svF, single(dx1, c), dz1_cast, single((float *)dy2, c), single(dx2, c), dx2_cast, late != nullptr) || on_side;
-    if (late && late->done && !ex.dry) cudaEventRecord(late->done, on_side ? ex.ctx->side_stream : ex.stream);
+    fn_backward(ex, g, single(x2, c, q), F, svF, single(dx1, c), dz1_cast, single((float *)dy2, c), single(dx2, c), dx2_cast);
     ex.ws.release(m0);
 }

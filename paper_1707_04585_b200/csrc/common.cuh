@@ -37,7 +37,6 @@ struct revnet_ctx {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaStream_t recon_stream = nullptr;     // a train step recomputes F here while the gradient steps of G run on the main stream
     cudaEvent_t ev_rfork = nullptr, ev_rjoin = nullptr;
-    cudaEvent_t ev_late[2] = {nullptr, nullptr};      // weight gradients of a unit whose successor does not wait for them (LateWgrad)
     // per-kernel timing (revnet_profile_*): one event after every launch while enabled
     bool profiling = false;
     bool prof_detail = false;   // summary lines per launch shape, not only per kernel name
@@ -175,7 +174,6 @@ struct Arena {
     char *base = nullptr;
     size_t off = 0, cap = 0, peak = 0;
     size_t high = 0;       // highest offset reached since the caller last set it (see block_backward)
-    size_t top = 0;        // the same for the stack driver (see LateWgrad)
     bool dry = true;
     bool overflow = false;
     void *alloc(size_t bytes) {
@@ -183,7 +181,6 @@ struct Arena {
         off = a + bytes;
         if (off > peak) peak = off;
         if (off > high) high = off;
-        if (off > top) top = off;
         if (!dry && off > cap) { overflow = true; return nullptr; }
         return dry ? (void *)(uintptr_t)(0x1000 + a) : base + a;   // non-null fake address in dry mode
     }
@@ -475,20 +472,8 @@ void fn_forward(Exec &ex, Geom g, Pair u, Moments *mom_in, const std::vector<Lay
 // dgin_out = add + (dFn/du)^T gup, parameter gradients written through the layers' pointers;
 // gup_cast: bf16 [P,C] copy of gup if the caller already has one; dgin_cast: if non-null, a bf16
 // [P,C] copy of dgin_out is written there as well
-// keep: what the weight gradients on the side stream read stays allocated and the main stream does not wait for them; the caller
-// does both.  Returns whether they run on the side stream.
-bool fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnSaved &saved, Pair gup, const bf16 *gup_cast,
-                 Pair add, Pair dgin_out, bf16 *dgin_cast, bool keep = false);
-// Weight gradients that the units of a stage do not wait for.  On small tensors the two side-stream launches of a function (a
-// partial sum of products, the sum of the partials) outlast the data gradient and the BN backward that they run beside, and the
-// main stream stood 6 to 8 us per function until they were done.  Instead a unit leaves them running: `done` is recorded behind
-// them; nothing they read (the unit's scratch, the bf16 gradient it was handed) may be overwritten before the main stream has waited
-// for it.  The units of a stage take two scratch regions in turn, and a unit waits for its predecessor's event (`before`) in front of
-// F's gradient steps.
-// kLateWgradElems: the largest half of a unit's pair for which they run on.  Both halves of a unit's scratch stay allocated for it; above, a
-// launch fills the GPU for so long that nothing is won by running two side by side.
-constexpr size_t kLateWgradElems = (size_t)1 << 23;
-struct LateWgrad { cudaEvent_t before = nullptr, done = nullptr; };      // (null: nothing to wait for, nothing to record)
+void fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnSaved &saved, Pair gup, const bf16 *gup_cast,
+                 Pair add, Pair dgin_out, bf16 *dgin_cast);
 struct FnSaved {
     std::vector<void *> a;        // activated input of each conv
     std::vector<float *> t;       // BN input of each layer beyond the first (conv outputs)
@@ -512,7 +497,6 @@ void block_backward(Exec &ex, Geom g, int c, const std::vector<Layer> &F, const 
                     const float *y1, const float *y2, const float *dy1, const float *dy2,
                     float *x1, float *x2, float *dx1, float *dx2,
                     Moments *m1 = nullptr, Moments *m2 = nullptr, Moments *m2_use = nullptr,
-                    const bf16 *dy2_cast = nullptr, bf16 *dx2_cast = nullptr, Moments *m1_out = nullptr, bool overlap = false,
-                    const LateWgrad *late = nullptr);
+                    const bf16 *dy2_cast = nullptr, bf16 *dx2_cast = nullptr, Moments *m1_out = nullptr, bool overlap = false);
 
 static inline int conv_out(int in, int k, int s) { return (in + 2 * (k / 2) - k) / s + 1; }

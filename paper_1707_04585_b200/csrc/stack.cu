@@ -148,7 +148,7 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
     // those of the stage's input x2, which the reversal of the first unit needs again
     struct StageMom { Moments m1, m2, cat, in_cat, in2, dy1; bool defer; };      // dy1: statistics of a down-sampling unit's y1, kept for its backward
     std::vector<StageMom> sm(S);
-    bf16 *gcast = nullptr, *gcast_alt = nullptr;      // bf16 copy of the gradient w.r.t. x2 / y2, handed from unit to unit (two in turn: LateWgrad)
+    bf16 *gcast = nullptr;          // bf16 copy of the gradient w.r.t. x2 / y2, handed from unit to unit
     float *x1_alt = nullptr;
     Moments m1_alt;
     bf16 *gcast2 = nullptr;         // stored-activation step: bf16 copy of the gradient w.r.t. z1 inside a unit
@@ -158,8 +158,6 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
     std::vector<std::vector<StoredUnit>> kept(S);
     std::vector<Pair> stage_out(S);
     const bool stored = d.store_activations != 0;
-    // the units of a stage leave their weight gradients running (see LateWgrad) where a launch is short
-    auto late_wgrad = [&](const StagePlan &s) { return ex.mode == 0 && !stored && (size_t)N * s.H * s.H * s.c <= kLateWgradElems; };
     uint64_t kept_bytes = 0;        // what the units keep, summed over the network
     {
         size_t cmax = 0;
@@ -181,9 +179,6 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
             size_t e = (size_t)N * s.H * s.H * s.c; if (e > cmax) cmax = e;
         }
         if (ex.mode == 0) gcast = ex.ws.get<bf16>(cmax);
-        size_t lmax = 0;
-        for (auto &st : pl->st) { const size_t e = (size_t)N * st.H * st.H * st.c; if (late_wgrad(st) && e > lmax) lmax = e; }
-        if (lmax) gcast_alt = ex.ws.get<bf16>(lmax);
         // the reversal writes x1 beside y1 instead of over it (the two buffers change roles from unit to unit), and the
         // statistics of x1 beside those of y1, so that F can be recomputed while G's gradient steps still read y1
         if (!d.store_activations) { x1_alt = ex.ws.get<float>(cmax); size_t c2 = 0; for (auto &st : pl->st) if ((size_t)st.c > c2) c2 = st.c; m1_alt = mom_alloc(ex, (int)c2); int cd = 0; for (int si = 0; si < S; si++) if (sm[si].defer && pl->st[si].c > cd) cd = pl->st[si].c; if (cd) mom_room(ex, m1_alt, cd); }
@@ -299,31 +294,16 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
             malt.mean = m1_alt.mean; malt.rstd = m1_alt.mean + s.c; malt.valid = false;
             if (mo.defer) { malt.part = m1_alt.part; malt.part_cap = m1_alt.part_cap; }
             float *cur1 = x1, *alt1 = x1_alt;
-            const bool late = late_wgrad(s), side = late && !ex.dry && ex.ctx->side_stream && !ex.ctx->profiling;
-            const size_t base = (ex.ws.mark() + 255) & ~size_t(255);
-            size_t span = 0;
-            bf16 *gc_in = gcast, *gc_out = late ? gcast_alt : gcast;
-            for (int u = s.units - 1, turn = 0; u >= 0; u--, turn ^= 1) {
-                LateWgrad lw;
-                if (side) { lw.done = ex.ctx->ev_late[turn]; lw.before = u == s.units - 1 ? nullptr : ex.ctx->ev_late[turn ^ 1]; }
-                if (late) { ex.ws.off = ex.ws.top = base + (turn ? span : 0); }
+            for (int u = s.units - 1; u >= 0; u--) {
                 // x1 alternates between the two buffers from unit to unit.  Nothing reads the statistics of the stage's input as the
                 // reversal returns it: the first unit's F takes those of the forward pass.  (The sizing run has them summed there as well:
                 // the scratch of a stage does not depend on its depth)
                 Moments none;
                 const bool unread = u == 0 && !ex.dry;
                 block_backward(ex, g, s.c, bind(s.F[u], params, grads), bind(s.G[u], params, grads), cur1, x2, d1, d2, alt1, x2, d1, d2,
-                               &mcur, unread ? nullptr : &mo.m2, u == 0 ? &mo.in2 : nullptr, u == s.units - 1 ? nullptr : gc_in, gc_out, unread ? &none : &malt, true, late ? &lw : nullptr);
-                if (late && !span) span = (ex.ws.top - base + 255) & ~size_t(255);
-                if (late) std::swap(gc_in, gc_out);
+                               &mcur, unread ? nullptr : &mo.m2, u == 0 ? &mo.in2 : nullptr, u == s.units - 1 ? nullptr : gcast, gcast, unread ? &none : &malt, true);
                 std::swap(cur1, alt1);
                 std::swap(mcur, malt);
-            }
-            if (late) {
-                // (a stage of one unit is planned like the deeper ones)
-                if (ex.dry && s.units) { ex.ws.off = base; ex.ws.alloc(2 * span); }
-                ex.ws.off = base;
-                if (side && s.units) cudaStreamWaitEvent(ex.stream, ex.ctx->ev_late[(s.units - 1) & 1], 0);
             }
             // after an odd number of units the stage's input sits in the other buffer: bring it home
             if (cur1 != x1 && !ex.dry) cudaMemcpyAsync(x1, cur1, g.P() * s.c * sizeof(float), cudaMemcpyDeviceToDevice, ex.stream);
