@@ -179,16 +179,6 @@ void fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
         const bool folded = sums.part != nullptr;
         bf16 *dt = folded ? ex.ws.get<bf16>(P * ly.cout) : nullptr;
         gq[l] = folded ? dt : gcur;
-        float *da = ex.ws.get<float>(P * ly.cin);
-        float *coef = ex.ws.get<float>((size_t)3 * ly.cin);
-        const Pair tl = l == 0 ? u : single(saved.t[l - 1], ly.cin);
-        const BnRef bn{ly.gamma, ly.beta, saved.bn[l].mean, saved.bn[l].rstd};
-        const BnBwdReq bb{tl, bn, ly.dgamma, ly.dbeta, coef};
-        // fold: the data gradient in front goes through this BN's backward; else the kernel between them adds the records
-        const bool fold = l > 0 && (l > 1 || u.c1 == 0) && conv_dgrad_fused_takes(ex, gin[l - 1], layers[l - 1], true);
-        const bool leave = b16 && (folded || conv_dgrad_fused_takes(ex, gin[l], ly, false)) && (fold || (bn_relu_bwd_sums_takes(P, ly.cin) && (l > 0 || plain)));
-        BwdSums mine;
-        if (leave) mine.part = ex.ws.get<float>(bwd_sums_floats(ex, ly.cin));
         auto wgrads = [&]() {            // as soon as every gradient operand exists
             if (!side) {
                 conv_wgrad(ex, gq[l], saved.a[l], gin[l], ly, ly.dW);
@@ -203,7 +193,17 @@ void fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
                 ex.stream = main;
             }
         };
-        if (!folded) wgrads();
+        if (!folded) wgrads();           // (in front of da: layer by layer their split partials are scratch that da takes over)
+        float *da = ex.ws.get<float>(P * ly.cin);
+        float *coef = ex.ws.get<float>((size_t)3 * ly.cin);
+        const Pair tl = l == 0 ? u : single(saved.t[l - 1], ly.cin);
+        const BnRef bn{ly.gamma, ly.beta, saved.bn[l].mean, saved.bn[l].rstd};
+        const BnBwdReq bb{tl, bn, ly.dgamma, ly.dbeta, coef};
+        // fold: the data gradient in front goes through this BN's backward; else the kernel between them adds the records
+        const bool fold = l > 0 && (l > 1 || u.c1 == 0) && conv_dgrad_fused_takes(ex, gin[l - 1], layers[l - 1], true);
+        const bool leave = b16 && (folded || conv_dgrad_fused_takes(ex, gin[l], ly, false)) && (fold || (bn_relu_bwd_sums_takes(P, ly.cin) && (l > 0 || plain)));
+        BwdSums mine;
+        if (leave) mine.part = ex.ws.get<float>(bwd_sums_floats(ex, ly.cin));
         bool sums_done = true;
         if (folded) {
             if (!conv_dgrad_fused_behind(ex, da_behind, behind, sums, dt, gin[l], ly, da, &bb, leave ? &mine : nullptr) && !ex.failed) {

@@ -143,3 +143,15 @@ def test_reversible_step_holds_a_fraction_of_what_ordinary_backprop_holds(ctx, n
         held.append(plan.activation_bytes + plan.workspace_bytes)
         plan.close()
     assert held[0] <= share * held[1]
+
+
+@pytest.mark.parametrize("kind,N,H,W,c,w,mode,ceiling", [
+    ("bottleneck", 64, 56, 56, 512, 128, 1, 1644823808),
+    ("basic", 128, 8, 8, 56, 0, 1, 12790272),
+    ("basic", 60, 41, 10, 100, 0, 0, 54856192),
+    ("single", 28, 39, 35, 12, 0, 0, 4598880),
+])
+def test_block_backward_asks_for_no_more_workspace(ctx, kind, N, H, W, c, w, mode, ceiling):
+    """Weight gradients layer by layer: their split partials and the next tensor of the data-gradient chain are not held at once."""
+    d = B.block_desc(syn.BlockCfg(N, H, W, c, w, kind, seed=0), mode, 0 if mode else 16)
+    assert B.revnet_block_workspace_bytes(ctx, d)[1] <= ceiling
