@@ -24,7 +24,7 @@ bool conv_fused_takes(Exec &ex, Geom gi, const Layer &L);
 bool conv_fprop_bn(Exec &ex, Pair t, BnRef bn, Geom gi, const Layer &L, Pair out, Moments *stats, bf16 *a_out);
 bool conv_fprop_fused(Exec &ex, Pair t, BnRef bn, Geom gi, const Layer &L, Pair out, Pair partner, int sign, Moments *stats, bf16 *a_out);
 bool conv_dgrad_fused(Exec &ex, const void *g, Geom gi, const Layer &L, float *da, const BnBwdReq *bb, BwdSums *sums);
-bool conv_dgrad_fused_takes(Exec &ex, Geom gi, const Layer &L, bool behind);
+bool conv_dgrad_fused_takes(Exec &ex, Geom gi, const Layer &L, bool behind, int *parts);
 bool conv_dgrad_fused_behind(Exec &ex, const float *g, const BnBwdReq &behind, const BwdSums &bsums, bf16 *g_out, Geom gi, const Layer &L, float *da, const BnBwdReq *bb,
                              BwdSums *sums);
 
@@ -41,6 +41,7 @@ static void conv_fprop(Exec &ex, const void *a, Geom gi, const Layer &L, Pair ou
 static bool conv_dgrad(Exec &ex, const void *g, Geom gi, const Layer &L, float *da, const BnBwdReq *bb, BwdSums *sums) {
     const bool b16 = ex.mode == 0;
     if (b16 && L.stride == 1 && conv_dgrad_fused(ex, g, gi, L, da, bb, sums)) return bb != nullptr;
+    if (sums) { if (!ex.failed) { ex.failed = true; ex.ctx->err = "conv_dgrad: a fused data gradient was refused"; } return true; }      // (does not happen: asked before)
     if (b16 && L.stride == 1 && conv_dgrad_tc(ex, g, gi, L, da, bb)) return bb != nullptr;
     // stride 2 on the tensor cores: the CTAs of one launch split into the parity classes of the input pixels
     bool fused = false;
@@ -170,6 +171,8 @@ void fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
     // Where the data gradients are fused kernels, the sums of a layer's BN backward stay the records of its data gradient's CTAs, and the data
     // gradient of the layer in front (or the last step, `add`) takes its input through that BN backward itself
     BwdSums sums;                        // pending sums of layer l + 1
+    int parts = 0, front_parts = 0;      // records that the data gradient of layer l leaves; of layer l - 1, if folded
+    size_t spare = wg_scratch ? wg_need : 0;
     const float *da_behind = nullptr;    // da of that layer
     BnBwdReq behind{};
     const bool plain = b16 && u.c1 == 0 && add.p0 && add.c1 == 0 && add.q == 0.f && dgin_out.p0 && dgin_out.c1 == 0 && dgin_out.q == 0.f;
@@ -195,15 +198,21 @@ void fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
         };
         if (!folded) wgrads();           // (in front of da: layer by layer their split partials are scratch that da takes over)
         float *da = ex.ws.get<float>(P * ly.cin);
-        float *coef = ex.ws.get<float>((size_t)3 * ly.cin);
+        // fold: the data gradient in front goes through this BN's backward; else the kernel between them adds the records
+        const bool fold = b16 && l > 0 && (l > 1 || u.c1 == 0) && conv_dgrad_fused_takes(ex, gin[l - 1], layers[l - 1], true, &front_parts);
+        const bool leave = b16 && (folded || conv_dgrad_fused_takes(ex, gin[l], ly, false, &parts)) && (fold || (bn_relu_bwd_sums_takes(P, ly.cin) && (l > 0 || plain)));
+        // (nobody has touched the weight gradients' partials yet: they start when the records of layer 1 are read)
+        BwdSums mine;
+        if (leave) {
+            const size_t need = (size_t)parts * 2 * ly.cin;
+            if (l > 0 && need <= spare) { mine.part = wg_scratch + (wg_need - spare); spare -= need; }
+            else mine.part = ex.ws.get<float>(need);
+        }
+        parts = front_parts;
+        float *coef = leave ? nullptr : ex.ws.get<float>((size_t)3 * ly.cin);
         const Pair tl = l == 0 ? u : single(saved.t[l - 1], ly.cin);
         const BnRef bn{ly.gamma, ly.beta, saved.bn[l].mean, saved.bn[l].rstd};
         const BnBwdReq bb{tl, bn, ly.dgamma, ly.dbeta, coef};
-        // fold: the data gradient in front goes through this BN's backward; else the kernel between them adds the records
-        const bool fold = l > 0 && (l > 1 || u.c1 == 0) && conv_dgrad_fused_takes(ex, gin[l - 1], layers[l - 1], true);
-        const bool leave = b16 && (folded || conv_dgrad_fused_takes(ex, gin[l], ly, false)) && (fold || (bn_relu_bwd_sums_takes(P, ly.cin) && (l > 0 || plain)));
-        BwdSums mine;
-        if (leave) mine.part = ex.ws.get<float>(bwd_sums_floats(ex, ly.cin));
         bool sums_done = true;
         if (folded) {
             if (!conv_dgrad_fused_behind(ex, da_behind, behind, sums, dt, gin[l], ly, da, &bb, leave ? &mine : nullptr) && !ex.failed) {

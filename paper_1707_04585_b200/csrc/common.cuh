@@ -379,7 +379,7 @@ struct Geom { int N, H, W; size_t P() const { return (size_t)N * H * W; } };
 
 // ---------------------------------------------------------------- elementwise.cu
 Moments mom_alloc(Exec &ex, int C, bool with_part = false);
-void mom_room(Exec &ex, Moments &m, int C);      // gives m room for pending records, and asks its producers to leave them
+size_t mom_records(const Exec &ex, int C);       // floats that the pending records of a tensor of C channels may take
 // pending statistics -> mean / rstd (one small kernel); no-op otherwise
 void mom_finalize(Exec &ex, Moments &m, int C);
 // batch statistics of t ([P,C]) -> mean, rstd (the convolution epilogues produce the same quantities for the
@@ -432,9 +432,7 @@ bool stem_wgrad(Exec &ex, const float *img, const float *gout, Geom gi, const La
 // own BN: its input t, its coefficients, and where dgamma, dbeta and coef[3][C] go.
 struct BnBwdReq { Pair t; BnRef bn; float *dgamma, *dbeta, *coef; };
 // Sums of a BN backward left as per-CTA records of 2C floats (layout as for Moments): their consumer adds them, and stores dgamma and dbeta.
-// part: room for bwd_sums_floats() floats
 struct BwdSums { float *part = nullptr; int parts = 0; double inv_count = 0; };
-inline size_t bwd_sums_floats(const Exec &ex, int C) { return (size_t)ex.ctx->sm_count * 2 * C; }
 // whether bn_relu_bwd_sums takes the shape; out = add + dt from pending sums, optionally with a bf16 copy, or (add.p0 == nullptr) the bf16
 // copy of dt alone (all plain tensors)
 bool bn_relu_bwd_sums_takes(size_t P, int C);

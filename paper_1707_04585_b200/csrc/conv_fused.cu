@@ -740,10 +740,12 @@ bool conv_dgrad_fused(Exec &ex, const void *g, Geom gi, const Layer &L, float *d
                      nullptr, sums);
 }
 
-// whether conv_dgrad_fused takes the data gradient of L, with a bf16 input or (behind) through the BN backward of the layer behind
-bool conv_dgrad_fused_takes(Exec &ex, Geom gi, const Layer &L, bool behind) {
+// whether conv_dgrad_fused takes the data gradient of L, with a bf16 input or (behind) through the BN backward of the layer behind; parts: the
+// records of 2 cin sums that it leaves
+bool conv_dgrad_fused_takes(Exec &ex, Geom gi, const Layer &L, bool behind, int *parts) {
     FusedShape s;
     if (L.stride != 1 || !fused_shape(gi, L.cout, L.cin, L.k, ex.ctx->sm_count, behind ? kInBwd : kInBf16, true, s) || !(ex.dry || tc_encoder(ex.ctx))) return false;
+    *parts = s.ctas;
     // Through the BN backward only where a build thread has few rows: its pass costs 0.3 us per row and thread, twice that of a bf16 input with
     // twice the threads per row, against 5 us for the launch that it saves.  Odd-sized block (24 channels, a tile per CTA, five and a half rows)
     // 151 -> 144.5 us; 56 channels at 8x8 (eleven rows) and 16 at 32x32 (twenty-one): 38-layer step 1665 -> 1686.

@@ -252,18 +252,14 @@ Moments mom_alloc(Exec &ex, int C, bool with_part) {
     float *p = ex.ws.get<float>((size_t)2 * C);
     m.mean = p; m.rstd = p + C;
     if (with_part) {
-        mom_room(ex, m, C);
-        m.defer = false;
+        m.part_cap = mom_records(ex, C);
+        m.part = ex.ws.get<float>(m.part_cap);
     }
     return m;
 }
-// room for the records of 2C floats that a producer may leave: one per CTA of a convolution (conv_tc_kernel runs at most two CTAs
-// per SM, the others one), kPendingRecords of a stand-alone reduction
-void mom_room(Exec &ex, Moments &m, int C) {
-    m.part_cap = (size_t)2 * ex.ctx->sm_count * 2 * C;
-    m.part = ex.ws.get<float>(m.part_cap);
-    m.defer = true;
-}
+// records of 2C floats that a producer may leave: one per CTA of a convolution (conv_tc_kernel runs at most two CTAs per SM, the
+// others one), kPendingRecords of a stand-alone reduction
+size_t mom_records(const Exec &ex, int C) { return (size_t)2 * ex.ctx->sm_count * 2 * C; }
 
 __global__ void __launch_bounds__(256) moments_finalize_kernel(const float *part, int parts, int C, double inv_count, float eps,
                                                              float *mean, float *rstd) {

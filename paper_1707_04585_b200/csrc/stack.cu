@@ -173,17 +173,31 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
             // Where a unit's functions start with a fused convolution, the statistics of the pair between units stay the records of the
             // convolution that coupled it: the next one adds them while its first rows are on the way (1.0 to 2.1 us), where the
             // reduction by the producer's last CTA kept every other SM waiting for 4 us (count, records, result).
-            sm[si].defer = ex.mode == 0 && s.units > 0 && conv_fused_takes(ex, Geom{N, s.H, s.H}, bind(s.F[0][0], params, grads)) &&
+            // Two sets of records in turn are enough (what a function leaves is read by the next one's first kernel), and they sit in
+            // a gradient buffer that is not in use meanwhile (pair_records), if it has the room.
+            sm[si].defer = ex.mode == 0 && s.units > 0 && 2 * mom_records(ex, s.c) <= gmax && conv_fused_takes(ex, Geom{N, s.H, s.H}, bind(s.F[0][0], params, grads)) &&
                            conv_fused_takes(ex, Geom{N, s.H, s.H}, bind(s.G[0][0], params, grads));
-            if (sm[si].defer) { mom_room(ex, sm[si].m1, s.c); mom_room(ex, sm[si].m2, s.c); }
             size_t e = (size_t)N * s.H * s.H * s.c; if (e > cmax) cmax = e;
         }
         if (ex.mode == 0) gcast = ex.ws.get<bf16>(cmax);
         // the reversal writes x1 beside y1 instead of over it (the two buffers change roles from unit to unit), and the
         // statistics of x1 beside those of y1, so that F can be recomputed while G's gradient steps still read y1
-        if (!d.store_activations) { x1_alt = ex.ws.get<float>(cmax); size_t c2 = 0; for (auto &st : pl->st) if ((size_t)st.c > c2) c2 = st.c; m1_alt = mom_alloc(ex, (int)c2); int cd = 0; for (int si = 0; si < S; si++) if (sm[si].defer && pl->st[si].c > cd) cd = pl->st[si].c; if (cd) mom_room(ex, m1_alt, cd); }
+        if (!d.store_activations) {
+            x1_alt = ex.ws.get<float>(cmax);
+            size_t c2 = 0;
+            for (auto &st : pl->st) if ((size_t)st.c > c2) c2 = st.c;
+            m1_alt = mom_alloc(ex, (int)c2);
+        }
         if (ex.mode == 0 && d.store_activations) gcast2 = ex.ws.get<bf16>(cmax);
     }
+    // set 0 or 1 of a stage's pending records: in either gradient buffer during the forward pass, in the one that holds no gradient while the
+    // units of the stage are walked back (the stage's own stored layers overwrite it afterwards)
+    auto pair_records = [&](int si, Moments &m, float *buf, int set) {
+        if (!sm[si].defer) return;
+        m.part_cap = mom_records(ex, pl->st[si].c);
+        m.part = buf + set * m.part_cap;
+        m.defer = true;
+    };
     float *recon = ex.ws.get<float>(REVNET_MAX_STAGES);
     if (recon_dev) *recon_dev = recon;
     if (d.verify_reconstruction) fill_zero(ex, recon, REVNET_MAX_STAGES * sizeof(float));
@@ -233,6 +247,8 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
             cudaMemcpyAsync(actf(s.off_v1), x1, b, cudaMemcpyDeviceToDevice, ex.stream);
             cudaMemcpyAsync(actf(s.off_v2), x2, b, cudaMemcpyDeviceToDevice, ex.stream);
         }
+        pair_records(si, mo.m1, gbuf[0], 0);
+        pair_records(si, mo.m2, gbuf[0], 1);
         if (!stored) {
             for (int u = 0; u < s.units; u++) {
                 // (the last unit's pair is read by a transition or a down-sampling unit, which want mean and rstd)
@@ -258,7 +274,10 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
                 k.y1 = ex.ws.get<float>(half); k.y2 = ex.ws.get<float>(half);
                 // the statistics of the stage's final pair go where the next transition expects them
                 if (last_unit) { k.my1 = mo.m1; k.my2 = mo.m2; k.my2.part = nullptr; k.my2.defer = false; }
-                else { k.my1 = mom_alloc(ex, s.c, mo.defer); k.my2 = mom_alloc(ex, s.c, mo.defer); k.my1.defer = k.my2.defer = mo.defer; }
+                else {
+                    k.my1 = mom_alloc(ex, s.c); k.my2 = mom_alloc(ex, s.c);
+                    pair_records(si, k.my1, gbuf[0], 0); pair_records(si, k.my2, gbuf[0], 1);
+                }
                 fn_forward(ex, g, single(c2, s.c, q), m_in, bind(s.F[u], params, grads), single(c1, s.c, q), single(k.y1, s.c, q), +1, &k.my1, &k.svF, false);
                 fn_forward(ex, g, single(k.y1, s.c, q), &k.my1, bind(s.G[u], params, grads), single(c2, s.c, q), single(k.y2, s.c, q), +1, &k.my2, &k.svG, false);
                 if (last_unit) { mo.m1 = k.my1; mo.m2 = k.my2; }
@@ -290,9 +309,11 @@ static void run_step(revnet_plan *pl, Exec &ex, const float *images, const int32
         float *d1 = gbuf[gi], *d2 = gbuf[gi] + half;
         StageMom &mo = sm[si];
         if (!stored) {
+            // (G's first kernel has added the records of y1 before F's last one leaves those of x1: they share a set)
+            pair_records(si, mo.m1, gbuf[gi ^ 1], 0);
+            pair_records(si, mo.m2, gbuf[gi ^ 1], 1);
             Moments mcur = mo.m1, malt = mo.m1;
             malt.mean = m1_alt.mean; malt.rstd = m1_alt.mean + s.c; malt.valid = false;
-            if (mo.defer) { malt.part = m1_alt.part; malt.part_cap = m1_alt.part_cap; }
             float *cur1 = x1, *alt1 = x1_alt;
             for (int u = s.units - 1; u >= 0; u--) {
                 // x1 alternates between the two buffers from unit to unit.  Nothing reads the statistics of the stage's input as the

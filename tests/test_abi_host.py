@@ -3,6 +3,7 @@ planning logic (parameter layout, stored-activation accounting) is right.  No ke
 import ctypes
 import os
 import re
+from dataclasses import replace
 
 import numpy as np
 import pytest
@@ -154,4 +155,25 @@ def test_reversible_step_holds_a_fraction_of_what_ordinary_backprop_holds(ctx, n
 def test_block_backward_asks_for_no_more_workspace(ctx, kind, N, H, W, c, w, mode, ceiling):
     """Weight gradients layer by layer: their split partials and the next tensor of the data-gradient chain are not held at once."""
     d = B.block_desc(syn.BlockCfg(N, H, W, c, w, kind, seed=0), mode, 0 if mode else 16)
+    assert B.revnet_block_workspace_bytes(ctx, d)[1] <= ceiling
+
+
+@pytest.mark.parametrize("name,N,stored,ceiling", [
+    ("revnet38", 23, False, 23758464), ("revnet38", 128, False, 113318144), ("revnet38", 80, True, 201538688),
+    ("revnet110", 128, False, 118021888), ("revnet110", 23, True, 166849280), ("revnet164", 80, False, 505738496),
+    ("paper_revnet38", 80, False, 71953152), ("paper_revnet164", 23, True, 459435008),
+])
+def test_records_of_statistics_and_sums_take_no_workspace_of_their_own(ctx, name, N, stored, ceiling):
+    """What the step planned when every producer reduced its records at once."""
+    plan = B.revnet_stack_plan(ctx, B.stack_desc(replace(syn.stack_config(name), N=N), 0, state_frac_bits=16, store_activations=stored))
+    assert plan.workspace_bytes <= ceiling
+    plan.close()
+
+
+@pytest.mark.parametrize("kind,N,H,W,c,w,ceiling", [
+    ("basic", 128, 32, 32, 16, 0, 47601920), ("basic", 37, 15, 21, 24, 0, 9386240), ("single", 4, 8, 8, 8, 0, 30848),
+    ("bottleneck", 121, 17, 36, 32, 8, 38283520), ("basic", 128, 8, 8, 56, 0, 15917824),
+])
+def test_block_backward_sums_take_no_workspace_of_their_own(ctx, kind, N, H, W, c, w, ceiling):
+    d = B.block_desc(syn.BlockCfg(N, H, W, c, w, kind, seed=0), 0, 16)
     assert B.revnet_block_workspace_bytes(ctx, d)[1] <= ceiling
