@@ -160,8 +160,10 @@ void fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
     // last layer's data gradient: by then every operand exists (the gradient entering layer 0 is the
     // last one produced).  One launch amortises set-up and split partials over the layers; the split
     // partials get a buffer of their own for that time.  Functions of more than four layers, shapes
-    // the tensor-core kernel does not take, and profiling runs go layer by layer on the main stream.
-    bool side = b16 && ex.use_side && L <= 4 && (ex.dry || (ex.ctx->side_stream && !ex.ctx->profiling));
+    // the tensor-core kernel does not take, and profiling runs go layer by layer on the main stream (a profiled run that has no
+    // workspace for that, ex.batch_wgrad: as one launch there).
+    bool side = b16 && L <= 4 && (ex.dry || (ex.ctx->side_stream && (!ex.ctx->profiling || ex.batch_wgrad)));
+    const bool fork = !ex.dry && !ex.ctx->profiling;
     size_t wg_need = 0;
     std::vector<const Layer *> lptr(L);
     std::vector<const void *> gq(L), aq(L);
@@ -187,7 +189,7 @@ void fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
                 conv_wgrad(ex, gq[l], saved.a[l], gin[l], ly, ly.dW);
             } else if (l == 0) {
                 cudaStream_t main = ex.stream;
-                if (!ex.dry) {
+                if (fork) {
                     cudaEventRecord(ex.ctx->ev_fork, main);
                     cudaStreamWaitEvent(ex.ctx->side_stream, ex.ctx->ev_fork, 0);
                     ex.stream = ex.ctx->side_stream;
@@ -234,7 +236,7 @@ void fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
             gcur = dtn;
         }
     }
-    if (side && !ex.dry) {
+    if (side && fork) {
         cudaEventRecord(ex.ctx->ev_join, ex.ctx->side_stream);
         cudaStreamWaitEvent(ex.stream, ex.ctx->ev_join, 0);
     }

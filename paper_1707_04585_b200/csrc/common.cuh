@@ -202,7 +202,7 @@ struct Exec {
     uint64_t launches = 0;
     bool failed = false;
     bool pdl = true;       // launch kernels with programmatic stream serialization (see launch())
-    bool use_side = true;  // run weight gradients on the context's side stream (never while profiling)
+    bool batch_wgrad = false;   // while profiling: one launch for the weight gradients of a function, as on the side stream, not layer by layer
     unsigned long long hold_ns = 0;   // profiling: the first mark() holds the stream this long so that launches queue up
     // called after every launch: error check, launch count and (when profiling) an event;
     // bytes / flops are the algorithmic traffic and work of that launch

@@ -534,11 +534,6 @@ extern "C" int revnet_stack_plan(revnet_ctx *ctx, const revnet_stack_desc *desc,
     ex.q = d.state_frac_bits ? ldexpf(1.f, -d.state_frac_bits) : 0.f;
     run_step(pl, ex, nullptr, nullptr, (float *)0x1000, (float *)0x1000, (float *)0x1000, (char *)0x1000, nullptr, nullptr, nullptr, nullptr, nullptr);
     pl->ws_bytes = ex.ws.peak + 256;
-    // and once more with the weight gradients layer by layer on the main stream, as profiling runs have them
-    Exec one = ex;
-    one.ws = Arena(); one.use_side = false;
-    run_step(pl, one, nullptr, nullptr, (float *)0x1000, (float *)0x1000, (float *)0x1000, (char *)0x1000, nullptr, nullptr, nullptr, nullptr, nullptr);
-    if (one.ws.peak + 256 > pl->ws_bytes) pl->ws_bytes = one.ws.peak + 256;
     if (param_count) *param_count = pl->n_params;
     if (activation_bytes) *activation_bytes = pl->act_bytes;
     if (workspace_bytes) *workspace_bytes = pl->ws_bytes;
@@ -602,6 +597,7 @@ extern "C" int revnet_train_step(revnet_ctx *ctx, revnet_plan *pl, const float *
     ex.stream = use_graph ? ctx->capture_stream : (cudaStream_t)stream;
     ex.q = pl->d.state_frac_bits ? ldexpf(1.f, -pl->d.state_frac_bits) : 0.f;
     ex.ws.dry = false; ex.ws.base = (char *)workspace; ex.ws.cap = pl->ws_bytes;
+    ex.batch_wgrad = pl->d.store_activations != 0;   // (layer by layer, the last unit's split partials would not fit beside what all units keep)
     if (ctx->profiling) ex.hold_ns = 5000000ull;     // the launches of a profiled step queue up behind a 5 ms hold
     if (use_graph) {
         if (pl->graph_exec) { cudaGraphExecDestroy(pl->graph_exec); pl->graph_exec = nullptr; }

@@ -161,7 +161,7 @@ def test_block_backward_asks_for_no_more_workspace(ctx, kind, N, H, W, c, w, mod
 @pytest.mark.parametrize("name,N,stored,ceiling", [
     ("revnet38", 23, False, 23758464), ("revnet38", 128, False, 113318144), ("revnet38", 80, True, 201538688),
     ("revnet110", 128, False, 118021888), ("revnet110", 23, True, 166849280), ("revnet164", 80, False, 505738496),
-    ("paper_revnet38", 80, False, 71953152), ("paper_revnet164", 23, True, 459435008),
+    ("paper_revnet38", 80, False, 71953152), ("paper_revnet164", 23, True, 459435008), ("revnet104", 23, True, 7489855488),
 ])
 def test_records_of_statistics_and_sums_take_no_workspace_of_their_own(ctx, name, N, stored, ceiling):
     """What the step planned when every producer reduced its records at once."""

@@ -138,3 +138,25 @@ def test_profiled_step_gives_the_same_result(ctx):
     assert torch.equal(res[0][2], res[1][2])
     for a, b in zip(res[0][:2], res[1][:2]):
         assert float((a - b).norm() / b.norm()) <= 1e-5
+
+
+def test_profiled_stored_step_fits_the_planned_workspace(ctx):
+    """Its weight gradients stay one launch per function, so every launch has the operands and splits of the ordinary step: the same bits."""
+    cfg = syn.shrink(syn.stack_config("revnet110"), N=23)
+    inp = syn.make_stack_inputs(cfg, affine_jitter=True)
+    res = []
+    for profiled in (False, True):
+        r = R.StackRunner(ctx, cfg, 0, store_activations=True)
+        r.load(inp["images"], inp["labels"], inp["params"])
+        B.revnet_profile_enable(ctx, 2 if profiled else 0)
+        try:
+            r.step()
+            torch.cuda.synchronize()
+            if profiled:
+                assert any(k.startswith("conv_wgrad_tc") for k in B.revnet_profile_summary(ctx))
+        finally:
+            B.revnet_profile_enable(ctx, 0)
+        res.append((r.grads.clone(), r.params.clone(), r.logits.clone()))
+        B.revnet_check_device(ctx)
+    for a, b in zip(*res):
+        assert torch.equal(a, b)
