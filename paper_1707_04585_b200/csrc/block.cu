@@ -60,10 +60,11 @@ static bool conv_dgrad(Exec &ex, const void *g, Geom gi, const Layer &L, float *
     conv_dgrad_simt(ex, g, b16, gi, L, da);
     return false;
 }
-static void conv_wgrad(Exec &ex, const void *g, const void *a, Geom gi, const Layer &L, float *dW) {
+// after: floats of the arena that the caller takes next, once the partials are given back
+static void conv_wgrad(Exec &ex, const void *g, const void *a, Geom gi, const Layer &L, float *dW, size_t after) {
     const bool b16 = ex.mode == 0;
     if (b16 && conv_wgrad_tc(ex, g, a, gi, L, dW, nullptr, nullptr)) return;
-    conv_wgrad_simt(ex, g, b16, a, b16, gi, L, dW);
+    conv_wgrad_simt(ex, g, b16, a, b16, gi, L, dW, after);
 }
 
 static size_t esz(const Exec &ex) { return ex.mode == 0 ? 2 : 4; }
@@ -186,7 +187,8 @@ void fn_backward(Exec &ex, Geom g, Pair u, const std::vector<Layer> &layers, FnS
         gq[l] = folded ? dt : gcur;
         auto wgrads = [&]() {            // as soon as every gradient operand exists
             if (!side) {
-                conv_wgrad(ex, gq[l], saved.a[l], gin[l], ly, ly.dW);
+                // (da; between layers also the next gradient operand and the da of the layer in front)
+                conv_wgrad(ex, gq[l], saved.a[l], gin[l], ly, ly.dW, P * ly.cin * (l && !b16 ? 2 : 1) + (l ? gin[l - 1].P() * layers[l - 1].cin : 0));
             } else if (l == 0) {
                 cudaStream_t main = ex.stream;
                 if (fork) {

@@ -420,7 +420,8 @@ void upsample_zero_bf16(Exec &ex, const bf16 *in, bf16 *out, int N, int Ho, int 
 // out = partner + sign*conv(a)   (sign 0: out = conv(a), partner unused)
 void conv_fprop_simt(Exec &ex, const void *a, bool a_bf16, Geom gi, const Layer &L, Pair out, Pair partner, int sign);
 void conv_dgrad_simt(Exec &ex, const void *g, bool g_bf16, Geom gi, const Layer &L, float *da);
-void conv_wgrad_simt(Exec &ex, const void *g, bool g_bf16, const void *a, bool a_bf16, Geom gi, const Layer &L, float *dW);
+// after: floats of the arena that the caller takes once the call's scratch is given back (scratch up to that costs no workspace)
+void conv_wgrad_simt(Exec &ex, const void *g, bool g_bf16, const void *a, bool a_bf16, Geom gi, const Layer &L, float *dW, size_t after = 0);
 
 // ---------------------------------------------------------------- stem.cu
 // the stem convolution of the image (few input channels), fp32; false: shape not taken, nothing launched

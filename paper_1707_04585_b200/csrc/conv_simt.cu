@@ -7,7 +7,7 @@
 //   wgrad: dW[co,kh,kw,ci] = sum_p g[p,co] * a[p (+) (kh,kw), ci]
 //
 // Four kernels.  conv3x3_direct_kernel takes fp32 3x3 stride-1 layers (forward and data gradient), wgrad3x3_strip_kernel the weight
-// gradients of those of at most 48, conv_gemm_kernel every other layer whose channel counts are multiples of four (all BN-ReLU-conv layers): quads of channels are loaded as vectors, a thread's pixel is decoded once, and the product is register-tiled.
+// gradients of most of those of at most 48 channels (see wg_strip_shape), conv_gemm_kernel every other layer whose channel counts are multiples of four (all BN-ReLU-conv layers): quads of channels are loaded as vectors, a thread's pixel is decoded once, and the product is register-tiled.
 // gemm_simt_kernel loads element by element and is left for the stem convolution's odd channel counts (an image has
 // three), where the kernels of stem.cu do not take its size.
 #include "common.cuh"
@@ -663,17 +663,20 @@ __global__ void splitk_reduce_kernel(const float *__restrict__ part, size_t n, i
 }
 
 // ------------------------------------------------------------------ weight gradient of fp32 3x3 stride-1 layers
-// dW[co, (kh, kw), ci] = sum over pixels of g[y, x, co] a[y + kh - 1, x + kw - 1, ci], of at most 48 x 48 channels.
+// dW[co, (kh, kw), ci] = sum over pixels of g[y, x, co] a[y + kh - 1, x + kw - 1, ci], of at most 64 channels on either
+// side and 144 pairs of channel quads (48 -> 48, 36 -> 64).
 // A lane keeps four input channels x four output channels x the three column taps of one row tap: walking along a row of the image
 // it reads one new quad of either tensor per pixel (the window of three input quads slides in registers) for 48 FMAs, where the
 // implicit GEMM above reads three per 32 and works out the pixel of every quad that it stages.
 // Warps: 3 row taps x nb blocks of 32 (input quad, output quad) pairs x R groups of rows; with at most 16 pairs a warp holds sl rows of
 // them.  The rows of a strip (BH rows of an image, and the halo rows of the input) arrive by asynchronous copies in two
 // buffers; the slices' sums are added through shared memory at the end, in order, and the CTAs' by splitk_reduce_kernel.
-// A lane's sum runs over its slice of the CTA's pixels: 64 products for 16 channels at 32x32.
-// Bound by the FMA pipes, and by launch, first copies and the two reductions for a third of the time.  Measured by events at batch 128: 16
-// channels at 32x32 57.9 -> 26.7 us, 32 at 16x16 33.7 -> 28.7 against the implicit GEMM; fp32 step of the
-// 38-layer network 5.61 -> 5.15 ms.
+// Sums.  A lane adds at most kWgStripRun products in a row, then the sum of that run to a second set of registers (one CTA of 384 to 480
+// threads per SM has them): rms error of dW against the runs of the implicit GEMM 0.98 (16 channels at 32x32, batch 128), 0.96
+// (batch 256), 0.89 (32 channels at 16x16), 0.91 and 0.82 (40 and 48 channels at 32x32); serial sums of 64 to 480 products had 1.1 to 1.9.
+// Bound by the FMA pipes, and by launch, first copies and the two reductions for a third of the time.  Block forward and backward, one layer per
+// function, against the implicit GEMM: 16 channels at 32x32, batch 128, 328 -> 267 us, batch 256 602 -> 462; 8 channels 229 -> 173; 48 channels
+// 1940 -> 1845; 32 channels at 16x16 267 -> 265; fp32 step of the 38-layer network 5.61 -> 5.18 ms.
 struct WgStrip {
     int N, H, W, Ci, Co;
     int cq, oq, pairs, sl, nb, R;         // quads per pixel, pairs of quads; slices per warp, blocks of pairs, row groups
@@ -681,11 +684,12 @@ struct WgStrip {
     int a_floats, g_floats;               // of a buffer
     FastDiv dcq, dw2, dpairs, dimg, dnb;  // by cq, by W + 2, by pairs, by per_img, by nb
 };
-constexpr int kWgStripThreads = 768;      // (at most 480 are launched; the bound keeps the kernel at 80 registers, two CTAs of 384 threads per SM)
+constexpr int kWgStripThreads = 480;
 // Most pairs of quads.  Above (56 channels and more) no two warps share a row and the implicit GEMM is as quick or quicker: 56 channels at
 // 8x8, batch 128, 24.6 against 24.5 us; fp32 stored step of the 110-layer network at batch 23 7.42 against 7.74 ms.
 constexpr int kWgStripPairs = 144;
-constexpr int kWgStripRun = 512;          // most products of one lane's sum (the error of a serial sum grows with it; see the runs of the implicit GEMM)
+constexpr int kWgStripRun = 33;           // products of a run; pieces of a row are multiples of the loop's three pixels
+constexpr int kWgStripRow = 512;          // longest row
 __device__ __forceinline__ void cp_async16(float *dst, const float *src, bool ok) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");
 }
@@ -734,11 +738,19 @@ __global__ void __launch_bounds__(kWgStripThreads, 1) wgrad3x3_strip_kernel(cons
     uint32_t oq, cq;
     p.dcq.divmod(pair, oq, cq);
     const int slice = (int)rg * p.sl + (int)sub, slices = p.R * p.sl;
-    float acc[3][16];
+    float acc[3][16], sum[3][16];            // products of the current run; sum of the runs before it
 #pragma unroll
     for (int k = 0; k < 3; k++)
 #pragma unroll
-        for (int i = 0; i < 16; i++) acc[k][i] = 0.f;
+        for (int i = 0; i < 16; i++) acc[k][i] = sum[k][i] = 0.f;
+    int run = 0;
+    auto flush = [&]() {
+        run = 0;
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+#pragma unroll
+            for (int i = 0; i < 16; i++) { sum[k][i] += acc[k][i]; acc[k][i] = 0.f; }
+    };
     fetch(s0, buf);
     for (int s = s0; s < s1; s++) {
         float *cur = buf + ((s - s0) & 1) * stage;
@@ -754,31 +766,37 @@ __global__ void __launch_bounds__(kWgStripThreads, 1) wgrad3x3_strip_kernel(cons
                 const float *pa = cur + (r + kh) * a_pitch + cq * 4, *pg = cur + p.a_floats + r * g_pitch + oq * 4;
                 float4 a0 = *reinterpret_cast<const float4 *>(pa), a1 = *reinterpret_cast<const float4 *>(pa + p.Ci), a2;
                 pa += 2 * p.Ci;
-                int x = 0;
 #pragma unroll 1
-                for (; x + 2 < p.W; x += 3) {
-                    float4 gv = *reinterpret_cast<const float4 *>(pg);
-                    a2 = *reinterpret_cast<const float4 *>(pa);
-                    wg_fma(acc[0], a0, gv); wg_fma(acc[1], a1, gv); wg_fma(acc[2], a2, gv);
-                    gv = *reinterpret_cast<const float4 *>(pg + p.Co);
-                    a0 = *reinterpret_cast<const float4 *>(pa + p.Ci);
-                    wg_fma(acc[0], a1, gv); wg_fma(acc[1], a2, gv); wg_fma(acc[2], a0, gv);
-                    gv = *reinterpret_cast<const float4 *>(pg + 2 * p.Co);
-                    a1 = *reinterpret_cast<const float4 *>(pa + 2 * p.Ci);
-                    wg_fma(acc[0], a2, gv); wg_fma(acc[1], a0, gv); wg_fma(acc[2], a1, gv);
-                    pa += 3 * p.Ci; pg += 3 * p.Co;
-                }
+                for (int x = 0, end; x < p.W; x = end) {
+                    end = x + kWgStripRun < p.W ? x + kWgStripRun : p.W;
+                    if (run + end - x > kWgStripRun) flush();
+                    run += end - x;
 #pragma unroll 1
-                for (; x < p.W; x++) {
-                    const float4 gv = *reinterpret_cast<const float4 *>(pg);
-                    a2 = *reinterpret_cast<const float4 *>(pa);
-                    wg_fma(acc[0], a0, gv); wg_fma(acc[1], a1, gv); wg_fma(acc[2], a2, gv);
-                    a0 = a1; a1 = a2;
-                    pa += p.Ci; pg += p.Co;
+                    for (; x + 2 < end; x += 3) {
+                        float4 gv = *reinterpret_cast<const float4 *>(pg);
+                        a2 = *reinterpret_cast<const float4 *>(pa);
+                        wg_fma(acc[0], a0, gv); wg_fma(acc[1], a1, gv); wg_fma(acc[2], a2, gv);
+                        gv = *reinterpret_cast<const float4 *>(pg + p.Co);
+                        a0 = *reinterpret_cast<const float4 *>(pa + p.Ci);
+                        wg_fma(acc[0], a1, gv); wg_fma(acc[1], a2, gv); wg_fma(acc[2], a0, gv);
+                        gv = *reinterpret_cast<const float4 *>(pg + 2 * p.Co);
+                        a1 = *reinterpret_cast<const float4 *>(pa + 2 * p.Ci);
+                        wg_fma(acc[0], a2, gv); wg_fma(acc[1], a0, gv); wg_fma(acc[2], a1, gv);
+                        pa += 3 * p.Ci; pg += 3 * p.Co;
+                    }
+#pragma unroll 1
+                    for (; x < end; x++) {
+                        const float4 gv = *reinterpret_cast<const float4 *>(pg);
+                        a2 = *reinterpret_cast<const float4 *>(pa);
+                        wg_fma(acc[0], a0, gv); wg_fma(acc[1], a1, gv); wg_fma(acc[2], a2, gv);
+                        a0 = a1; a1 = a2;
+                        pa += p.Ci; pg += p.Co;
+                    }
                 }
             }
         __syncthreads();
     }
+    flush();
     const int n_out = 9 * p.Ci * p.Co;
     float *out = part + (size_t)blockIdx.x * n_out, *dst = slices > 1 ? buf + (size_t)slice * n_out : out;
     if (active)
@@ -787,7 +805,7 @@ __global__ void __launch_bounds__(kWgStripThreads, 1) wgrad3x3_strip_kernel(cons
 #pragma unroll
             for (int j = 0; j < 4; j++)
                 *reinterpret_cast<float4 *>(dst + ((oq * 4 + j) * 9 + kh * 3 + k) * p.Ci + cq * 4) =
-                    make_float4(acc[k][4 * j], acc[k][4 * j + 1], acc[k][4 * j + 2], acc[k][4 * j + 3]);
+                    make_float4(sum[k][4 * j], sum[k][4 * j + 1], sum[k][4 * j + 2], sum[k][4 * j + 3]);
     if (slices > 1) {
         __syncthreads();
         for (int i = tid; i < n_out / 4; i += nt) {
@@ -800,43 +818,57 @@ __global__ void __launch_bounds__(kWgStripThreads, 1) wgrad3x3_strip_kernel(cons
         }
     }
 }
-// The shape of that launch; false: not taken (other kernels and strides, more channels, rows too long for the shared memory)
-static bool wg_strip_shape(const ConvGeom &g, int sm, WgStrip &p, int &ctas, int &threads, int &smem) {
-    if (g.k != 3 || g.s != 1 || g.Ci % 4 || g.Co % 4 || g.Ci > 64 || g.Co > 64 || g.W > kWgStripRun) return false;
+// The shape of that launch; false: not taken (other kernels and strides, more channels, rows too long for the shared memory, tensors too small).
+// most: CTAs whose partials there is room for
+static bool wg_strip_shape(const ConvGeom &g, int sm, int most, WgStrip &p, int &ctas, int &threads, int &smem) {
+    if (g.k != 3 || g.s != 1 || g.Ci % 4 || g.Co % 4 || g.Ci > 64 || g.Co > 64 || g.W > kWgStripRow) return false;
     p.N = g.N; p.H = g.H; p.W = g.W; p.Ci = g.Ci; p.Co = g.Co;
     p.cq = g.Ci / 4; p.oq = g.Co / 4; p.pairs = p.cq * p.oq;
     if (p.pairs > kWgStripPairs) return false;
     p.sl = p.pairs <= 16 ? 32 / p.pairs : 1;
     p.nb = p.sl > 1 ? 1 : (p.pairs + 31) / 32;
     if (p.sl > p.H) p.sl = p.H;
-    p.R = 4 / p.nb < 1 ? 1 : 4 / p.nb;               // about twelve warps
-    while (p.R > 1 && (p.R * p.sl > p.H || p.N * ((p.H + p.R * p.sl - 1) / (p.R * p.sl)) < sm)) p.R--;      // (few images: smaller CTAs)
-    threads = 96 * p.nb * p.R;
+    // strips: two buffers of as many rows, a multiple of the slices, as there is shared memory for; one round of the slices at least
+    const size_t room = 200 * 1024;
+    auto bytes_of = [&](int bh) { return 2 * ((size_t)(bh + 2) * (g.W + 2) * g.Ci + (size_t)bh * g.W * g.Co) * sizeof(float); };
+    while (p.sl > 1 && bytes_of(p.sl) > room) p.sl--;
+    if (bytes_of(p.sl) > room) return false;
+    // Groups of rows: as many as make about twelve warps.  Where those CTAs would not fill the SMs, the number that gives an SM the shortest run of
+    // rows.  CTAs per SM: one, or two to five of fewer warps where their buffers fit side by side.  (An SM counts as idle in part below six warps)
+    int fit = 0, side = 1;             // CTAs in all, CTAs side by side on an SM
+    long long least = -1;
+    for (int R = 4 / p.nb < 1 ? 1 : 4 / p.nb; R >= 1; R--) {
+        const int sl = R * p.sl, n = 96 * p.nb * R;
+        if (R > 1 && (sl > p.H || bytes_of(sl) > room)) continue;
+        int per_sm = kWgStripThreads / n;
+        while (per_sm > 1 && bytes_of(sl) > room / per_sm) per_sm--;
+        const int f = most < sm * per_sm ? most : sm * per_sm, strips = p.N * ((p.H + sl - 1) / sl), ctas1 = strips < f ? strips : f;
+        const int warps = 3 * p.nb * R * ((ctas1 + sm - 1) / sm);
+        const long long cost = (long long)((strips + f - 1) / f) * (warps < 6 ? 6 : warps);
+        if (least < 0 || cost < least) { least = cost; p.R = R; fit = f; side = per_sm; threads = n; }
+        if (strips >= sm) break;
+    }
     const int slices = p.R * p.sl;
-    // strips: as many rows, a multiple of the slices, as two CTAs per SM have room for in two buffers; a strip of one round of the slices at least
-    auto floats = [&](int bh) { return (size_t)(bh + 2) * (g.W + 2) * g.Ci + (size_t)bh * g.W * g.Co; };
-    // (of these the height that gives a CTA the fewest rows, its strips' halos counted as one each)
-    const int room = sm * (threads <= 384 ? 2 : 1);
+    // (of the heights the one that gives a CTA the fewest rows, its strips' halos counted as one each)
     long long best = -1;
     for (int bh = slices;; bh += slices) {
         const int h = bh < p.H ? bh : p.H, strips = p.N * ((p.H + h - 1) / h);
-        const long long cost = (long long)((strips + room - 1) / room) * (h + 1);
+        const long long cost = (long long)((strips + fit - 1) / fit) * (h + 1);
         if (best < 0 || cost <= best) { best = cost; p.BH = h; }
-        if (h == p.H || 2 * floats(bh + slices) * 4 > 100 * 1024 || (bh / slices + 1) * g.W > kWgStripRun) break;
+        if (h == p.H || bytes_of(bh + slices) > room / side) break;
     }
     p.a_floats = (p.BH + 2) * (g.W + 2) * g.Ci; p.g_floats = p.BH * g.W * g.Co;
-    size_t bytes = 2 * floats(p.BH) * 4;
+    size_t bytes = bytes_of(p.BH);
     const size_t red = slices > 1 ? (size_t)slices * 9 * g.Ci * g.Co * 4 : 0;
     if (bytes < red) bytes = red;
-    if (bytes > 200 * 1024) return false;
+    if (bytes > room) return false;                  // (a few rows beside a large reduction: fewer CTAs per SM than counted on)
     smem = (int)bytes;
     p.per_img = (p.H + p.BH - 1) / p.BH; p.strips = p.N * p.per_img;
-    // as many CTAs as there is room for, with the same number of strips each
-    const int fit = smem <= 112 * 1024 ? room : sm;
-    p.per_cta = (p.strips + fit - 1) / fit;
-    const int run = (p.BH + slices - 1) / slices * g.W;              // products of a lane's sum per strip
-    if (p.per_cta * run > kWgStripRun) p.per_cta = kWgStripRun / run;
+    p.per_cta = (p.strips + fit - 1) / fit;          // the same number of strips each
     ctas = (p.strips + p.per_cta - 1) / p.per_cta;
+    // Partials for too few SMs: the implicit GEMM spreads its tiles of dW as well.  Few channels gain most from strips: 24 channels, 40 images of 13x12,
+    // 299 us with the GEMM against 286 with strips on 54 % of the SMs; 40 channels, 40 of 31x25, 692 against 714 on 65 %.
+    if (most < sm && ctas * 4 <= sm * (p.pairs <= 36 ? 2 : 3)) return false;
     p.dcq = fast_div(p.cq); p.dw2 = fast_div(g.W + 2); p.dpairs = fast_div(p.pairs); p.dimg = fast_div(p.per_img); p.dnb = fast_div(p.nb);
     return true;
 }
@@ -852,13 +884,23 @@ static void wgrad_launch(Exec &ex, const TG *gq, const TA *a, ConvGeom g, float 
     else if (N <= 32) launch_tile<1, 2, 4>(ex, al, bl, ep, M, N, K, splits, kps);
     else launch_tile<1, 4, 2>(ex, al, bl, ep, M, N, K, splits, kps);
 }
-void conv_wgrad_simt(Exec &ex, const void *gq, bool g_bf16, const void *a, bool a_bf16, Geom gi, const Layer &L, float *dW) {
+void conv_wgrad_simt(Exec &ex, const void *gq, bool g_bf16, const void *a, bool a_bf16, Geom gi, const Layer &L, float *dW, size_t after) {
     ConvGeom g = geom_of(gi, L);
     const int Co = g.Co, KC = g.k * g.k * g.Ci, P = g.N * g.Ho * g.Wo;
     ex.flops += 2ull * Co * KC * (size_t)P;
+    const bool quads = g.Ci % 4 == 0 && g.Co % 4 == 0;
+    const int bn = Co <= 16 ? 16 : (Co <= 32 ? 32 : 64);
+    const int tiles = quads ? ((KC + 63) / 64) * ((Co + bn - 1) / bn) : ((Co + 63) / 64) * ((KC + 63) / 64);
+    int splits = (ex.ctx->sm_count * (quads ? 4 : 2) + tiles - 1) / tiles;
+    int max_splits = (P + 255) / 256; if (splits > max_splits) splits = max_splits; if (splits < 1) splits = 1;
+    int kps = (((P + splits - 1) / splits) + 15) / 16 * 16;
+    splits = (P + kps - 1) / kps;
+    // partials of strips: as many as the implicit GEMM would have, or as take no more workspace than what the caller allocates behind them
+    const size_t room = after / ((size_t)Co * KC);
+    const int most = (size_t)splits > room ? splits : (int)(room < (size_t)P ? room : (size_t)P);
     WgStrip st;
     int ctas, threads, smem;
-    if (!g_bf16 && !a_bf16 && wg_strip_shape(g, ex.ctx->sm_count, st, ctas, threads, smem)) {
+    if (!g_bf16 && !a_bf16 && wg_strip_shape(g, ex.ctx->sm_count, most, st, ctas, threads, smem)) {
         size_t m = ex.ws.mark();
         float *part = ctas > 1 ? ex.ws.get<float>((size_t)ctas * Co * KC) : dW;
         if (!ex.dry) {
@@ -875,13 +917,6 @@ void conv_wgrad_simt(Exec &ex, const void *gq, bool g_bf16, const void *a, bool 
         ex.ws.release(m);
         return;
     }
-    const bool quads = g.Ci % 4 == 0 && g.Co % 4 == 0;
-    const int bn = Co <= 16 ? 16 : (Co <= 32 ? 32 : 64);
-    const int tiles = quads ? ((KC + 63) / 64) * ((Co + bn - 1) / bn) : ((Co + 63) / 64) * ((KC + 63) / 64);
-    int splits = (ex.ctx->sm_count * (quads ? 4 : 2) + tiles - 1) / tiles;
-    int max_splits = (P + 255) / 256; if (splits > max_splits) splits = max_splits; if (splits < 1) splits = 1;
-    int kps = (((P + splits - 1) / splits) + 15) / 16 * 16;
-    splits = (P + kps - 1) / kps;
     size_t m = ex.ws.mark();
     float *part = splits > 1 ? ex.ws.get<float>((size_t)splits * Co * KC) : dW;
     if (!ex.dry) {

@@ -151,6 +151,7 @@ def test_reversible_step_holds_a_fraction_of_what_ordinary_backprop_holds(ctx, n
     ("basic", 128, 8, 8, 56, 0, 1, 12790272),
     ("basic", 60, 41, 10, 100, 0, 0, 54856192),
     ("single", 28, 39, 35, 12, 0, 0, 4598880),
+    ("basic", 37, 15, 21, 24, 0, 1, 6729344), ("single", 57, 13, 8, 32, 0, 1, 1644032), ("single", 75, 40, 17, 40, 0, 1, 16488960), ("basic", 6, 25, 40, 36, 0, 1, 5442048),
 ])
 def test_block_backward_asks_for_no_more_workspace(ctx, kind, N, H, W, c, w, mode, ceiling):
     """Weight gradients layer by layer: their split partials and the next tensor of the data-gradient chain are not held at once."""
