@@ -519,7 +519,7 @@ void bn_relu_bwd(Exec &ex, const float *da, Pair t, size_t P, BnRef bn, float *d
 constexpr int kSumsRows = 4;
 template <bool ADD, bool CAST>
 __global__ void __launch_bounds__(256, 2) bn_relu_bwd_sums_kernel(const float *__restrict__ da, Pair t, int P, int rows, BnRef bn, float *__restrict__ dgamma,
-                                                                  float *__restrict__ dbeta, const float *__restrict__ add, float *__restrict__ out,
+                                                                  float *__restrict__ dbeta, const float *add, float *out,
                                                                   bf16 *__restrict__ cast, unsigned long long *stamp) {
     __shared__ double red[256 * 4], tot[32 * 4];
     __shared__ __align__(16) float cf[7][64];
@@ -531,7 +531,8 @@ __global__ void __launch_bounds__(256, 2) bn_relu_bwd_sums_kernel(const float *_
     auto load = [&](int rb) {
 #pragma unroll
         for (int j = 0; j < kSumsRows; j++) {
-            int row = rb + j * rpp; if (row >= r1) row = r1 - 1;
+            const int row = rb + j * rpp;
+            if (row >= r1) continue;          // (out may be add: a row is read by the thread that stores it, and by no other)
             const size_t off = (size_t)row * C + q * 4;
             v[j] = ld4(t.p0 + off); g[j] = ld4(da + off);
             if (ADD) a[j] = ld4(add + off);
