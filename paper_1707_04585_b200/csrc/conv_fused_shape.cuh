@@ -82,7 +82,8 @@ static inline bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count,
     g.BN = cout_pad <= 16 ? 16 : (cout_pad <= 32 ? 32 : 64);
     // few tiles (late stages): split the output channels so that more SMs take part
     while (g.BN > 16 && tiles * ((cout_pad + g.BN - 1) / g.BN) * 2 <= sm_count) g.BN /= 2;
-    for (;; g.BN /= 2) {
+    bool tight = false;          // (very long rows: one shortest piece of the input at a time leaves the most to the operand)
+    for (;; tight ? (void)0 : (void)(g.BN /= 2)) {
         s.n_tiles = (cout_pad + g.BN - 1) / g.BN;
         g.groups = g.BN / NC;
         s.EW = g.BN == 64 ? 16 : 8;
@@ -97,10 +98,10 @@ static inline bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count,
         // Six build warps, or ten where a CTA has a tile at most and so waits for its build (24 channels, 8 images of 9x17, forward: 19.7 against 18.8 us);
         // with more tiles they cost the epilogue beside them more than they give (16 channels, 14 images of 47x44: 21.6 against 22.6 us), and beside sixteen
         // epilogue warps there are no registers for them.
-        s.NBT = s.EW == 8 && g.chunk <= 128 ? 320 : 192;
+        s.NBT = s.EW == 8 && g.chunk <= 128 && !tight ? 320 : 192;
         g.RS = s.NBT / g.nit; g.step_r = g.RS / g.pitch; g.step_c = g.RS % g.pitch;
         g.piece = g.RS;
-        while (2 * g.piece * g.rowb * tensors <= 12800) g.piece *= 2;
+        while (!tight && 2 * g.piece * g.rowb * tensors <= 12800) g.piece *= 2;
         g.raw_bytes = round_up(g.piece * g.rowb, 128) * tensors;
         g.wtile_bytes = (g.BN * g.KC * 2 + 1023) & ~1023;
         const int T = (g.chunk + 127) / 128, fixed = 1024 + k * k * g.wtile_bytes + (int)sizeof(FusedShared) + 64;
@@ -116,14 +117,19 @@ static inline bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count,
         auto tabs_of = [&](int nseg) { return nseg == 2 && 32 % g.nit != 0 ? 2 : 1; };
         auto fits = [&](int S, int nseg) {
             const int op = nseg * seg_of(S);
-            return (op < least ? least : op) + (T <= S && pieces_of(S) < 2 ? 1 : 2) * g.raw_bytes + aux1 + tabs_of(nseg) * tab_of(S) <= room;
+            return (op < least ? least : op) + (tight || (T <= S && pieces_of(S) < 2) ? 1 : 2) * g.raw_bytes + aux1 + tabs_of(nseg) * tab_of(S) <= room;
         };
         // (1x1: no halo to build twice, short segments leave the room to the rings)
         if (T <= (k == 1 ? 2 : kFullBars) && fits(T, 1)) { g.S = T; g.nseg = 1; }
         else {
             g.nseg = 2; g.S = k == 1 ? 2 : kFullBars / 2;
             while (g.S > 1 && !fits(g.S, 2)) g.S--;
-            if (!fits(g.S, 2)) g.nseg = 1;
+            // One buffer of longer segments, where the 2 halo rows that every segment builds again cost more than the wait for the MMAs at each
+            // end of a segment, about as long as two rounds of RS rows
+            int S1 = kFullBars;
+            while (S1 > 1 && !fits(S1, 1)) S1--;
+            const int segs1 = (T + S1 - 1) / S1, segs2 = (T + g.S - 1) / g.S;
+            if (!fits(g.S, 2) || (k == 3 && g.halo * (segs2 - segs1) >= g.RS * (segs1 - 1))) { g.nseg = 1; g.S = (T + segs1 - 1) / segs1; }
         }
         g.plane16 = plane_of(g.S);
         g.seg_bytes = seg_of(g.S);
@@ -136,16 +142,23 @@ static inline bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count,
         // what is left goes to more pieces and more partner rows in flight, whichever has less
         // (a range that fits in two pieces beside two tiles of partner rows comes in two, the first with the first tile's rows at least:
         // every piece costs a build warp 0.3 us)
-        if (T <= g.S) {
+        if (T <= g.S && !tight) {
             const int rows = g.chunk + 2 * g.halo, first = 128 + 2 * g.halo, half = (rows + 1) / 2;
             const int R = round_up(half < first && first < rows ? first : half, g.RS), bytes = round_up(R * g.rowb, 128) * tensors;
             if (R > g.piece && g.op_bytes + tab + (R >= rows ? 1 : 2) * bytes + 2 * aux1 <= room) {
                 g.piece = R; g.raw_bytes = bytes; g.pps = g.pieces = pieces_of(g.S); g.dpps = fast_div(g.pps);
             }
         }
+        // several segments: pieces as long as two of them fit, at most two thirds of a segment (24 -> 48 KB: 64 channels at 32x32, batch 128, forward 174 -> 170 us)
+        if (T > g.S && !tight) {
+            while (g.op_bytes + tab + 2 * round_up(2 * g.piece * g.rowb, 128) * tensors + aux1 <= room && 3 * g.piece <= g.S * 128 + 2 * g.halo) {
+                g.piece *= 2; g.raw_bytes = round_up(g.piece * g.rowb, 128) * tensors;
+            }
+            g.pps = pieces_of(g.S); g.dpps = fast_div(g.pps);
+        }
         const int most_raw = T <= g.S ? (pieces_of(g.S) < kRawSlots ? pieces_of(g.S) : kRawSlots) : kRawSlots;
         const int most_aux = !aux ? 0 : (own_tiles < kAuxSlots ? own_tiles : kAuxSlots);
-        g.raw_slots = most_raw < 2 ? most_raw : 2; g.aux_slots = aux ? 1 : 0;
+        g.raw_slots = most_raw < 2 || tight ? 1 : 2; g.aux_slots = aux ? 1 : 0;
         int left = room - g.op_bytes - tab - g.raw_slots * g.raw_bytes - g.aux_slots * aux1;
         s.smem = 227 * 1024 - left;
         if (left >= 0 && g.plane16 < (1 << 14)) {
@@ -158,6 +171,6 @@ static inline bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count,
             s.smem = 227 * 1024 - left;
             return true;
         }
-        if (g.BN < 32) return false;
+        if (g.BN < 32) { if (tight) return false; tight = true; }
     }
 }

@@ -35,24 +35,30 @@ def test_fused_layers_at_ring_edges(ctx, kind, N, H, W, c, w):
     tp.run_block_case(ctx, syn.BlockCfg(N, H, W, c, w, kind, seed=700 + c), 0, jitter=True, inplace=True)
 
 
-# 3x3 layers whose CTAs take their range in several operand segments, two buffers in turn (tests/test_fused_shapes_host.py holds the last
-# number, their segments, against the launch geometry).  With 24, 40, 48 and 56 channels the threads of a row sit in two warps
+# 3x3 layers whose CTAs take their range in several operand segments, in one buffer or two in turn (tests/test_fused_shapes_host.py holds the last
+# two numbers, segments and buffers, against the launch geometry).  With 24, 40, 48 and 56 channels the threads of a row sit in two warps
 SEGMENTED = [
-    ("single", 3, 133, 485, 24, 11),
-    ("basic", 3, 226, 119, 40, 5),
-    ("single", 37, 46, 64, 48, 3),
-    ("basic", 7, 114, 77, 56, 4),
-    ("single", 100, 24, 30, 64, 3),
+    ("single", 2415, 31, 3, 24, 3, 2),
+    ("basic", 935, 31, 3, 40, 3, 2),
+    ("single", 935, 31, 3, 48, 3, 2),
+    ("basic", 213, 31, 11, 56, 3, 2),
+    ("single", 3, 133, 485, 24, 2, 1),
+    ("basic", 3, 226, 119, 40, 2, 1),
+    ("single", 2, 17, 691, 40, 4, 1),
+    ("basic", 7, 114, 77, 56, 2, 1),
+    ("single", 100, 24, 30, 64, 2, 1),
+    ("single", 2, 9, 600, 64, 3, 1),      # rows so long that one piece of the input at a time is all that fits beside the operand
 ]
 
 
-@pytest.mark.parametrize("kind,N,H,W,c,segments", SEGMENTED)
-def test_segments_in_turn(ctx, kind, N, H, W, c, segments):
+@pytest.mark.parametrize("kind,N,H,W,c,segments,buffers", SEGMENTED)
+def test_segments_in_turn(ctx, kind, N, H, W, c, segments, buffers):
     tp.run_block_case(ctx, syn.BlockCfg(N, H, W, c, 0, kind, seed=750 + c), 0, jitter=True, inplace=True)
 
 
-def test_segments_in_turn_give_the_same_bits_every_time(ctx):
-    b = syn.BlockCfg(3, 226, 119, 40, 0, "single", seed=790)
+@pytest.mark.parametrize("N,H,W,c", [(3, 226, 119, 40), (935, 31, 3, 48)])
+def test_segments_in_turn_give_the_same_bits_every_time(ctx, N, H, W, c):
+    b = syn.BlockCfg(N, H, W, c, 0, "single", seed=790)
     r, inp = R.BlockRunner(ctx, b, 0), syn.make_block_inputs(b)
     r.load(inp["params"])
     first = None
