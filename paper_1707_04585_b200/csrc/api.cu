@@ -110,12 +110,13 @@ extern "C" int revnet_block_workspace_bytes(revnet_ctx *ctx, const revnet_block_
     Geom g{d->N, d->H, d->W};
     float *fake = (float *)0x1000;
     for (int pass = 0; pass < 2; pass++) {
+        size_t *o = pass == 0 ? fwd_bytes : bwd_bytes;
+        if (!o) continue;          // (every block call asks for its own direction)
         Exec ex; ex.ctx = ctx; ex.dry = true; ex.ws.dry = true; ex.mode = d->mode; ex.eps = d->eps;
         auto F = layers_of(d->F, nullptr, nullptr), G = layers_of(d->G, nullptr, nullptr);
         if (pass == 0) block_forward(ex, g, d->c, F, G, fake, fake, fake, fake);
         else block_backward(ex, g, d->c, F, G, fake, fake, fake, fake, fake, fake, fake, fake);
-        size_t *o = pass == 0 ? fwd_bytes : bwd_bytes;
-        if (o) *o = ex.ws.peak + 256;
+        *o = ex.ws.peak + 256;
     }
     return REVNET_OK;
 }

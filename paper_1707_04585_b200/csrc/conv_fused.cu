@@ -633,6 +633,23 @@ __global__ void __launch_bounds__(EW == 8 ? 640 : fused_threads(EW, NBT), 1) con
     }
 }
 
+// fused_shape, which a call asks for every layer several times over (sizing run, launch, whether a neighbour can leave its records): the last
+// shapes of a thread are at hand.  (16 channels at 32x32: sizing a block backward 4.0 -> 2.4 us on the host)
+const FusedShape *shape_of(Geom geo, int cin, int cout, int k, int sm_count, int in_mode, bool aux) {
+    struct Entry { int key[8]; bool ok; FusedShape s; };
+    constexpr int kEntries = 16;
+    static thread_local Entry memo[kEntries];          // (an empty entry has k = 0)
+    static thread_local int next = 0;
+    if (in_mode == kInFixed) in_mode = kInFloat;       // the same rows
+    const int key[8] = {geo.N, geo.H, geo.W, cin, cout, k, sm_count, in_mode * 2 + (aux ? 1 : 0)};
+    for (const Entry &e : memo) if (!memcmp(e.key, key, sizeof key)) return e.ok ? &e.s : nullptr;
+    Entry &e = memo[next];
+    next = (next + 1) % kEntries;
+    memcpy(e.key, key, sizeof key);
+    e.ok = fused_shape(geo, cin, cout, k, sm_count, in_mode, aux, e.s);
+    return e.ok ? &e.s : nullptr;
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
                                   const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -643,10 +660,11 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
 bool run_fused(Exec &ex, const char *what, int in_mode, const void *in, float in_q, BnRef bn, Geom geo, int cin, int cout, int k,
                const float *Wsrc, const bf16 *prepacked, bool transposed, Pair out, Pair partner, int sign, EpiReq req, bf16 *a_out,
                const BnBwdReq *behind = nullptr, BwdSums *sums = nullptr) {
-    FusedShape s;
     if (out.c1 != 0 || (sign && partner.c1 != 0) || (req.bnbwd && req.bnbwd->t.c1 != 0)) return false;
     const bool aux = sign != 0 || req.bnbwd;
-    if (!fused_shape(geo, cin, cout, k, ex.ctx->sm_count, in_mode, aux, s)) return false;
+    const FusedShape *sp = shape_of(geo, cin, cout, k, ex.ctx->sm_count, in_mode, aux);
+    if (!sp) return false;
+    const FusedShape &s = *sp;
     EncodeTiledFn enc = nullptr;
     if (!ex.dry) { enc = (EncodeTiledFn)tc_encoder(ex.ctx); if (!enc) return false; }
     const int taps = k * k;
@@ -721,8 +739,7 @@ bool run_fused(Exec &ex, const char *what, int in_mode, const void *in, float in
 
 // whether conv_fprop_fused takes layer L on images gi (and so adds pending statistics of its input itself)
 bool conv_fused_takes(Exec &ex, Geom gi, const Layer &L) {
-    FusedShape s;
-    return L.stride == 1 && fused_shape(gi, L.cin, L.cout, L.k, ex.ctx->sm_count, kInFloat, true, s);
+    return L.stride == 1 && shape_of(gi, L.cin, L.cout, L.k, ex.ctx->sm_count, kInFloat, true);
 }
 
 // out = partner + sign * conv(ReLU(BN(t)));  a_out (optional): the activated tensor, for the weight gradient
@@ -743,13 +760,13 @@ bool conv_dgrad_fused(Exec &ex, const void *g, Geom gi, const Layer &L, float *d
 // whether conv_dgrad_fused takes the data gradient of L, with a bf16 input or (behind) through the BN backward of the layer behind; parts: the
 // records of 2 cin sums that it leaves
 bool conv_dgrad_fused_takes(Exec &ex, Geom gi, const Layer &L, bool behind, int *parts) {
-    FusedShape s;
-    if (L.stride != 1 || !fused_shape(gi, L.cout, L.cin, L.k, ex.ctx->sm_count, behind ? kInBwd : kInBf16, true, s) || !(ex.dry || tc_encoder(ex.ctx))) return false;
-    *parts = s.ctas;
+    const FusedShape *s = L.stride == 1 ? shape_of(gi, L.cout, L.cin, L.k, ex.ctx->sm_count, behind ? kInBwd : kInBf16, true) : nullptr;
+    if (!s || !(ex.dry || tc_encoder(ex.ctx))) return false;
+    *parts = s->ctas;
     // Through the BN backward only where a build thread has few rows: its pass costs 0.3 us per row and thread, twice that of a bf16 input with
     // twice the threads per row, against 5 us for the launch that it saves.  Odd-sized block (24 channels, a tile per CTA, five and a half rows)
     // 151 -> 144.5 us; 56 channels at 8x8 (eleven rows) and 16 at 32x32 (twenty-one): 38-layer step 1665 -> 1686.
-    return !behind || (long long)(s.g.chunk + 2 * s.g.halo) * s.g.nit <= 6 * 192;
+    return !behind || (long long)(s->g.chunk + 2 * s->g.halo) * s->g.nit <= 6 * 192;
 }
 
 // The same where the gradient still has to go through the BN + ReLU backward of the layer behind L: g is da of that layer (float), `behind` its
