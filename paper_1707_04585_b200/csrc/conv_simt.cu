@@ -12,6 +12,7 @@
 // three), where the kernels of stem.cu do not take its size.
 #include "common.cuh"
 #include "conv_direct.cuh"
+#include "conv_strips.cuh"
 #include <algorithm>
 
 template <class T> __device__ __forceinline__ float ldf(const T *p);
@@ -677,19 +678,6 @@ __global__ void splitk_reduce_kernel(const float *__restrict__ part, size_t n, i
 // Bound by the FMA pipes, and by launch, first copies and the two reductions for a third of the time.  Block forward and backward, one layer per
 // function, against the implicit GEMM: 16 channels at 32x32, batch 128, 328 -> 267 us, batch 256 602 -> 462; 8 channels 229 -> 173; 48 channels
 // 1940 -> 1845; 32 channels at 16x16 267 -> 265; fp32 step of the 38-layer network 5.61 -> 5.18 ms.
-struct WgStrip {
-    int N, H, W, Ci, Co;
-    int cq, oq, pairs, sl, nb, R;         // quads per pixel, pairs of quads; slices per warp, blocks of pairs, row groups
-    int BH, strips, per_img, per_cta;
-    int a_floats, g_floats;               // of a buffer
-    FastDiv dcq, dw2, dpairs, dimg, dnb;  // by cq, by W + 2, by pairs, by per_img, by nb
-};
-constexpr int kWgStripThreads = 480;
-// Most pairs of quads.  Above (56 channels and more) no two warps share a row and the implicit GEMM is as quick or quicker: 56 channels at
-// 8x8, batch 128, 24.6 against 24.5 us; fp32 stored step of the 110-layer network at batch 23 7.42 against 7.74 ms.
-constexpr int kWgStripPairs = 144;
-constexpr int kWgStripRun = 33;           // products of a run; pieces of a row are multiples of the loop's three pixels
-constexpr int kWgStripRow = 512;          // longest row
 __device__ __forceinline__ void cp_async16(float *dst, const float *src, bool ok) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 16 : 0) : "memory");
 }
@@ -818,61 +806,6 @@ __global__ void __launch_bounds__(kWgStripThreads, 1) wgrad3x3_strip_kernel(cons
         }
     }
 }
-// The shape of that launch; false: not taken (other kernels and strides, more channels, rows too long for the shared memory, tensors too small).
-// most: CTAs whose partials there is room for
-static bool wg_strip_shape(const ConvGeom &g, int sm, int most, WgStrip &p, int &ctas, int &threads, int &smem) {
-    if (g.k != 3 || g.s != 1 || g.Ci % 4 || g.Co % 4 || g.Ci > 64 || g.Co > 64 || g.W > kWgStripRow) return false;
-    p.N = g.N; p.H = g.H; p.W = g.W; p.Ci = g.Ci; p.Co = g.Co;
-    p.cq = g.Ci / 4; p.oq = g.Co / 4; p.pairs = p.cq * p.oq;
-    if (p.pairs > kWgStripPairs) return false;
-    p.sl = p.pairs <= 16 ? 32 / p.pairs : 1;
-    p.nb = p.sl > 1 ? 1 : (p.pairs + 31) / 32;
-    if (p.sl > p.H) p.sl = p.H;
-    // strips: two buffers of as many rows, a multiple of the slices, as there is shared memory for; one round of the slices at least
-    const size_t room = 200 * 1024;
-    auto bytes_of = [&](int bh) { return 2 * ((size_t)(bh + 2) * (g.W + 2) * g.Ci + (size_t)bh * g.W * g.Co) * sizeof(float); };
-    while (p.sl > 1 && bytes_of(p.sl) > room) p.sl--;
-    if (bytes_of(p.sl) > room) return false;
-    // Groups of rows: as many as make about twelve warps.  Where those CTAs would not fill the SMs, the number that gives an SM the shortest run of
-    // rows.  CTAs per SM: one, or two to five of fewer warps where their buffers fit side by side.  (An SM counts as idle in part below six warps)
-    int fit = 0, side = 1;             // CTAs in all, CTAs side by side on an SM
-    long long least = -1;
-    for (int R = 4 / p.nb < 1 ? 1 : 4 / p.nb; R >= 1; R--) {
-        const int sl = R * p.sl, n = 96 * p.nb * R;
-        if (R > 1 && (sl > p.H || bytes_of(sl) > room)) continue;
-        int per_sm = kWgStripThreads / n;
-        while (per_sm > 1 && bytes_of(sl) > room / per_sm) per_sm--;
-        const int f = most < sm * per_sm ? most : sm * per_sm, strips = p.N * ((p.H + sl - 1) / sl), ctas1 = strips < f ? strips : f;
-        const int warps = 3 * p.nb * R * ((ctas1 + sm - 1) / sm);
-        const long long cost = (long long)((strips + f - 1) / f) * (warps < 6 ? 6 : warps);
-        if (least < 0 || cost < least) { least = cost; p.R = R; fit = f; side = per_sm; threads = n; }
-        if (strips >= sm) break;
-    }
-    const int slices = p.R * p.sl;
-    // (of the heights the one that gives a CTA the fewest rows, its strips' halos counted as one each)
-    long long best = -1;
-    for (int bh = slices;; bh += slices) {
-        const int h = bh < p.H ? bh : p.H, strips = p.N * ((p.H + h - 1) / h);
-        const long long cost = (long long)((strips + fit - 1) / fit) * (h + 1);
-        if (best < 0 || cost <= best) { best = cost; p.BH = h; }
-        if (h == p.H || bytes_of(bh + slices) > room / side) break;
-    }
-    p.a_floats = (p.BH + 2) * (g.W + 2) * g.Ci; p.g_floats = p.BH * g.W * g.Co;
-    size_t bytes = bytes_of(p.BH);
-    const size_t red = slices > 1 ? (size_t)slices * 9 * g.Ci * g.Co * 4 : 0;
-    if (bytes < red) bytes = red;
-    if (bytes > room) return false;                  // (a few rows beside a large reduction: fewer CTAs per SM than counted on)
-    smem = (int)bytes;
-    p.per_img = (p.H + p.BH - 1) / p.BH; p.strips = p.N * p.per_img;
-    p.per_cta = (p.strips + fit - 1) / fit;          // the same number of strips each
-    ctas = (p.strips + p.per_cta - 1) / p.per_cta;
-    // Partials for too few SMs: the implicit GEMM spreads its tiles of dW as well.  Few channels gain most from strips: 24 channels, 40 images of 13x12,
-    // 299 us with the GEMM against 286 with strips on 54 % of the SMs; 40 channels, 40 of 31x25, 692 against 714 on 65 %.
-    if (most < sm && ctas * 4 <= sm * (p.pairs <= 36 ? 2 : 3)) return false;
-    p.dcq = fast_div(p.cq); p.dw2 = fast_div(g.W + 2); p.dpairs = fast_div(p.pairs); p.dimg = fast_div(p.per_img); p.dnb = fast_div(p.nb);
-    return true;
-}
-
 // dW as a GEMM of M = (tap, ci), N = co over the pixels; the pixels are split so that the grid fills the machine twice
 template <class TG, class TA>
 static void wgrad_launch(Exec &ex, const TG *gq, const TA *a, ConvGeom g, float *part, int splits, int kps) {
@@ -900,7 +833,7 @@ void conv_wgrad_simt(Exec &ex, const void *gq, bool g_bf16, const void *a, bool 
     const int most = (size_t)splits > room ? splits : (int)(room < (size_t)P ? room : (size_t)P);
     WgStrip st;
     int ctas, threads, smem;
-    if (!g_bf16 && !a_bf16 && wg_strip_shape(g, ex.ctx->sm_count, most, st, ctas, threads, smem)) {
+    if (g.k == 3 && g.s == 1 && !g_bf16 && !a_bf16 && wg_strip_shape(g.N, g.H, g.W, g.Ci, g.Co, ex.ctx->sm_count, most, st, ctas, threads, smem)) {
         size_t m = ex.ws.mark();
         float *part = ctas > 1 ? ex.ws.get<float>((size_t)ctas * Co * KC) : dW;
         if (!ex.dry) {

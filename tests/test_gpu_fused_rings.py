@@ -20,11 +20,19 @@ def ctx():
     c.close()
 
 
+# Basic blocks whose inner data gradient takes its input through the BN backward of the layer behind, or does not (tests/test_fused_shapes_host.py)
+FOLDS = [
+    (37, 15, 21, 24, True),               # one tile per CTA
+    (3, 5, 110, 16, True),                # the largest halo: six rows per build thread, and
+    (3, 5, 111, 16, False),               # one size on
+]
+
+
 @pytest.mark.parametrize("kind,N,H,W,c,w", [
     ("basic", 1, 1, 1, 8, 0),             # one pixel; one piece
-    ("basic", 37, 15, 21, 24, 0),         # one tile per CTA: the inner data gradient goes through the BN backward itself
-    ("basic", 3, 5, 78, 16, 0),           # the largest halo for which it does (six rows per build thread), and
-    ("basic", 3, 5, 79, 16, 0),           # one size on, where it does not
+    ("basic", 3, 5, 110, 16, 0),          # (see FOLDS)
+    ("basic", 3, 5, 111, 16, 0),
+    ("basic", 37, 15, 21, 24, 0),
     ("basic", 150, 33, 31, 16, 0),        # nine tiles per CTA: the range as one segment, the partner ring goes round
     ("basic", 64, 32, 32, 64, 0),         # four tiles per CTA as one segment, two pieces of the input in flight
     ("basic", 3, 40, 150, 48, 0),         # long rows: a halo of 152 rows, six planes
@@ -70,13 +78,20 @@ def test_segments_in_turn_give_the_same_bits_every_time(ctx, N, H, W, c):
         assert all(np.array_equal(out[k], first[k]) for k in first)
 
 
-@pytest.mark.parametrize("kind,N,H,W,c", [
-    ("basic", 2, 9, 5, 12),               # nine pairs of quads: three row slices of a warp, five idle lanes; rows of 3 + 2 pixels
-    ("basic", 3, 1, 7, 4),                # one row: one slice
-    ("basic", 150, 17, 16, 16),           # several strips per CTA, the last strip of an image one row
-    ("basic", 5, 6, 9, 44),               # 121 pairs in four blocks, the last of 25
-    ("basic", 2, 3, 31, 48),              # the most pairs that it takes: five blocks, 15 warps
-    ("basic", 2, 3, 31, 52),              # one quad more: the implicit GEMM
-])
-def test_strict_weight_gradient_strips(ctx, kind, N, H, W, c):
+# Strict weight gradients; the last value: in strips (held against the launch geometry by tests/test_strip_shapes_host.py), or by the implicit GEMM
+STRIPS = [
+    ("basic", 2, 9, 5, 12, False),        # a few pixels: the GEMM
+    ("basic", 300, 9, 5, 12, True),       # nine pairs of quads: three row slices of a warp, five idle lanes; rows of 3 + 2 pixels
+    ("basic", 700, 1, 7, 4, True),        # one row: one slice
+    ("basic", 150, 17, 16, 16, True),     # strips of a whole image, the last round of slices one row
+    ("single", 250, 26, 9, 44, True),     # 121 pairs in four blocks, the last of 25
+    ("single", 20, 60, 61, 48, True),     # the most pairs that it takes: five blocks, 15 warps; rows of two runs of products
+    ("single", 20, 60, 61, 52, False),    # one quad more: the implicit GEMM
+    ("single", 40, 31, 70, 8, True),      # three runs per row, the last of four pixels
+    ("single", 1, 275, 275, 16, False),   # rows too long for a warp's slices in two buffers
+]
+
+
+@pytest.mark.parametrize("kind,N,H,W,c,strips", STRIPS)
+def test_strict_weight_gradient_strips(ctx, kind, N, H, W, c, strips):
     tp.run_block_case(ctx, syn.BlockCfg(N, H, W, c, 0, kind, seed=800 + c), 1, jitter=True, inplace=True)

@@ -25,7 +25,7 @@ def ctx():
 
 @pytest.mark.parametrize("kind,N,H,W,c,w", [
     ("basic", 2, 3, 3, 8, 0),             # one operand plane, less than one tile
-    ("basic", 2, 281, 283, 8, 0),         # rows longer than a tile; more tiles per CTA than one operand segment holds
+    ("basic", 2, 281, 283, 8, 0),         # rows longer than a tile; nine tiles per CTA, one operand segment
     ("basic", 3, 2, 200, 24, 0),          # three planes, two-row images
     ("basic", 6, 9, 11, 40, 0),           # five planes
     ("basic", 4, 13, 13, 56, 0),          # seven planes, 56 of 64 output columns
@@ -47,8 +47,8 @@ def test_bf16_blocks_at_tile_edges(ctx, kind, N, H, W, c, w):
 @pytest.mark.parametrize("kind,N,H,W,c,w", [
     ("basic", 1, 5, 13, 4, 0),            # direct 3x3: one tile, half of it inside the image, outputs 4 of 16; 65 pixels in the weight gradient
     ("basic", 1, 275, 275, 16, 0),        # direct 3x3: 16-row tiles, the last one of 3 rows
-    ("basic", 1, 150, 253, 20, 0),        # direct 3x3: 20 of 32 outputs; weight gradient in 32-column tiles
-    ("basic", 1, 139, 137, 36, 0),        # direct 3x3: two groups of outputs, the second of 4; weight gradient in 64-column tiles
+    ("basic", 1, 150, 253, 20, 0),        # direct 3x3: 20 of 32 outputs; weight gradient by the GEMM, in 32-column tiles (rows too long for strips)
+    ("basic", 1, 139, 137, 36, 0),        # direct 3x3: two groups of outputs, the second of 4; weight gradient of the first layer by the GEMM, in 64-column tiles
     ("basic", 2, 11, 7, 68, 0),           # two column tiles, the second of 4 columns
     ("basic", 16, 5, 4, 8, 0),            # direct 3x3: eight images per tile, one column of warps
     ("basic", 5, 7, 6, 20, 0),            # two images per tile, the last one of a tile missing
