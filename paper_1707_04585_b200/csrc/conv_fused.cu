@@ -763,10 +763,7 @@ bool conv_dgrad_fused_takes(Exec &ex, Geom gi, const Layer &L, bool behind, int 
     const FusedShape *s = L.stride == 1 ? shape_of(gi, L.cout, L.cin, L.k, ex.ctx->sm_count, behind ? kInBwd : kInBf16, true) : nullptr;
     if (!s || !(ex.dry || tc_encoder(ex.ctx))) return false;
     *parts = s->ctas;
-    // Through the BN backward only where a build thread has few rows: its pass costs 0.3 us per row and thread, twice that of a bf16 input with
-    // twice the threads per row, against 5 us for the launch that it saves.  Odd-sized block (24 channels, a tile per CTA, five and a half rows)
-    // 151 -> 144.5 us; 56 channels at 8x8 (eleven rows) and 16 at 32x32 (twenty-one): 38-layer step 1665 -> 1686.
-    return !behind || (long long)(s->g.chunk + 2 * s->g.halo) * s->g.nit <= 6 * 192;
+    return !behind || fused_folds(*s);
 }
 
 // The same where the gradient still has to go through the BN + ReLU backward of the layer behind L: g is da of that layer (float), `behind` its

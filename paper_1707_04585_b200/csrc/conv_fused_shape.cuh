@@ -174,3 +174,9 @@ static inline bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count,
         if (g.BN < 32) { if (tight) return false; tight = true; }
     }
 }
+
+// Whether a data gradient takes its input through the BN backward of the layer behind (s: its shape as kInBwd).
+// Only where a build thread has few rows: its pass costs 0.3 us per row and thread, twice that of a bf16 input with
+// twice the threads per row, against 5 us for the launch that it saves.  Odd-sized block (24 channels, a tile per CTA, five and a half rows)
+// 151 -> 144.5 us; 56 channels at 8x8 (eleven rows) and 16 at 32x32 (twenty-one): 38-layer step 1665 -> 1686.
+static inline bool fused_folds(const FusedShape &s) { return (long long)(s.g.chunk + 2 * s.g.halo) * s.g.nit <= 6 * 192; }

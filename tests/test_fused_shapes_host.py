@@ -35,7 +35,7 @@ int main(int argc, char **) {
         while (scanf("%d %d %d %d %d %d %d", &N, &H, &W, &ci, &co, &k, &mode) == 7) {
             FusedShape s;
             if (!fused_shape(Geom{N, H, W}, ci, co, k, 148, mode, true, s)) { printf("0 0 0\n"); continue; }
-            printf("%d %d %d\n", tiles_of(s.g), s.g.S, s.g.nseg);
+            printf("%d %d %d\n", tiles_of(s.g), s.g.S, mode == kInBwd ? (int)fused_folds(s) : s.g.nseg);
         }
         return 0;
     }
@@ -80,3 +80,9 @@ def test_segmented_cases_have_the_segments_that_they_claim(program, kind, N, H, 
     out = subprocess.run([program, "-"], input=shapes, capture_output=True, text=True, check=True).stdout.split()
     for tiles, S, nseg in (map(int, out[i:i + 3]) for i in (0, 3)):
         assert nseg == buffers and -(-tiles // S) == segments
+
+
+def test_fold_cases_fold_or_not_as_they_claim(program):
+    shapes = "".join(f"{N} {H} {W} {c} {c} 3 3\n" for N, H, W, c, _ in rings.FOLDS)
+    out = subprocess.run([program, "-"], input=shapes, capture_output=True, text=True, check=True).stdout.split()
+    assert [int(v) for v in out[2::3]] == [int(folds) for *_, folds in rings.FOLDS]
