@@ -409,8 +409,8 @@ __device__ __forceinline__ void column_sums(float (&a)[NC], int lane) {
     a[0] += __shfl_xor_sync(0xffffffffu, a[0], 16);
 }
 
-// Registers: with eight epilogue warps 96 for 512 or 640 threads; of 512 (the bound asks for it) that leaves an SM room for a CTA of the
-// weight gradients (72 for 192 threads) that run on another stream.
+// Registers: with eight epilogue warps 96, for 512 or 640 threads (80, for a bound of 672 threads, spill: 38-layer step 12 % slower).  No CTA of
+// another stream shares the SM, the rings take what shared memory there is: weight gradients run on the SMs that a layer leaves empty.
 template <int EW, int NBT>
 __global__ void __launch_bounds__(EW == 8 ? 640 : fused_threads(EW, NBT), 1) conv_fused_kernel(const __grid_constant__ FusedArgs A) {
     extern __shared__ uint8_t smem_raw[];

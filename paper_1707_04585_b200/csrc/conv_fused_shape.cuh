@@ -90,8 +90,9 @@ static inline bool fused_shape(Geom geo, int cin, int cout, int k, int sm_count,
         g.nacc = g.BN == 64 ? 2 : 4; g.acc_shift = g.BN == 64 ? 1 : 2;
         int ctas = sm_count / s.n_tiles; if (ctas < 1) ctas = 1;
         // A contiguous range of positions per CTA, a tile at least.  (Half tiles would put a small layer on every SM, but take as long and
-        // leave none to the launches beside it: 110-layer step 4964 -> 4877 us, odd-sized basic block 167 -> 164 with whole ones.)  A layer
-        // of so few tiles that half ones leave half of the SMs takes those: 64 channels, 10 images of 22x8, forward 20.6 -> 19.2 us.
+        // leave none to the launches of other streams beside it: 38-layer step 1680 -> 1635 us, 110-layer 4542 -> 4429, odd-sized basic block 153 -> 143
+        // with whole ones.)  A layer of so few tiles that half ones leave half of the SMs takes those: 24 channels, 8 images of 9x17, block forward
+        // 32.5 -> 31.2 us.
         const int least_chunk = tiles * 4 * s.n_tiles <= sm_count ? 64 : 128;
         g.chunk = round_up((g.total + ctas - 1) / ctas, 8); if (g.chunk < least_chunk) g.chunk = least_chunk;
         s.ctas = (g.total + g.chunk - 1) / g.chunk;
